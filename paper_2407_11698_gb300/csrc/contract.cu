@@ -15,7 +15,7 @@ struct nitro_conv {
     LayerGeom g{};
     TcLayer t;
     int max_batch = 0;
-    uint32_t* words = nullptr;   // [0] max|W| [1] max|delta| [2] status
+    uint32_t* words = nullptr;   // [0] max|W| [1] max|delta| [2] status [4, 5] tc_maxabs scratch
     std::vector<void*> allocs;
     std::vector<void*> host_allocs;
 };
@@ -24,7 +24,7 @@ struct nitro_gemm {
     int max_m = 0, max_n = 0, max_k = 0;
     uint16_t* a = nullptr;       // bf16 [M][K]
     uint16_t* b = nullptr;       // bf16 limb planes [4][N][K]
-    uint32_t* words = nullptr;   // [0] max|B| [1] status
+    uint32_t* words = nullptr;   // [0] max|B| [1] status [2, 3] tc_maxabs scratch
     std::vector<void*> allocs;
 };
 
@@ -76,10 +76,10 @@ nitro_status nitro_conv3x3_create(int max_batch, int h, int w, int cin, int cout
     if (!c) return NITRO_ERR_CUDA;
     c->g = LayerGeom{NITRO_CONV3X3, cin, cout, h, w, 0, h, w};
     c->max_batch = max_batch;
-    bool ok = dalloc(c->allocs, &c->words, 4) &&
+    bool ok = dalloc(c->allocs, &c->words, 6) &&
               tc_layer_init(c->t, c->g, max_batch, true, c->words, c->words + 1, c->allocs,
                             c->host_allocs);
-    if (ok) ok = cudaMemset(c->words, 0, 16) == cudaSuccess;
+    if (ok) ok = cudaMemset(c->words, 0, 24) == cudaSuccess;
     if (!ok) {
         free_all(c->allocs);
         free_host(c->host_allocs);
@@ -107,7 +107,7 @@ nitro_status nitro_conv3x3_contract(nitro_conv* c, int mode, const void* x, cons
     bool done = false, fused = false;
     if (mode == NITRO_CONTRACT_FWD) {
         const int8_t* a = static_cast<const int8_t*>(x);
-        TRY(tc_maxabs(y, (int64_t)g.cout * 9 * g.cin, c->words, s));
+        TRY(tc_maxabs(y, (int64_t)g.cout * 9 * g.cin, c->words, c->words + 4, s));
         TRY(tc_refresh_weights(c->t, g, y, c->words, s));
         TRY(tc_pack_input(c->t, g, a, batch, false, s));
         TRY(tc_conv_forward(c->t, g, batch, out, nullptr, status, s, &done, &fused));
@@ -115,14 +115,14 @@ nitro_status nitro_conv3x3_contract(nitro_conv* c, int mode, const void* x, cons
     } else if (mode == NITRO_CONTRACT_WGRAD) {
         const int8_t* a = static_cast<const int8_t*>(x);
         TRY(tc_pack_input(c->t, g, a, batch, false, s));
-        TRY(tc_maxabs(y, (int64_t)batch * g.h * g.w * g.cout, c->words + 1, s));
+        TRY(tc_maxabs(y, (int64_t)batch * g.h * g.w * g.cout, c->words + 1, c->words + 4, s));
         TRY(tc_conv_wgrad(c->t, g, y, c->words + 1, batch, out, status, s, &done));
         if (!done) TRY(simt_gemm(GM_CONV_WGRAD, a, y, nullptr, out, batch, g.h, g.w, g.cin, g.cout, s));
     } else {
         const int32_t* d = static_cast<const int32_t*>(x);
-        TRY(tc_maxabs(y, (int64_t)g.cout * 9 * g.cin, c->words, s));
+        TRY(tc_maxabs(y, (int64_t)g.cout * 9 * g.cin, c->words, c->words + 4, s));
         TRY(tc_refresh_weights(c->t, g, y, c->words, s));
-        TRY(tc_maxabs(d, (int64_t)batch * g.h * g.w * g.cout, c->words + 1, s));
+        TRY(tc_maxabs(d, (int64_t)batch * g.h * g.w * g.cout, c->words + 1, c->words + 4, s));
         TRY(tc_pack_delta(c->t, g, d, c->words + 1, batch, s));
         TRY(tc_conv_dgrad(c->t, g, batch, out, nullptr, status, s, &done, &fused));
         if (!done) TRY(simt_gemm(GM_CONV_DGRAD, nullptr, d, y, out, batch, g.h, g.w, g.cin, g.cout, s));
@@ -161,8 +161,8 @@ nitro_status nitro_gemm_create(int max_m, int max_n, int max_k, nitro_gemm** out
     g->max_k = max_k;
     bool ok = dalloc(g->allocs, &g->a, (size_t)max_m * max_k) &&
               dalloc(g->allocs, &g->b, (size_t)kMaxLimbs * max_n * max_k) &&
-              dalloc(g->allocs, &g->words, 2);
-    if (ok) ok = cudaMemset(g->words, 0, 8) == cudaSuccess;
+              dalloc(g->allocs, &g->words, 4);
+    if (ok) ok = cudaMemset(g->words, 0, 16) == cudaSuccess;
     if (!ok) {
         free_all(g->allocs);
         delete g;
@@ -188,8 +188,8 @@ nitro_status nitro_gemm_run(nitro_gemm* g, const int8_t* a, const int32_t* b, in
         TRY(simt_gemm(GM_LIN_FWD, a, nullptr, b, c, m, 1, 1, k, n, s));
         return NITRO_OK;
     }
-    TRY(tc_pack_int8(a, m, k, g->a, s));
-    TRY(tc_maxabs(b, (int64_t)n * k, g->words, s));
+    TRY(tc_pack_int8(a, m, k, g->a, s, tc_gemm_adds(m, n, k) ? c : nullptr, (int64_t)m * n));
+    TRY(tc_maxabs(b, (int64_t)n * k, g->words, g->words + 2, s));
     TRY(tc_pack_limbs(b, (int64_t)n * k, g->words, g->b, s));
     TRY(tc_gemm_run(g->a, g->b, m, n, k, g->words, c, g->words + 1, s));
     return NITRO_OK;

@@ -79,6 +79,8 @@ uint32_t* w_gl(nitro_block* b) { return b->words + 3 + (int)b->L.size(); }
 uint32_t* w_delta(nitro_block* b, int i) { return b->words + 4 + (int)b->L.size() + i; }
 int sse_word(int n_layers) { return (4 + 2 * n_layers + 1) & ~1; }   // 8-byte aligned
 int n_words(int n_layers) { return sse_word(n_layers) + 2; }
+// behind them, IntegerSGD's scratch (zero between launches)
+uint32_t* w_sgd(nitro_block* b) { return b->words + n_words((int)b->L.size()); }
 
 template <typename T>
 bool dalloc(nitro_block* b, T** p, size_t count) {
@@ -275,7 +277,7 @@ nitro_status nitro_init_block(const nitro_block_desc* desc, uint64_t seed, void*
     }
     ok = ok && dalloc(b, &b->Wlr, (size_t)b->G * b->d) && dalloc(b, &b->dWlr, (size_t)b->G * b->d) &&
          dalloc(b, &b->grad_l, (size_t)MB * b->G) && dalloc(b, &b->zsum, simt_learn_scratch(MB, (int)b->d, b->G)) && dalloc(b, &b->z64, z_need) &&
-         dalloc(b, &b->words, n_words(desc->n_layers));
+         dalloc(b, &b->words, n_words(desc->n_layers) + kSgdScratchWords);
     if (ok) {
         b->sse = reinterpret_cast<unsigned long long*>(b->words + sse_word(desc->n_layers));
         void* h = nullptr;
@@ -302,7 +304,7 @@ nitro_status nitro_init_block(const nitro_block_desc* desc, uint64_t seed, void*
         return NITRO_ERR_CUDA;
     }
     std::vector<int32_t> wlr = draw_weights((int64_t)b->G * b->d, b->d, seed, kLearningTensorId);
-    std::vector<uint32_t> words(n_words(desc->n_layers), 0);
+    std::vector<uint32_t> words(n_words(desc->n_layers) + kSgdScratchWords, 0);
     words[2] = host_maxabs(wlr.data(), wlr.size());
     cudaError_t e = cudaSuccess;
     for (int i = 0; i < desc->n_layers && e == cudaSuccess; ++i) {
@@ -322,7 +324,7 @@ nitro_status nitro_init_block(const nitro_block_desc* desc, uint64_t seed, void*
             e = tc_pack_limbs(b->L[i].W, b->L[i].wcount, w_w(b, i), b->L[i].lin_planes, s);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess) std::memcpy(b->words_host, words.data(), words.size() * 4);
+    if (e == cudaSuccess) std::memcpy(b->words_host, words.data(), 4 * (size_t)n_words(desc->n_layers));
     if (e != cudaSuccess) {
         free_all(b);
         delete b;
@@ -366,7 +368,9 @@ nitro_status nitro_block_forward(nitro_block* b, const int8_t* a_in, int batch, 
         NITRO_TRY(tc_conv_forward(ly.tc, g, batch, b->z64, &fo, w_status(b), s, &done, &fused));
         if (ly.lin_planes) {
             // linear: z = a W^T on the tcgen05 GEMM (weight planes kept by IntegerSGD)
-            NITRO_TRY(tc_pack_int8(x, batch, g.cin, ly.lin_a, s));
+            const bool adds = tc_gemm_adds(batch, g.cout, g.cin);
+            NITRO_TRY(tc_pack_int8(x, batch, g.cin, ly.lin_a, s, adds ? b->z64 : nullptr,
+                                   (int64_t)batch * g.cout));
             NITRO_TRY(tc_gemm_run(ly.lin_a, ly.lin_planes, batch, g.cout, g.cin, w_w(b, i), b->z64,
                                   w_status(b), s));
             done = true;
@@ -414,9 +418,9 @@ nitro_status block_backward(nitro_block* b, const int8_t* a_in, const int32_t* l
     const int n = (int)b->L.size();
     const int G = b->G;
     const int64_t d = b->d;
-    // reset the per-step range words and the SSE (one contiguous range)
-    NITRO_TRY(cudaMemsetAsync(w_gl(b), 0, 4 * (size_t)(n_words(n) - (3 + n)), s));
     if (batch == 0) {
+        // the per-step range words and the SSE (one contiguous range)
+        NITRO_TRY(cudaMemsetAsync(w_gl(b), 0, 4 * (size_t)(n_words(n) - (3 + n)), s));
         NITRO_TRY(cudaMemsetAsync(b->dWlr, 0, (size_t)G * d * 8, s));
         for (int i = 0; i < n; ++i) NITRO_TRY(cudaMemsetAsync(b->L[i].dW, 0, (size_t)b->L[i].wcount * 8, s));
         if (loss_dev) NITRO_TRY(cudaMemsetAsync(loss_dev, 0, 8, s));
@@ -430,8 +434,10 @@ nitro_status block_backward(nitro_block* b, const int8_t* a_in, const int32_t* l
                                    b->lp.ph, b->lp.pw, b->zmp, b->lr_am, s));
         a_last = b->zmp;
     }
+    // also resets the max |delta| words and dW_lr for the kernels below
     NITRO_TRY(simt_learn_fwd(a_last, b->Wlr, labels, batch, (int)d, G, b->zsum, b->grad_l, b->sse,
-                             loss_dev, w_gl(b), w_status(b), s));
+                             loss_dev, w_gl(b), w_status(b), w_gl(b) + 1, n,
+                             simt_lr_backward_ok(G) ? b->dWlr : nullptr, s));
     if (b->zmp) {
         // learning-weight gradient from z^mp, then delta_fw back through the
         // learning pool into the last layer's delta (pre-update W_lr)
@@ -577,17 +583,16 @@ nitro_status block_sgd(nitro_block* b, void* stream, const std::vector<char>* sk
             st.row_k = 9 * b->L[i].g.cin;
             st.tap_k = b->L[i].g.cin;
         }
-        if (skip) NITRO_TRY(cudaMemsetAsync(w_w(b, i), 0, 4, s));
         bt.t[bt.count++] = st;
     }
     bt.t[bt.count++] = SgdTensor{b->Wlr, b->dWlr, (int64_t)b->G * b->d, b->desc.gamma_inv_lr,
                                  b->desc.eta_inv_lr, w_wlr(b), {}, {}, nullptr, 0, 0, 0, 0, {}};
-    // max |W_lr| and every updated layer's max |W| start from zero: one range
-    // unless some layers were updated in their weight-gradient kernels
-    NITRO_TRY(cudaMemsetAsync(w_wlr(b), 0, 4 * (size_t)(skip ? 1 : 1 + n), s));
+    // the launch's last CTA also refreshes the kernel-variant hints of the next step
+    bt.scratch = w_sgd(b);
+    bt.words = b->words;
+    bt.host_words = b->words_host;
+    bt.n_words = n_words(n);
     NITRO_TRY(simt_integersgd(bt, s));
-    // the kernel-variant hints of the next step: one copy of all the words
-    NITRO_TRY(cudaMemcpyAsync(b->words_host, b->words, 4 * (size_t)n_words(n), cudaMemcpyDeviceToHost, s));
     return NITRO_OK;
 }
 

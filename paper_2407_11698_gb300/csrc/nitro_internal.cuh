@@ -225,12 +225,16 @@ cudaError_t simt_lrpool_to_delta(const int32_t* gl, const int32_t* wlr, int G, i
 // Learning layer forward + loss: grad_l = floor(a W^T / (256 d)) - 32 onehot,
 // sse = sum grad_l^2 (mod 2^64), loss = floor(sse / 2) (if loss != NULL),
 // max|grad_l| into *maxabs_gl, status bits.  scratch: int64 buffer of
-// simt_learn_scratch(max_batch, d, G) words (partial sums and tickets,
-// cleared by each call); *sse must be zero on entry.
+// simt_learn_scratch(max_batch, d, G) words (partial sums, tickets, SSE and
+// maximum), zero before the first call and left zero by every call.
+// The launch also clears what the rest of the backward accumulates into, which
+// saves a memset each: zero_words[0..n_zero) and, when zero_dwlr is not null,
+// the G d values of dW_lr.
 size_t simt_learn_scratch(int max_batch, int d, int G);
 cudaError_t simt_learn_fwd(const int8_t* a, const int32_t* wlr, const int32_t* labels, int B,
                            int d, int G, int64_t* scratch, int32_t* grad_l, unsigned long long* sse,
-                           int64_t* loss, uint32_t* maxabs_gl, uint32_t* status, cudaStream_t s);
+                           int64_t* loss, uint32_t* maxabs_gl, uint32_t* status,
+                           uint32_t* zero_words, int n_zero, int64_t* zero_dwlr, cudaStream_t s);
 
 // dW_lr[g][j] = sum_b grad_l[b][g] a[b][j]
 cudaError_t simt_learn_dw(const int8_t* a, const int32_t* grad_l, int B, int d, int G,
@@ -262,7 +266,8 @@ cudaError_t simt_conv_small_fwd(const int8_t* x, const int32_t* w, const LayerGe
 cudaError_t simt_conv_small_wgrad(const int8_t* x, const int32_t* d, const LayerGeom& g, int B,
                                   int64_t* dw, cudaStream_t s);
 
-// Learning-layer backward for G <= 16, fused: dW_lr (overwritten) and, when
+// Learning-layer backward for G <= 16, fused: dW_lr (added to; zero on entry,
+// see simt_learn_fwd) and, when
 // lg (geometry of the block's last forward layer) is not null, that layer's
 // delta from delta_fw = grad_L W_lr (pre-update), with the int32 storage
 // rule, the int64 bound check, max-pool and NITRO-ReLU backward.  d: features
@@ -297,7 +302,17 @@ struct SgdBatch {
     int round_trunc;
     uint32_t* status;
     uint32_t* step;        // block step counter, incremented once per launch (or null)
+    // kMaxSgdTensors maxima and a CTA ticket, zero before the first launch and
+    // left zero by every launch: the last CTA stores the finished maxima into
+    // each tensor's maxabs_w and copies words[0..n_words) to host_words (pinned
+    // host memory; null: no copy)
+    uint32_t* scratch;
+    const uint32_t* words;
+    uint32_t* host_words;
+    int n_words;
+    int first[kMaxSgdTensors + 1];   // first CTA of each tensor (filled by simt_integersgd)
 };
+constexpr int kSgdScratchWords = kMaxSgdTensors + 1;
 cudaError_t simt_integersgd(const SgdBatch& b, cudaStream_t s);
 
 

@@ -1042,10 +1042,25 @@ __device__ __forceinline__ uint16_t bf16_bits(int v) {
     return __bfloat16_as_ushort(__float2bfloat16_rn((float)v));   // exact for |v| <= 256
 }
 
+// Clears n int64 values: the pack kernels do it for the contraction that runs
+// after them and adds K-split partial sums, instead of a memset between the two.
+__device__ __forceinline__ void zero_fill(int64_t* z, int64_t n) {
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    if (!z) return;
+    if (((uintptr_t)z & 15) == 0 && (n & 1) == 0) {
+        for (int64_t i = tid; i < n / 2; i += stride)
+            reinterpret_cast<uint4*>(z)[i] = make_uint4(0, 0, 0, 0);
+    } else {
+        for (int64_t i = tid; i < n; i += stride) z[i] = 0;
+    }
+}
+
 // int8 NHWC [P][C] -> bf16 NHWC [P][Cp] copy, zero in channels C..Cp-1
 __global__ void k_pack_act_nhwc(const int8_t* __restrict__ x, int64_t P, int C, int Cp,
-                                uint16_t* __restrict__ out) {
+                                uint16_t* __restrict__ out, int64_t* zero, int64_t n_zero) {
     pdl_wait();
+    zero_fill(zero, n_zero);
     const int64_t n = P * Cp;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -1133,8 +1148,10 @@ __global__ void k_pack_act_nhwc8(const int8_t* __restrict__ x, int64_t n8,
 // input is read as 16-byte words when `d` is 16-byte aligned (vec != 0).
 __global__ void __launch_bounds__(256) k_pack_delta_nhwc(const int32_t* __restrict__ d, int64_t n,
                                                          int vec, const uint32_t* maxabs,
-                                                         uint16_t* __restrict__ out) {
+                                                         uint16_t* __restrict__ out, int64_t* zero,
+                                                         int64_t n_zero) {
     pdl_wait();
+    zero_fill(zero, n_zero);
     const int L = limb_count(*maxabs);
     const int64_t n8 = n / 8;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n8;
@@ -1486,7 +1503,8 @@ cudaError_t tc_pack_input(TcLayer& t, const LayerGeom& g, const int8_t* x, int b
         launch_k(k_pack_act_nhwc8, grid1d(P * g.cin / 8), 256, 0, s, x, P * g.cin / 8, t.act_nhwc);
         return cudaGetLastError();
     }
-    launch_k(k_pack_act_nhwc, grid1d(P * t.cin8), 256, 0, s, x, P, g.cin, t.cin8, t.act_nhwc);
+    launch_k(k_pack_act_nhwc, grid1d(P * t.cin8), 256, 0, s, x, P, g.cin, t.cin8, t.act_nhwc,
+             (int64_t*)nullptr, (int64_t)0);
     return cudaGetLastError();
 }
 
@@ -1554,7 +1572,7 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
 
 cudaError_t tc_pack_delta(TcLayer& t, const LayerGeom& g, const int32_t* delta,
                           const uint32_t* maxabs_delta, int batch, cudaStream_t s,
-                          bool planes_done) {
+                          bool planes_done, int64_t* zero, int64_t n_zero) {
     if (batch <= 0 || (!t.wgrad && !t.dgrad)) return cudaSuccess;
     // limb planes of delta (NHWC, read by the wgrad and dgrad passes), unless
     // an earlier call split this delta already
@@ -1562,7 +1580,9 @@ cudaError_t tc_pack_delta(TcLayer& t, const LayerGeom& g, const int32_t* delta,
     if (!planes_done) {
         ProfScope ps(K_TC_PACK_D, s, 0.0, (double)n * 4 * 2);
         launch_k(k_pack_delta_nhwc, grid1d(n / 8), 256, 0, s, delta, n, ((uintptr_t)delta & 15) == 0,
-                                                       maxabs_delta, t.d_nhwc);
+                                                       maxabs_delta, t.d_nhwc, zero, n_zero);
+    } else if (zero) {
+        return cudaMemsetAsync(zero, 0, sizeof(int64_t) * (size_t)n_zero, s);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !t.own_hints) return e;
@@ -1576,9 +1596,7 @@ cudaError_t tc_conv_wgrad(TcLayer& t, const LayerGeom& g, const int32_t* delta,
     *done = false;
     if (sgd_done) *sgd_done = false;
     if (batch <= 0 || (!t.wgrad && !t.dgrad)) return cudaSuccess;
-    cudaError_t pe = tc_pack_delta(t, g, delta, maxabs_delta, batch, s, planes_done);
-    if (pe != cudaSuccess) return pe;
-    if (!t.wgrad) return cudaSuccess;
+    if (!t.wgrad) return tc_pack_delta(t, g, delta, maxabs_delta, batch, s, planes_done);
     // A linear layer is one image of height 1 and width `batch` with a single
     // centred tap: rows = input features, K = the samples.
     const bool lin = g.kind == NITRO_LINEAR;
@@ -1609,6 +1627,10 @@ cudaError_t tc_conv_wgrad(TcLayer& t, const LayerGeom& g, const int32_t* delta,
     a.out = dW;
     a.status = status;
     a.atomic_out = splits > 1;
+    // the pack also clears dW for the partial sums of a K split
+    cudaError_t pe = tc_pack_delta(t, g, delta, maxabs_delta, batch, s, planes_done,
+                                   a.atomic_out ? dW : nullptr, a.cstride * g.cout);
+    if (pe != cudaSuccess) return pe;
     // The update is folded in only without a K split: the sums are then final
     // in the accumulators.  With a split, the warp that completes an output
     // slot would have to read its sums back and update after every other
@@ -1643,10 +1665,6 @@ cudaError_t tc_conv_wgrad(TcLayer& t, const LayerGeom& g, const int32_t* delta,
     const uint32_t bb[5] = {64, (uint32_t)a.wb, (uint32_t)a.hb, 1, (uint32_t)pb};
     if (!make_map(&ma, t.act_nhwc, 4, da, sa, ba) || !make_map(&mb, t.d_nhwc, 5, db, sb, bb))
         return cudaErrorInvalidValue;
-    if (a.atomic_out) {
-        cudaError_t e = cudaMemsetAsync(dW, 0, sizeof(int64_t) * (size_t)a.cstride * g.cout, s);
-        if (e != cudaSuccess) return e;
-    }
     const double ops = 2.0 * nimg * hw * g.cout * (double)a.cstride;
     ProfScope ps(lin ? K_TC_LIN_WGRAD : K_TC_CONV_WGRAD, s, ops, 0.0);
     cudaError_t e = launch_gemm_pb<TC_WGRAD>(n, pb, ma, mb, a, s);
@@ -1729,7 +1747,9 @@ cudaError_t tc_timeout_probe(uint32_t* status, uint64_t limit_ns, cudaStream_t s
 
 // ------------------------------------------------------------------ plain GEMM
 namespace {
-__global__ void k_maxabs(const int32_t* __restrict__ x, int64_t n, uint32_t* out) {
+// *out = max |x|: maximum and CTA ticket in scratch[0], scratch[1] (zero
+// between launches), so no memset of *out precedes the launch.
+__global__ void k_maxabs(const int32_t* __restrict__ x, int64_t n, uint32_t* out, uint32_t* scratch) {
     pdl_wait();
     uint32_t m = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -1737,22 +1757,31 @@ __global__ void k_maxabs(const int32_t* __restrict__ x, int64_t n, uint32_t* out
         m = max(m, abs_u32(x[i]));
 #pragma unroll
     for (int off = 16; off; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
+    if ((threadIdx.x & 31) == 0) {
+        if (m) atomicMax(&scratch[0], m);
+        __threadfence();     // this warp's maximum, before the CTA's ticket
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&scratch[1], 1u) == gridDim.x - 1) {
+        __threadfence();
+        *out = atomicExch(&scratch[0], 0u);
+        scratch[1] = 0;
+    }
 }
 }  // namespace
 
-cudaError_t tc_maxabs(const int32_t* x, int64_t n, uint32_t* out, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(out, 0, sizeof(uint32_t), s);
-    if (e != cudaSuccess || n <= 0) return e;
+cudaError_t tc_maxabs(const int32_t* x, int64_t n, uint32_t* out, uint32_t* scratch, cudaStream_t s) {
+    if (n <= 0) return cudaMemsetAsync(out, 0, sizeof(uint32_t), s);
     ProfScope ps(K_TC_PACK, s, 0.0, (double)n * 4);
-    launch_k(k_maxabs, grid1d(n), 256, 0, s, x, n, out);
+    launch_k(k_maxabs, grid1d(n), 256, 0, s, x, n, out, scratch);
     return cudaGetLastError();
 }
 
-cudaError_t tc_pack_int8(const int8_t* x, int64_t rows, int cols, uint16_t* out, cudaStream_t s) {
+cudaError_t tc_pack_int8(const int8_t* x, int64_t rows, int cols, uint16_t* out, cudaStream_t s,
+                         int64_t* zero, int64_t n_zero) {
     if (rows <= 0) return cudaSuccess;
     ProfScope ps(K_TC_PACK, s, 0.0, (double)rows * cols * 3);
-    launch_k(k_pack_act_nhwc, grid1d(rows * cols), 256, 0, s, x, rows, cols, cols, out);
+    launch_k(k_pack_act_nhwc, grid1d(rows * cols), 256, 0, s, x, rows, cols, cols, out, zero, n_zero);
     return cudaGetLastError();
 }
 
@@ -1760,8 +1789,29 @@ cudaError_t tc_pack_limbs(const int32_t* x, int64_t n, const uint32_t* maxabs, u
                           cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     ProfScope ps(K_TC_PACK, s, 0.0, (double)n * 4 * 2);
-    launch_k(k_pack_delta_nhwc, grid1d(n / 8), 256, 0, s, x, n, ((uintptr_t)x & 15) == 0, maxabs, planes);
+    launch_k(k_pack_delta_nhwc, grid1d(n / 8), 256, 0, s, x, n, ((uintptr_t)x & 15) == 0, maxabs, planes,
+             (int64_t*)nullptr, (int64_t)0);
     return cudaGetLastError();
+}
+
+namespace {
+// K split of the GEMM over CTAs: with few output tiles (a batch of 64 against a
+// linear layer) about one wave of CTAs, at least four K-blocks per split.
+int gemm_splits(int M, int N, int K, int* kb_per_split) {
+    const int n = pick_n(N);
+    const int tiles = (M + kBM - 1) / kBM * ((N + n - 1) / n);
+    const int kb_total = (K + kBK - 1) / kBK;
+    int splits = sm_count() / tiles;
+    const int max_splits = (kb_total + 3) / 4;
+    splits = splits < 1 ? 1 : (splits > max_splits ? max_splits : splits);
+    *kb_per_split = (kb_total + splits - 1) / splits;
+    return (kb_total + *kb_per_split - 1) / *kb_per_split;
+}
+}  // namespace
+
+bool tc_gemm_adds(int M, int N, int K) {
+    int kbs = 0;
+    return M > 0 && N > 0 && gemm_splits(M, N, K, &kbs) > 1;
 }
 
 cudaError_t tc_gemm_run(const uint16_t* a_bf16, const uint16_t* b_planes, int M, int N, int K,
@@ -1776,25 +1826,14 @@ cudaError_t tc_gemm_run(const uint16_t* a_bf16, const uint16_t* b_planes, int M,
     a.tiles_m = (M + kBM - 1) / kBM;
     a.tiles_n = (N + n - 1) / n;
     a.kb_total = (K + kBK - 1) / kBK;
-    // few output tiles (a batch of 64 against a linear layer): split K so that
-    // about one wave of CTAs runs, at least four K-blocks per split, partial
-    // sums added with 64-bit atomics into a zeroed C
-    const int tiles = a.tiles_m * a.tiles_n;
-    int splits = sm_count() / tiles;
-    const int max_splits = (a.kb_total + 3) / 4;
-    splits = splits < 1 ? 1 : (splits > max_splits ? max_splits : splits);
-    a.kb_per_split = (a.kb_total + splits - 1) / splits;
-    splits = (a.kb_total + a.kb_per_split - 1) / a.kb_per_split;
-    a.total_tiles = tiles * splits;
+    // a K split adds its partial sums with 64-bit atomics into a zeroed C
+    const int splits = gemm_splits(M, N, K, &a.kb_per_split);
+    a.total_tiles = a.tiles_m * a.tiles_n * splits;
     a.atomic_out = splits > 1;
     a.max_a = nullptr;
     a.max_b = max_b;
     a.out = out;
     a.status = status;
-    if (a.atomic_out) {
-        cudaError_t e = cudaMemsetAsync(out, 0, sizeof(int64_t) * (size_t)M * N, s);
-        if (e != cudaSuccess) return e;
-    }
     CUtensorMap ma, mb;
     const uint64_t da[2] = {(uint64_t)K, (uint64_t)M};
     const uint64_t sa[1] = {(uint64_t)K};

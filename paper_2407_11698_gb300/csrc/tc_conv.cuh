@@ -137,12 +137,12 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
 
 // Splits delta into NHWC limb planes for the wgrad and dgrad passes (limb
 // count from *maxabs_delta), unless planes_done (an earlier call split this
-// delta already); then refreshes the host hint of max |delta|.  Writing the
+// delta already), and clears zero[0..n_zero); then refreshes the host hint of max |delta|.  Writing the
 // planes from the kernels that produce delta instead (the dgrad epilogue,
 // the learning-layer backward) was measured slower than this pass.
 cudaError_t tc_pack_delta(TcLayer& t, const LayerGeom& g, const int32_t* delta,
                           const uint32_t* maxabs_delta, int batch, cudaStream_t s,
-                          bool planes_done = false);
+                          bool planes_done = false, int64_t* zero = nullptr, int64_t n_zero = 0);
 
 // tc_pack_delta, then, if wgrad runs on tcgen05, dW = sum_p delta (x)
 // im2col(a).  Must precede tc_conv_dgrad.
@@ -186,13 +186,18 @@ cudaError_t tc_conv_dgrad(TcLayer& t, const LayerGeom& g, int batch, int64_t* g6
 cudaError_t tc_timeout_probe(uint32_t* status, uint64_t limit_ns, cudaStream_t s);
 
 // Helpers of the kernel-level entry points (contract.cu).
-cudaError_t tc_maxabs(const int32_t* x, int64_t n, uint32_t* out, cudaStream_t s);
-cudaError_t tc_pack_int8(const int8_t* x, int64_t rows, int cols, uint16_t* out, cudaStream_t s);
+// (scratch: two words, zero before the first call and left zero)
+cudaError_t tc_maxabs(const int32_t* x, int64_t n, uint32_t* out, uint32_t* scratch, cudaStream_t s);
+// also clears zero[0..n_zero)
+cudaError_t tc_pack_int8(const int8_t* x, int64_t rows, int cols, uint16_t* out, cudaStream_t s,
+                         int64_t* zero = nullptr, int64_t n_zero = 0);
 // n % 8 == 0; planes [4][n], limb count from *maxabs
 cudaError_t tc_pack_limbs(const int32_t* x, int64_t n, const uint32_t* maxabs, uint16_t* planes,
                           cudaStream_t s);
 // C[m][n] (int64) = sum_k A[m][k] B[n][k]; A bf16 [M][K] (int8 values), B limb
-// planes [4][N][K] (limb count from *max_b); K % 8 == 0.
+// planes [4][N][K] (limb count from *max_b); K % 8 == 0.  Where tc_gemm_adds
+// says so, K is split and C must be zero before the call (tc_pack_int8 clears it).
+bool tc_gemm_adds(int M, int N, int K);
 cudaError_t tc_gemm_run(const uint16_t* a_bf16, const uint16_t* b_planes, int M, int N, int K,
                         const uint32_t* max_b, int64_t* out, uint32_t* status, cudaStream_t s);
 
