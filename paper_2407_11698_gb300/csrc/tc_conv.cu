@@ -4,8 +4,9 @@
 //
 // A persistent CTA computes 128 x N output tiles, each over a range of
 // K-blocks (64 elements each).  Warp 0 issues TMA loads into an S-stage shared-memory ring,
-// warp 1 allocates TMEM and issues the MMAs, warps 2..17 drain the fp32 TMEM
-// accumulator every <= 16 K-blocks into int64 registers (four warps per TMEM
+// warp 1 allocates TMEM and issues the MMAs, warps 4..19 drain the fp32 TMEM
+// accumulator every <= 16 K-blocks into int64 registers (the fused forward: into
+// z modulo 2^32 and an fp32 sum; four warps per TMEM
 // lane quadrant, each owning a quarter of the N columns).  Four TMEM accumulators
 // rotate so the MMAs run up to three chunks ahead of the drain.
 // Every wait on an mbarrier is bounded in time; on expiry the kernel raises
@@ -22,7 +23,9 @@
 namespace nitro {
 namespace {
 
-enum TcMode : int { TC_FWD = 0, TC_WGRAD = 1, TC_DGRAD = 2, TC_GEMM = 3 };
+// TC_FWD: forward with the fused NITRO-Scaling / NITRO-ReLU / max-pool epilogue;
+// TC_FWDZ: the same contraction with int64 sums as its output.
+enum TcMode : int { TC_FWD = 0, TC_WGRAD = 1, TC_DGRAD = 2, TC_GEMM = 3, TC_FWDZ = 4 };
 
 constexpr int kBM = 128;              // rows per tile (TMEM lanes)
 constexpr int kBK = 64;               // K elements per block (one 128-byte row)
@@ -40,6 +43,11 @@ constexpr int kEpiWarp0 = 4;          // first epilogue warp
 constexpr int kEpiWarps = 16;         // 4 per TMEM lane quadrant
 constexpr int kThreads = 32 * (kEpiWarp0 + kEpiWarps);
 constexpr int kRegsProducer = 32, kRegsEpilogue = 112;
+constexpr int kTabHalf = 256;         // half the fused forward's table of z*
+// K-blocks of a fused forward (Cin <= 896): with four weight limbs and eight chunks
+// its fp32 sums are off by less than 2^24 1.02 8 (8 + 4.2) = 1.67e9, so that the
+// remainder taken modulo 2^32 is exact
+constexpr int kFwdMaxBlocks = 128;
 constexpr uint64_t kWaitNs = 2000000000ull;   // 2 s bound on any wait
 
 // ------------------------------------------------------------------ PTX
@@ -237,11 +245,12 @@ struct TcArgs {
     uint32_t* status;
     int atomic_out;
     int out_vec;           // out is 16-byte aligned: pairs of int64 stored together
+    int fuse;              // input gradient: fused epilogue
     // forward with fused NITRO-Scaling / NITRO-ReLU / max-pool epilogue
-    int fuse;
     FloorDiv alpha;        // divide by alpha_inv
-    FloorDiv32 sf32;       // divide by 9 * Cin (after the shift by 8)
-    int64_t z_hi, z_lo;    // z >= 128 SF: piece 3; z < -127 SF: piece 0
+    int32_t sf;            // SF = 2^8 9 Cin
+    float sf_inv;          // 1 / SF
+    int out32;             // outputs and their rows are 32-byte aligned
     int mu, pool, oh, ow;
     int8_t* act;           // layer output (post-pool) int8 NHWC
     int8_t* out2;          // optional second copy of the output (caller's buffer)
@@ -275,15 +284,40 @@ struct TcArgs {
 __device__ __forceinline__ void st16(int8_t* dst, const uint32_t* w) {
     *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
 }
-// 16 int8 values (4 packed words) -> 16 bf16 values (two 16-byte stores),
-// through the 256-entry table of bf16 bits indexed by byte ^ 0x80
-__device__ __forceinline__ void st16_bf16(uint16_t* dst, const uint32_t* w, const uint16_t* tab) {
+// 32 int8 values (8 packed words): one 32-byte store (a whole sector) when the
+// destination is 32-byte aligned, else two of 16 bytes
+__device__ __forceinline__ void st32(int8_t* dst, const uint32_t* w, bool aligned32) {
+    if (aligned32) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]),
+                     "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                     : "memory");
+    } else {
+        st16(dst, w);
+        st16(dst + 16, w + 4);
+    }
+}
+// larger of each pair of signed 16-bit halves
+__device__ __forceinline__ uint32_t max_s16x2(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("max.s16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+// two int8 values v (bytes i, i + 1 of a word whose bytes hold v + 128) -> two bf16:
+// 2^23 + (v + 128) is the float 0x4B0000xx, and subtracting 2^23 + 128 leaves v
+// exactly, whose upper half is its bf16
+__device__ __forceinline__ uint32_t bf16x2(uint32_t biased, int i) {
+    const float f0 = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7540 + i)) - 8388736.0f;
+    const float f1 = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7541 + i)) - 8388736.0f;
+    return __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+}
+// 16 int8 values (4 packed words) -> 16 bf16 values (two 16-byte stores)
+__device__ __forceinline__ void st16_bf16(uint16_t* dst, const uint32_t* w) {
     uint32_t o[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const uint32_t lo = (w[k >> 1] >> (16 * (k & 1))) & 255u;
-        const uint32_t hi = (w[k >> 1] >> (16 * (k & 1) + 8)) & 255u;
-        o[k] = (uint32_t)tab[lo ^ 0x80u] | ((uint32_t)tab[hi ^ 0x80u] << 16);
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t u = w[k] ^ 0x80808080u;
+        o[2 * k] = bf16x2(u, 0);
+        o[2 * k + 1] = bf16x2(u, 2);
     }
     reinterpret_cast<uint4*>(dst)[0] = make_uint4(o[0], o[1], o[2], o[3]);
     reinterpret_cast<uint4*>(dst)[1] = make_uint4(o[4], o[5], o[6], o[7]);
@@ -301,7 +335,7 @@ struct TcCfg {
     // up to 14% in the kernel-level contractions (more TMA writes in flight
     // compete with the MMA's shared-memory reads)
     static constexpr int S = S_FIT > 6 ? 6 : S_FIT;
-    static constexpr int SMEM = 1024 + S * STAGE + 1024;
+    static constexpr int SMEM = 1024 + S * STAGE + 2048;   // alignment, ring, barriers and table
     static constexpr int NBUF = (512 / (PB * N)) > 4 ? 4 : (512 / (PB * N));   // accumulator sets
     static constexpr int TCOLS = NBUF * PB * N;                                  // 256 or 512
 };
@@ -332,6 +366,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     using C = TcCfg<N, PB>;
     constexpr int S = C::S;
     constexpr int NH = N / 4;            // columns per epilogue warp
+    constexpr bool kFwd = MODE == TC_FWD || MODE == TC_FWDZ;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -341,9 +376,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 2 * NBUF);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     int* hiskip_slot = reinterpret_cast<int*>(tmem_slot + 2);
-    int8_t* relu_tab = reinterpret_cast<int8_t*>(smem + S * C::STAGE + 256);   // 255 entries
-    // bf16 bits of every int8 value v, at index (v + 128) = byte ^ 0x80
-    uint16_t* bf16_tab = reinterpret_cast<uint16_t*>(smem + S * C::STAGE + 512);
+    // fused forward: NITRO-ReLU value (high byte) and piece (low byte) of every
+    // z* in [-kTabHalf, kTabHalf), at index z* + kTabHalf
+    uint16_t* relu_tab = reinterpret_cast<uint16_t*>(smem + S * C::STAGE + 256);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t bar0 = smem_u32(bars);
@@ -364,12 +399,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // NITRO-ReLU value of every z* in [-127, 127] (fused forward epilogue)
-    if (MODE == TC_FWD && args.fuse) {
-        for (int i = threadIdx.x; i < 255; i += kThreads)
-            relu_tab[i] = (int8_t)relu_value((int64_t)i - 127, args.alpha, args.mu);
-        for (int i = threadIdx.x; i < 256; i += kThreads)
-            bf16_tab[i] = __bfloat16_as_ushort(__float2bfloat16_rn((float)(i - 128)));
+    if (MODE == TC_FWD) {
+        for (int i = threadIdx.x; i < 2 * kTabHalf; i += kThreads) {
+            const int zs = i - kTabHalf;
+            relu_tab[i] = (uint16_t)((uint32_t)(uint8_t)relu_value((int64_t)zs, args.alpha, args.mu) << 8 |
+                                     (uint32_t)relu_region(zs));
+        }
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -451,9 +486,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     // forward / input gradient: K-block kb = (tap t, 64-channel block cb),
                     // cb fastest, walked incrementally
-                    const int knc = MODE == TC_FWD ? args.cin_k / kBK : (args.Cout + kBK - 1) / kBK;
+                    const int knc = kFwd ? args.cin_k / kBK : (args.Cout + kBK - 1) / kBK;
                     int kt = 0, kcb = 0;
-                    if (MODE == TC_FWD || MODE == TC_DGRAD) {
+                    if (kFwd || MODE == TC_DGRAD) {
                         kt = T.kb0 / knc;
                         kcb = T.kb0 - kt * knc;
                     }
@@ -471,7 +506,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                             tma_load_2d(a_dst, &tmA, fb, kb * kBK, T.mt * kBM);
                             for (int j = 0; j < nb; ++j)
                                 tma_load_3d(b_dst + j * C::B_BYTES, &tmB, fb, kb * kBK, n0, lb0 + j);
-                        } else if (MODE == TC_FWD) {
+                        } else if (kFwd) {
                             const int t = kt, cb = kcb;
                             const int tc = args.taps == 1 ? 4 : t;   // im2col rows: centre tap
                             const int ky = tc / 3, kx = tc - 3 * ky;
@@ -599,12 +634,32 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int q = warp & 3;                     // TMEM lane quadrant this warp may read
         const int half = (warp - kEpiWarp0) >> 2;   // which quarter of the N columns
         int chunk = 0;
+        // Fused forward: bound of the error of its fp32 sums.  A chunk of csz K-blocks
+        // has limb sums below csz 2^20 2^(8 limb).  Per chunk at most two roundings (of
+        // 2^-24) hit the running sum, which stays below c csz 2^20 2^(8 (LB - 1)) (1 +
+        // 2^-6) after c chunks, one hits a limb pair, and the product with 1 / SF adds
+        // 2^-23 of the sum: together csz / 16 2^(8 (LB - 1)) cpp (cpp + 1 + 1 + 2.01).
+        const int fcpp = (args.kb_total + kChunkBlocks - 1) / kChunkBlocks;
+        const int fcsz = fcpp ? (args.kb_total + fcpp - 1) / fcpp : 0;
+        const float err = (float)(1 << (8 * (LB - 1))) * 1.02f * (1.0f / 16.0f) * (float)fcsz *
+                          (float)fcpp * ((float)fcpp + 4.2f);
+        const bool tight = err <= 0.25f * (float)args.sf;
+        const float far = err + 400.0f * (float)args.sf;
         for (int tile = blockIdx.x; tile < args.total_tiles; tile += gridDim.x) {
             const Tile T = decode_tile(args, tile);
             const int cpp = (T.kb1 - T.kb0 + kChunkBlocks - 1) / kChunkBlocks;
-            uint64_t acc[NH];
+            uint64_t acc[MODE == TC_FWD ? 1 : NH];
+            uint32_t lo[MODE == TC_FWD ? NH : 1];   // fused forward: z modulo 2^32
+            float zf[MODE == TC_FWD ? NH : 1];      // and z rounded to fp32
 #pragma unroll
-            for (int i = 0; i < NH; ++i) acc[i] = 0;
+            for (int i = 0; i < NH; ++i) {
+                if constexpr (MODE == TC_FWD) {
+                    lo[i] = 0;
+                    zf[i] = 0.0f;
+                } else {
+                    acc[i] = 0;
+                }
+            }
             for (int la = 0; la < LA; ++la)
             for (int lb0 = 0; lb0 < lb_limit(la); lb0 += PB) {
                 const int nb = min(PB, lb_limit(la) - lb0);
@@ -644,7 +699,35 @@ __global__ void __launch_bounds__(kThreads, 1)
                     };
                     // 32 values per TMEM round trip: two loads issued back to
                     // back, then one wait (16 columns: two limbs at once)
-                    if (NH == 16) {
+                    if constexpr (MODE == TC_FWD) {
+#pragma unroll
+                        for (int j = 0; j < NH / 16; ++j)
+                            for (int jb = 0; jb < nb; jb += 2) {
+                                const bool two = jb + 1 < nb;
+                                const int m = 1 << (shift0 + 8 * jb);
+                                const float mf = (float)m;
+                                uint32_t r[32];
+                                tmem_ld16_nowait(limb_base(jb) + 16 * j, r);
+                                if (two) tmem_ld16_nowait(limb_base(jb + 1) + 16 * j, r + 16);
+                                tmem_wait_ld<32>(r);
+                                if (two) {
+#pragma unroll
+                                    for (int i = 0; i < 16; ++i) {
+                                        const float v0 = __uint_as_float(r[i]), v1 = __uint_as_float(r[16 + i]);
+                                        const uint32_t w = ((uint32_t)__float2int_rz(v1) << 8) + (uint32_t)__float2int_rz(v0);
+                                        lo[16 * j + i] += w * (uint32_t)m;
+                                        zf[16 * j + i] = fmaf(fmaf(v1, 256.0f, v0), mf, zf[16 * j + i]);
+                                    }
+                                } else {
+#pragma unroll
+                                    for (int i = 0; i < 16; ++i) {
+                                        const float v0 = __uint_as_float(r[i]);
+                                        lo[16 * j + i] += (uint32_t)__float2int_rz(v0) * (uint32_t)m;
+                                        zf[16 * j + i] = fmaf(v0, mf, zf[16 * j + i]);
+                                    }
+                                }
+                            }
+                    } else if constexpr (NH == 16) {
                         for (int jb = 0; jb < nb; jb += 2) {
                             uint32_t r[32];
                             tmem_ld16_nowait(limb_base(jb), r);
@@ -675,7 +758,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             {
                 const int r = 32 * q + lane;   // output row of this thread
                 const int col0 = T.nt * N + half * NH;
-                if (MODE == TC_GEMM) {
+                if constexpr (MODE == TC_GEMM) {
                     const int m = T.mt * kBM + r;      // C[m][n], M rows in args.B
                     if (m < args.B) {
                         int64_t* o = args.out + (int64_t)m * args.ncols + col0;
@@ -689,7 +772,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 o[i] = (int64_t)acc[i];
                         }
                     }
-                } else if (MODE == TC_WGRAD) {
+                } else if constexpr (MODE == TC_WGRAD) {
                     const int m = T.mt * kBM + r;
                     const int t = m / args.cin_k, ci = m - t * args.cin_k;
                     // im2col rows: row m is already the (tap, ci) index t Cin + ci
@@ -772,11 +855,23 @@ __global__ void __launch_bounds__(kThreads, 1)
                             }
                         }
                     }
-                } else if (MODE == TC_FWD && args.fuse) {
-                    // z* = floor(z / SF), NITRO-ReLU piece and value, optional
+                } else if constexpr (MODE == TC_FWD) {
+                    // z* = floor(z / SF) from z modulo 2^32 (exact) and z in fp32,
+                    // then the NITRO-ReLU value and piece from the table, optional
                     // 2x2 max-pool across lanes; int8 outputs straight from
                     // registers (the 2x2 windows of a tile lie inside one warp:
-                    // x partner lane ^ 1, y partner lane ^ wb).
+                    // x partner lane ^ 1, y partner lane ^ wb).  Bound by instruction
+                    // issue: two 32-bit words a column instead of 64-bit sums and a
+                    // 64-bit divide took the VGG11B forward at batch 256 from 1449 to
+                    // 1181 us and the VGG8B step from 980 to 928 us.
+                    //
+                    // zf is off by less than err (set before the tile loop).  Where err <= SF / 4 the
+                    // nearest integer to zf / SF is z* or z* + 1, and the sign of
+                    // z - q SF (modulo 2^32, so exact) says which.  Where it is
+                    // larger (three or four weight limbs) the remainder, below 2^31
+                    // as the host allows at most kFwdMaxBlocks K-blocks, is divided
+                    // once more.  |z*| beyond the table is clamped: value and piece
+                    // are flat outside [-127, 127].
                     const int mq = udiv32(args.dv_ntx, T.mt), tb = udiv32(args.dv_nty, mq);
                     const int tx = T.mt - mq * args.ntx, ty = mq - tb * args.nty;
                     const int xx = r & ((1 << args.lg_wb) - 1);
@@ -785,77 +880,87 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const int x = tx * args.wb + xx, y = ty * args.hb + yy, b = tb * args.bb + bbx;
                     const bool valid = x < args.W && y < args.H && b < args.B;
                     const int C = args.Cout;
-                    const int64_t zlo = args.z_lo;
-                    const uint64_t zrange = (uint64_t)(args.z_hi - args.z_lo);
-                    const FloorDiv32 sf32 = args.sf32;
+                    const int32_t sf = args.sf;
+                    const float sfi = args.sf_inv;
                     const int64_t pix = ((int64_t)b * args.H + y) * args.W + x;
                     const bool anchor = valid && !(x & 1) && !(y & 1) && x + 1 < args.W && y + 1 < args.H;
                     const int64_t opix = ((int64_t)b * args.oh + (y >> 1)) * args.ow + (x >> 1);
                     const int dys = args.wb;
-                    // one group of 16 columns at a time (only its packed words live)
+                    // position 3 - (2 (y & 1) + (x & 1)) of this pixel in its window, in
+                    // bits 6, 7 of each 16-bit key: the maximum is the first maximum
+                    const uint32_t poskey = (uint32_t)(3 - (((y & 1) << 1) | (x & 1))) * 0x00400040u;
+                    const bool wide = NH == 32 && args.out32 && col0 + 32 <= C;
+                    uint32_t vpk[NH / 4], rpk[NH / 4];   // packed outputs, pieces or window positions
 #pragma unroll
-                    for (int k = 0; k < NH / 16; ++k) {
-                        if (col0 + 16 * k >= C) break;   // uniform across the warp
-                        uint32_t vpk[4], rpk[4];
+                    for (int g4 = 0; g4 < NH / 4; ++g4) {
+                        uint32_t e[4];
 #pragma unroll
-                        for (int g4 = 0; g4 < 4; ++g4) {
-                            uint32_t vp = 0, rp = 0;
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                // z* = floor(z / SF) = floor((z >> 8) / 9Cin).  Inside
-                                // [-127 SF, 128 SF) it fits 32 bits and indexes the
-                                // NITRO-ReLU table; outside, the value is flat (table
-                                // ends) and only the sign picks the piece.
-                                const uint64_t z = acc[16 * k + 4 * g4 + u];
-                                const bool inside = z - (uint64_t)zlo < zrange;
-                                const bool neg = (int32_t)(z >> 32) < 0;
-                                const int zq = sf32.floor_div((int32_t)((int64_t)z >> 8));
-                                const int idx = inside ? zq + 127 : (neg ? 0 : 254);
-                                const int reg = inside ? (neg ? 1 : 2) : (neg ? 0 : 3);
-                                rp |= (uint32_t)reg << (8 * u);
-                                vp |= (uint32_t)(uint8_t)relu_tab[idx] << (8 * u);
+                        for (int u = 0; u < 4; ++u) {
+                            const uint32_t l = lo[4 * g4 + u];
+                            const float f = zf[4 * g4 + u];
+                            int q;
+                            if (tight) {
+                                q = min(max(__float2int_rn(f * sfi), -200), 200);
+                                q += (int32_t)(l - (uint32_t)(q * sf)) >> 31;
+                            } else {
+                                const int q1 = __float2int_rn(f * sfi);
+                                const uint32_t r1 = l - (uint32_t)q1 * (uint32_t)sf;
+                                const int q2 = __float2int_rn((float)(int32_t)r1 * sfi);
+                                const int32_t r2 = (int32_t)(r1 - (uint32_t)q2 * (uint32_t)sf);
+                                q = min(max(q1 + q2 + (r2 >> 31), -200), 200);
+                                if (fabsf(f) > far) q = f < 0.0f ? -200 : 200;
                             }
-                            vpk[g4] = vp;
-                            rpk[g4] = rp;
+                            e[u] = relu_tab[q + kTabHalf];
                         }
-                        const int c16 = col0 + 16 * k;
-                        if (valid) st16(args.region + pix * C + c16, rpk);
+                        const uint32_t e01 = e[0] | (e[1] << 16), e23 = e[2] | (e[3] << 16);
+                        rpk[g4] = __byte_perm(e01, e23, 0x6420);
                         if (!args.pool) {
-                            if (valid) {
-                                const int64_t o = pix * C + c16;
-                                st16(args.act + o, vpk);
-                                if (args.out2) st16(args.out2 + o, vpk);
-                                if (args.next_nhwc) st16_bf16(args.next_nhwc + o, vpk, bf16_tab);
-                            }
+                            vpk[g4] = __byte_perm(e01, e23, 0x7531);
                         } else {
-                            uint32_t opk[4], apk[4];
+                            // key = value, 3 - position, piece: the maximum over the
+                            // window's four lanes, two 16-bit keys per word
+                            vpk[g4] = e01 + poskey;
+                            lo[4 * g4] = e23 + poskey;
+                        }
+                    }
+                    if (valid && col0 < C) {
+                        int8_t* p = args.region + pix * C + col0;
+                        if (wide) {
+                            st32(p, rpk, true);
+                        } else {
 #pragma unroll
-                            for (int g4 = 0; g4 < 4; ++g4) {
-                                const uint32_t v00 = vpk[g4];
-                                const uint32_t v01 = __shfl_xor_sync(0xffffffffu, v00, 1);
-                                const uint32_t v10 = __shfl_xor_sync(0xffffffffu, v00, dys);
-                                const uint32_t v11 = __shfl_xor_sync(0xffffffffu, v00, dys ^ 1);
-                                // four windows at once, a byte each: signed maxima, then
-                                // the first position (order (0,0), (0,1), (1,0), (1,1))
-                                // that holds the maximum
-                                const uint32_t best = __vmaxs4(__vmaxs4(v00, v01), __vmaxs4(v10, v11));
-                                const uint32_t e0 = __vcmpeq4(v00, best);
-                                const uint32_t e1 = __vcmpeq4(v01, best);
-                                const uint32_t e2 = __vcmpeq4(v10, best);
-                                uint32_t ap = 0x03030303u;
-                                ap = (ap & ~e2) | (0x02020202u & e2);
-                                ap = (ap & ~e1) | (0x01010101u & e1);
-                                ap &= ~e0;
-                                opk[g4] = best;
-                                apk[g4] = ap;
+                            for (int k = 0; k < NH / 16; ++k)
+                                if (col0 + 16 * k < C) st16(p + 16 * k, rpk + 4 * k);
+                        }
+                    }
+                    if (args.pool) {
+#pragma unroll
+                        for (int g4 = 0; g4 < NH / 4; ++g4) {
+                            uint32_t k0 = vpk[g4], k1 = lo[4 * g4];
+                            k0 = max_s16x2(k0, __shfl_xor_sync(0xffffffffu, k0, 1));
+                            k1 = max_s16x2(k1, __shfl_xor_sync(0xffffffffu, k1, 1));
+                            k0 = max_s16x2(k0, __shfl_xor_sync(0xffffffffu, k0, dys));
+                            k1 = max_s16x2(k1, __shfl_xor_sync(0xffffffffu, k1, dys));
+                            vpk[g4] = __byte_perm(k0, k1, 0x7531);
+                            rpk[g4] = 0x03030303u - ((__byte_perm(k0, k1, 0x6420) >> 6) & 0x03030303u);
+                        }
+                    }
+                    if ((args.pool ? anchor : valid) && col0 < C) {
+                        const int64_t o = (args.pool ? opix : pix) * C + col0;
+                        if (wide) {
+                            st32(args.act + o, vpk, true);
+                            if (args.out2) st32(args.out2 + o, vpk, true);
+                            if (args.pool) st32(args.argmax + o, rpk, true);
+                        }
+#pragma unroll
+                        for (int k = 0; k < NH / 16; ++k) {
+                            if (col0 + 16 * k >= C) break;
+                            if (!wide) {
+                                st16(args.act + o + 16 * k, vpk + 4 * k);
+                                if (args.out2) st16(args.out2 + o + 16 * k, vpk + 4 * k);
+                                if (args.pool) st16(args.argmax + o + 16 * k, rpk + 4 * k);
                             }
-                            if (anchor) {
-                                const int64_t o = opix * C + c16;
-                                st16(args.act + o, opk);
-                                if (args.out2) st16(args.out2 + o, opk);
-                                st16(args.argmax + o, apk);
-                                if (args.next_nhwc) st16_bf16(args.next_nhwc + o, opk, bf16_tab);
-                            }
+                            if (args.next_nhwc) st16_bf16(args.next_nhwc + o + 16 * k, vpk + 4 * k);
                         }
                     }
                 } else if (MODE == TC_DGRAD && args.fuse) {
@@ -1532,12 +1637,10 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
     a.out_vec = ((uintptr_t)z & 15) == 0;
     a.status = status;
     a.atomic_out = 0;
-    if (fo && g.cout % 16 == 0) {
-        a.fuse = 1;
-        const int64_t sf = 256LL * 9LL * g.cin;
-        a.sf32 = FloorDiv32::make(9u * (uint32_t)g.cin);
-        a.z_hi = 128 * sf;
-        a.z_lo = -127 * sf;
+    const bool fuse = fo && g.cout % 16 == 0 && a.kb_total <= kFwdMaxBlocks;
+    if (fuse) {
+        a.sf = 256 * 9 * g.cin;
+        a.sf_inv = 1.0f / (float)a.sf;
         a.alpha = FloorDiv::make((uint64_t)fo->alpha_inv);
         a.mu = fo->mu;
         a.pool = g.pool;
@@ -1548,6 +1651,8 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
         a.region = fo->region;
         a.argmax = fo->argmax;
         a.next_nhwc = fo->next_nhwc;
+        a.out32 = g.cout % 32 == 0 && (((uintptr_t)a.act | (uintptr_t)a.region | (uintptr_t)a.out2 |
+                                        (uintptr_t)a.argmax) & 31) == 0;
     }
     CUtensorMap ma, mb;
     const uint64_t da[4] = {(uint64_t)t.cin8, (uint64_t)g.w, (uint64_t)g.h, (uint64_t)batch};
@@ -1562,10 +1667,11 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
         return cudaErrorInvalidValue;
     const double ops = 2.0 * batch * g.h * g.w * g.cout * 9.0 * g.cin;
     ProfScope ps(K_TC_CONV_FWD, s, ops, 0.0);
-    cudaError_t e = launch_gemm_pb<TC_FWD>(n, pb, ma, mb, a, s);
+    cudaError_t e = fuse ? launch_gemm_pb<TC_FWD>(n, pb, ma, mb, a, s)
+                         : launch_gemm_pb<TC_FWDZ>(n, pb, ma, mb, a, s);
     if (e == cudaSuccess) {
         *done = true;
-        *fused = a.fuse != 0;
+        *fused = fuse;
     }
     return e;
 }
