@@ -358,7 +358,7 @@ nitro_status nitro_block_forward(nitro_block* b, const int8_t* a_in, int batch, 
         // is filled by a copy after the last layer instead
         int8_t* out2 = (i == n - 1 && ((uintptr_t)a_out & 15) == 0) ? a_out : nullptr;
         bool done = false, fused = false;
-        NITRO_TRY(tc_pack_input(ly.tc, g, x, batch, nhwc_done, s));
+        if (!ly.lin_planes) NITRO_TRY(tc_pack_input(ly.tc, g, x, batch, nhwc_done, s));
         // the epilogue also writes the next layer's bf16 forward operand
         uint16_t* next_nhwc = nullptr;
         if (i + 1 < n && b->L[i + 1].tc.act_nhwc && !b->L[i + 1].tc.im2col &&
