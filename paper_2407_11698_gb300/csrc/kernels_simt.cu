@@ -19,6 +19,22 @@
 namespace nitro {
 namespace {
 
+// The CTA's maximum into *word (one atomic a CTA: thousands of warps on one word
+// take longer than most of these kernels) and its overflow flag into *status.
+// Every thread of the CTA calls it.
+__device__ __forceinline__ void block_maximum(uint32_t mx, bool ovf, uint32_t* word, uint32_t* status) {
+    __shared__ uint32_t cta_max;
+    if (threadIdx.x == 0) cta_max = 0;
+    const bool any = __syncthreads_or(ovf);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0 && mx) atomicMax(&cta_max, mx);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (cta_max) atomicMax(word, cta_max);
+        if (any) atomicOr(status, ST_OVERFLOW);
+    }
+}
+
 constexpr int kTile = 64;   // M and N tile
 constexpr int kTK = 16;     // K slab
 constexpr unsigned kFull = 0xffffffffu;
@@ -552,78 +568,116 @@ __global__ void k_lrpool_to_delta(const int32_t* __restrict__ gl, const int32_t*
     }
 }
 
-// Same, four channels per thread (C % 4 == 0): one 4-byte load of each code
-// array and of the region bytes, one 16-byte delta store, 32-bit index
-// arithmetic (B h w C < 2^31) through invariant dividers; the pool windows
-// are powers of two, so their divisions are shifts.
-__global__ void k_lrpool_to_delta4(const int32_t* __restrict__ gl, const int32_t* __restrict__ wlr,
-                                   int G, int d, LayerGeom g, LrPoolGeom lp, int lg_kh, int lg_kw,
-                                   int B, FloorDiv32 dv_c4, FloorDiv32 dv_w, FloorDiv32 dv_h,
-                                   const uint8_t* __restrict__ lam,
-                                   const int8_t* __restrict__ argmax,
-                                   const int8_t* __restrict__ region, FloorDiv32 alpha,
-                                   int32_t* __restrict__ delta, const uint32_t* maxabs_gl,
-                                   const uint32_t* maxabs_wlr, uint32_t* maxabs_delta,
-                                   uint32_t* status) {
+// Same by windows, four channels per thread (C % 4 == 0): a thread takes the
+// learning feature of one (sample, window, four channels), finds the one
+// pre-pool position each of its channels routes to (window maximum, then 2x2
+// maximum), forms its delta there and writes the window, zeros elsewhere, 16
+// bytes a position; the last window of a row or column also writes what the
+// floor-sized pools drop.  blockIdx.y takes a share of the window's rows.  Bound by
+// the delta stores: looking the codes up per pre-pool element instead cost a
+// chain of dependent loads for each of 8.4 M or 16.8 M elements.
+// With planes != null the thread also writes delta's bf16 limb planes (the weight
+// gradient's operand), as many as the bound G max|grad_L| max|W_lr| can need, so
+// that no pass reads delta again; and the launch clears zero[0..n_zero).
+__global__ void __launch_bounds__(256) k_lrpool_to_delta4(
+    const int32_t* __restrict__ gl, const int32_t* __restrict__ wlr, int G, int d, LayerGeom g,
+    LrPoolGeom lp, int B, FloorDiv32 dv_c4, FloorDiv32 dv_pw, FloorDiv32 dv_ph,
+    const uint8_t* __restrict__ lam, const int8_t* __restrict__ argmax,
+    const int8_t* __restrict__ region, FloorDiv32 alpha, int32_t* __restrict__ delta,
+    uint16_t* __restrict__ planes, int64_t plane, int64_t* zero, int64_t n_zero,
+    const uint32_t* maxabs_gl, const uint32_t* maxabs_wlr, uint32_t* maxabs_delta,
+    uint32_t* status) {
     pdl_wait();
     const int C = g.cout, C4 = g.cout >> 2;
-    const uint32_t n4 = (uint32_t)B * g.h * g.w * C4;
-    if (blockIdx.x == 0 && threadIdx.x == 0 && int64_bound_exceeded(*maxabs_gl, *maxabs_wlr, G))
+    const uint32_t n4 = (uint32_t)B * lp.ph * lp.pw * C4;
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    {
+        const int64_t cta = blockIdx.x + (int64_t)blockIdx.y * gridDim.x;
+        const int64_t step = (int64_t)gridDim.x * gridDim.y * blockDim.x;
+        for (int64_t k = cta * blockDim.x + threadIdx.x; k < n_zero; k += step) zero[k] = 0;
+    }
+    if (i == 0 && blockIdx.y == 0 && int64_bound_exceeded(*maxabs_gl, *maxabs_wlr, G))
         atomicOr(status, ST_OVERFLOW);
+    int L = 0;
+    if (planes) {
+        const uint64_t gb = (uint64_t)*maxabs_gl * (uint64_t)G;           // < 2^38
+        const uint64_t wb = *maxabs_wlr;
+        const uint64_t bound = wb && gb > 0xffffffffull / wb ? 0xffffffffull : gb * wb;
+        L = limb_count((uint32_t)bound);
+    }
     uint32_t mx = 0;
     bool ovf = false;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += gridDim.x * blockDim.x) {
-        const uint32_t pix = dv_c4.udiv(i);
-        const int c = (int)(i - pix * C4) * 4;
-        const uint32_t r = dv_w.udiv(pix);
-        const int x = (int)(pix - r * g.w);
-        const uint32_t b = dv_h.udiv(r);
-        const int y = (int)(r - b * g.h);
-        int qy = y, qx = x;
-        bool any = true;
-        uint32_t am2 = 0, code2 = 0;
-        if (g.pool) {
-            qy = y >> 1;
-            qx = x >> 1;
-            any = qy < g.oh && qx < g.ow;
-            if (any) {
-                am2 = *reinterpret_cast<const uint32_t*>(argmax + ((b * g.oh + qy) * g.ow + qx) * C + c);
-                code2 = (uint32_t)(((y & 1) << 1) | (x & 1));
+    if (i < n4) {
+        const uint32_t win = dv_c4.udiv(i);
+        const int c = (int)(i - win * C4) * 4;
+        const uint32_t r = dv_pw.udiv(win);
+        const int wx = (int)(win - r * lp.pw);
+        const uint32_t b = dv_ph.udiv(r);
+        const int wy = (int)(r - b * lp.ph);
+        const int lg_kw = 31 - __clz(lp.kw);
+        const uint32_t lw = *reinterpret_cast<const uint32_t*>(lam + (size_t)win * C + c);
+        const int f0 = (wy * lp.pw + wx) * C + c;
+        uint64_t acc[4] = {0, 0, 0, 0};       // modulo 2^64, exact below the bound
+        const int32_t* wp = wlr + f0;
+#pragma unroll 5
+        for (int k = 0; k < G; ++k) {
+            const int4 w = *reinterpret_cast<const int4*>(wp + (int64_t)k * d);
+            const int64_t gv = gl[b * G + k];
+            acc[0] += (uint64_t)(gv * w.x);
+            acc[1] += (uint64_t)(gv * w.y);
+            acc[2] += (uint64_t)(gv * w.z);
+            acc[3] += (uint64_t)(gv * w.w);
+        }
+        int pos[4], v[4];                     // row << 16 | column of the hit, and delta there
+        uint32_t rg[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int code = (int)((lw >> (8 * j)) & 255u);
+            int y = wy * lp.kh + (code >> lg_kw), x = wx * lp.kw + (code & (lp.kw - 1));
+            if (g.pool) {
+                const int am = argmax[((size_t)(b * g.oh + y) * g.ow + x) * C + c + j];
+                y = 2 * y + (am >> 1);
+                x = 2 * x + (am & 1);
+            }
+            rg[j] = (uint8_t)region[((size_t)(b * g.h + y) * g.w + x) * C + c + j];
+            pos[j] = (y << 16) | x;
+        }
+        uint32_t h01[4], h23[4];              // bf16 limbs of the four deltas
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int64_t gv = (int64_t)acc[j];
+            const bool mine = blockIdx.y == 0;
+            ovf |= mine && !fits_i32(gv);
+            const int32_t gs = (int32_t)gv;
+            v[j] = rg[j] == 1 ? alpha.floor_div(gs) : (rg[j] == 2 ? gs : 0);
+            mx = max(mx, mine ? abs_u32(v[j]) : 0u);
+        }
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+            h01[l] = limb_bf16x2(v[0], v[1], l);
+            h23[l] = limb_bf16x2(v[2], v[3], l);
+        }
+        const int s2 = g.pool ? 2 : 1;
+        const int y0 = wy * lp.kh * s2, y1 = wy + 1 == lp.ph ? g.h : y0 + lp.kh * s2;
+        const int x0 = wx * lp.kw * s2, x1 = wx + 1 == lp.pw ? g.w : x0 + lp.kw * s2;
+        for (int y = y0 + blockIdx.y; y < y1; y += gridDim.y) {
+            size_t o = ((size_t)(b * g.h + y) * g.w + x0) * C + c;
+            for (int x = x0; x < x1; ++x, o += C) {
+                const int at = (y << 16) | x;
+                const bool k0 = pos[0] == at, k1 = pos[1] == at, k2 = pos[2] == at, k3 = pos[3] == at;
+                *reinterpret_cast<int4*>(delta + o) =
+                    make_int4(k0 ? v[0] : 0, k1 ? v[1] : 0, k2 ? v[2] : 0, k3 ? v[3] : 0);
+                const uint32_t m01 = (k0 ? 0xffffu : 0u) | (k1 ? 0xffff0000u : 0u);
+                const uint32_t m23 = (k2 ? 0xffffu : 0u) | (k3 ? 0xffff0000u : 0u);
+#pragma unroll
+                for (int l = 0; l < 4; ++l) {
+                    if (l >= L) break;
+                    *reinterpret_cast<uint2*>(planes + l * plane + o) = make_uint2(h01[l] & m01, h23[l] & m23);
+                }
             }
         }
-        int v[4] = {0, 0, 0, 0};
-        const int wy = qy >> lg_kh, wx = qx >> lg_kw;
-        if (any && wy < lp.ph && wx < lp.pw) {
-            const uint32_t lw =
-                *reinterpret_cast<const uint32_t*>(lam + ((b * lp.ph + wy) * lp.pw + wx) * C + c);
-            const uint32_t code = (uint32_t)(((qy - (wy << lg_kh)) << lg_kw) + (qx - (wx << lg_kw)));
-            const uint32_t rw = *reinterpret_cast<const uint32_t*>(region + 4 * (size_t)i);
-            const int f0 = (wy * lp.pw + wx) * C + c;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const bool hit = (!g.pool || ((am2 >> (8 * j)) & 255u) == code2) &&
-                                 ((lw >> (8 * j)) & 255u) == code;
-                if (!hit) continue;
-                uint64_t acc = 0;   // modulo 2^64, exact below the bound
-                for (int k = 0; k < G; ++k)
-                    acc += (uint64_t)((int64_t)gl[b * G + k] * wlr[(int64_t)k * d + f0 + j]);
-                const int64_t gv = (int64_t)acc;
-                ovf |= !fits_i32(gv);
-                const int32_t gs = (int32_t)gv;
-                const int rg = (int8_t)(rw >> (8 * j));
-                v[j] = rg == 1 ? alpha.floor_div(gs) : (rg == 2 ? gs : 0);
-                mx = max(mx, abs_u32(v[j]));
-            }
-        }
-        reinterpret_cast<int4*>(delta)[i] = make_int4(v[0], v[1], v[2], v[3]);
     }
-#pragma unroll
-    for (int off = 16; off; off >>= 1) mx = max(mx, __shfl_xor_sync(kFull, mx, off));
-    ovf = __any_sync(kFull, ovf);
-    if ((threadIdx.x & 31) == 0) {
-        if (mx) atomicMax(maxabs_delta, mx);
-        if (ovf) atomicOr(status, ST_OVERFLOW);
-    }
+    block_maximum(mx, ovf, maxabs_delta, status);
 }
 
 // ---------------------------------------------------------------------------
@@ -1252,7 +1306,8 @@ cudaError_t simt_lr_pool_fwd(const int8_t* a, int B, int H, int W, int C, int kh
 cudaError_t simt_lrpool_to_delta(const int32_t* gl, const int32_t* wlr, int G, int d,
                                  const LayerGeom& g, const LrPoolGeom& lp, int B,
                                  const uint8_t* am, const int8_t* argmax, const int8_t* region,
-                                 int alpha_inv, int32_t* delta, const uint32_t* maxabs_gl,
+                                 int alpha_inv, int32_t* delta, uint16_t* planes, int64_t* zero,
+                                 int64_t n_zero, bool* planes_done, const uint32_t* maxabs_gl,
                                  const uint32_t* maxabs_wlr, uint32_t* maxabs_delta,
                                  uint32_t* status, cudaStream_t s) {
     const int64_t n = (int64_t)B * g.h * g.w * g.cout;
@@ -1265,17 +1320,24 @@ cudaError_t simt_lrpool_to_delta(const int32_t* gl, const int32_t* wlr, int G, i
     ProfScope ps(K_LRPOOL_TO_DELTA, s, 2.0 * B * d * G,
                  5.0 * n + (double)B * g.oh * g.ow * g.cout * (g.pool ? 1 : 0) + (double)B * d +
                      4.0 * G * (B + (double)d));
-    int lg_kh = 0, lg_kw = 0;
-    while ((1 << lg_kh) < lp.kh) ++lg_kh;
-    while ((1 << lg_kw) < lp.kw) ++lg_kw;
-    const bool aligned = (((uintptr_t)am | (uintptr_t)region | (uintptr_t)delta |
+    const bool aligned = (((uintptr_t)am | (uintptr_t)region | (uintptr_t)delta | (uintptr_t)wlr |
                            (uintptr_t)(g.pool ? argmax : region)) & 15) == 0;
-    if (g.cout % 4 == 0 && aligned && (1 << lg_kh) == lp.kh && (1 << lg_kw) == lp.kw) {
-        launch_k(k_lrpool_to_delta4, grid_for(n / 4, 256), 256, 0, s,
-            gl, wlr, G, d, g, lp, lg_kh, lg_kw, B, FloorDiv32::make((uint32_t)(g.cout / 4)),
-            FloorDiv32::make((uint32_t)g.w), FloorDiv32::make((uint32_t)g.h), am, argmax, region,
-            FloorDiv32::make((uint32_t)alpha_inv), delta, maxabs_gl, maxabs_wlr, maxabs_delta,
-            status);
+    const bool pow2 = (lp.kh & (lp.kh - 1)) == 0 && (lp.kw & (lp.kw - 1)) == 0;
+    *planes_done = false;
+    if (g.cout % 4 == 0 && aligned && pow2) {   // d = ph pw cout is then a multiple of 4
+        // a thread per (sample, window, four channels); the rows of a window are
+        // shared out until about 200 k threads store
+        const int64_t threads = (int64_t)B * d / 4;
+        const int rows = lp.kh * (g.pool ? 2 : 1);
+        int64_t parts = 200000 / threads;
+        parts = parts < 1 ? 1 : (parts > rows ? rows : parts);
+        dim3 grid((unsigned)((threads + 255) / 256), (unsigned)parts);
+        launch_k(k_lrpool_to_delta4, grid, 256, 0, s,
+            gl, wlr, G, d, g, lp, B, FloorDiv32::make((uint32_t)(g.cout / 4)),
+            FloorDiv32::make((uint32_t)lp.pw), FloorDiv32::make((uint32_t)lp.ph), am, argmax, region,
+            FloorDiv32::make((uint32_t)alpha_inv), delta, planes, n, zero, zero ? n_zero : (int64_t)0,
+            maxabs_gl, maxabs_wlr, maxabs_delta, status);
+        *planes_done = planes != nullptr;
     } else {
         launch_k(k_lrpool_to_delta, grid_for(n, 256), 256, 0, s,
             gl, wlr, G, d, g, lp, B, am, argmax, region,

@@ -427,6 +427,7 @@ nitro_status block_backward(nitro_block* b, const int8_t* a_in, const int32_t* l
         return NITRO_OK;
     }
     const int8_t* a_last = n ? b->L[n - 1].act : a_in;
+    bool planes_done = false;   // the last layer's delta is already in limb planes
     if (b->zmp) {
         // z^mp: the block output max-pooled for the learning layer (Sec. 3.3)
         const LayerGeom& lg = b->L[n - 1].g;
@@ -447,10 +448,13 @@ nitro_status block_backward(nitro_block* b, const int8_t* a_in, const int32_t* l
                                        w_gl(b), w_wlr(b), nullptr, w_status(b), s));
         else
             NITRO_TRY(simt_learn_dw(a_last, b->grad_l, batch, (int)d, G, b->dWlr, s));
+        // (and its limb planes; the launch also clears dW for a split weight gradient)
         Layer& ly = b->L[n - 1];
         NITRO_TRY(simt_lrpool_to_delta(b->grad_l, b->Wlr, G, (int)d, ly.g, b->lp, batch, b->lr_am,
-                                       ly.argmax, ly.region, b->desc.alpha_inv, ly.delta, w_gl(b),
-                                       w_wlr(b), w_delta(b, n - 1), w_status(b), s));
+                                       ly.argmax, ly.region, b->desc.alpha_inv, ly.delta,
+                                       ly.tc.d_nhwc, tc_wgrad_adds(ly.tc, ly.g, batch, ly.dW),
+                                       ly.wcount, &planes_done, w_gl(b), w_wlr(b), w_delta(b, n - 1),
+                                       w_status(b), s));
     } else if (simt_lr_backward_ok(G)) {
         // learning-weight gradient and (below a forward layer) delta_fw -> that
         // layer's delta in one pass
@@ -502,7 +506,7 @@ nitro_status block_backward(nitro_block* b, const int8_t* a_in, const int32_t* l
 
             } else {
                 NITRO_TRY(tc_conv_wgrad(ly.tc, g, ly.delta, w_delta(b, i), batch, ly.dW, w_status(b), s,
-                                        &done));
+                                        &done, planes_done && i == n - 1));
             }
             if (!done && simt_small_conv_ok(g)) {
                 NITRO_TRY(simt_conv_small_wgrad(x, ly.delta, g, batch, ly.dW, s));
@@ -515,7 +519,7 @@ nitro_status block_backward(nitro_block* b, const int8_t* a_in, const int32_t* l
             return NITRO_OK;
         };
         if (fuse_sgd) {
-            NITRO_TRY(tc_pack_delta(ly.tc, g, ly.delta, w_delta(b, i), batch, s));
+            NITRO_TRY(tc_pack_delta(ly.tc, g, ly.delta, w_delta(b, i), batch, s, planes_done && i == n - 1));
         } else {
             nitro_status st = wgrad();
             if (st != NITRO_OK) return st;

@@ -163,6 +163,44 @@ __host__ __device__ __forceinline__ bool int64_bound_exceeded(uint32_t ma, uint3
 }
 
 // ---------------------------------------------------------------------------
+// The signed base-256 split behind the tensor-core operands (bf16 limb planes).
+// ---------------------------------------------------------------------------
+// Limbs of a tensor with max |x| = m.  The split is canonical: limbs 0..2 are
+// the digits ((x + 128) & 255) - 128 of successive base-256 remainders and
+// limb 3 takes the rest (in [-128, 128] for int32).  With the thresholds below
+// every limb at index >= L is zero, so the first L planes of the 4-limb split
+// are exact and producers may write all four without knowing L.
+__host__ __device__ __forceinline__ int limb_count(uint32_t m) {
+    return m <= 127u ? 1 : (m <= 32639u ? 2 : (m <= 8355711u ? 3 : 4));
+}
+
+#ifdef __CUDACC__
+// two int8 values v (bytes i, i + 1 of a word whose bytes hold v + 128) -> two bf16:
+// 2^23 + (v + 128) is the float 0x4B0000xx, and subtracting 2^23 + 128 leaves v
+// exactly, whose upper half is its bf16
+__device__ __forceinline__ uint32_t bf16x2(uint32_t biased, int i) {
+    const float f0 = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7540 + i)) - 8388736.0f;
+    const float f1 = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7541 + i)) - 8388736.0f;
+    return __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+}
+
+// Limb l of two values as two bf16.  Adding 0x808080 moves the digits 0..2 of
+// the signed base-256 split into [0, 255] with all their carries at once: byte l of
+// the sum is digit l + 128.  Limb 3 is what remains, with the carry of the low
+// 24 bits (the sum itself may wrap).
+__device__ __forceinline__ uint32_t limb_bf16x2(int32_t a, int32_t b, int l) {
+    if (l < 3) {
+        const uint32_t ta = (uint32_t)a + 0x808080u, tb = (uint32_t)b + 0x808080u;
+        return bf16x2(__byte_perm(ta, tb, l | ((4 + l) << 4)), 0);
+    }
+    const int32_t da = (a >> 24) + (int32_t)((((uint32_t)a & 0xffffffu) + 0x808080u) >> 24);
+    const int32_t db = (b >> 24) + (int32_t)((((uint32_t)b & 0xffffffu) + 0x808080u) >> 24);
+    return __byte_perm(__float_as_uint((float)da), __float_as_uint((float)db), 0x7632);
+}
+
+#endif
+
+// ---------------------------------------------------------------------------
 // Layer geometry as the kernels see it.
 // ---------------------------------------------------------------------------
 struct LayerGeom {
@@ -211,14 +249,17 @@ cudaError_t simt_lr_pool_fwd(const int8_t* a, int B, int H, int W, int C, int kh
 // delta_fw = grad_l W_lr at the pooled learning features (int32 storage rule,
 // int64 bound check), routed back through the learning-layer pool (window
 // maximum am), the 2x2 max-pool of conv layer g (argmax) and NITRO-ReLU
-// backward into g's delta [B][h][w][cout]; every element is written.
+// backward into g's delta [B][h][w][cout]; every element is written.  planes (may
+// be null): delta's limb planes [4][n], written too where the channel count
+// allows (*planes_done); zero[0..n_zero) is then cleared as well.
 struct LrPoolGeom {
     int kh, kw, ph, pw;
 };
 cudaError_t simt_lrpool_to_delta(const int32_t* gl, const int32_t* wlr, int G, int d,
                                  const LayerGeom& g, const LrPoolGeom& lp, int B,
                                  const uint8_t* am, const int8_t* argmax, const int8_t* region,
-                                 int alpha_inv, int32_t* delta, const uint32_t* maxabs_gl,
+                                 int alpha_inv, int32_t* delta, uint16_t* planes, int64_t* zero,
+                                 int64_t n_zero, bool* planes_done, const uint32_t* maxabs_gl,
                                  const uint32_t* maxabs_wlr, uint32_t* maxabs_delta,
                                  uint32_t* status, cudaStream_t s);
 

@@ -217,15 +217,6 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t* r) {
     for (int j = 0; j < n / 16; ++j) reg_touch16(r + 16 * j);
 }
 
-// Limbs of a tensor with max |x| = m.  The split is canonical: limbs 0..2 are
-// the digits ((x + 128) & 255) - 128 of successive base-256 remainders and
-// limb 3 takes the rest (in [-128, 128] for int32).  With the thresholds below
-// every limb at index >= L is zero, so the first L planes of the 4-limb split
-// are exact and producers may write all four without knowing L.
-__host__ __device__ __forceinline__ int limb_count(uint32_t m) {
-    return m <= 127u ? 1 : (m <= 32639u ? 2 : (m <= 8355711u ? 3 : 4));
-}
-
 // ------------------------------------------------------------------ kernel
 struct TcArgs {
     int B, H, W, Cin, Cout, Bp;
@@ -309,14 +300,6 @@ __device__ __forceinline__ uint32_t max_s16x2(uint32_t a, uint32_t b) {
     uint32_t d;
     asm("max.s16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
     return d;
-}
-// two int8 values v (bytes i, i + 1 of a word whose bytes hold v + 128) -> two bf16:
-// 2^23 + (v + 128) is the float 0x4B0000xx, and subtracting 2^23 + 128 leaves v
-// exactly, whose upper half is its bf16
-__device__ __forceinline__ uint32_t bf16x2(uint32_t biased, int i) {
-    const float f0 = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7540 + i)) - 8388736.0f;
-    const float f1 = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7541 + i)) - 8388736.0f;
-    return __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
 }
 // 16 int8 values (4 packed words) -> 16 bf16 values, packed
 __device__ __forceinline__ void cvt16_bf16(uint32_t* o, const uint32_t* w) {
@@ -1263,20 +1246,6 @@ __global__ void __launch_bounds__(256) k_pack_act_flat(const int8_t* __restrict_
     for (int64_t i = 16 * n16 + tid; i < n; i += stride) out[i] = bf16_bits(x[i]);
 }
 
-// Limb l of two values as two bf16.  Adding 0x808080 moves the digits 0..2 of
-// the signed base-256 split into [0, 255] with all their carries at once: byte l of
-// the sum is digit l + 128.  Limb 3 is what remains, with the carry of the low
-// 24 bits (the sum itself may wrap).
-__device__ __forceinline__ uint32_t limb_bf16x2(int32_t a, int32_t b, int l) {
-    if (l < 3) {
-        const uint32_t ta = (uint32_t)a + 0x808080u, tb = (uint32_t)b + 0x808080u;
-        return bf16x2(__byte_perm(ta, tb, l | ((4 + l) << 4)), 0);
-    }
-    const int32_t da = (a >> 24) + (int32_t)((((uint32_t)a & 0xffffffu) + 0x808080u) >> 24);
-    const int32_t db = (b >> 24) + (int32_t)((((uint32_t)b & 0xffffffu) + 0x808080u) >> 24);
-    return __byte_perm(__float_as_uint((float)da), __float_as_uint((float)db), 0x7632);
-}
-
 // int32 delta NHWC (n values, n % 8 == 0) -> limb planes [L][n], eight values
 // per thread and one 16-byte store per plane (L from *maxabs).  The
 // input is read 32 bytes at a time when `d` is 32-byte aligned (vec != 0).
@@ -1490,8 +1459,8 @@ int wgrad_splits(int tiles, int kb_total, int* kb_per_split) {
 
 }  // namespace
 
-bool tc_wgrad_fusable(const TcLayer& t, const LayerGeom& g, int batch) {
-    if (!t.wgrad || batch <= 0) return false;
+namespace {
+int wgrad_split_count(const TcLayer& t, const LayerGeom& g, int batch) {
     const bool lin = g.kind == NITRO_LINEAR;
     const int gh = lin ? 1 : g.h, gw = lin ? batch : g.w;
     const int wb = gw <= 8 ? 8 : (gw <= 16 ? 16 : (gw <= 32 ? 32 : 64)), hb = 64 / wb;
@@ -1499,7 +1468,16 @@ bool tc_wgrad_fusable(const TcLayer& t, const LayerGeom& g, int batch) {
     const int tiles = (taps * t.cin_k + kBM - 1) / kBM * ((g.cout + pick_n(g.cout) - 1) / pick_n(g.cout));
     const int kb_total = (lin ? 1 : batch) * ((gw + wb - 1) / wb) * ((gh + hb - 1) / hb);
     int kbs = 0;
-    return wgrad_splits(tiles, kb_total, &kbs) == 1;
+    return wgrad_splits(tiles, kb_total, &kbs);
+}
+}  // namespace
+
+bool tc_wgrad_fusable(const TcLayer& t, const LayerGeom& g, int batch) {
+    return t.wgrad && batch > 0 && wgrad_split_count(t, g, batch) == 1;
+}
+
+int64_t* tc_wgrad_adds(const TcLayer& t, const LayerGeom& g, int batch, int64_t* dW) {
+    return t.wgrad && batch > 0 && wgrad_split_count(t, g, batch) > 1 ? dW : nullptr;
 }
 
 bool tc_layer_init(TcLayer& t, const LayerGeom& g, int max_batch, bool has_dgrad,
@@ -1703,8 +1681,6 @@ cudaError_t tc_pack_delta(TcLayer& t, const LayerGeom& g, const int32_t* delta,
         ProfScope ps(K_TC_PACK_D, s, 0.0, (double)n * 4 * 2);
         launch_k(k_pack_delta_nhwc, grid1d(n / 8), 256, 0, s, delta, n, ((uintptr_t)delta & 31) == 0,
                                                        maxabs_delta, t.d_nhwc, zero, n_zero);
-    } else if (zero) {
-        return cudaMemsetAsync(zero, 0, sizeof(int64_t) * (size_t)n_zero, s);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !t.own_hints) return e;

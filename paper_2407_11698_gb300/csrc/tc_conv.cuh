@@ -137,7 +137,7 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
 
 // Splits delta into NHWC limb planes for the wgrad and dgrad passes (limb
 // count from *maxabs_delta), unless planes_done (an earlier call split this
-// delta already), and clears zero[0..n_zero); then refreshes the host hint of max |delta|.  Writing the
+// delta already), and clears zero[0..n_zero) (not with planes_done); then refreshes the host hint of max |delta|.  Writing the
 // planes from the kernels that produce delta instead (the dgrad epilogue,
 // the learning-layer backward) was measured slower than this pass.
 cudaError_t tc_pack_delta(TcLayer& t, const LayerGeom& g, const int32_t* delta,
@@ -146,6 +146,10 @@ cudaError_t tc_pack_delta(TcLayer& t, const LayerGeom& g, const int32_t* delta,
 
 // tc_pack_delta, then, if wgrad runs on tcgen05, dW = sum_p delta (x)
 // im2col(a).  Must precede tc_conv_dgrad.
+// dW when tc_conv_wgrad adds K-split partial sums into it at this batch (it must
+// be zero before), else null.
+int64_t* tc_wgrad_adds(const TcLayer& t, const LayerGeom& g, int batch, int64_t* dW);
+
 // True when the layer's weight gradient runs on tcgen05 without a K split at
 // this batch, i.e. when tc_conv_wgrad can fold IntegerSGD into it.
 bool tc_wgrad_fusable(const TcLayer& t, const LayerGeom& g, int batch);
