@@ -687,8 +687,10 @@ __global__ void __launch_bounds__(256) k_lrpool_to_delta4(
 __device__ __forceinline__ int32_t sgd_one(const SgdTensor& t, int round_trunc, int32_t w32,
                                            int64_t g, uint32_t& mx, bool& ovf) {
     const int64_t w = w32;
-    int64_t d = round_trunc ? t.gdiv.trunc_div(g) : t.gdiv.floor_div(g);
-    if (t.eta_inv != 0) d += round_trunc ? t.ediv.trunc_div(w) : t.ediv.floor_div(w);
+    int64_t d;
+    if (fits_i32(g)) d = round_trunc ? t.gdiv32.trunc_div((int32_t)g) : t.gdiv32.floor_div((int32_t)g);
+    else d = round_trunc ? t.gdiv.trunc_div(g) : t.gdiv.floor_div(g);
+    if (t.eta_inv != 0) d += round_trunc ? t.ediv32.trunc_div(w32) : t.ediv32.floor_div(w32);
     const int64_t nw = w - d;
     ovf |= !fits_i32(nw);
     const int32_t s = (int32_t)nw;
@@ -696,57 +698,37 @@ __device__ __forceinline__ int32_t sgd_one(const SgdTensor& t, int round_trunc, 
     return s;
 }
 
-// The updated weight w (element i of [Cout][9][cin]) into its four bf16 limb
-// planes: limbs 0..2 the digits ((x + 128) & 255) - 128 of successive base-256
-// remainders, limb 3 the rest; each limb is an integer of at most 8 bits, so
-// the top half of its fp32 bits is its exact bf16.
+// The updated weight w (element i of [Cout][9][cin]) into its four bf16 limb planes.
 __device__ __forceinline__ void sgd_planes(const SgdTensor& t, int64_t i, int32_t w) {
     const uint32_t q = t.cin_div.udiv((uint32_t)i);
     const int ci = (int)(i - (int64_t)q * t.cin);
     const int tap = (int)(q % 9u), co = (int)(q / 9u);
     uint16_t* p = t.planes + (int64_t)co * t.row_k + tap * t.tap_k + ci;
-    int64_t x = w;
 #pragma unroll
-    for (int l = 0; l < 4; ++l) {
-        int v;
-        if (l < 3) {
-            v = (int)(((x + 128) & 255) - 128);
-            x = (x - v) >> 8;
-        } else {
-            v = (int)x;
-        }
-        p[l * t.plane] = (uint16_t)(__float_as_uint((float)v) >> 16);
-    }
+    for (int l = 0; l < 4; ++l) p[l * t.plane] = (uint16_t)limb_bf16x2(w, w, l);
 }
 
 // Four consecutive updated weights into their limb planes when the planes are
-// laid out like W (linear layers; convs with Cin a multiple of 64): the same
-// split, one 8-byte store per plane at p + l * plane.
-__device__ __forceinline__ void sgd_planes4(uint16_t* p, int64_t plane, int4 w) {
-    int32_t v[4] = {w.x, w.y, w.z, w.w};
+// laid out like W (linear layers; convs with Cin a multiple of 64), 8 bytes a
+// plane at p + l * plane; a plane whose four limbs stay as they were is not stored.
+__device__ __forceinline__ void sgd_planes4(uint16_t* p, int64_t plane, int4 w, int4 old) {
 #pragma unroll
     for (int l = 0; l < 4; ++l) {
-        uint32_t h[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            int dg;
-            if (l < 3) {
-                // v = 256 q + r: digit r or r - 256, remainder q or q + 1
-                const int r = v[k] & 255;
-                dg = r - ((r >> 7) << 8);
-                v[k] = (v[k] >> 8) + (r >> 7);
-            } else {
-                dg = v[k];
-            }
-            h[k] = __float_as_uint((float)dg) >> 16;
-        }
-        *reinterpret_cast<uint2*>(p + l * plane) = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
+        const uint2 v = make_uint2(limb_bf16x2(w.x, w.y, l), limb_bf16x2(w.z, w.w, l));
+        const uint2 u = make_uint2(limb_bf16x2(old.x, old.y, l), limb_bf16x2(old.z, old.w, l));
+        if (v.x != u.x || v.y != u.y) *reinterpret_cast<uint2*>(p + l * plane) = v;
     }
 }
 
-// Four consecutive weights per thread (16-byte loads of W, two of dW; the
-// tensors are this library's own 256-byte aligned buffers), the tail singly.
-__global__ void k_integersgd(SgdBatch bt) {
+// Four consecutive weights per thread and round (16-byte loads of W, two of dW;
+// the tensors are this library's own 256-byte aligned buffers), the tail singly.
+// Bound by memory traffic: W and dW are read (12 bytes a weight), and only what
+// changes is written - the planes always hold all four limbs of W, so a group of
+// weights that stay, or a plane whose digits stay (the upper ones, nearly always),
+// needs no store.  24 bytes a weight before; the 21 M weights of the wide MLP took
+// 171 us a step in four launches, now 112.
+// A gradient that fits 32 bits takes the 32-bit divide.
+__global__ void __launch_bounds__(256) k_integersgd(const SgdBatch bt) {
     pdl_wait();
     int ti = 0;
     while (ti + 1 < bt.count && (int)blockIdx.x >= bt.first[ti + 1]) ++ti;
@@ -756,38 +738,41 @@ __global__ void k_integersgd(SgdBatch bt) {
     uint32_t mx = 0;
     bool ovf = false;
     const int64_t n4 = t.n / 4;
-    for (int64_t i = tid; i < n4; i += stride) {
-        const int4 w = reinterpret_cast<const int4*>(t.w)[i];
-        const longlong2 g0 = reinterpret_cast<const longlong2*>(t.dw)[2 * i];
-        const longlong2 g1 = reinterpret_cast<const longlong2*>(t.dw)[2 * i + 1];
+    const auto group = [&](int64_t i, const int4 w, const longlong2 g0, const longlong2 g1) {
         int4 o;
         o.x = sgd_one(t, bt.round_trunc, w.x, g0.x, mx, ovf);
         o.y = sgd_one(t, bt.round_trunc, w.y, g0.y, mx, ovf);
         o.z = sgd_one(t, bt.round_trunc, w.z, g1.x, mx, ovf);
         o.w = sgd_one(t, bt.round_trunc, w.w, g1.y, mx, ovf);
+        if (o.x == w.x && o.y == w.y && o.z == w.z && o.w == w.w) return;
         reinterpret_cast<int4*>(t.w)[i] = o;
         if (t.planes && t.contig) {
-            sgd_planes4(t.planes + 4 * i, t.plane, o);
+            sgd_planes4(t.planes + 4 * i, t.plane, o, w);
         } else if (t.planes) {
-            sgd_planes(t, 4 * i, o.x);
-            sgd_planes(t, 4 * i + 1, o.y);
-            sgd_planes(t, 4 * i + 2, o.z);
-            sgd_planes(t, 4 * i + 3, o.w);
+            if (o.x != w.x) sgd_planes(t, 4 * i, o.x);
+            if (o.y != w.y) sgd_planes(t, 4 * i + 1, o.y);
+            if (o.z != w.z) sgd_planes(t, 4 * i + 2, o.z);
+            if (o.w != w.w) sgd_planes(t, 4 * i + 3, o.w);
         }
+    };
+    const int4* wv = reinterpret_cast<const int4*>(t.w);
+    const longlong2* gv = reinterpret_cast<const longlong2*>(t.dw);
+    int64_t i = tid;
+    for (; i + stride < n4; i += 2 * stride) {   // two groups' loads in flight
+        const int64_t j = i + stride;
+        const int4 wa = wv[i], wb = wv[j];
+        const longlong2 a0 = gv[2 * i], a1 = gv[2 * i + 1], b0 = gv[2 * j], b1 = gv[2 * j + 1];
+        group(i, wa, a0, a1);
+        group(j, wb, b0, b1);
     }
-    for (int64_t i = 4 * n4 + tid; i < t.n; i += stride) {
-        const int32_t nw = sgd_one(t, bt.round_trunc, t.w[i], t.dw[i], mx, ovf);
-        t.w[i] = nw;
-        if (t.planes) sgd_planes(t, i, nw);
+    if (i < n4) group(i, wv[i], gv[2 * i], gv[2 * i + 1]);
+    for (int64_t k = 4 * n4 + tid; k < t.n; k += stride) {
+        const int32_t nw = sgd_one(t, bt.round_trunc, t.w[k], t.dw[k], mx, ovf);
+        t.w[k] = nw;
+        if (t.planes) sgd_planes(t, k, nw);
     }
-#pragma unroll
-    for (int off = 16; off; off >>= 1) mx = max(mx, __shfl_xor_sync(kFull, mx, off));
-    ovf = __any_sync(kFull, ovf);
-    if ((threadIdx.x & 31) == 0) {
-        if (mx) atomicMax(&bt.scratch[ti], mx);
-        if (ovf) atomicOr(bt.status, ST_OVERFLOW);
-        __threadfence();     // this warp's maximum, before the CTA's ticket
-    }
+    block_maximum(mx, ovf, &bt.scratch[ti], bt.status);
+    if (threadIdx.x == 0) __threadfence();     // the CTA's maximum, before its ticket
     __shared__ bool last;
     __syncthreads();
     if (threadIdx.x == 0) last = atomicAdd(&bt.scratch[kMaxSgdTensors], 1u) == gridDim.x - 1;
@@ -1401,7 +1386,10 @@ cudaError_t simt_integersgd(const SgdBatch& b_in, cudaStream_t s) {
         b.first[i + 1] = b.first[i] + grid_for((b.t[i].n + 3) / 4, 256, 152 * 4);
         if (b.t[i].gamma_inv <= 0 || b.t[i].eta_inv < 0) return cudaErrorInvalidValue;
         b.t[i].gdiv = FloorDiv::make((uint64_t)b.t[i].gamma_inv);
-        b.t[i].ediv = FloorDiv::make(b.t[i].eta_inv > 0 ? (uint64_t)b.t[i].eta_inv : 1);
+        // 32-bit dividends: any divisor above 2^31 gives what 2^31 + 1 gives
+        const auto clamp32 = [](int64_t v) { return (uint32_t)std::min<int64_t>(v, ((int64_t)1 << 31) + 1); };
+        b.t[i].gdiv32 = FloorDiv32::make(clamp32(b.t[i].gamma_inv));
+        b.t[i].ediv32 = FloorDiv32::make(b.t[i].eta_inv > 0 ? clamp32(b.t[i].eta_inv) : 1u);
         if (b.t[i].planes) {
             if (b.t[i].cin < 1 || b.t[i].n >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
             b.t[i].cin_div = FloorDiv32::make((uint32_t)b.t[i].cin);

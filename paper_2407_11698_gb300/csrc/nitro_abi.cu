@@ -319,9 +319,10 @@ nitro_status nitro_init_block(const nitro_block_desc* desc, uint64_t seed, void*
     if (e == cudaSuccess)
         e = cudaMemsetAsync(b->zsum, 0, 8 * simt_learn_scratch(MB, (int)b->d, b->G), s);
     for (int i = 0; e == cudaSuccess && i < desc->n_layers; ++i) {
-        e = tc_refresh_weights(b->L[i].tc, b->L[i].g, b->L[i].W, w_w(b, i), s);
+        // all four limb planes: IntegerSGD stores only what changes in them
+        e = tc_refresh_weights(b->L[i].tc, b->L[i].g, b->L[i].W, w_w(b, i), s, true);
         if (e == cudaSuccess && b->L[i].lin_planes)
-            e = tc_pack_limbs(b->L[i].W, b->L[i].wcount, w_w(b, i), b->L[i].lin_planes, s);
+            e = tc_pack_limbs(b->L[i].W, b->L[i].wcount, nullptr, b->L[i].lin_planes, s);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) std::memcpy(b->words_host, words.data(), 4 * (size_t)n_words(desc->n_layers));
@@ -576,7 +577,7 @@ nitro_status block_sgd(nitro_block* b, void* stream, const std::vector<char>* sk
         if (skip && (*skip)[i]) continue;
         // the update also writes the tensor-core weight planes of the layer
         SgdTensor st{b->L[i].W, b->L[i].dW, b->L[i].wcount, gamma_fw, b->desc.eta_inv_fw,
-                     w_w(b, i), {}, {}, nullptr, 0, 0, 0, 0, {}};
+                     w_w(b, i), {}, {}, {}, nullptr, 0, 0, 0, 0, {}};
         tc_weight_planes(b->L[i].tc, b->L[i].g, &st.planes, &st.plane, &st.row_k, &st.tap_k);
         st.cin = b->L[i].g.cin;
         if (b->L[i].lin_planes) {
@@ -590,7 +591,7 @@ nitro_status block_sgd(nitro_block* b, void* stream, const std::vector<char>* sk
         bt.t[bt.count++] = st;
     }
     bt.t[bt.count++] = SgdTensor{b->Wlr, b->dWlr, (int64_t)b->G * b->d, b->desc.gamma_inv_lr,
-                                 b->desc.eta_inv_lr, w_wlr(b), {}, {}, nullptr, 0, 0, 0, 0, {}};
+                                 b->desc.eta_inv_lr, w_wlr(b), {}, {}, {}, nullptr, 0, 0, 0, 0, {}};
     // the launch's last CTA also refreshes the kernel-variant hints of the next step
     bt.scratch = w_sgd(b);
     bt.words = b->words;
@@ -765,10 +766,10 @@ nitro_status nitro_block_set_tensor(nitro_block* b, int which, int layer, const 
         uint32_t* word = which == NITRO_T_W ? w_w(b, layer) : w_wlr(b);
         if (cudaMemcpy(word, &m, 4, cudaMemcpyHostToDevice) != cudaSuccess) return NITRO_ERR_CUDA;
         if (which == NITRO_T_W &&
-            tc_refresh_weights(b->L[layer].tc, b->L[layer].g, b->L[layer].W, word, 0) != cudaSuccess)
+            tc_refresh_weights(b->L[layer].tc, b->L[layer].g, b->L[layer].W, word, 0, true) != cudaSuccess)
             return NITRO_ERR_CUDA;
         if (which == NITRO_T_W && b->L[layer].lin_planes &&
-            tc_pack_limbs(b->L[layer].W, b->L[layer].wcount, word, b->L[layer].lin_planes, 0) !=
+            tc_pack_limbs(b->L[layer].W, b->L[layer].wcount, nullptr, b->L[layer].lin_planes, 0) !=
                 cudaSuccess)
             return NITRO_ERR_CUDA;
     }

@@ -86,6 +86,10 @@ struct FloorDiv32 {
 #endif
         return (t + ((n - t) >> sh1)) >> sh2;
     }
+    __host__ __device__ __forceinline__ int32_t trunc_div(int32_t x) const {
+        const uint32_t q = udiv(x < 0 ? 0u - (uint32_t)x : (uint32_t)x);
+        return x < 0 ? (int32_t)(0u - q) : (int32_t)q;
+    }
     // branch-free: for x < 0, ~x = -(x + 1) and ~q = -q - 1
     __host__ __device__ __forceinline__ int32_t floor_div(int32_t x) const {
         const uint32_t ux = x >= 0 ? (uint32_t)x : ~(uint32_t)x;
@@ -328,9 +332,13 @@ struct SgdTensor {
     int64_t n;
     int64_t gamma_inv, eta_inv;
     uint32_t* maxabs_w;
-    FloorDiv gdiv, ediv;   // dividers for gamma_inv and eta_inv (filled by simt_integersgd)
+    // dividers for gamma_inv and eta_inv (filled by simt_integersgd): 64-bit gradients,
+    // gradients that fit 32 bits, weights
+    FloorDiv gdiv;
+    FloorDiv32 gdiv32, ediv32;
     // optional bf16 limb planes of a conv weight [Cout][9][cin] that the update
-    // writes itself: planes[l plane + co row_k + t tap_k + ci], all four limbs
+    // keeps itself: planes[l plane + co row_k + t tap_k + ci].  They hold all four
+    // limbs of W before and after (so that only what changes is stored)
     uint16_t* planes;
     int64_t plane;
     int row_k, tap_k, cin;

@@ -1255,7 +1255,7 @@ __global__ void __launch_bounds__(256) k_pack_delta_nhwc(const int32_t* __restri
                                                          int64_t n_zero) {
     pdl_wait();
     zero_fill(zero, n_zero);
-    const int L = limb_count(*maxabs);
+    const int L = maxabs ? limb_count(*maxabs) : kMaxLimbs;
     const int64_t n8 = n / 8;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n8;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -1287,7 +1287,7 @@ __global__ void __launch_bounds__(256) k_pack_delta_nhwc(const int32_t* __restri
 __global__ void k_pack_weights(const int32_t* __restrict__ W, int Cout, int Cin, int row_k,
                                int tap_k, const uint32_t* maxabs, uint16_t* __restrict__ wp) {
     pdl_wait();
-    const int L = limb_count(*maxabs);
+    const int L = maxabs ? limb_count(*maxabs) : kMaxLimbs;
     const int64_t n = (int64_t)Cout * 9 * Cin;
     const int64_t nk = (int64_t)Cout * row_k;
     auto split = [L](int64_t x, uint16_t* dst, int64_t plane) {
@@ -1570,14 +1570,14 @@ void tc_weight_planes(const TcLayer& t, const LayerGeom& g, uint16_t** planes, i
 }
 
 cudaError_t tc_refresh_weights(TcLayer& t, const LayerGeom& g, const int32_t* W,
-                               const uint32_t* maxabs_w, cudaStream_t s) {
+                               const uint32_t* maxabs_w, cudaStream_t s, bool all_planes) {
     if (!t.w_planes) return cudaSuccess;
     const int64_t n = (int64_t)g.cout * 9 * g.cin;
     {
         ProfScope ps(K_TC_PACK_W, s, 0.0, (double)n * 4 * 2);
         const int row_k = t.im2col ? kBK : 9 * t.cin_k, tap_k = t.im2col ? g.cin : t.cin_k;
-        launch_k(k_pack_weights, grid1d(n), 256, 0, s, W, g.cout, g.cin, row_k, tap_k, maxabs_w,
-                                                 t.w_planes);
+        launch_k(k_pack_weights, grid1d(n), 256, 0, s, W, g.cout, g.cin, row_k, tap_k,
+                 all_planes ? (const uint32_t*)nullptr : maxabs_w, t.w_planes);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !t.own_hints) return e;

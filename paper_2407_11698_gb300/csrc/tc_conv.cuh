@@ -108,9 +108,9 @@ void tc_weight_planes(const TcLayer& t, const LayerGeom& g, uint16_t** planes, i
 cudaError_t tc_weights_hint(TcLayer& t, cudaStream_t s);
 
 // Re-splits the layer's int32 weights into limb planes (after init, an update
-// or a checkpoint load); the limb count follows *maxabs_w.
+// or a checkpoint load); the limb count follows *maxabs_w unless all_planes.
 cudaError_t tc_refresh_weights(TcLayer& t, const LayerGeom& g, const int32_t* W,
-                               const uint32_t* maxabs_w, cudaStream_t s);
+                               const uint32_t* maxabs_w, cudaStream_t s, bool all_planes = false);
 
 // bf16 NHWC copy of the layer's int8 input for the forward and wgrad operands
 // (skipped when the previous layer's epilogue wrote it).
@@ -195,7 +195,7 @@ cudaError_t tc_maxabs(const int32_t* x, int64_t n, uint32_t* out, uint32_t* scra
 // also clears zero[0..n_zero)
 cudaError_t tc_pack_int8(const int8_t* x, int64_t rows, int cols, uint16_t* out, cudaStream_t s,
                          int64_t* zero = nullptr, int64_t n_zero = 0);
-// n % 8 == 0; planes [4][n], limb count from *maxabs
+// n % 8 == 0; planes [4][n], limb count from *maxabs (null: all four)
 cudaError_t tc_pack_limbs(const int32_t* x, int64_t n, const uint32_t* maxabs, uint16_t* planes,
                           cudaStream_t s);
 // C[m][n] (int64) = sum_k A[m][k] B[n][k]; A bf16 [M][K] (int8 values), B limb
