@@ -9,6 +9,7 @@
 // or small layers, linear weight and input gradients, linear forwards whose
 // input width is not a multiple of 8); the learning layer (G = 10 outputs) and
 // the element-wise stages always run here.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -216,159 +217,267 @@ __global__ void k_fwd_epilogue(const int64_t* __restrict__ z, LayerGeom g, int B
 }
 
 // ---------------------------------------------------------------------------
-// Learning layer forward + RSS loss, in one kernel.  A CTA (128-feature
-// slice, 16 samples) adds its partial sums of z[b][g] = sum_j a[b][j] W_lr[g][j]
-// into zsum with int64 atomics (exact, order independent).  The last CTA of
-// a sample group (per-group ticket) turns that group's z into
-// y_hat = floor(z / (256 d)) and grad_L = y_hat - 32 onehot and adds its part
-// of the SSE; the last of those (final ticket) writes the loss.
-// Behind zsum lie the tickets (zsum[B G + y] per group, then the final one),
-// the SSE and the maximum of |grad_L|.  All of it is zero between launches: the
-// CTA that consumes a word puts it back to zero, so no memset precedes the
-// launch, and the launch clears what the kernels after it accumulate into.
-// Six stream operations fewer per block step (with IntegerSGD's last CTA doing
-// the same for its words): the small MLP's step went from 152 to 109 us, the small CNN's
-// from 170 to 121 us, the VGG8B step from 1127 to 980 us.
-// Splitting this into a partial-sum kernel and a separate finish kernel
-// (per-slice partials with plain stores, or the atomic partials with a
-// one-read-per-output finish) was measured no faster: the second launch costs
-// what the fence and tickets save.
+// Learning layer forward: z[b][g] = sum_j a[b][j] W_lr[g][j], y_hat = floor(z /
+// (256 d)), grad_L = y_hat - 32 onehot.  A cluster takes eight samples; its CTAs
+// (up to eight) share out the features and exchange their partial sums through
+// distributed shared memory, so that no atomic, fence or ticket stands between
+// the sums and grad_L.  Warp u of a CTA takes sample u, 256 features a tile,
+// eight a lane, against W_lr split into signed 8-bit limbs in shared memory: one
+// dp4a a limb and four features, exact in 32 bits over 256 tiles.  W_lr with four
+// limbs (the top one may be +128, not a signed byte) takes 64-bit products.
+// Bound by latency (the loads of a tile go out before the one before it is summed)
+// and by launch overhead.  The kernel before it (64-bit products, 64-bit atomics into
+// a sum array, one ticket a sample group and one for the loss) took 15.3 us a launch
+// in the VGG8B step and 29 us with 47 classes, this one 10.7 and 17 (events included).
+// The loss, the SSE and max |grad_L| are left to the kernel after it (loss_tail),
+// off the chain; the launch clears what the rest of the backward adds into.
 // ---------------------------------------------------------------------------
-constexpr int kLrSamples = 16;   // samples per CTA
-constexpr int kLpSlice = 128;    // features per CTA
-static_assert(kLpSlice == 16 * 8, "k_learn_partial: 16 lanes of 8 features per sample");
+constexpr int kLfSamples = 8;      // samples per cluster, one warp each
+constexpr int kLfTile = 256;       // features per tile
+constexpr int kLfCluster = 8;      // CTAs per cluster at most
+constexpr int kLfG = 16;           // classes per pass
+constexpr int kMaxClasses = 64;
+constexpr int kLfSpan = 256;       // tiles per 32-bit sum
 
-__global__ void __launch_bounds__(256) k_learn_partial(const int8_t* __restrict__ a,
-                                                       const int32_t* __restrict__ wlr, int B,
-                                                       int d, int G, int vec8,
-                                                       unsigned long long* __restrict__ zsum,
-                                                       FloorDiv dv, const int32_t* __restrict__ labels,
-                                                       int32_t* __restrict__ grad_l,
-                                                       unsigned long long* sse, int64_t* loss,
-                                                       uint32_t* maxabs_gl, uint32_t* status,
-                                                       uint32_t* zero_words, int n_zero,
-                                                       int64_t* zero_dwlr) {
-    pdl_wait();
-    // nothing in this launch reads what is cleared here
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < n_zero) zero_words[threadIdx.x] = 0;
-    if (zero_dwlr) {
-        const int n = min(kLpSlice, d - (int)blockIdx.x * kLpSlice);
-        for (int g = blockIdx.y; g < G; g += gridDim.y)
-            if (threadIdx.x < n)
-                zero_dwlr[(int64_t)g * d + blockIdx.x * kLpSlice + threadIdx.x] = 0;
-    }
-    // thread (u, k): sample u of the group, features 8k .. 8k + 7 of the slice,
-    // read as one 8-byte word when the rows allow it (vec8: d % 8 == 0 and an
-    // 8-byte aligned a).  The slice of W_lr is staged in shared memory with
-    // feature 8k + m at column 16m + k, so the lanes of a sample read
-    // consecutive words; classes in chunks of kLpG.
-    constexpr int kLpG = 16;
-    __shared__ int32_t ws[kLpG][kLpSlice + 1];
-    const int u = threadIdx.x >> 4, k = threadIdx.x & 15;
-    const int b = blockIdx.y * kLrSamples + u;
-    const int j0 = blockIdx.x * kLpSlice;
-    const int jb = j0 + 8 * k;
-    int av[8];
-    if (vec8 && b < B && jb + 8 <= d) {
-        const uint2 w = *reinterpret_cast<const uint2*>(a + (int64_t)b * d + jb);
+struct LearnArgs {
+    const int8_t* a;
+    const int32_t* wlr;
+    int B, d, G, per;              // per: features per CTA, a multiple of the tile
+    int vec_a, vec_w;              // 8-byte rows of a, 16-byte rows of W_lr
+};
+
+// Eight features of one sample as bytes, zero past the row or the batch.
+__device__ __forceinline__ uint2 learn_load_a(const LearnArgs& p, int b, int j) {
+    uint2 v = make_uint2(0, 0);
+    if (b >= p.B || j >= p.d) return v;
+    const int8_t* src = p.a + (int64_t)b * p.d + j;
+    if (p.vec_a) return *reinterpret_cast<const uint2*>(src);
+    const int n = min(8, p.d - j);
+    for (int m = 0; m < n; ++m)
+        (m < 4 ? v.x : v.y) |= (uint32_t)(uint8_t)src[m] << (8 * (m & 3));
+    return v;
+}
+__device__ __forceinline__ int4 learn_load_w(const LearnArgs& p, int g, int j) {
+    int4 v = make_int4(0, 0, 0, 0);
+    if (g >= p.G || j >= p.d) return v;
+    const int32_t* src = p.wlr + (int64_t)g * p.d + j;
+    if (p.vec_w) return *reinterpret_cast<const int4*>(src);
+    v.x = src[0];
+    if (j + 1 < p.d) v.y = src[1];
+    if (j + 2 < p.d) v.z = src[2];
+    if (j + 3 < p.d) v.w = src[3];
+    return v;
+}
+
+// z of classes gc .. gc + GM - 1 for this warp's sample over features [j0, j1): lane
+// g returns class gc + g.  ws: GM rows of one tile, L limb words of four features.
+template <int GM, int L>
+__device__ __forceinline__ long long learn_dots(const LearnArgs& p, int b, int gc, int j0, int j1,
+                                                uint32_t* ws) {
+    constexpr int kPer = (GM * (kLfTile / 4) + 255) / 256;   // groups of four weights a thread
+    const int lane = threadIdx.x & 31, wd = threadIdx.x & 63, gr = threadIdx.x >> 6;
+    long long z = 0;
+    int acc[GM][L];
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            av[m] = (int8_t)(w.x >> (8 * m));
-            av[4 + m] = (int8_t)(w.y >> (8 * m));
-        }
-    } else {
+    for (int g = 0; g < GM; ++g)
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            const int j = jb + m;
-            av[m] = (b < B && j < d) ? a[(int64_t)b * d + j] : 0;
-        }
-    }
-    for (int gc = 0; gc < G; gc += kLpG) {
-        const int ng = min(kLpG, G - gc);
-        if (gc) __syncthreads();
-        for (int i = threadIdx.x; i < ng * kLpSlice; i += blockDim.x) {
-            const int g = i / kLpSlice, j = i - g * kLpSlice;
-            ws[g][(j & 7) * 16 + (j >> 3)] = j0 + j < d ? wlr[(int64_t)(gc + g) * d + j0 + j] : 0;
+        for (int l = 0; l < L; ++l) acc[g][l] = 0;
+    uint2 av = learn_load_a(p, b, j0 + 8 * lane);
+    int4 wv[kPer];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) wv[i] = learn_load_w(p, gc + gr + 4 * i, j0 + 4 * wd);
+    int tile = 0;
+    for (int j = j0; j < j1; j += kLfTile) {
+        __syncthreads();                       // readers of the tile before are done
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int g = gr + 4 * i;
+            if (g >= GM) break;
+            // byte l of w + 0x808080 is digit l + 128; xor 0x80 makes it signed
+            const uint32_t t0 = (uint32_t)wv[i].x + 0x808080u, t1 = (uint32_t)wv[i].y + 0x808080u;
+            const uint32_t t2 = (uint32_t)wv[i].z + 0x808080u, t3 = (uint32_t)wv[i].w + 0x808080u;
+#pragma unroll
+            for (int l = 0; l < L; ++l) {
+                const uint32_t sel = l | ((4 + l) << 4);
+                const uint32_t lo = __byte_perm(t0, t1, sel), hi = __byte_perm(t2, t3, sel);
+                ws[(l * GM + g) * 64 + wd] = __byte_perm(lo, hi, 0x5410) ^ 0x80808080u;
+            }
         }
         __syncthreads();
-        for (int g = 0; g < ng; ++g) {
-            long long t = 0;
+        const uint2 ac = av;
+        if (j + kLfTile < j1) {
+            av = learn_load_a(p, b, j + kLfTile + 8 * lane);
 #pragma unroll
-            for (int m = 0; m < 8; ++m) t += (long long)ws[g][16 * m + k] * av[m];
+            for (int i = 0; i < kPer; ++i)
+                wv[i] = learn_load_w(p, gc + gr + 4 * i, j + kLfTile + 4 * wd);
+        }
 #pragma unroll
-            for (int off = 8; off; off >>= 1) t += __shfl_xor_sync(kFull, t, off);
-            if (k == 0 && b < B && t != 0)
-                atomicAdd(&zsum[(int64_t)b * G + gc + g], (unsigned long long)t);
+        for (int g = 0; g < GM; ++g)
+#pragma unroll
+            for (int l = 0; l < L; ++l) {
+                const uint2 w = *reinterpret_cast<const uint2*>(&ws[(l * GM + g) * 64 + 2 * lane]);
+                acc[g][l] = __dp4a((int)ac.x, (int)w.x, acc[g][l]);
+                acc[g][l] = __dp4a((int)ac.y, (int)w.y, acc[g][l]);
+            }
+        if (++tile == kLfSpan || j + kLfTile >= j1) {
+            // at most 256 tiles x 256 features x 2^14 = 2^30 a limb
+            tile = 0;
+#pragma unroll
+            for (int g = 0; g < GM; ++g) {
+                long long t = 0;
+#pragma unroll
+                for (int l = 0; l < L; ++l) {
+                    t += (long long)__reduce_add_sync(kFull, acc[g][l]) << (8 * l);
+                    acc[g][l] = 0;
+                }
+                if (lane == g) z += t;
+            }
         }
     }
-    __shared__ int last;
-    __shared__ unsigned long long red_s[8];
-    __shared__ uint32_t red_m[8];
-    __shared__ int flags;
-    unsigned long long* tickets = zsum + (int64_t)B * G;
-    unsigned long long* total = tickets + gridDim.y + 1;   // SSE, then max |grad_L|
-    if (k == 0) __threadfence();     // the lanes that added into zsum
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        flags = 0;
-        last = atomicAdd(&tickets[blockIdx.y], 1ull) == (unsigned long long)gridDim.x - 1;
+    return z;
+}
+
+// The same with 64-bit products of the whole weights (four limbs); ws: one tile of
+// kLfG rows, one class at a time.
+__device__ __noinline__ long long learn_dots_wide(const LearnArgs& p, int b, int gc, int j0, int j1) {
+    const int lane = threadIdx.x & 31;
+    long long z = 0;
+    for (int g = 0; g < min(kLfG, p.G - gc); ++g) {
+        long long t = 0;
+        for (int j = j0 + lane; j < min(j1, p.d); j += 32)
+            if (b < p.B)
+                t += (long long)p.a[(int64_t)b * p.d + j] * p.wlr[(int64_t)(gc + g) * p.d + j];
+#pragma unroll
+        for (int off = 16; off; off >>= 1) t += __shfl_xor_sync(kFull, t, off);
+        if (lane == g) z = t;
     }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    // this sample group's z is complete: y_hat, grad_L, its share of the SSE
+    return z;
+}
+
+template <int GM>
+__device__ __forceinline__ long long learn_pass(const LearnArgs& p, int limbs, int b, int gc, int j0,
+                                                int j1, uint32_t* ws) {
+    if (limbs == 1) return learn_dots<GM, 1>(p, b, gc, j0, j1, ws);
+    if (limbs == 2) return learn_dots<GM, 2>(p, b, gc, j0, j1, ws);
+    if (limbs == 3) return learn_dots<GM, 3>(p, b, gc, j0, j1, ws);
+    return learn_dots_wide(p, b, gc, j0, j1);
+}
+
+__global__ void __launch_bounds__(256) k_learn_fwd(const LearnArgs p, FloorDiv dv,
+                                                   const int32_t* __restrict__ labels,
+                                                   int32_t* __restrict__ grad_l,
+                                                   const uint32_t* maxabs_wlr, uint32_t* status,
+                                                   uint32_t* zero_words, int n_zero,
+                                                   int64_t* zero_dwlr) {
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    __shared__ __align__(16) uint32_t ws[3 * kLfG * 64];
+    __shared__ long long part[kLfSamples][kMaxClasses];
+    const int u = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int group = blockIdx.x / S, groups = gridDim.x / S;
+    const int b = group * kLfSamples + u;
+    pdl_wait();
+    const int limbs = limb_count(*maxabs_wlr);
+    // nothing in this launch reads what is cleared here
+    if (blockIdx.x == 0 && threadIdx.x < n_zero) zero_words[threadIdx.x] = 0;
+    const int j0 = rank * p.per, j1 = min(p.d, j0 + p.per);
+    if (zero_dwlr)
+        for (int g = group; g < p.G; g += groups)
+            for (int j = j0 + threadIdx.x; j < j1; j += 256) zero_dwlr[(int64_t)g * p.d + j] = 0;
+    for (int gc = 0; gc < p.G; gc += kLfG) {
+        const long long z = p.G <= 10 ? learn_pass<10>(p, limbs, b, gc, j0, j1, ws)
+                                      : learn_pass<kLfG>(p, limbs, b, gc, j0, j1, ws);
+        if (lane < min(kLfG, p.G - gc)) part[u][gc + lane] = z;
+    }
+    cluster.sync();
+    // sample v of the group is finished by CTA v mod S
+    for (int i = threadIdx.x; i < kLfSamples * p.G; i += 256) {
+        const int v = i / p.G, g = i - v * p.G, bb = group * kLfSamples + v;
+        if (v % S != rank || bb >= p.B) continue;
+        long long z = 0;
+        for (int r = 0; r < S; ++r) z += *cluster.map_shared_rank(&part[v][g], r);
+        const int lab = labels[bb];
+        const bool bad = lab < 0 || lab >= p.G;
+        // NITRO-Scaling, SF = 2^8 d: floor(floor(z / 256) / d)
+        const int64_t yhat = dv.floor_div((int64_t)z >> 8);
+        const int64_t t = yhat - ((!bad && g == lab) ? 32 : 0);
+        if (bad && g == 0) atomicOr(status, ST_BAD_LABEL);
+        if (!fits_i32(t)) atomicOr(status, ST_OVERFLOW);
+        grad_l[(int64_t)bb * p.G + g] = (int32_t)t;
+    }
+    cluster.sync();      // the partial sums stay until every CTA has read them
+}
+
+// The last CTA column of the kernel after k_learn_fwd: SSE, loss = floor(SSE / 2),
+// max |grad_L| and, with wlr_max != null, the int64 exactness bound of grad_L W_lr.
+// One CTA forms them up to kTailValues values; above, the column's CTAs add their
+// shares into *sse and *maxabs_gl (cleared by k_learn_fwd) and the last one ends.
+struct LossTail {
+    const int32_t* grad_l;
+    int B, G;
+    unsigned long long* sse;
+    int64_t* loss;               // may be null
+    uint32_t* maxabs_gl;
+    uint32_t* ticket;            // cleared by k_learn_fwd
+    const uint32_t* wlr_max;
+    uint32_t* status;
+};
+constexpr int kTailValues = 8192;
+__device__ __forceinline__ void loss_tail(const LossTail& t) {
+    const int64_t n = (int64_t)t.B * t.G;
+    const int ctas = (int)min((int64_t)gridDim.y, (n + kTailValues - 1) / kTailValues);
+    if ((int)blockIdx.y >= ctas) return;
     unsigned long long ss = 0;
     uint32_t mx = 0;
-    int fl = 0;
-    const int nb = min(kLrSamples, B - (int)blockIdx.y * kLrSamples);
-    for (int i = threadIdx.x; i < nb * G; i += blockDim.x) {
-        const int bb = blockIdx.y * kLrSamples + i / G, g = i % G;
-        const int lab = labels[bb];
-        const bool bad = lab < 0 || lab >= G;
-        if (bad && g == 0) fl |= ST_BAD_LABEL;
-        // NITRO-Scaling, SF = 2^8 d: floor(floor(z / 256) / d)
-        const int64_t yhat = dv.floor_div((int64_t)__ldcg(zsum + (int64_t)bb * G + g) >> 8);
-        zsum[(int64_t)bb * G + g] = 0;
-        const int64_t v = yhat - ((!bad && g == lab) ? 32 : 0);
-        if (!fits_i32(v)) fl |= ST_OVERFLOW;
-        const int32_t sv = (int32_t)v;
-        grad_l[(int64_t)bb * G + g] = sv;
-        ss += (unsigned long long)((int64_t)sv * sv);
-        mx = max(mx, abs_u32(sv));
+    for (int64_t i = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; i < n; i += (int64_t)ctas * blockDim.x) {
+        const int32_t v = t.grad_l[i];
+        ss += (unsigned long long)((int64_t)v * v);              // modulo 2^64
+        mx = max(mx, abs_u32(v));
     }
+    __shared__ unsigned long long sum;
+    __shared__ uint32_t top;
+    if (threadIdx.x == 0) {
+        sum = 0;
+        top = 0;
+    }
+    __syncthreads();
 #pragma unroll
-    for (int off = 16; off; off >>= 1) {
-        ss += __shfl_xor_sync(kFull, ss, off);
-        mx = max(mx, __shfl_xor_sync(kFull, mx, off));
+    for (int off = 16; off; off >>= 1) ss += __shfl_xor_sync(kFull, ss, off);
+    mx = __reduce_max_sync(kFull, mx);
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&sum, ss);
+        atomicMax(&top, mx);
     }
-    if (fl) atomicOr(&flags, fl);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) { red_s[warp] = ss; red_m[warp] = mx; }
     __syncthreads();
     if (threadIdx.x == 0) {
-        unsigned long long t = 0;
-        uint32_t m = 0;
-        for (int w = 0; w < 8; ++w) { t += red_s[w]; m = max(m, red_m[w]); }
-        tickets[blockIdx.y] = 0;
-        atomicAdd(&total[0], t);                             // modulo 2^64
-        if (m) atomicMax(&total[1], (unsigned long long)m);
-        if (flags) atomicOr(status, (uint32_t)flags);
-        __threadfence();
-        if (atomicAdd(&tickets[gridDim.y], 1ull) == (unsigned long long)gridDim.y - 1) {
+        unsigned long long total = sum;
+        uint32_t most = top;
+        if (ctas > 1) {
+            atomicAdd(t.sse, total);
+            atomicMax(t.maxabs_gl, most);
             __threadfence();
-            const unsigned long long tot = atomicExch(&total[0], 0ull);
-            *sse = tot;
-            *maxabs_gl = (uint32_t)atomicExch(&total[1], 0ull);
-            if (loss) *loss = fdiv64((int64_t)tot, 2);
-            tickets[gridDim.y] = 0;
+            if (atomicAdd(t.ticket, 1u) != (uint32_t)ctas - 1) return;
+            __threadfence();
+            total = atomicAdd(t.sse, 0ull);
+            most = atomicMax(t.maxabs_gl, 0u);
+        } else {
+            *t.sse = total;
+            *t.maxabs_gl = most;
         }
+        if (t.loss) *t.loss = fdiv64((int64_t)total, 2);
+        if (t.wlr_max && int64_bound_exceeded(most, *t.wlr_max, t.G)) atomicOr(t.status, ST_OVERFLOW);
     }
 }
 
-// dW_lr[g][j] = sum_b grad_l[b][g] * a[b][j]
+// dW_lr[g][j] = sum_b grad_l[b][g] * a[b][j]; the last CTA column forms the loss
 __global__ void k_learn_dw(const int8_t* __restrict__ a, const int32_t* __restrict__ grad_l,
-                           int B, int d, int G, int64_t* __restrict__ dwlr) {
+                           int B, int d, int G, int64_t* __restrict__ dwlr, const LossTail tail) {
     pdl_wait();
+    if (blockIdx.x == gridDim.x - 1) {
+        loss_tail(tail);
+        return;
+    }
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     const int g = blockIdx.y;
     if (j >= d) return;
@@ -428,13 +537,7 @@ __global__ void k_grad_to_delta(DeltaSrc src, LayerGeom g, int B, int alpha_inv,
             mx = max(mx, abs_u32(dv));
         }
     }
-#pragma unroll
-    for (int off = 16; off; off >>= 1) mx = max(mx, __shfl_xor_sync(kFull, mx, off));
-    ovf = __any_sync(kFull, ovf);
-    if ((threadIdx.x & 31) == 0) {
-        if (mx) atomicMax(maxabs_delta, mx);
-        if (ovf) atomicOr(status, ST_OVERFLOW);
-    }
+    block_maximum(mx, ovf, maxabs_delta, status);
 }
 
 // ---------------------------------------------------------------------------
@@ -559,13 +662,7 @@ __global__ void k_lrpool_to_delta(const int32_t* __restrict__ gl, const int32_t*
         delta[i] = dv;
         mx = max(mx, abs_u32(dv));
     }
-#pragma unroll
-    for (int off = 16; off; off >>= 1) mx = max(mx, __shfl_xor_sync(kFull, mx, off));
-    ovf = __any_sync(kFull, ovf);
-    if ((threadIdx.x & 31) == 0) {
-        if (mx) atomicMax(maxabs_delta, mx);
-        if (ovf) atomicOr(status, ST_OVERFLOW);
-    }
+    block_maximum(mx, ovf, maxabs_delta, status);
 }
 
 // Same by windows, four channels per thread (C % 4 == 0): a thread takes the
@@ -972,10 +1069,13 @@ __global__ void __launch_bounds__(256) k_lr_backward(const int8_t* __restrict__ 
                                                      const int8_t* __restrict__ argmax,
                                                      int32_t* __restrict__ delta,
                                                      unsigned long long* __restrict__ dwlr,
-                                                     const uint32_t* maxabs_gl,
-                                                     const uint32_t* maxabs_wlr,
-                                                     uint32_t* maxabs_delta, uint32_t* status) {
+                                                     uint32_t* maxabs_delta, uint32_t* status,
+                                                     const LossTail tail) {
     pdl_wait();
+    if (blockIdx.x == gridDim.x - 1) {        // the last column of the grid: the loss
+        loss_tail(tail);
+        return;
+    }
     __shared__ int32_t gls[kLbSamples][GM];
     __shared__ int8_t as[kLbSamples][kLbQ];
     const int ql = threadIdx.x % kLbQ, sl = threadIdx.x / kLbQ;
@@ -991,9 +1091,6 @@ __global__ void __launch_bounds__(256) k_lr_backward(const int8_t* __restrict__ 
         const int u = sl + kLbLanes * i;
         as[u][ql] = (u < nb && q < d) ? a[(int64_t)(b0 + u) * d + q] : (int8_t)0;
     }
-    if (has_delta && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 &&
-        int64_bound_exceeded(*maxabs_gl, *maxabs_wlr, G))
-        atomicOr(status, ST_OVERFLOW);
     // loads of the delta path (W_lr column, argmax, region bytes) go out with
     // the staging loads, before the barrier
     const bool act = has_delta && q < d;
@@ -1068,13 +1165,7 @@ __global__ void __launch_bounds__(256) k_lr_backward(const int8_t* __restrict__ 
             }
         }
     }
-#pragma unroll
-    for (int off = 16; off; off >>= 1) mx = max(mx, __shfl_xor_sync(kFull, mx, off));
-    ovf = __any_sync(kFull, ovf);
-    if ((threadIdx.x & 31) == 0) {
-        if (mx) atomicMax(maxabs_delta, mx);
-        if (ovf) atomicOr(status, ST_OVERFLOW);
-    }
+    block_maximum(mx, ovf, maxabs_delta, status);
 }
 
 // Same, four features per thread when the last layer's channel count is a
@@ -1093,10 +1184,13 @@ __global__ void __launch_bounds__(16 * NS) k_lr_backward4(const int8_t* __restri
                                                       const int8_t* __restrict__ argmax,
                                                       int32_t* __restrict__ delta,
                                                       unsigned long long* __restrict__ dwlr,
-                                                      const uint32_t* maxabs_gl,
-                                                      const uint32_t* maxabs_wlr,
-                                                      uint32_t* maxabs_delta, uint32_t* status) {
+                                                      uint32_t* maxabs_delta, uint32_t* status,
+                                                      const LossTail tail) {
     pdl_wait();
+    if (blockIdx.x == gridDim.x - 1) {        // the last column of the grid: the loss
+        loss_tail(tail);
+        return;
+    }
     __shared__ int32_t gls[NS][GM];
     __shared__ int8_t as[NS][kLbQ];
     __shared__ __align__(16) int32_t wsl[GM][kLbQ];
@@ -1116,9 +1210,6 @@ __global__ void __launch_bounds__(16 * NS) k_lr_backward4(const int8_t* __restri
         const int g = i / kLbQ, qq = i % kLbQ;
         wsl[g][qq] = (g < G && q0 + qq < d) ? wlr[(int64_t)g * d + q0 + qq] : 0;
     }
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 &&
-        int64_bound_exceeded(*maxabs_gl, *maxabs_wlr, G))
-        atomicOr(status, ST_OVERFLOW);
     // loads of the delta path go out with the staging loads, before the barrier
     const bool act = q < d && u < nb;      // d % 4 == 0: all four features valid
     int64_t base = 0, dx = 0, dy = 0;
@@ -1188,13 +1279,7 @@ __global__ void __launch_bounds__(16 * NS) k_lr_backward4(const int8_t* __restri
             *reinterpret_cast<int4*>(delta + base) = make_int4(dv[0], dv[1], dv[2], dv[3]);
         }
     }
-#pragma unroll
-    for (int off = 16; off; off >>= 1) mx = max(mx, __shfl_xor_sync(kFull, mx, off));
-    ovf = __any_sync(kFull, ovf);
-    if ((threadIdx.x & 31) == 0) {
-        if (mx) atomicMax(maxabs_delta, mx);
-        if (ovf) atomicOr(status, ST_OVERFLOW);
-    }
+    block_maximum(mx, ovf, maxabs_delta, status);
 }
 
 inline int grid_for(int64_t n, int threads, int cap = 152 * 16) {
@@ -1332,33 +1417,34 @@ cudaError_t simt_lrpool_to_delta(const int32_t* gl, const int32_t* wlr, int G, i
     return cudaGetLastError();
 }
 
-size_t simt_learn_scratch(int max_batch, int d, int G) {
-    (void)d;
-    return (size_t)max_batch * G + (max_batch + kLrSamples - 1) / kLrSamples + 3;
+cudaError_t simt_learn_fwd(const int8_t* a, const int32_t* wlr, const int32_t* labels, int B,
+                           int d, int G, int32_t* grad_l, const uint32_t* maxabs_wlr,
+                           uint32_t* status, uint32_t* zero_words, int n_zero, int64_t* zero_dwlr,
+                           cudaStream_t s) {
+    if (B <= 0) return cudaSuccess;
+    if (n_zero > 256 || G > kMaxClasses) return cudaErrorInvalidValue;
+    int S = 1;
+    while (S < kLfCluster && S * kLfTile < d) S *= 2;
+    LearnArgs p{a, wlr, B, d, G, 0, d % 8 == 0 && ((uintptr_t)a & 7) == 0,
+                d % 4 == 0 && ((uintptr_t)wlr & 15) == 0};
+    p.per = ((d + S - 1) / S + kLfTile - 1) / kLfTile * kLfTile;
+    ProfScope ps(K_LEARN_FWD, s, 2.0 * B * d * G, 0.0);
+    return launch_cluster(k_learn_fwd, S * ((B + kLfSamples - 1) / kLfSamples), 256, S, s, p,
+                          FloorDiv::make((uint64_t)d), labels, grad_l, maxabs_wlr, status, zero_words,
+                          n_zero, zero_dwlr);
 }
 
-cudaError_t simt_learn_fwd(const int8_t* a, const int32_t* wlr, const int32_t* labels, int B,
-                           int d, int G, int64_t* zsum, int32_t* grad_l, unsigned long long* sse,
-                           int64_t* loss, uint32_t* maxabs_gl, uint32_t* status,
-                           uint32_t* zero_words, int n_zero, int64_t* zero_dwlr, cudaStream_t s) {
-    if (B <= 0) return cudaSuccess;
-    if (n_zero > 256) return cudaErrorInvalidValue;
-    const int groups = (B + kLrSamples - 1) / kLrSamples;
-    dim3 grid((d + kLpSlice - 1) / kLpSlice, groups);
-    ProfScope ps(K_LEARN_FWD, s, 2.0 * B * d * G, 0.0);
-    const int vec8 = d % 8 == 0 && ((uintptr_t)a & 7) == 0;
-    launch_k(k_learn_partial, grid, 256, 0, s, a, wlr, B, d, G, vec8,
-                                         reinterpret_cast<unsigned long long*>(zsum),
-                                         FloorDiv::make((uint64_t)d), labels, grad_l, sse, loss,
-                                         maxabs_gl, status, zero_words, n_zero, zero_dwlr);
-    return cudaGetLastError();
+namespace {
+LossTail loss_args(const int32_t* gl, int B, int G, const LossOut& o) {
+    return LossTail{gl, B, G, o.sse, o.loss, o.maxabs_gl, o.ticket, o.wlr_max, o.status};
 }
+}  // namespace
 
 cudaError_t simt_learn_dw(const int8_t* a, const int32_t* grad_l, int B, int d, int G,
-                          int64_t* dwlr, cudaStream_t s) {
-    dim3 grid((d + 255) / 256, G);
+                          int64_t* dwlr, const LossOut& lo, cudaStream_t s) {
+    dim3 grid((d + 255) / 256 + 1, G);
     ProfScope ps(K_LEARN_DW, s, 2.0 * B * d * G, 0.0);
-    launch_k(k_learn_dw, grid, 256, 0, s, a, grad_l, B, d, G, dwlr);
+    launch_k(k_learn_dw, grid, 256, 0, s, a, grad_l, B, d, G, dwlr, loss_args(grad_l, B, G, lo));
     return cudaGetLastError();
 }
 
@@ -1463,19 +1549,20 @@ bool simt_lr_backward_ok(int G) { return G <= kLbMaxG; }
 cudaError_t simt_lr_backward(const int8_t* a, const int32_t* gl, const int32_t* wlr, int B, int G,
                              int d, const LayerGeom* lg, int alpha_inv, const int8_t* region,
                              const int8_t* argmax, int32_t* delta, int64_t* dwlr,
-                             const uint32_t* maxabs_gl, const uint32_t* maxabs_wlr,
-                             uint32_t* maxabs_delta, uint32_t* status, cudaStream_t s) {
+                             uint32_t* maxabs_delta, uint32_t* status, const LossOut& lo,
+                             cudaStream_t s) {
     cudaError_t e = cudaSuccess;
     if (B <= 0) return e;
     if (lg && lg->pool && ((lg->h & 1) || (lg->w & 1))) {   // rows / columns the pool dropped
         e = cudaMemsetAsync(delta, 0, sizeof(int32_t) * (size_t)B * lg->h * lg->w * lg->cout, s);
         if (e != cudaSuccess) return e;
     }
-    dim3 grid((d + kLbQ - 1) / kLbQ, (B + kLbSamples - 1) / kLbSamples);
+    dim3 grid((d + kLbQ - 1) / kLbQ + 1, (B + kLbSamples - 1) / kLbSamples);   // + the loss column
     // the four-feature kernel takes 32 samples per CTA (half the weight-gradient
     // atomics of 16) when the batch fills them
     constexpr int kLb4Samples = 32;
-    dim3 grid4((d + kLbQ - 1) / kLbQ, (B + kLb4Samples - 1) / kLb4Samples);
+    dim3 grid4((d + kLbQ - 1) / kLbQ + 1, (B + kLb4Samples - 1) / kLb4Samples);
+    const LossTail tail = loss_args(gl, B, G, lo);
     ProfScope ps(K_LR_BACKWARD, s, (lg ? 4.0 : 2.0) * B * d * G, 0.0);
     const FloorDiv32 al = FloorDiv32::make((uint32_t)(alpha_inv > 0 ? alpha_inv : 1));
     auto* dw64 = reinterpret_cast<unsigned long long*>(dwlr);
@@ -1488,22 +1575,19 @@ cudaError_t simt_lr_backward(const int8_t* a, const int32_t* gl, const int32_t* 
     if (quad) {
         if (G <= 10)
             launch_k(k_lr_backward4<10, kLb4Samples>, grid4, 16 * kLb4Samples, 0, s,
-                a, gl, wlr, B, G, d, g0, al, region, argmax, delta, dw64, maxabs_gl, maxabs_wlr,
-                maxabs_delta, status);
+                a, gl, wlr, B, G, d, g0, al, region, argmax, delta, dw64, maxabs_delta, status, tail);
         else
             launch_k(k_lr_backward4<kLbMaxG, kLb4Samples>, grid4, 16 * kLb4Samples, 0, s,
-                a, gl, wlr, B, G, d, g0, al, region, argmax, delta, dw64, maxabs_gl, maxabs_wlr,
-                maxabs_delta, status);
+                a, gl, wlr, B, G, d, g0, al, region, argmax, delta, dw64, maxabs_delta, status, tail);
         return cudaGetLastError();
     }
     if (G <= 10)
         launch_k(k_lr_backward<10>, grid, 256, 0, s, a, gl, wlr, B, G, d, lg != nullptr, g0, al, region,
-                                               argmax, delta, dw64, maxabs_gl, maxabs_wlr,
-                                               maxabs_delta, status);
+                                               argmax, delta, dw64, maxabs_delta, status, tail);
     else
         launch_k(k_lr_backward<kLbMaxG>, grid, 256, 0, s, a, gl, wlr, B, G, d, lg != nullptr, g0, al,
-                                                    region, argmax, delta, dw64, maxabs_gl,
-                                                    maxabs_wlr, maxabs_delta, status);
+                                                    region, argmax, delta, dw64, maxabs_delta, status,
+                                                    tail);
     return cudaGetLastError();
 }
 

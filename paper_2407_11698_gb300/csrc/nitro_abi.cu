@@ -50,13 +50,13 @@ struct nitro_block {
     int32_t* Wlr = nullptr;
     int64_t* dWlr = nullptr;
     int32_t* grad_l = nullptr;      // [max_batch x G]
-    int64_t* zsum = nullptr;        // learning-layer partial sums and ticket (simt_learn_scratch)
     int64_t* z64 = nullptr;         // scratch, int64 pre-activations / dgrad outputs
     size_t z64_elems = 0;
     uint32_t* words = nullptr;      // [0] status [1] step counter (dropout masks)
                                     // [2] max|W_lr| [3 + i] max|W_i|    (reset by the update)
                                     // [3 + n] max|grad_l| [4 + n + i] max|delta_i|, then the
-                                    // SSE (8-byte aligned)              (reset by the backward)
+                                    // SSE (8-byte aligned) and the loss ticket (reset by the
+                                    // backward)
     uint32_t* words_host = nullptr; // pinned copy of the words, refreshed once per step: the
                                     // limb-count hints that pick kernel variants
     uint64_t seed = 0;
@@ -78,7 +78,7 @@ uint32_t* w_w(nitro_block* b, int i) { return b->words + 3 + i; }
 uint32_t* w_gl(nitro_block* b) { return b->words + 3 + (int)b->L.size(); }
 uint32_t* w_delta(nitro_block* b, int i) { return b->words + 4 + (int)b->L.size() + i; }
 int sse_word(int n_layers) { return (4 + 2 * n_layers + 1) & ~1; }   // 8-byte aligned
-int n_words(int n_layers) { return sse_word(n_layers) + 2; }
+int n_words(int n_layers) { return sse_word(n_layers) + 3; }   // + the loss ticket
 // behind them, IntegerSGD's scratch (zero between launches)
 uint32_t* w_sgd(nitro_block* b) { return b->words + n_words((int)b->L.size()); }
 
@@ -276,7 +276,7 @@ nitro_status nitro_init_block(const nitro_block_desc* desc, uint64_t seed, void*
         }
     }
     ok = ok && dalloc(b, &b->Wlr, (size_t)b->G * b->d) && dalloc(b, &b->dWlr, (size_t)b->G * b->d) &&
-         dalloc(b, &b->grad_l, (size_t)MB * b->G) && dalloc(b, &b->zsum, simt_learn_scratch(MB, (int)b->d, b->G)) && dalloc(b, &b->z64, z_need) &&
+         dalloc(b, &b->grad_l, (size_t)MB * b->G) && dalloc(b, &b->z64, z_need) &&
          dalloc(b, &b->words, n_words(desc->n_layers) + kSgdScratchWords);
     if (ok) {
         b->sse = reinterpret_cast<unsigned long long*>(b->words + sse_word(desc->n_layers));
@@ -316,8 +316,6 @@ nitro_status nitro_init_block(const nitro_block_desc* desc, uint64_t seed, void*
     if (e == cudaSuccess) e = cudaMemsetAsync(b->dWlr, 0, (size_t)b->G * b->d * 8, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->words, words.data(), words.size() * 4, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->sse, 0, 8, s);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(b->zsum, 0, 8 * simt_learn_scratch(MB, (int)b->d, b->G), s);
     for (int i = 0; e == cudaSuccess && i < desc->n_layers; ++i) {
         // all four limb planes: IntegerSGD stores only what changes in them
         e = tc_refresh_weights(b->L[i].tc, b->L[i].g, b->L[i].W, w_w(b, i), s, true);
@@ -436,19 +434,23 @@ nitro_status block_backward(nitro_block* b, const int8_t* a_in, const int32_t* l
                                    b->lp.ph, b->lp.pw, b->zmp, b->lr_am, s));
         a_last = b->zmp;
     }
-    // also resets the max |delta| words and dW_lr for the kernels below
-    NITRO_TRY(simt_learn_fwd(a_last, b->Wlr, labels, batch, (int)d, G, b->zsum, b->grad_l, b->sse,
-                             loss_dev, w_gl(b), w_status(b), w_gl(b) + 1, n,
+    // also resets the per-step words and dW_lr for the kernels below
+    NITRO_TRY(simt_learn_fwd(a_last, b->Wlr, labels, batch, (int)d, G, b->grad_l, w_wlr(b),
+                             w_status(b), w_gl(b), n_words(n) - (3 + n),
                              simt_lr_backward_ok(G) ? b->dWlr : nullptr, s));
+    // the kernel after it forms the loss; where that kernel also forms delta_fw, it
+    // checks the bound of grad_L W_lr as well
+    LossOut lo{b->sse, loss_dev, w_gl(b), b->words + n_words(n) - 1, n && !b->zmp && simt_lr_backward_ok(G) ? w_wlr(b) : nullptr,
+               w_status(b)};
     if (b->zmp) {
         // learning-weight gradient from z^mp, then delta_fw back through the
         // learning pool into the last layer's delta (pre-update W_lr)
         if (simt_lr_backward_ok(G))
             NITRO_TRY(simt_lr_backward(a_last, b->grad_l, b->Wlr, batch, G, (int)d, nullptr,
                                        b->desc.alpha_inv, nullptr, nullptr, nullptr, b->dWlr,
-                                       w_gl(b), w_wlr(b), nullptr, w_status(b), s));
+                                       nullptr, w_status(b), lo, s));
         else
-            NITRO_TRY(simt_learn_dw(a_last, b->grad_l, batch, (int)d, G, b->dWlr, s));
+            NITRO_TRY(simt_learn_dw(a_last, b->grad_l, batch, (int)d, G, b->dWlr, lo, s));
         // (and its limb planes; the launch also clears dW for a split weight gradient)
         Layer& ly = b->L[n - 1];
         NITRO_TRY(simt_lrpool_to_delta(b->grad_l, b->Wlr, G, (int)d, ly.g, b->lp, batch, b->lr_am,
@@ -463,9 +465,9 @@ nitro_status block_backward(nitro_block* b, const int8_t* a_in, const int32_t* l
         NITRO_TRY(simt_lr_backward(a_last, b->grad_l, b->Wlr, batch, G, (int)d, ly ? &ly->g : nullptr,
                                    b->desc.alpha_inv, ly ? ly->region : nullptr,
                                    ly ? ly->argmax : nullptr, ly ? ly->delta : nullptr, b->dWlr,
-                                   w_gl(b), w_wlr(b), n ? w_delta(b, n - 1) : nullptr, w_status(b), s));
+                                   n ? w_delta(b, n - 1) : nullptr, w_status(b), lo, s));
     } else {
-        NITRO_TRY(simt_learn_dw(a_last, b->grad_l, batch, (int)d, G, b->dWlr, s));
+        NITRO_TRY(simt_learn_dw(a_last, b->grad_l, batch, (int)d, G, b->dWlr, lo, s));
     }
     if (n == 0) return NITRO_OK;
     // delta_fw = grad_L W_lr (pre-update), into the last layer

@@ -267,23 +267,30 @@ cudaError_t simt_lrpool_to_delta(const int32_t* gl, const int32_t* wlr, int G, i
                                  const uint32_t* maxabs_wlr, uint32_t* maxabs_delta,
                                  uint32_t* status, cudaStream_t s);
 
-// Learning layer forward + loss: grad_l = floor(a W^T / (256 d)) - 32 onehot,
-// sse = sum grad_l^2 (mod 2^64), loss = floor(sse / 2) (if loss != NULL),
-// max|grad_l| into *maxabs_gl, status bits.  scratch: int64 buffer of
-// simt_learn_scratch(max_batch, d, G) words (partial sums, tickets, SSE and
-// maximum), zero before the first call and left zero by every call.
-// The launch also clears what the rest of the backward accumulates into, which
-// saves a memset each: zero_words[0..n_zero) and, when zero_dwlr is not null,
-// the G d values of dW_lr.
-size_t simt_learn_scratch(int max_batch, int d, int G);
+// Learning layer forward: grad_l = floor(a W^T / (256 d)) - 32 onehot (the limbs of
+// W from *maxabs_wlr) and status bits.  The launch also clears what the rest of the
+// backward accumulates into, which saves a memset each: zero_words[0..n_zero) and,
+// when zero_dwlr is not null, the G d values of dW_lr.
 cudaError_t simt_learn_fwd(const int8_t* a, const int32_t* wlr, const int32_t* labels, int B,
-                           int d, int G, int64_t* scratch, int32_t* grad_l, unsigned long long* sse,
-                           int64_t* loss, uint32_t* maxabs_gl, uint32_t* status,
-                           uint32_t* zero_words, int n_zero, int64_t* zero_dwlr, cudaStream_t s);
+                           int d, int G, int32_t* grad_l, const uint32_t* maxabs_wlr,
+                           uint32_t* status, uint32_t* zero_words, int n_zero, int64_t* zero_dwlr,
+                           cudaStream_t s);
+
+// Written by the kernel that follows it (simt_lr_backward or simt_learn_dw): sse =
+// sum grad_l^2 (mod 2^64), loss = floor(sse / 2) (may be null), max |grad_l|, and
+// OVERFLOW when max |grad_l| *wlr_max G reaches 2^63 (wlr_max null: not checked).
+struct LossOut {
+    unsigned long long* sse;
+    int64_t* loss;
+    uint32_t* maxabs_gl;
+    uint32_t* ticket;          // sse, maxabs_gl and ticket: zero before (simt_learn_fwd clears them)
+    const uint32_t* wlr_max;
+    uint32_t* status;
+};
 
 // dW_lr[g][j] = sum_b grad_l[b][g] a[b][j]
 cudaError_t simt_learn_dw(const int8_t* a, const int32_t* grad_l, int B, int d, int G,
-                          int64_t* dwlr, cudaStream_t s);
+                          int64_t* dwlr, const LossOut& lo, cudaStream_t s);
 
 // Gradient at the output of layer g (post-pool) -> delta at its
 // pre-activation: max-pool backward, NITRO-ReLU backward, STE.  The source
@@ -321,8 +328,8 @@ bool simt_lr_backward_ok(int G);
 cudaError_t simt_lr_backward(const int8_t* a, const int32_t* gl, const int32_t* wlr, int B, int G,
                              int d, const LayerGeom* lg, int alpha_inv, const int8_t* region,
                              const int8_t* argmax, int32_t* delta, int64_t* dwlr,
-                             const uint32_t* maxabs_gl, const uint32_t* maxabs_wlr,
-                             uint32_t* maxabs_delta, uint32_t* status, cudaStream_t s);
+                             uint32_t* maxabs_delta, uint32_t* status, const LossOut& lo,
+                             cudaStream_t s);
 
 // IntegerSGD (Algorithm 1) over up to kMaxSgdTensors tensors in one launch.
 constexpr int kMaxSgdTensors = 16;
@@ -401,6 +408,26 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
+// launch_k with clusters of `cluster` CTAs along x (no dynamic shared memory).
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_cluster(void (*kernel)(KArgs...), int grid, int block, int cluster,
+                                  cudaStream_t s, Args&&... args) {
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
