@@ -1,13 +1,13 @@
 // CUDA-core kernels of the NITRO-D block step: an exact int64 implicit GEMM
-// for every contraction shape (conv 3x3 fwd / dgrad / wgrad, linear fwd /
-// dgrad / wgrad), and the element-wise stages fused around it (NITRO-Scaling,
+// (conv 3x3 fwd / dgrad / wgrad, linear fwd / dgrad), the linear layers of few
+// products, and the element-wise stages fused around it (NITRO-Scaling,
 // NITRO-ReLU and max-pool forward, with dropout for linear layers; max-pool,
 // NITRO-ReLU backward and STE; the learning layer, its max-pool to d_lr and
 // the RSS loss; IntegerSGD).
 //
 // The GEMM serves the contractions the tensor-core path does not take (narrow
-// or small layers, linear weight and input gradients, linear forwards whose
-// input width is not a multiple of 8); the learning layer (G = 10 outputs) and
+// or small conv layers, linear input gradients, the kernel-level matrix product
+// where K is not a multiple of 8); the learning layer (G = 10 outputs) and
 // the element-wise stages always run here.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
@@ -68,10 +68,8 @@ __device__ __forceinline__ int32_t load_a(const GemmParams& p, int m, int k) {
         return p.grad[(int64_t)k * p.Cout + m];
     } else if (MODE == GM_LIN_FWD) {
         return p.act[(int64_t)m * p.Cin + k];
-    } else if (MODE == GM_LIN_DGRAD) {
+    } else {  // GM_LIN_DGRAD
         return p.grad[(int64_t)m * p.Cout + k];
-    } else {  // GM_LIN_WGRAD
-        return p.grad[(int64_t)k * p.Cout + m];
     }
 }
 
@@ -91,10 +89,8 @@ __device__ __forceinline__ int32_t load_b(const GemmParams& p, int n, int k) {
         return p.act[((int64_t)(b * p.H + iy) * p.W + ix) * p.Cin + ci];
     } else if (MODE == GM_LIN_FWD) {
         return p.wts[(int64_t)n * p.Cin + k];
-    } else if (MODE == GM_LIN_DGRAD) {
+    } else {  // GM_LIN_DGRAD
         return p.wts[(int64_t)k * p.Cin + n];
-    } else {  // GM_LIN_WGRAD
-        return p.act[(int64_t)k * p.Cin + n];
     }
 }
 
@@ -222,9 +218,9 @@ __global__ void k_fwd_epilogue(const int64_t* __restrict__ z, LayerGeom g, int B
 // (up to eight) share out the features and exchange their partial sums through
 // distributed shared memory, so that no atomic, fence or ticket stands between
 // the sums and grad_L.  Warp u of a CTA takes sample u, 256 features a tile,
-// eight a lane, against W_lr split into signed 8-bit limbs in shared memory: one
-// dp4a a limb and four features, exact in 32 bits over 256 tiles.  W_lr with four
-// limbs (the top one may be +128, not a signed byte) takes 64-bit products.
+// eight a lane, against the bytes of W_lr in shared memory (two's complement: as
+// many bytes as max |W_lr| needs, the top one signed, those below unsigned): one
+// dp4a a byte and four features, exact in 32 bits over 128 tiles.
 // Bound by latency (the loads of a tile go out before the one before it is summed)
 // and by launch overhead.  The kernel before it (64-bit products, 64-bit atomics into
 // a sum array, one ticket a sample group and one for the loss) took 15.3 us a launch
@@ -237,7 +233,13 @@ constexpr int kLfTile = 256;       // features per tile
 constexpr int kLfCluster = 8;      // CTAs per cluster at most
 constexpr int kLfG = 16;           // classes per pass
 constexpr int kMaxClasses = 64;
-constexpr int kLfSpan = 256;       // tiles per 32-bit sum
+constexpr int kLfSpan = 128;       // tiles per 32-bit sum
+// Products up to which a linear layer that could run on the tensor cores runs on
+// k_lin_fwd / k_lin_wgrad.  Forward, us, here against there, weights of two limbs: 16 M
+// (batch 16, 1024 x 1024) 7.6 / 10.9, 32 M 9.8 / 12.3, 64 M 13.4 / 14.6 and 17.0 / 18.9
+// (batch 256, 512 x 512), 128 M 23.6 / 20.0; four limbs at 64 M 18.3 / 16.8.  Whole
+// backward: 16 M 18.2 / 19.5, 32 M 18.6 / 19.6, 64 M 26.1 / 19.5.
+constexpr int64_t kLinFwdMacs = (int64_t)48 << 20, kLinWgradMacs = (int64_t)32 << 20;
 
 struct LearnArgs {
     const int8_t* a;
@@ -269,8 +271,15 @@ __device__ __forceinline__ int4 learn_load_w(const LearnArgs& p, int g, int j) {
     return v;
 }
 
+// c + sum of four products of a signed byte of a and an unsigned byte of b
+__device__ __forceinline__ int dp4a_su(uint32_t a, uint32_t b, int c) {
+    int d;
+    asm("dp4a.s32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+
 // z of classes gc .. gc + GM - 1 for this warp's sample over features [j0, j1): lane
-// g returns class gc + g.  ws: GM rows of one tile, L limb words of four features.
+// g returns class gc + g.  ws: GM rows of one tile, byte l of four features a word.
 template <int GM, int L>
 __device__ __forceinline__ long long learn_dots(const LearnArgs& p, int b, int gc, int j0, int j1,
                                                 uint32_t* ws) {
@@ -293,14 +302,12 @@ __device__ __forceinline__ long long learn_dots(const LearnArgs& p, int b, int g
         for (int i = 0; i < kPer; ++i) {
             const int g = gr + 4 * i;
             if (g >= GM) break;
-            // byte l of w + 0x808080 is digit l + 128; xor 0x80 makes it signed
-            const uint32_t t0 = (uint32_t)wv[i].x + 0x808080u, t1 = (uint32_t)wv[i].y + 0x808080u;
-            const uint32_t t2 = (uint32_t)wv[i].z + 0x808080u, t3 = (uint32_t)wv[i].w + 0x808080u;
 #pragma unroll
             for (int l = 0; l < L; ++l) {
                 const uint32_t sel = l | ((4 + l) << 4);
-                const uint32_t lo = __byte_perm(t0, t1, sel), hi = __byte_perm(t2, t3, sel);
-                ws[(l * GM + g) * 64 + wd] = __byte_perm(lo, hi, 0x5410) ^ 0x80808080u;
+                const uint32_t lo = __byte_perm((uint32_t)wv[i].x, (uint32_t)wv[i].y, sel);
+                const uint32_t hi = __byte_perm((uint32_t)wv[i].z, (uint32_t)wv[i].w, sel);
+                ws[(l * GM + g) * 64 + wd] = __byte_perm(lo, hi, 0x5410);
             }
         }
         __syncthreads();
@@ -316,11 +323,16 @@ __device__ __forceinline__ long long learn_dots(const LearnArgs& p, int b, int g
 #pragma unroll
             for (int l = 0; l < L; ++l) {
                 const uint2 w = *reinterpret_cast<const uint2*>(&ws[(l * GM + g) * 64 + 2 * lane]);
-                acc[g][l] = __dp4a((int)ac.x, (int)w.x, acc[g][l]);
-                acc[g][l] = __dp4a((int)ac.y, (int)w.y, acc[g][l]);
+                if (l == L - 1) {
+                    acc[g][l] = __dp4a((int)ac.x, (int)w.x, acc[g][l]);
+                    acc[g][l] = __dp4a((int)ac.y, (int)w.y, acc[g][l]);
+                } else {
+                    acc[g][l] = dp4a_su(ac.x, w.x, acc[g][l]);
+                    acc[g][l] = dp4a_su(ac.y, w.y, acc[g][l]);
+                }
             }
         if (++tile == kLfSpan || j + kLfTile >= j1) {
-            // at most 256 tiles x 256 features x 2^14 = 2^30 a limb
+            // at most 128 tiles x 256 features x 128 x 255 < 2^30 a byte
             tile = 0;
 #pragma unroll
             for (int g = 0; g < GM; ++g) {
@@ -337,30 +349,13 @@ __device__ __forceinline__ long long learn_dots(const LearnArgs& p, int b, int g
     return z;
 }
 
-// The same with 64-bit products of the whole weights (four limbs); ws: one tile of
-// kLfG rows, one class at a time.
-__device__ __noinline__ long long learn_dots_wide(const LearnArgs& p, int b, int gc, int j0, int j1) {
-    const int lane = threadIdx.x & 31;
-    long long z = 0;
-    for (int g = 0; g < min(kLfG, p.G - gc); ++g) {
-        long long t = 0;
-        for (int j = j0 + lane; j < min(j1, p.d); j += 32)
-            if (b < p.B)
-                t += (long long)p.a[(int64_t)b * p.d + j] * p.wlr[(int64_t)(gc + g) * p.d + j];
-#pragma unroll
-        for (int off = 16; off; off >>= 1) t += __shfl_xor_sync(kFull, t, off);
-        if (lane == g) z = t;
-    }
-    return z;
-}
-
 template <int GM>
 __device__ __forceinline__ long long learn_pass(const LearnArgs& p, int limbs, int b, int gc, int j0,
                                                 int j1, uint32_t* ws) {
     if (limbs == 1) return learn_dots<GM, 1>(p, b, gc, j0, j1, ws);
     if (limbs == 2) return learn_dots<GM, 2>(p, b, gc, j0, j1, ws);
     if (limbs == 3) return learn_dots<GM, 3>(p, b, gc, j0, j1, ws);
-    return learn_dots_wide(p, b, gc, j0, j1);
+    return learn_dots<GM, 4>(p, b, gc, j0, j1, ws);
 }
 
 __global__ void __launch_bounds__(256) k_learn_fwd(const LearnArgs p, FloorDiv dv,
@@ -372,7 +367,7 @@ __global__ void __launch_bounds__(256) k_learn_fwd(const LearnArgs p, FloorDiv d
     namespace cg = cooperative_groups;
     const cg::cluster_group cluster = cg::this_cluster();
     const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-    __shared__ __align__(16) uint32_t ws[3 * kLfG * 64];
+    __shared__ __align__(16) uint32_t ws[4 * kLfG * 64];
     __shared__ long long part[kLfSamples][kMaxClasses];
     const int u = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int group = blockIdx.x / S, groups = gridDim.x / S;
@@ -407,6 +402,104 @@ __global__ void __launch_bounds__(256) k_learn_fwd(const LearnArgs p, FloorDiv d
         grad_l[(int64_t)bb * p.G + g] = (int32_t)t;
     }
     cluster.sync();      // the partial sums stay until every CTA has read them
+}
+
+// ---------------------------------------------------------------------------
+// Linear forward layer, one launch: the learning layer's contraction over 16 outputs
+// a cluster, then NITRO-Scaling, NITRO-ReLU and dropout on the summed values.  For
+// few products it is bound by latency: 64 x 784 x 100 takes 4.3 us where input pack,
+// tensor-core GEMM and epilogue as three launches took 9.8 us, 64 x 100 x 50 4.1
+// against 17.1 us on the general CUDA-core GEMM.
+// ---------------------------------------------------------------------------
+struct LinFwdArgs {
+    int alpha_inv, mu;
+    FloorDiv dv;                   // divide by the input width (after >> 8)
+    int8_t* act;
+    int8_t* out2;                  // may be null
+    int8_t* region;
+};
+__global__ void __launch_bounds__(256) k_lin_fwd(const LearnArgs p, const LinFwdArgs o,
+                                                 const uint32_t* maxabs_w, DropoutArgs drop) {
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    __shared__ __align__(16) uint32_t ws[4 * kLfG * 64];
+    __shared__ long long part[kLfSamples][kLfG];
+    const int u = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int groups = (p.B + kLfSamples - 1) / kLfSamples;
+    const int chunk = (int)(blockIdx.x / S) / groups, group = (int)(blockIdx.x / S) - chunk * groups;
+    const int gc = chunk * kLfG;
+    pdl_wait();
+    const int limbs = limb_count(*maxabs_w);
+    const int j0 = rank * p.per, j1 = min(p.d, j0 + p.per);
+    const long long z = learn_pass<kLfG>(p, limbs, group * kLfSamples + u, gc, j0, j1, ws);
+    if (lane < kLfG) part[u][lane] = z;
+    cluster.sync();
+    for (int i = threadIdx.x; i < kLfSamples * kLfG; i += 256) {
+        const int v = i / kLfG, g = i - v * kLfG, b = group * kLfSamples + v;
+        if (v % S != rank || b >= p.B || gc + g >= p.G) continue;
+        long long t = 0;
+        for (int r = 0; r < S; ++r) t += *cluster.map_shared_rank(&part[v][g], r);
+        const int64_t zs = o.dv.floor_div((int64_t)t >> 8);
+        const int64_t e = (int64_t)b * p.G + gc + g;
+        int rg = relu_region(zs);
+        int8_t val = (int8_t)relu_value(zs, o.alpha_inv, o.mu);
+        if (drop.p16 && dropout_drop(drop.seed, *drop.step, drop.layer, (uint64_t)e, drop.p16)) {
+            rg = kRegionDropped;
+            val = 0;
+        }
+        o.region[e] = (int8_t)rg;
+        o.act[e] = val;
+        if (o.out2) o.out2[e] = val;
+    }
+    cluster.sync();      // the partial sums stay until every CTA has read them
+}
+
+// Weight gradient of a linear layer: dW[o][i] = sum_b d[b][o] a[b][i], 16 outputs x
+// 64 inputs per CTA, four inputs a thread, the samples in slabs through shared
+// memory; every sum is finished in one thread (no K split, no clearing).  Few
+// products: bound by latency.  A backward of 64 x 784 x 100 with it takes 13.7 us,
+// 19.7 us with the general CUDA-core GEMM, which decodes an index for every operand
+// it stages.
+constexpr int kLwB = 32;           // samples per slab
+__global__ void __launch_bounds__(256) k_lin_wgrad(const int8_t* __restrict__ a,
+                                                   const int32_t* __restrict__ dl, int B, int in,
+                                                   int out, int64_t* __restrict__ dw) {
+    pdl_wait();
+    __shared__ int32_t ds[kLwB][16];
+    __shared__ __align__(4) int8_t as[kLwB][64];
+    const int ti = (in + 63) / 64;
+    const int i0 = (int)(blockIdx.x % ti) * 64, o0 = (int)(blockIdx.x / ti) * 16;
+    const int oi = threadIdx.x >> 4, q = threadIdx.x & 15;
+    int64_t acc[4] = {0, 0, 0, 0};
+    for (int b0 = 0; b0 < B; b0 += kLwB) {
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kLwB * 16 / 256; ++k) {
+            const int e = threadIdx.x + 256 * k, b = e >> 4, c = e & 15;
+            ds[b][c] = b0 + b < B && o0 + c < out ? dl[(int64_t)(b0 + b) * out + o0 + c] : 0;
+        }
+#pragma unroll
+        for (int k = 0; k < kLwB * 64 / 256; ++k) {
+            const int e = threadIdx.x + 256 * k, b = e >> 6, c = e & 63;
+            as[b][c] = b0 + b < B && i0 + c < in ? a[(int64_t)(b0 + b) * in + i0 + c] : (int8_t)0;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int b = 0; b < kLwB; ++b) {
+            const int32_t d = ds[b][oi];
+            const char4 v = *reinterpret_cast<const char4*>(&as[b][4 * q]);
+            acc[0] += (int64_t)d * v.x;
+            acc[1] += (int64_t)d * v.y;
+            acc[2] += (int64_t)d * v.z;
+            acc[3] += (int64_t)d * v.w;
+        }
+    }
+    if (o0 + oi >= out) return;
+    int64_t* row = dw + (int64_t)(o0 + oi) * in;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (i0 + 4 * q + k < in) row[i0 + 4 * q + k] = acc[k];
 }
 
 // The last CTA column of the kernel after k_learn_fwd: SSE, loss = floor(SSE / 2),
@@ -1299,7 +1392,6 @@ cudaError_t simt_gemm(int mode, const int8_t* act, const int32_t* grad, const in
         case GM_CONV_WGRAD: p.M = Cout; p.N = 9 * Cin; p.K = P; break;
         case GM_LIN_FWD: p.M = B; p.N = Cout; p.K = Cin; break;
         case GM_LIN_DGRAD: p.M = B; p.N = Cin; p.K = Cout; break;
-        case GM_LIN_WGRAD: p.M = Cout; p.N = Cin; p.K = B; break;
         default: return cudaErrorInvalidValue;
     }
     if (p.M <= 0 || p.N <= 0) return cudaSuccess;
@@ -1311,7 +1403,7 @@ cudaError_t simt_gemm(int mode, const int8_t* act, const int32_t* grad, const in
     // batch of 64 against a linear layer, a 4 x 4 conv map).
     int splits = 1;
     const int64_t tiles = (int64_t)tiles_m * tiles_n;
-    if (mode == GM_CONV_WGRAD || mode == GM_LIN_WGRAD || tiles < 2 * 152) {
+    if (mode == GM_CONV_WGRAD || tiles < 2 * 152) {
         const int64_t want = (4 * 152 + tiles - 1) / tiles;
         const int64_t maxs = (p.K + 255) / 256;
         splits = (int)(want < maxs ? want : maxs);
@@ -1326,16 +1418,15 @@ cudaError_t simt_gemm(int mode, const int8_t* act, const int32_t* grad, const in
         if (p.K == 0) return cudaSuccess;
     }
     dim3 grid(tiles_n, tiles_m, splits);
-    static const int kIds[6] = {K_SIMT_CONV_FWD, K_SIMT_CONV_DGRAD, K_SIMT_CONV_WGRAD,
-                                K_SIMT_LIN_FWD, K_SIMT_LIN_DGRAD, K_SIMT_LIN_WGRAD};
+    static const int kIds[5] = {K_SIMT_CONV_FWD, K_SIMT_CONV_DGRAD, K_SIMT_CONV_WGRAD,
+                                K_SIMT_LIN_FWD, K_SIMT_LIN_DGRAD};
     ProfScope ps(kIds[mode], s, 2.0 * p.M * p.N * p.K, 0.0);
     switch (mode) {
         case GM_CONV_FWD: launch_k(k_gemm<GM_CONV_FWD>, grid, 256, 0, s, p); break;
         case GM_CONV_DGRAD: launch_k(k_gemm<GM_CONV_DGRAD>, grid, 256, 0, s, p); break;
         case GM_CONV_WGRAD: launch_k(k_gemm<GM_CONV_WGRAD>, grid, 256, 0, s, p); break;
         case GM_LIN_FWD: launch_k(k_gemm<GM_LIN_FWD>, grid, 256, 0, s, p); break;
-        case GM_LIN_DGRAD: launch_k(k_gemm<GM_LIN_DGRAD>, grid, 256, 0, s, p); break;
-        default: launch_k(k_gemm<GM_LIN_WGRAD>, grid, 256, 0, s, p); break;
+        default: launch_k(k_gemm<GM_LIN_DGRAD>, grid, 256, 0, s, p); break;
     }
     return cudaGetLastError();
 }
@@ -1417,21 +1508,62 @@ cudaError_t simt_lrpool_to_delta(const int32_t* gl, const int32_t* wlr, int G, i
     return cudaGetLastError();
 }
 
+namespace {
+// CTAs that share one sample group's features: as many as have a tile each, up to
+// eight, while the launch stays below about two CTAs an SM (more would each do less
+// than their launch and cluster barriers cost)
+int learn_cluster(int64_t ctas, int d) {
+    int S = 1;
+    while (S < kLfCluster && S * kLfTile < d && ctas * S < 300) S *= 2;
+    return S;
+}
+}  // namespace
+
 cudaError_t simt_learn_fwd(const int8_t* a, const int32_t* wlr, const int32_t* labels, int B,
                            int d, int G, int32_t* grad_l, const uint32_t* maxabs_wlr,
                            uint32_t* status, uint32_t* zero_words, int n_zero, int64_t* zero_dwlr,
                            cudaStream_t s) {
     if (B <= 0) return cudaSuccess;
     if (n_zero > 256 || G > kMaxClasses) return cudaErrorInvalidValue;
-    int S = 1;
-    while (S < kLfCluster && S * kLfTile < d) S *= 2;
+    const int S = learn_cluster((B + kLfSamples - 1) / kLfSamples, d);
     LearnArgs p{a, wlr, B, d, G, 0, d % 8 == 0 && ((uintptr_t)a & 7) == 0,
                 d % 4 == 0 && ((uintptr_t)wlr & 15) == 0};
     p.per = ((d + S - 1) / S + kLfTile - 1) / kLfTile * kLfTile;
     ProfScope ps(K_LEARN_FWD, s, 2.0 * B * d * G, 0.0);
-    return launch_cluster(k_learn_fwd, S * ((B + kLfSamples - 1) / kLfSamples), 256, S, s, p,
+    return launch_cluster(k_learn_fwd, dim3(S * ((B + kLfSamples - 1) / kLfSamples)), 256, S, s, p,
                           FloorDiv::make((uint64_t)d), labels, grad_l, maxabs_wlr, status, zero_words,
                           n_zero, zero_dwlr);
+}
+
+bool simt_lin_fwd_ok(const LayerGeom& g, int B, bool tc) {
+    return g.kind == NITRO_LINEAR && (!tc || (int64_t)B * g.cin * g.cout <= kLinFwdMacs);
+}
+
+cudaError_t simt_lin_fwd(const int8_t* a, const int32_t* w, const uint32_t* maxabs_w, const LayerGeom& g,
+                         int B, int alpha_inv, int mu, int8_t* act, int8_t* out2, int8_t* region,
+                         const DropoutArgs* drop, cudaStream_t s) {
+    if (B <= 0) return cudaSuccess;
+    const int d = g.cin;
+    const int S = learn_cluster((B + kLfSamples - 1) / kLfSamples * ((g.cout + kLfG - 1) / kLfG), d);
+    LearnArgs p{a, w, B, d, g.cout, 0, d % 8 == 0 && ((uintptr_t)a & 7) == 0,
+                d % 4 == 0 && ((uintptr_t)w & 15) == 0};
+    p.per = ((d + S - 1) / S + kLfTile - 1) / kLfTile * kLfTile;
+    LinFwdArgs o{alpha_inv, mu, FloorDiv::make((uint64_t)d), act, out2, region};
+    ProfScope ps(K_SIMT_LIN_FWD, s, 2.0 * B * d * g.cout, 0.0);
+    return launch_cluster(k_lin_fwd,
+                          dim3(S * ((B + kLfSamples - 1) / kLfSamples) * ((g.cout + kLfG - 1) / kLfG)), 256,
+                          S, s, p, o, maxabs_w, drop ? *drop : DropoutArgs{});
+}
+
+bool simt_lin_wgrad_ok(const LayerGeom& g, int B, bool tc) {
+    return g.kind == NITRO_LINEAR && (!tc || (int64_t)B * g.cin * g.cout <= kLinWgradMacs);
+}
+
+cudaError_t simt_lin_wgrad(const int8_t* a, const int32_t* delta, const LayerGeom& g, int B, int64_t* dw,
+                           cudaStream_t s) {
+    ProfScope ps(K_SIMT_LIN_WGRAD, s, 2.0 * B * g.cin * (double)g.cout, 0.0);
+    return launch_k(k_lin_wgrad, dim3((unsigned)((g.cin + 63) / 64) * (unsigned)((g.cout + 15) / 16)), 256, 0,
+                    s, a, delta, B, g.cin, g.cout, dw);
 }
 
 namespace {

@@ -357,6 +357,16 @@ nitro_status nitro_block_forward(nitro_block* b, const int8_t* a_in, int batch, 
         // is filled by a copy after the last layer instead
         int8_t* out2 = (i == n - 1 && ((uintptr_t)a_out & 15) == 0) ? a_out : nullptr;
         bool done = false, fused = false;
+        // dropout of the linear layers (App. B, p_l)
+        const DropoutArgs da{b->seed, (uint32_t)b->desc.dropout_p16, i, w_step(b)};
+        const DropoutArgs* drop = g.kind == NITRO_LINEAR && b->desc.dropout_p16 > 0 ? &da : nullptr;
+        if (simt_lin_fwd_ok(g, batch, ly.lin_planes != nullptr)) {
+            NITRO_TRY(simt_lin_fwd(x, ly.W, w_w(b, i), g, batch, b->desc.alpha_inv, b->mu, ly.act, out2,
+                                   ly.region, drop, s));
+            nhwc_done = false;
+            x = ly.act;
+            continue;
+        }
         if (!ly.lin_planes) NITRO_TRY(tc_pack_input(ly.tc, g, x, batch, nhwc_done, s));
         // the epilogue also writes the next layer's bf16 forward operand
         uint16_t* next_nhwc = nullptr;
@@ -380,16 +390,11 @@ nitro_status nitro_block_forward(nitro_block* b, const int8_t* a_in, int batch, 
                                           ly.region, ly.argmax, next_nhwc, s));
             done = fused = true;
         }
-        if (!done) {
-            const int mode = g.kind == NITRO_CONV3X3 ? GM_CONV_FWD : GM_LIN_FWD;
-            NITRO_TRY(simt_gemm(mode, x, nullptr, ly.W, b->z64, batch, g.h, g.w, g.cin, g.cout, s));
-        }
+        if (!done)
+            NITRO_TRY(simt_gemm(GM_CONV_FWD, x, nullptr, ly.W, b->z64, batch, g.h, g.w, g.cin, g.cout, s));
         if (!fused) {
-            // dropout of the linear layers (App. B, p_l)
-            DropoutArgs da{b->seed, (uint32_t)b->desc.dropout_p16, i, w_step(b)};
-            const bool drop = g.kind == NITRO_LINEAR && b->desc.dropout_p16 > 0;
             NITRO_TRY(simt_fwd_epilogue(b->z64, g, batch, b->desc.alpha_inv, b->mu, ly.act, out2,
-                                        ly.region, ly.argmax, s, drop ? &da : nullptr));
+                                        ly.region, ly.argmax, s, drop));
         }
         nhwc_done = fused && next_nhwc != nullptr;
         x = ly.act;
@@ -488,9 +493,17 @@ nitro_status block_backward(nitro_block* b, const int8_t* a_in, const int32_t* l
         // fused update: the input gradient reads the pre-update weights, so it
         // runs first (after the delta split), then the weight gradient with
         // IntegerSGD; otherwise weight gradient first, as the split requires
-        const bool fuse_sgd = updated && tc_wgrad_fusable(ly.tc, g, batch);
+        const bool small = simt_lin_wgrad_ok(g, batch, ly.tc.wgrad);
+        const bool fuse_sgd = updated && !small && tc_wgrad_fusable(ly.tc, g, batch);
+        // the tensor-core weight gradient of a linear layer reads the bf16 copy of its
+        // input, which the forward makes only where it runs on the tensor cores too
+        if (ly.lin_a && !small && simt_lin_fwd_ok(g, batch, true))
+            NITRO_TRY(tc_pack_int8(x, batch, g.cin, ly.lin_a, s));
         auto wgrad = [&]() -> nitro_status {
-            if (fuse_sgd) {
+            if (small) {
+                NITRO_TRY(simt_lin_wgrad(x, ly.delta, g, batch, ly.dW, s));
+                done = true;
+            } else if (fuse_sgd) {
                 NITRO_TRY(cudaMemsetAsync(w_w(b, i), 0, 4, s));
                 TcSgd sg{gamma_fw, b->desc.eta_inv_fw, b->desc.sgd_round == NITRO_ROUND_TRUNC, ly.W,
                          w_w(b, i), nullptr, 0, 0, 0};
@@ -515,10 +528,9 @@ nitro_status block_backward(nitro_block* b, const int8_t* a_in, const int32_t* l
                 NITRO_TRY(simt_conv_small_wgrad(x, ly.delta, g, batch, ly.dW, s));
                 done = true;
             }
-            if (!done) {
-                const int mode = g.kind == NITRO_CONV3X3 ? GM_CONV_WGRAD : GM_LIN_WGRAD;
-                NITRO_TRY(simt_gemm(mode, x, ly.delta, nullptr, ly.dW, batch, g.h, g.w, g.cin, g.cout, s));
-            }
+            if (!done)
+                NITRO_TRY(simt_gemm(GM_CONV_WGRAD, x, ly.delta, nullptr, ly.dW, batch, g.h, g.w, g.cin,
+                                    g.cout, s));
             return NITRO_OK;
         };
         if (fuse_sgd) {

@@ -227,8 +227,7 @@ enum GemmMode : int {
     GM_CONV_DGRAD = 1,  // C[p][ci]      = sum_(t,co) g[p - tap t][co] * W[co][t][ci]
     GM_CONV_WGRAD = 2,  // C[co][(t,ci)] = sum_p g[p][co] * a[p + tap t][ci]
     GM_LIN_FWD = 3,     // C[b][o] = sum_i a[b][i] * W[o][i]
-    GM_LIN_DGRAD = 4,   // C[b][i] = sum_o g[b][o] * W[o][i]
-    GM_LIN_WGRAD = 5    // C[o][i] = sum_b g[b][o] * a[b][i]
+    GM_LIN_DGRAD = 4    // C[b][i] = sum_o g[b][o] * W[o][i]
 };
 
 // Exact int64 implicit GEMM on CUDA cores.  act: int8 activations, grad:
@@ -291,6 +290,17 @@ struct LossOut {
 // dW_lr[g][j] = sum_b grad_l[b][g] a[b][j]
 cudaError_t simt_learn_dw(const int8_t* a, const int32_t* grad_l, int B, int d, int G,
                           int64_t* dwlr, const LossOut& lo, cudaStream_t s);
+
+// Linear layer on the CUDA cores: the whole forward (scaling, NITRO-ReLU, dropout; the
+// limbs of w from *maxabs_w) and the weight gradient (dw overwritten), one launch
+// each.  _ok: the layer has few products, or no tensor-core form (tc false).
+bool simt_lin_fwd_ok(const LayerGeom& g, int B, bool tc);
+cudaError_t simt_lin_fwd(const int8_t* a, const int32_t* w, const uint32_t* maxabs_w, const LayerGeom& g,
+                         int B, int alpha_inv, int mu, int8_t* act, int8_t* out2, int8_t* region,
+                         const DropoutArgs* drop, cudaStream_t s);
+bool simt_lin_wgrad_ok(const LayerGeom& g, int B, bool tc);
+cudaError_t simt_lin_wgrad(const int8_t* a, const int32_t* delta, const LayerGeom& g, int B, int64_t* dw,
+                           cudaStream_t s);
 
 // Gradient at the output of layer g (post-pool) -> delta at its
 // pre-activation: max-pool backward, NITRO-ReLU backward, STE.  The source
@@ -413,7 +423,7 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
 
 // launch_k with clusters of `cluster` CTAs along x (no dynamic shared memory).
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_cluster(void (*kernel)(KArgs...), int grid, int block, int cluster,
+inline cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, int block, int cluster,
                                   cudaStream_t s, Args&&... args) {
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -423,7 +433,7 @@ inline cudaError_t launch_cluster(void (*kernel)(KArgs...), int grid, int block,
     attr[1].val.clusterDim.y = 1;
     attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)block);
     cfg.stream = s;
     cfg.attrs = attr;
