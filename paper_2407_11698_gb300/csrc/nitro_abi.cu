@@ -384,12 +384,6 @@ nitro_status nitro_block_forward(nitro_block* b, const int8_t* a_in, int batch, 
                                   w_status(b), s));
             done = true;
         }
-        if (!done && simt_small_conv_ok(g)) {
-            // narrow input (image channels): fused CUDA-core forward
-            NITRO_TRY(simt_conv_small_fwd(x, ly.W, g, batch, b->desc.alpha_inv, b->mu, ly.act, out2,
-                                          ly.region, ly.argmax, next_nhwc, s));
-            done = fused = true;
-        }
         if (!done)
             NITRO_TRY(simt_gemm(GM_CONV_FWD, x, nullptr, ly.W, b->z64, batch, g.h, g.w, g.cin, g.cout, s));
         if (!fused) {
@@ -523,10 +517,6 @@ nitro_status block_backward(nitro_block* b, const int8_t* a_in, const int32_t* l
             } else {
                 NITRO_TRY(tc_conv_wgrad(ly.tc, g, ly.delta, w_delta(b, i), batch, ly.dW, w_status(b), s,
                                         &done, planes_done && i == n - 1));
-            }
-            if (!done && simt_small_conv_ok(g)) {
-                NITRO_TRY(simt_conv_small_wgrad(x, ly.delta, g, batch, ly.dW, s));
-                done = true;
             }
             if (!done)
                 NITRO_TRY(simt_gemm(GM_CONV_WGRAD, x, ly.delta, nullptr, ly.dW, batch, g.h, g.w, g.cin,

@@ -235,6 +235,9 @@ enum GemmMode : int {
 cudaError_t simt_gemm(int mode, const int8_t* act, const int32_t* grad, const int32_t* wts,
                       int64_t* out, int B, int H, int W, int Cin, int Cout, cudaStream_t s);
 
+// Brings the kernels of a conv forward (GEMM, epilogue) onto the current device.
+cudaError_t simt_preload_conv_fwd();
+
 // z (int64, pre-pool NHWC) -> NITRO-Scaling -> NITRO-ReLU -> region codes,
 // optional 2x2 max-pool with argmax codes, int8 outputs (out2 may be NULL).
 // With drop.p16 > 0 (linear layers, no pool) dropped outputs are stored as 0
@@ -317,16 +320,6 @@ struct DeltaSrc {
 cudaError_t simt_grad_to_delta(const DeltaSrc& src, const LayerGeom& g, int B, int alpha_inv,
                                const int8_t* region, const int8_t* argmax, int32_t* delta,
                                uint32_t* maxabs_delta, uint32_t* status, cudaStream_t s);
-
-// Narrow-input conv (Cin <= 8, Cout % 16 == 0): fused forward (writes act,
-// out2, region, argmax and, if next_nhwc != null, a bf16 copy of act) and
-// weight gradient (dw overwritten).
-bool simt_small_conv_ok(const LayerGeom& g);
-cudaError_t simt_conv_small_fwd(const int8_t* x, const int32_t* w, const LayerGeom& g, int B,
-                                int alpha_inv, int mu, int8_t* act, int8_t* out2, int8_t* region,
-                                int8_t* argmax, uint16_t* next_nhwc, cudaStream_t s);
-cudaError_t simt_conv_small_wgrad(const int8_t* x, const int32_t* d, const LayerGeom& g, int B,
-                                  int64_t* dw, cudaStream_t s);
 
 // Learning-layer backward for G <= 16, fused: dW_lr (added to; zero on entry,
 // see simt_learn_fwd) and, when

@@ -242,7 +242,7 @@ struct TcArgs {
     FloorDiv alpha;        // divide by alpha_inv
     int32_t sf;            // SF = 2^8 9 Cin
     float sf_inv;          // 1 / SF
-    int out32;             // outputs and their rows are 32-byte aligned
+    int out_align;         // outputs and their rows are aligned to 32, 16 or 8 bytes
     int mu, pool, oh, ow;
     int8_t* act;           // layer output (post-pool) int8 NHWC
     int8_t* out2;          // optional second copy of the output (caller's buffer)
@@ -272,6 +272,10 @@ struct TcArgs {
     uint32_t* maxabs_w;        // max |new W| (atomic max, zeroed by the caller)
 };
 
+// 8 int8 values (2 packed words) -> one 8-byte store
+__device__ __forceinline__ void st8(int8_t* dst, const uint32_t* w) {
+    *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
+}
 // 16 int8 values (4 packed words) -> one 16-byte store
 __device__ __forceinline__ void st16(int8_t* dst, const uint32_t* w) {
     *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
@@ -310,12 +314,10 @@ __device__ __forceinline__ void cvt16_bf16(uint32_t* o, const uint32_t* w) {
         o[2 * k + 1] = bf16x2(u, 2);
     }
 }
-// the same to memory (two 16-byte stores)
-__device__ __forceinline__ void st16_bf16(uint16_t* dst, const uint32_t* w) {
-    uint32_t o[8];
-    cvt16_bf16(o, w);
-    reinterpret_cast<uint4*>(dst)[0] = make_uint4(o[0], o[1], o[2], o[3]);
-    reinterpret_cast<uint4*>(dst)[1] = make_uint4(o[4], o[5], o[6], o[7]);
+// 8 int8 values (2 packed words) -> 8 bf16 values, one 16-byte store
+__device__ __forceinline__ void st8_bf16(uint16_t* dst, const uint32_t* w) {
+    const uint32_t u = w[0] ^ 0x80808080u, v = w[1] ^ 0x80808080u;
+    *reinterpret_cast<uint4*>(dst) = make_uint4(bf16x2(u, 0), bf16x2(u, 2), bf16x2(v, 0), bf16x2(v, 2));
 }
 
 // PB = B-operand limbs carried per stage: one A tile feeds PB limb tiles of B
@@ -889,7 +891,21 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // position 3 - (2 (y & 1) + (x & 1)) of this pixel in its window, in
                     // bits 6, 7 of each 16-bit key: the maximum is the first maximum
                     const uint32_t poskey = (uint32_t)(3 - (((y & 1) << 1) | (x & 1))) * 0x00400040u;
-                    const bool wide = NH == 32 && args.out32 && col0 + 32 <= C;
+                    const bool wide = NH == 32 && args.out_align == 32 && col0 + 32 <= C;
+                    // this thread's columns of one row: 32, 16 or 8 bytes a store
+                    const auto put = [&](int8_t* p, const uint32_t* w) {
+                        if (wide) {
+                            st32(p, w, true);
+                        } else if (args.out_align >= 16) {
+#pragma unroll
+                            for (int k = 0; k < NH / 16; ++k)
+                                if (col0 + 16 * k < C) st16(p + 16 * k, w + 4 * k);
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < NH / 8; ++k)
+                                if (col0 + 8 * k < C) st8(p + 8 * k, w + 2 * k);
+                        }
+                    };
                     uint32_t vpk[NH / 4], rpk[NH / 4];   // packed outputs, pieces or window positions
 #pragma unroll
                     for (int g4 = 0; g4 < NH / 4; ++g4) {
@@ -923,16 +939,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                             lo[4 * g4] = e23 + poskey;
                         }
                     }
-                    if (valid && col0 < C) {
-                        int8_t* p = args.region + pix * C + col0;
-                        if (wide) {
-                            st32(p, rpk, true);
-                        } else {
-#pragma unroll
-                            for (int k = 0; k < NH / 16; ++k)
-                                if (col0 + 16 * k < C) st16(p + 16 * k, rpk + 4 * k);
-                        }
-                    }
+                    if (valid && col0 < C) put(args.region + pix * C + col0, rpk);
                     if (args.pool) {
 #pragma unroll
                         for (int g4 = 0; g4 < NH / 4; ++g4) {
@@ -947,20 +954,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     if ((args.pool ? anchor : valid) && col0 < C) {
                         const int64_t o = (args.pool ? opix : pix) * C + col0;
-                        if (wide) {
-                            st32(args.act + o, vpk, true);
-                            if (args.out2) st32(args.out2 + o, vpk, true);
-                            if (args.pool) st32(args.argmax + o, rpk, true);
-                        }
+                        put(args.act + o, vpk);
+                        if (args.out2) put(args.out2 + o, vpk);
+                        if (args.pool) put(args.argmax + o, rpk);
+                        if (args.next_nhwc) {
 #pragma unroll
-                        for (int k = 0; k < NH / 16; ++k) {
-                            if (col0 + 16 * k >= C) break;
-                            if (!wide) {
-                                st16(args.act + o + 16 * k, vpk + 4 * k);
-                                if (args.out2) st16(args.out2 + o + 16 * k, vpk + 4 * k);
-                                if (args.pool) st16(args.argmax + o + 16 * k, rpk + 4 * k);
-                            }
-                            if (args.next_nhwc) st16_bf16(args.next_nhwc + o + 16 * k, vpk + 4 * k);
+                            for (int k = 0; k < NH / 8; ++k)
+                                if (col0 + 8 * k < C) st8_bf16(args.next_nhwc + o + 8 * k, vpk + 2 * k);
                         }
                     }
                 } else if (MODE == TC_DGRAD && args.fuse) {
@@ -1315,6 +1315,44 @@ __global__ void k_pack_weights(const int32_t* __restrict__ W, int Cout, int Cin,
 
 }
 
+// The same into all four planes, eight entries a thread, zeros where the rows are
+// padded, and *out = max |W| (maximum and CTA ticket in scratch[0], scratch[1],
+// zero between launches): one launch for planes whose memory holds anything.
+__global__ void __launch_bounds__(256) k_pack_weights_pad(const int32_t* __restrict__ W, int Cout, int Cin,
+                                                          int row_k, int tap_k, uint16_t* __restrict__ wp,
+                                                          uint32_t* out, uint32_t* scratch) {
+    pdl_wait();
+    const int64_t nk = (int64_t)Cout * row_k;
+    uint32_t mx = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nk / 8;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int co = (int)(8 * i / row_k), e0 = (int)(8 * i - (int64_t)co * row_k);
+        int32_t v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int e = e0 + k, t = e / tap_k, ci = e - t * tap_k;
+            v[k] = t < 9 && ci < Cin ? W[((int64_t)co * 9 + t) * Cin + ci] : 0;
+            mx = max(mx, abs_u32(v[k]));
+        }
+#pragma unroll
+        for (int l = 0; l < kMaxLimbs; ++l)
+            reinterpret_cast<uint4*>(wp + l * nk)[i] =
+                make_uint4(limb_bf16x2(v[0], v[1], l), limb_bf16x2(v[2], v[3], l),
+                           limb_bf16x2(v[4], v[5], l), limb_bf16x2(v[6], v[7], l));
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0) {
+        if (mx) atomicMax(&scratch[0], mx);
+        __threadfence();     // this warp's maximum, before the CTA's ticket
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&scratch[1], 1u) == gridDim.x - 1) {
+        __threadfence();
+        *out = atomicExch(&scratch[0], 0u);
+        scratch[1] = 0;
+    }
+}
+
 // ------------------------------------------------------------------ host side
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -1480,6 +1518,79 @@ int64_t* tc_wgrad_adds(const TcLayer& t, const LayerGeom& g, int batch, int64_t*
     return t.wgrad && batch > 0 && wgrad_split_count(t, g, batch) > 1 ? dW : nullptr;
 }
 
+namespace {
+// Which passes of a conv layer run on tcgen05, and its operand layout.
+void tc_layer_shape(TcLayer& t, const LayerGeom& g, bool has_dgrad) {
+    if (g.kind != NITRO_CONV3X3 || !encode_fn()) return;
+    // Inputs with 9 Cin <= 64 run as one 64-wide K-block of im2col rows, others with
+    // each tap padded to a multiple of 64 channels; maps of any size, a 128-pixel tile
+    // overhanging small ones.  Both waste MMA work and still beat the CUDA-core GEMM,
+    // which such layers ran on before: a training step of a 7 x 7, 64 -> 64 layer at
+    // batch 128 took 150 us, now 51; 16 x 16, 8 -> 64 at batch 64 213, now 73; 12 x 12,
+    // 20 -> 16 at batch 8 154, now 49.
+    t.im2col = 9 * g.cin <= kBK && im2col_smem(g.w, g.cin) <= 48 * 1024;
+    t.fwd = true;
+    t.wgrad = g.cout % 8 == 0;
+    // the input gradient reads the forward planes, which im2col layers lay out
+    // without taps
+    t.dgrad = has_dgrad && g.cout % 8 == 0 && !t.im2col;
+    t.cin8 = t.im2col ? kBK : round_up(g.cin, 8);
+    t.cin_k = round_up(g.cin, 64);
+}
+
+// The forward's fused epilogue: rows of 8-byte multiples, and few enough K-blocks
+// for its error bound.
+bool tc_fwd_fused(const TcLayer& t, const LayerGeom& g) {
+    return t.fwd && g.cout % 8 == 0 && (t.im2col ? 1 : 9) * (t.cin_k / kBK) <= kFwdMaxBlocks;
+}
+
+size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
+}  // namespace
+
+size_t tc_fwd_scratch(const LayerGeom& g, int batch) {
+    TcLayer t;
+    tc_layer_shape(t, g, false);
+    if (!tc_fwd_fused(t, g)) return 0;
+    const size_t nwk = (size_t)g.cout * (t.im2col ? kBK : 9 * t.cin_k);
+    return align256(2 * kMaxLimbs * nwk) + align256(2 * (size_t)batch * g.h * g.w * t.cin8);
+}
+
+cudaError_t tc_fwd_in_scratch(const LayerGeom& g, int batch, const int8_t* x, const int32_t* W,
+                              const TcFwdOut& fo, void* scratch, uint32_t* words, cudaStream_t s) {
+    TcLayer t;
+    tc_layer_shape(t, g, false);
+    const int row_k = t.im2col ? kBK : 9 * t.cin_k, tap_k = t.im2col ? g.cin : t.cin_k;
+    const size_t nwk = (size_t)g.cout * row_k;
+    t.w_planes = static_cast<uint16_t*>(scratch);
+    t.act_nhwc = reinterpret_cast<uint16_t*>(static_cast<char*>(scratch) + align256(2 * kMaxLimbs * nwk));
+    t.maxabs_w = words;
+    static const uint32_t two_limbs = 32639;       // any hint is exact
+    tc_use_external_hints(t, &two_limbs, &two_limbs);
+    {
+        ProfScope ps(K_TC_PACK_W, s, 0.0, (double)nwk * 12);
+        launch_k(k_pack_weights_pad, grid1d((int64_t)nwk / 8), 256, 0, s, W, g.cout, g.cin, row_k, tap_k,
+                 t.w_planes, words, words + 1);
+    }
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = tc_pack_input(t, g, x, batch, false, s);
+    bool done = false, fused = false;
+    if (e == cudaSuccess) e = tc_conv_forward(t, g, batch, nullptr, &fo, words + 3, s, &done, &fused);
+    return e == cudaSuccess && !fused ? cudaErrorInvalidValue : e;
+}
+
+cudaError_t tc_fwd_preload() {
+    cudaFuncAttributes fa{};
+    const void* const fns[] = {
+        reinterpret_cast<const void*>(k_tc_gemm<TC_FWD, 64, 2>), reinterpret_cast<const void*>(k_tc_gemm<TC_FWD, 128, 2>),
+        reinterpret_cast<const void*>(k_pack_weights_pad), reinterpret_cast<const void*>(k_pack_im2col),
+        reinterpret_cast<const void*>(k_pack_act_flat), reinterpret_cast<const void*>(k_pack_act_nhwc)};
+    for (const void* f : fns) {
+        const cudaError_t e = cudaFuncGetAttributes(&fa, f);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 bool tc_layer_init(TcLayer& t, const LayerGeom& g, int max_batch, bool has_dgrad,
                    const uint32_t* maxabs_w, const uint32_t* maxabs_d,
                    std::vector<void*>& allocs, std::vector<void*>& host_allocs) {
@@ -1487,20 +1598,7 @@ bool tc_layer_init(TcLayer& t, const LayerGeom& g, int max_batch, bool has_dgrad
     t.maxabs_w = maxabs_w;
     t.maxabs_d = maxabs_d;
     if (g.kind != NITRO_CONV3X3 || max_batch < 1 || !encode_fn()) return true;
-    // Narrow inputs (Cin < 32, e.g. image channels) stay on the CUDA-core
-    // kernels: zero-padding them to a 64-wide K-block wastes most MMA work.
-    // Inputs with 9 Cin <= 64 run as one 64-wide K-block of im2col rows.
-    const bool pix_ok = g.h >= 8 && g.w >= 8;
-    const bool pix4 = g.h == 4 && g.w == 4;       // forward only: 4 x 4 x 8-image tiles
-    const bool wide = g.cin >= 32;
-    t.im2col = pix_ok && 9 * g.cin <= kBK && im2col_smem(g.w, g.cin) <= 48 * 1024;
-    t.fwd = (pix_ok && (wide || t.im2col)) || (pix4 && wide);
-    t.wgrad = (wide || t.im2col) && g.cout % 8 == 0;
-    // the input gradient reads the forward planes, which im2col layers lay out
-    // without taps
-    t.dgrad = has_dgrad && pix_ok && g.cout % 8 == 0 && !t.im2col;
-    t.cin8 = t.im2col ? kBK : round_up(g.cin, 8);
-    t.cin_k = round_up(g.cin, 64);
+    tc_layer_shape(t, g, has_dgrad);
     const size_t hw = (size_t)g.h * g.w;
     const size_t nwk = (size_t)g.cout * (t.im2col ? kBK : 9 * t.cin_k);
     bool ok = true;
@@ -1631,7 +1729,7 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
     a.out_vec = ((uintptr_t)z & 31) == 0 && g.cout % 4 == 0;
     a.status = status;
     a.atomic_out = 0;
-    const bool fuse = fo && g.cout % 16 == 0 && a.kb_total <= kFwdMaxBlocks;
+    const bool fuse = fo && tc_fwd_fused(t, g);
     if (fuse) {
         a.sf = 256 * 9 * g.cin;
         a.sf_inv = 1.0f / (float)a.sf;
@@ -1645,8 +1743,10 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
         a.region = fo->region;
         a.argmax = fo->argmax;
         a.next_nhwc = fo->next_nhwc;
-        a.out32 = g.cout % 32 == 0 && (((uintptr_t)a.act | (uintptr_t)a.region | (uintptr_t)a.out2 |
-                                        (uintptr_t)a.argmax) & 31) == 0;
+        const uintptr_t low = (uintptr_t)a.act | (uintptr_t)a.region | (uintptr_t)a.out2 |
+                              (uintptr_t)a.argmax | (uintptr_t)g.cout;
+        a.out_align = (low & 31) == 0 ? 32 : ((low & 15) == 0 ? 16 : 8);
+        if (low & 7) return cudaErrorInvalidValue;
     }
     CUtensorMap ma, mb;
     const uint64_t da[4] = {(uint64_t)t.cin8, (uint64_t)g.w, (uint64_t)g.h, (uint64_t)batch};

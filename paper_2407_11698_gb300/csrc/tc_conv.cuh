@@ -128,7 +128,7 @@ struct TcFwdOut {
 };
 
 // Forward contraction on tcgen05; *done = false if the layer does not run
-// there.  With fo != null and Cout % 16 == 0 the epilogue applies
+// there.  With fo != null and Cout % 8 == 0 (and at most 128 K-blocks) the epilogue applies
 // NITRO-Scaling, NITRO-ReLU and the max-pool and writes fo's outputs
 // (*fused = true); otherwise z[p][co] (int64) is written.
 cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* z,
@@ -183,6 +183,16 @@ struct TcDgradOut {
 cudaError_t tc_conv_dgrad(TcLayer& t, const LayerGeom& g, int batch, int64_t* g64,
                           const TcDgradOut* fo, uint32_t* status, cudaStream_t s, bool* done,
                           bool* fused);
+
+// A conv layer's fused forward with its operands in the caller's memory: bytes of
+// 256-byte aligned scratch it needs at this batch (0: the layer does not run there),
+// and the call (words: [0] max |W|, [1, 2] zero before the first call and left zero,
+// [3] status; outputs 8-byte aligned).  The preload brings every kernel that the
+// calls use onto the device.
+size_t tc_fwd_scratch(const LayerGeom& g, int batch);
+cudaError_t tc_fwd_in_scratch(const LayerGeom& g, int batch, const int8_t* x, const int32_t* W,
+                              const TcFwdOut& fo, void* scratch, uint32_t* words, cudaStream_t s);
+cudaError_t tc_fwd_preload();
 
 // One CTA that holds TMEM and waits, through the contraction kernel's bounded
 // mbarrier wait, on a barrier nothing completes: after limit_ns it raises
