@@ -17,6 +17,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "prof.cuh"
 #include "tc_conv.cuh"
@@ -33,17 +34,20 @@ constexpr int kBK = 64;               // K elements per block (one 128-byte row)
 constexpr int kChunkBlocks = 16;      // 16 x 64 = 1024 products per exact chunk
 // Warp roles: warpgroup 0 = TMA warp, MMA warp and two idle warps; warpgroups
 // 1 to 4 = the epilogue, four warps per TMEM lane quadrant, each holding a
-// quarter of the N columns as int64 accumulators.  The epilogue is bound by
-// memory latency, so it gets as many warps as the register file allows; the
-// warpgroups split it with setmaxnreg: 128 x kRegsProducer + 32 x kEpiWarps x
-// kRegsEpilogue must not exceed kThreads x the registers the kernel is
-// launched with (checked on the host before the first launch).  A layout with
-// eight epilogue warps (half the N columns each, 224 registers, no spills) was
-// measured slower: 175k against 257k images/s on the VGG-style step.
+// quarter of the N columns.  The epilogue is bound by latency, so it gets as many
+// warps as the register file allows; the warpgroups split it with setmaxnreg: 128
+// x kRegsProducer + 32 x kEpiWarps x kRegsEpilogue must not exceed kThreads x the
+// registers the kernel is launched with (checked on the host before the first
+// launch).  64 / 104 with TMEM loads of 8 columns (16 where a warp holds 16) spills
+// nothing in the forward, GEMM and kernel-level variants: at 32 / 112 the TMA and
+// MMA warps reloaded spilled values on their per-K-block path, which the small L1
+// beside 227 KB of shared memory does not hold (VGG11B forward at batch 256 1154 us,
+// now 1098; 4096^3 GEMM 264, now 247; conv contractions 784, now 751).  Eight
+// epilogue warps (half the N columns each, 224 registers) were slower.
 constexpr int kEpiWarp0 = 4;          // first epilogue warp
 constexpr int kEpiWarps = 16;         // 4 per TMEM lane quadrant
 constexpr int kThreads = 32 * (kEpiWarp0 + kEpiWarps);
-constexpr int kRegsProducer = 32, kRegsEpilogue = 112;
+constexpr int kRegsProducer = 64, kRegsEpilogue = 104;
 constexpr int kTabHalf = 256;         // half the fused forward's table of z*
 // K-blocks of a fused forward (Cin <= 896): with four weight limbs and eight chunks
 // its fp32 sums are off by less than 2^24 1.02 8 (8 + 4.2) = 1.67e9, so that the
@@ -202,19 +206,25 @@ __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t* r) {
         : "r"(taddr));
 }
 
+__device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t* r) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+        : "r"(taddr));
+}
+
 // Wait for this thread's outstanding tcgen05.ld, then mark the n destination
 // registers as written here, so that no use of them is placed before the wait.
-__device__ __forceinline__ void reg_touch16(uint32_t* r) {
+__device__ __forceinline__ void reg_touch8(uint32_t* r) {
     asm volatile(""
                  : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
-                   "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]),
-                   "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]));
+                   "+r"(r[6]), "+r"(r[7]));
 }
 template <int n>
 __device__ __forceinline__ void tmem_wait_ld(uint32_t* r) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int j = 0; j < n / 16; ++j) reg_touch16(r + 16 * j);
+    for (int j = 0; j < n / 8; ++j) reg_touch8(r + 8 * j);
 }
 
 // ------------------------------------------------------------------ kernel
@@ -678,49 +688,57 @@ __global__ void __launch_bounds__(kThreads, 1)
                     };
                     // acc += v 2^shift: one 32 x 32 -> 64 multiply-add below 2^32, an
                     // add to the high word above (shift is a multiple of 8)
-                    auto accumulate = [&](const uint32_t* r, int j, int shift) {
+                    auto accumulate = [&](const uint32_t* r, int col, int shift, auto n) {
                         if (shift < 32) {
                             const int m = 1 << shift;
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) {
+                            for (int i = 0; i < n(); ++i) {
                                 const int v = __float2int_rz(__uint_as_float(r[i]));   // exact integer
-                                acc[16 * j + i] += (uint64_t)((long long)v * (long long)m);
+                                acc[col + i] += (uint64_t)((long long)v * (long long)m);
                             }
                         } else {
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) {
+                            for (int i = 0; i < n(); ++i) {
                                 const int v = __float2int_rz(__uint_as_float(r[i]));
-                                acc[16 * j + i] += (uint64_t)((uint32_t)v << (shift - 32)) << 32;
+                                acc[col + i] += (uint64_t)((uint32_t)v << (shift - 32)) << 32;
                             }
                         }
                     };
-                    // 32 values per TMEM round trip: two loads issued back to
-                    // back, then one wait (16 columns: two limbs at once)
+                    // 16 or 32 values per TMEM round trip, as the registers beside the
+                    // sums allow without spills
                     if constexpr (MODE == TC_FWD) {
+                        // CW columns of a limb pair at once: 16 values in flight beside the
+                        // 64 words of 32 columns' sums, 32 beside 16 columns' sums
+                        constexpr int CW = NH == 16 ? 16 : 8;
 #pragma unroll
-                        for (int j = 0; j < NH / 16; ++j)
+                        for (int j = 0; j < NH / CW; ++j)
                             for (int jb = 0; jb < nb; jb += 2) {
                                 const bool two = jb + 1 < nb;
                                 const int m = 1 << (shift0 + 8 * jb);
                                 const float mf = (float)m;
-                                uint32_t r[32];
-                                tmem_ld16_nowait(limb_base(jb) + 16 * j, r);
-                                if (two) tmem_ld16_nowait(limb_base(jb + 1) + 16 * j, r + 16);
-                                tmem_wait_ld<32>(r);
+                                uint32_t r[2 * CW];
+                                if constexpr (CW == 16) {
+                                    tmem_ld16_nowait(limb_base(jb) + CW * j, r);
+                                    if (two) tmem_ld16_nowait(limb_base(jb + 1) + CW * j, r + CW);
+                                } else {
+                                    tmem_ld8_nowait(limb_base(jb) + CW * j, r);
+                                    if (two) tmem_ld8_nowait(limb_base(jb + 1) + CW * j, r + CW);
+                                }
+                                tmem_wait_ld<2 * CW>(r);
                                 if (two) {
 #pragma unroll
-                                    for (int i = 0; i < 16; ++i) {
-                                        const float v0 = __uint_as_float(r[i]), v1 = __uint_as_float(r[16 + i]);
+                                    for (int i = 0; i < CW; ++i) {
+                                        const float v0 = __uint_as_float(r[i]), v1 = __uint_as_float(r[CW + i]);
                                         const uint32_t w = ((uint32_t)__float2int_rz(v1) << 8) + (uint32_t)__float2int_rz(v0);
-                                        lo[16 * j + i] += w * (uint32_t)m;
-                                        zf[16 * j + i] = fmaf(fmaf(v1, 256.0f, v0), mf, zf[16 * j + i]);
+                                        lo[CW * j + i] += w * (uint32_t)m;
+                                        zf[CW * j + i] = fmaf(fmaf(v1, 256.0f, v0), mf, zf[CW * j + i]);
                                     }
                                 } else {
 #pragma unroll
-                                    for (int i = 0; i < 16; ++i) {
+                                    for (int i = 0; i < CW; ++i) {
                                         const float v0 = __uint_as_float(r[i]);
-                                        lo[16 * j + i] += (uint32_t)__float2int_rz(v0) * (uint32_t)m;
-                                        zf[16 * j + i] = fmaf(v0, mf, zf[16 * j + i]);
+                                        lo[CW * j + i] += (uint32_t)__float2int_rz(v0) * (uint32_t)m;
+                                        zf[CW * j + i] = fmaf(v0, mf, zf[CW * j + i]);
                                     }
                                 }
                             }
@@ -730,20 +748,19 @@ __global__ void __launch_bounds__(kThreads, 1)
                             tmem_ld16_nowait(limb_base(jb), r);
                             if (jb + 1 < nb) tmem_ld16_nowait(limb_base(jb + 1), r + 16);
                             tmem_wait_ld<32>(r);
-                            accumulate(r, 0, shift0 + 8 * jb);
-                            if (jb + 1 < nb) accumulate(r + 16, 0, shift0 + 8 * (jb + 1));
+                            accumulate(r, 0, shift0 + 8 * jb, std::integral_constant<int, 16>());
+                            if (jb + 1 < nb)
+                                accumulate(r + 16, 0, shift0 + 8 * (jb + 1), std::integral_constant<int, 16>());
                         }
                     } else {
                         for (int jb = 0; jb < nb; ++jb) {
                             const uint32_t base = limb_base(jb);
 #pragma unroll
-                            for (int j2 = 0; j2 < NH / 32; ++j2) {
-                                uint32_t r[32];
-                                tmem_ld16_nowait(base + 32 * j2, r);
-                                tmem_ld16_nowait(base + 32 * j2 + 16, r + 16);
-                                tmem_wait_ld<32>(r);
-                                accumulate(r, 2 * j2, shift0 + 8 * jb);
-                                accumulate(r + 16, 2 * j2 + 1, shift0 + 8 * jb);
+                            for (int j = 0; j < NH / 8; ++j) {
+                                uint32_t r[8];
+                                tmem_ld8_nowait(base + 8 * j, r);
+                                tmem_wait_ld<8>(r);
+                                accumulate(r, 8 * j, shift0 + 8 * jb, std::integral_constant<int, 8>());
                             }
                         }
                     }
@@ -865,7 +882,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // x partner lane ^ 1, y partner lane ^ wb).  Bound by instruction
                     // issue: two 32-bit words a column instead of 64-bit sums and a
                     // 64-bit divide took the VGG11B forward at batch 256 from 1449 to
-                    // 1181 us and the VGG8B step from 980 to 928 us.
+                    // 1181 us and the VGG8B step from 980 to 928 us, the branches taken
+                    // out of its loops the forward to 1154 us.
                     //
                     // zf is off by less than err (set before the tile loop).  Where err <= SF / 4 the
                     // nearest integer to zf / SF is z* or z* + 1, and the sign of
@@ -884,13 +902,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const int C = args.Cout;
                     const int32_t sf = args.sf;
                     const float sfi = args.sf_inv;
-                    const int64_t pix = ((int64_t)b * args.H + y) * args.W + x;
+                    // element offsets fit 32 bits (checked when the block is made)
+                    const uint32_t pix = (uint32_t)((b * args.H + y) * args.W + x);
                     const bool anchor = valid && !(x & 1) && !(y & 1) && x + 1 < args.W && y + 1 < args.H;
-                    const int64_t opix = ((int64_t)b * args.oh + (y >> 1)) * args.ow + (x >> 1);
-                    const int dys = args.wb;
-                    // position 3 - (2 (y & 1) + (x & 1)) of this pixel in its window, in
-                    // bits 6, 7 of each 16-bit key: the maximum is the first maximum
-                    const uint32_t poskey = (uint32_t)(3 - (((y & 1) << 1) | (x & 1))) * 0x00400040u;
                     const bool wide = NH == 32 && args.out_align == 32 && col0 + 32 <= C;
                     // this thread's columns of one row: 32, 16 or 8 bytes a store
                     const auto put = [&](int8_t* p, const uint32_t* w) {
@@ -906,44 +920,53 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 if (col0 + 8 * k < C) st8(p + 8 * k, w + 2 * k);
                         }
                     };
-                    uint32_t vpk[NH / 4], rpk[NH / 4];   // packed outputs, pieces or window positions
-#pragma unroll
-                    for (int g4 = 0; g4 < NH / 4; ++g4) {
-                        uint32_t e[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const uint32_t l = lo[4 * g4 + u];
-                            const float f = zf[4 * g4 + u];
-                            int q;
-                            if (tight) {
-                                q = min(max(__float2int_rn(f * sfi), -200), 200);
-                                q += (int32_t)(l - (uint32_t)(q * sf)) >> 31;
-                            } else {
-                                const int q1 = __float2int_rn(f * sfi);
-                                const uint32_t r1 = l - (uint32_t)q1 * (uint32_t)sf;
-                                const int q2 = __float2int_rn((float)(int32_t)r1 * sfi);
-                                const int32_t r2 = (int32_t)(r1 - (uint32_t)q2 * (uint32_t)sf);
-                                q = min(max(q1 + q2 + (r2 >> 31), -200), 200);
-                                if (fabsf(f) > far) q = f < 0.0f ? -200 : 200;
-                            }
-                            e[u] = relu_tab[q + kTabHalf];
-                        }
-                        const uint32_t e01 = e[0] | (e[1] << 16), e23 = e[2] | (e[3] << 16);
-                        rpk[g4] = __byte_perm(e01, e23, 0x6420);
-                        if (!args.pool) {
-                            vpk[g4] = __byte_perm(e01, e23, 0x7531);
-                        } else {
-                            // key = value, 3 - position, piece: the maximum over the
-                            // window's four lanes, two 16-bit keys per word
-                            vpk[g4] = e01 + poskey;
-                            lo[4 * g4] = e23 + poskey;
-                        }
-                    }
-                    if (valid && col0 < C) put(args.region + pix * C + col0, rpk);
-                    if (args.pool) {
+                    // table entries of four columns, two 16-bit ones a word, into lo[4 g],
+                    // lo[4 g + 1]: the sums are not needed after
+                    if (tight) {
 #pragma unroll
                         for (int g4 = 0; g4 < NH / 4; ++g4) {
-                            uint32_t k0 = vpk[g4], k1 = lo[4 * g4];
+                            uint32_t e[4];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                int q = min(max(__float2int_rn(zf[4 * g4 + u] * sfi), -200), 200);
+                                q += (int32_t)(lo[4 * g4 + u] - (uint32_t)(q * sf)) >> 31;
+                                e[u] = relu_tab[q + kTabHalf];
+                            }
+                            lo[4 * g4] = e[0] | (e[1] << 16);
+                            lo[4 * g4 + 1] = e[2] | (e[3] << 16);
+                        }
+                    } else {
+#pragma unroll
+                        for (int g4 = 0; g4 < NH / 4; ++g4) {
+                            uint32_t e[4];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                const float f = zf[4 * g4 + u];
+                                const int q1 = __float2int_rn(f * sfi);
+                                const uint32_t r1 = lo[4 * g4 + u] - (uint32_t)q1 * (uint32_t)sf;
+                                const int q2 = __float2int_rn((float)(int32_t)r1 * sfi);
+                                const int32_t r2 = (int32_t)(r1 - (uint32_t)q2 * (uint32_t)sf);
+                                int q = min(max(q1 + q2 + (r2 >> 31), -200), 200);
+                                if (fabsf(f) > far) q = f < 0.0f ? -200 : 200;
+                                e[u] = relu_tab[q + kTabHalf];
+                            }
+                            lo[4 * g4] = e[0] | (e[1] << 16);
+                            lo[4 * g4 + 1] = e[2] | (e[3] << 16);
+                        }
+                    }
+                    uint32_t vpk[NH / 4], rpk[NH / 4];   // packed outputs, pieces or window positions
+#pragma unroll
+                    for (int g4 = 0; g4 < NH / 4; ++g4) rpk[g4] = __byte_perm(lo[4 * g4], lo[4 * g4 + 1], 0x6420);
+                    if (valid && col0 < C) put(args.region + pix * (uint32_t)C + col0, rpk);
+                    if (args.pool) {
+                        // key = value, 3 - position (2 (y & 1) + (x & 1)) in its window, piece:
+                        // the maximum over the window's four lanes is the first maximum, two
+                        // 16-bit keys a word
+                        const uint32_t poskey = (uint32_t)(3 - (((y & 1) << 1) | (x & 1))) * 0x00400040u;
+                        const int dys = args.wb;
+#pragma unroll
+                        for (int g4 = 0; g4 < NH / 4; ++g4) {
+                            uint32_t k0 = lo[4 * g4] + poskey, k1 = lo[4 * g4 + 1] + poskey;
                             k0 = max_s16x2(k0, __shfl_xor_sync(0xffffffffu, k0, 1));
                             k1 = max_s16x2(k1, __shfl_xor_sync(0xffffffffu, k1, 1));
                             k0 = max_s16x2(k0, __shfl_xor_sync(0xffffffffu, k0, dys));
@@ -951,12 +974,24 @@ __global__ void __launch_bounds__(kThreads, 1)
                             vpk[g4] = __byte_perm(k0, k1, 0x7531);
                             rpk[g4] = 0x03030303u - ((__byte_perm(k0, k1, 0x6420) >> 6) & 0x03030303u);
                         }
-                    }
-                    if ((args.pool ? anchor : valid) && col0 < C) {
-                        const int64_t o = (args.pool ? opix : pix) * C + col0;
+                        if (anchor && col0 < C) {
+                            const uint32_t o =
+                                (uint32_t)((b * args.oh + (y >> 1)) * args.ow + (x >> 1)) * (uint32_t)C + col0;
+                            put(args.act + o, vpk);
+                            if (args.out2) put(args.out2 + o, vpk);
+                            put(args.argmax + o, rpk);
+                            if (args.next_nhwc) {
+#pragma unroll
+                                for (int k = 0; k < NH / 8; ++k)
+                                    if (col0 + 8 * k < C) st8_bf16(args.next_nhwc + o + 8 * k, vpk + 2 * k);
+                            }
+                        }
+                    } else if (valid && col0 < C) {
+#pragma unroll
+                        for (int g4 = 0; g4 < NH / 4; ++g4) vpk[g4] = __byte_perm(lo[4 * g4], lo[4 * g4 + 1], 0x7531);
+                        const uint32_t o = pix * (uint32_t)C + col0;
                         put(args.act + o, vpk);
                         if (args.out2) put(args.out2 + o, vpk);
-                        if (args.pool) put(args.argmax + o, rpk);
                         if (args.next_nhwc) {
 #pragma unroll
                             for (int k = 0; k < NH / 8; ++k)
