@@ -1382,7 +1382,7 @@ cudaError_t simt_learn_fwd(const int8_t* a, const int32_t* wlr, const int32_t* l
                 d % 4 == 0 && ((uintptr_t)wlr & 15) == 0};
     p.per = ((d + S - 1) / S + kLfTile - 1) / kLfTile * kLfTile;
     ProfScope ps(K_LEARN_FWD, s, 2.0 * B * d * G, 0.0);
-    return launch_cluster(k_learn_fwd, dim3(S * ((B + kLfSamples - 1) / kLfSamples)), 256, S, s, p,
+    return launch_cluster(k_learn_fwd, dim3(S * ((B + kLfSamples - 1) / kLfSamples)), 256, S, s, 0, p,
                           FloorDiv::make((uint64_t)d), labels, grad_l, maxabs_wlr, status, zero_words,
                           n_zero, zero_dwlr);
 }
@@ -1404,7 +1404,7 @@ cudaError_t simt_lin_fwd(const int8_t* a, const int32_t* w, const uint32_t* maxa
     ProfScope ps(K_SIMT_LIN_FWD, s, 2.0 * B * d * g.cout, 0.0);
     return launch_cluster(k_lin_fwd,
                           dim3(S * ((B + kLfSamples - 1) / kLfSamples) * ((g.cout + kLfG - 1) / kLfG)), 256,
-                          S, s, p, o, maxabs_w, drop ? *drop : DropoutArgs{});
+                          S, s, 0, p, o, maxabs_w, drop ? *drop : DropoutArgs{});
 }
 
 bool simt_lin_wgrad_ok(const LayerGeom& g, int B, bool tc) {

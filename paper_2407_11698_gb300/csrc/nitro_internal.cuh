@@ -414,10 +414,10 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// launch_k with clusters of `cluster` CTAs along x (no dynamic shared memory).
+// launch_k with clusters of `cluster` CTAs along x.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, int block, int cluster,
-                                  cudaStream_t s, Args&&... args) {
+                                  cudaStream_t s, size_t smem, Args&&... args) {
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
@@ -428,6 +428,7 @@ inline cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, int block
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 2;

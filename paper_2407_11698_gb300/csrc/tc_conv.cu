@@ -26,8 +26,9 @@ namespace nitro {
 namespace {
 
 // TC_FWD: forward with the fused NITRO-Scaling / NITRO-ReLU / max-pool epilogue;
-// TC_FWDZ: the same contraction with int64 sums as its output.
-enum TcMode : int { TC_FWD = 0, TC_WGRAD = 1, TC_DGRAD = 2, TC_GEMM = 3, TC_FWDZ = 4 };
+// TC_FWDK: the same with a tile's K shared out over a cluster; TC_FWDZ: the forward
+// contraction with int64 sums as its output.
+enum TcMode : int { TC_FWD = 0, TC_WGRAD = 1, TC_DGRAD = 2, TC_GEMM = 3, TC_FWDZ = 4, TC_FWDK = 5 };
 
 constexpr int kBM = 128;              // rows per tile (TMEM lanes)
 constexpr int kBK = 64;               // K elements per block (one 128-byte row)
@@ -248,6 +249,7 @@ struct TcArgs {
     int atomic_out;
     int out_vec;           // int64 rows are 32-byte aligned: four values a store
     int fuse;              // input gradient: fused epilogue
+    int ksplit;            // fused forward: CTAs of a cluster that share a tile's K (1: none)
     // forward with fused NITRO-Scaling / NITRO-ReLU / max-pool epilogue
     FloorDiv alpha;        // divide by alpha_inv
     int32_t sf;            // SF = 2^8 9 Cin
@@ -281,6 +283,26 @@ struct TcArgs {
     int decay, trunc;
     uint32_t* maxabs_w;        // max |new W| (atomic max, zeroed by the caller)
 };
+
+// Cluster-wide barrier, and shared memory of another CTA of the cluster.
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t remote_smem(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_remote4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c),
+                 "r"(d)
+                 : "memory");
+}
 
 // 8 int8 values (2 packed words) -> one 8-byte store
 __device__ __forceinline__ void st8(int8_t* dst, const uint32_t* w) {
@@ -358,7 +380,7 @@ __device__ __forceinline__ Tile decode_tile(const TcArgs& a, int tile) {
     t.nt = tile - r * a.tiles_n;
     const int split = udiv32(a.dv_tm, r);
     t.mt = r - split * a.tiles_m;
-    t.kb0 = split * a.kb_per_split;
+    t.kb0 = min(a.kb_total, split * a.kb_per_split);
     t.kb1 = min(a.kb_total, t.kb0 + a.kb_per_split);
     return t;
 }
@@ -373,7 +395,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     using C = TcCfg<N, PB>;
     constexpr int S = C::S;
     constexpr int NH = N / 4;            // columns per epilogue warp
-    constexpr bool kFwd = MODE == TC_FWD || MODE == TC_FWDZ;
+    constexpr bool kFused = MODE == TC_FWD || MODE == TC_FWDK;
+    constexpr bool kFwd = kFused || MODE == TC_FWDZ;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -406,7 +429,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (MODE == TC_FWD) {
+    if (kFused) {
         for (int i = threadIdx.x; i < 2 * kTabHalf; i += kThreads) {
             const int zs = i - kTabHalf;
             relu_tab[i] = (uint16_t)((uint32_t)(uint8_t)relu_value((int64_t)zs, args.alpha, args.mu) << 8 |
@@ -449,6 +472,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int LA = args.max_a ? limb_count(*args.max_a) : 1;
     const int LB = args.max_b ? limb_count(*args.max_b) : 1;
     const int hiskip = *hiskip_slot;
+    // Tiles of this CTA: every gridDim.x-th one, or, where a cluster shares a tile's K
+    // (the ranks are the splits), one.
+    const int KS = MODE == TC_FWDK ? args.ksplit : 1;
+    const int rank = MODE == TC_FWDK ? (int)cluster_rank() : 0;
+    const int tile0 =
+        MODE == TC_FWDK ? rank * (args.tiles_m * args.tiles_n) + (int)blockIdx.x / KS : (int)blockIdx.x;
+    const int tile_step = MODE == TC_FWDK ? args.total_tiles : (int)gridDim.x;
     // B limbs that pair with A limb la: all, or those with la + lb <= 3
     auto lb_limit = [&](int la) { return hiskip ? min(LB, 4 - la) : LB; };
 
@@ -459,7 +489,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) {
             // ---------------- TMA producer
             int it = 0;
-            for (int tile = blockIdx.x; tile < args.total_tiles; tile += gridDim.x) {
+            for (int tile = tile0; tile < args.total_tiles; tile += tile_step) {
                 const Tile T = decode_tile(args, tile);
                 const int n0 = T.nt * N;
                 const int mq = udiv32(args.dv_ntx, T.mt), tb = udiv32(args.dv_nty, mq);
@@ -582,7 +612,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             int st = 0;          // ring stage of the next K-block
             uint32_t ph = 0;     // and the parity of the phase it waits for
             int chunk = 0;
-            for (int tile = blockIdx.x; tile < args.total_tiles; tile += gridDim.x) {
+            for (int tile = tile0; tile < args.total_tiles; tile += tile_step) {
                 const Tile T = decode_tile(args, tile);
                 // chunks of equal length (at most kChunkBlocks K-blocks each), so
                 // that no short chunk costs a full drain for little MMA work
@@ -635,6 +665,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             pdl_trigger();
         }
     }
+    if constexpr (MODE == TC_FWDK) {
+        cluster_barrier();      // the two of the epilogue's exchange
+        cluster_barrier();
+    }
     } else {
         // ---------------- epilogue: warpgroups 1 and 2
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpilogue));
@@ -646,21 +680,25 @@ __global__ void __launch_bounds__(kThreads, 1)
         // 2^-24) hit the running sum, which stays below c csz 2^20 2^(8 (LB - 1)) (1 +
         // 2^-6) after c chunks, one hits a limb pair, and the product with 1 / SF adds
         // 2^-23 of the sum: together csz / 16 2^(8 (LB - 1)) cpp (cpp + 1 + 1 + 2.01).
-        const int fcpp = (args.kb_total + kChunkBlocks - 1) / kChunkBlocks;
-        const int fcsz = fcpp ? (args.kb_total + fcpp - 1) / fcpp : 0;
+        // With the K range in KS parts the parts' roundings and the KS - 1 additions stay
+        // below what cpp = all the parts' chunks gives.
+        const int pcpp = (args.kb_per_split + kChunkBlocks - 1) / kChunkBlocks;
+        const int fcpp = KS * pcpp;
+        const int fcsz = pcpp ? (args.kb_per_split + pcpp - 1) / pcpp : 0;
         const float err = (float)(1 << (8 * (LB - 1))) * 1.02f * (1.0f / 16.0f) * (float)fcsz *
                           (float)fcpp * ((float)fcpp + 4.2f);
         const bool tight = err <= 0.25f * (float)args.sf;
         const float far = err + 400.0f * (float)args.sf;
-        for (int tile = blockIdx.x; tile < args.total_tiles; tile += gridDim.x) {
+        int barriers = MODE == TC_FWDK ? 2 : 0;     // cluster barriers this thread still owes
+        for (int tile = tile0; tile < args.total_tiles; tile += tile_step) {
             const Tile T = decode_tile(args, tile);
             const int cpp = (T.kb1 - T.kb0 + kChunkBlocks - 1) / kChunkBlocks;
-            uint64_t acc[MODE == TC_FWD ? 1 : NH];
-            uint32_t lo[MODE == TC_FWD ? NH : 1];   // fused forward: z modulo 2^32
-            float zf[MODE == TC_FWD ? NH : 1];      // and z rounded to fp32
+            uint64_t acc[kFused ? 1 : NH];
+            uint32_t lo[kFused ? NH : 1];   // fused forward: z modulo 2^32
+            float zf[kFused ? NH : 1];      // and z rounded to fp32
 #pragma unroll
             for (int i = 0; i < NH; ++i) {
-                if constexpr (MODE == TC_FWD) {
+                if constexpr (kFused) {
                     lo[i] = 0;
                     zf[i] = 0.0f;
                 } else {
@@ -706,7 +744,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     };
                     // 16 or 32 values per TMEM round trip, as the registers beside the
                     // sums allow without spills
-                    if constexpr (MODE == TC_FWD) {
+                    if constexpr (kFused) {
                         // CW columns of a limb pair at once: 16 values in flight beside the
                         // 64 words of 32 columns' sums, 32 beside 16 columns' sums
                         constexpr int CW = NH == 16 ? 16 : 8;
@@ -767,6 +805,41 @@ __global__ void __launch_bounds__(kThreads, 1)
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tempty_bar(buf));
+                }
+            }
+            if constexpr (MODE == TC_FWDK) {
+                // Partial sums of a cluster's K parts: each quarter of the columns is
+                // finished by one CTA, and the others write theirs into its ring
+                // memory, which is idle once every CTA has drained its last chunk.
+                const int owner = KS == 2 ? half >> 1 : half;
+                const int per_owner = KS == 2 ? 2 : 1;
+                constexpr uint32_t kSlot = NH * 2 * 32 * 4;      // one warp's sums
+                const auto slot = [&](int src) {
+                    return smem_u32(smem) + (uint32_t)((src * per_owner + half % per_owner) * 4 + q) * kSlot;
+                };
+                cluster_barrier();
+                if (owner != rank) {
+                    const uint32_t dst = remote_smem(slot(rank), (uint32_t)owner) + 16u * lane;
+#pragma unroll
+                    for (int i = 0; i < NH; i += 4) {
+                        st_remote4(dst + 128u * i, lo[i], lo[i + 1], lo[i + 2], lo[i + 3]);
+                        st_remote4(dst + 128u * (NH + i), __float_as_uint(zf[i]), __float_as_uint(zf[i + 1]),
+                                   __float_as_uint(zf[i + 2]), __float_as_uint(zf[i + 3]));
+                    }
+                }
+                cluster_barrier();
+                barriers = 0;
+                if (owner != rank) continue;
+                for (int src = 0; src < KS; ++src) {
+                    if (src == rank) continue;
+                    const uint8_t* from = smem + (slot(src) - smem_u32(smem)) + 16 * lane;
+#pragma unroll
+                    for (int i = 0; i < NH; i += 4) {
+                        const uint4 a = *reinterpret_cast<const uint4*>(from + 128 * i);
+                        const float4 b = *reinterpret_cast<const float4*>(from + 128 * (NH + i));
+                        lo[i] += a.x; lo[i + 1] += a.y; lo[i + 2] += a.z; lo[i + 3] += a.w;
+                        zf[i] += b.x; zf[i + 1] += b.y; zf[i + 2] += b.z; zf[i + 3] += b.w;
+                    }
                 }
             }
             {
@@ -874,7 +947,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                             }
                         }
                     }
-                } else if constexpr (MODE == TC_FWD) {
+                } else if constexpr (kFused) {
                     // z* = floor(z / SF) from z modulo 2^32 (exact) and z in fp32,
                     // then the NITRO-ReLU value and piece from the table, optional
                     // 2x2 max-pool across lanes; int8 outputs straight from
@@ -1117,7 +1190,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
         }
-    epi_done:;
+    epi_done:
+        for (; barriers > 0; --barriers) cluster_barrier();   // a wait gave up: the peers still count on it
     }
     tc_fence_before();
     __syncthreads();
@@ -1469,6 +1543,9 @@ cudaError_t launch_gemm(const CUtensorMap& a, const CUtensorMap& b, const TcArgs
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
+    if constexpr (MODE == TC_FWDK)
+        return launch_cluster(k_tc_gemm<MODE, N, PB>, dim3(args.total_tiles), kThreads, args.ksplit, s, C::SMEM,
+                              a, b, args);
     const int grid = args.total_tiles < sm_count() ? args.total_tiles : sm_count();
     launch_k(k_tc_gemm<MODE, N, PB>, grid, kThreads, C::SMEM, s, a, b, args);
     return cudaGetLastError();
@@ -1617,6 +1694,7 @@ cudaError_t tc_fwd_preload() {
     cudaFuncAttributes fa{};
     const void* const fns[] = {
         reinterpret_cast<const void*>(k_tc_gemm<TC_FWD, 64, 2>), reinterpret_cast<const void*>(k_tc_gemm<TC_FWD, 128, 2>),
+        reinterpret_cast<const void*>(k_tc_gemm<TC_FWDK, 64, 2>), reinterpret_cast<const void*>(k_tc_gemm<TC_FWDK, 128, 2>),
         reinterpret_cast<const void*>(k_pack_weights_pad), reinterpret_cast<const void*>(k_pack_im2col),
         reinterpret_cast<const void*>(k_pack_act_flat), reinterpret_cast<const void*>(k_pack_act_nhwc)};
     for (const void* f : fns) {
@@ -1740,6 +1818,28 @@ cudaError_t tc_pack_input(TcLayer& t, const LayerGeom& g, const int8_t* x, int b
     return cudaGetLastError();
 }
 
+namespace {
+// K split of the fused forward over a cluster, for layers with few output tiles (one
+// image, 4 x 4 maps): two, four or, with 64-column tiles, eight CTAs a tile while all
+// are resident at once and each has at least four K-blocks, from sixteen K-blocks on (a
+// cluster launch costs the host 1 us).  Clusters of eight, one CTA an SM, do not fill
+// a GPC: up to 104 CTAs, 128 ran in two rounds.  64-column tiles where even four CTAs
+// for each 128-column tile would leave half the SMs idle.  *n: tile width.  Us a launch, events included, unsplit against split: one image 512 ->
+// 512 at 8 x 8 and 4 x 4 34.8 against 14.4 and 16.3, 128 -> 256 at 32 x 32 19.7 against
+// 14.1; 64 images 512 -> 512 at 4 x 4 35.7 against 22.6.
+void fwd_split(TcArgs& a, int cout, int* n) {
+    const auto tiles = [&](int w) { return a.tiles_m * ((cout + w - 1) / w); };
+    if (a.kb_total < 16 || tiles(*n) * 2 > sm_count()) return;
+    if (*n == 128 && tiles(128) * 8 < sm_count()) *n = 64;
+    for (const int s : {8, 4, 2}) {
+        if ((s == 8 && (*n == 128 || tiles(*n) * 8 > 104)) || tiles(*n) * s > sm_count() || a.kb_total < 4 * s)
+            continue;
+        a.ksplit = s;
+        return;
+    }
+}
+}  // namespace
+
 cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* z,
                             const TcFwdOut* fo, uint32_t* status, cudaStream_t s, bool* done,
                             bool* fused) {
@@ -1752,11 +1852,14 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
     a.cin_k = t.cin_k;
     a.taps = t.im2col ? 1 : 9;
     pixel_tiling(g, batch, a);
-    const int n = pick_n(g.cout);
-    a.tiles_n = (g.cout + n - 1) / n;
-    a.total_tiles = a.tiles_m * a.tiles_n;
     a.kb_total = a.taps * (t.cin_k / kBK);
-    a.kb_per_split = a.kb_total;
+    const bool fuse = fo && tc_fwd_fused(t, g);
+    int n = pick_n(g.cout);
+    a.ksplit = 1;
+    if (fuse) fwd_split(a, g.cout, &n);
+    a.tiles_n = (g.cout + n - 1) / n;
+    a.total_tiles = a.tiles_m * a.tiles_n * a.ksplit;
+    a.kb_per_split = (a.kb_total + a.ksplit - 1) / a.ksplit;
     a.ncols = g.cout;
     a.max_a = nullptr;
     a.max_b = t.maxabs_w;
@@ -1764,7 +1867,6 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
     a.out_vec = ((uintptr_t)z & 31) == 0 && g.cout % 4 == 0;
     a.status = status;
     a.atomic_out = 0;
-    const bool fuse = fo && tc_fwd_fused(t, g);
     if (fuse) {
         a.sf = 256 * 9 * g.cin;
         a.sf_inv = 1.0f / (float)a.sf;
@@ -1796,8 +1898,9 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
         return cudaErrorInvalidValue;
     const double ops = 2.0 * batch * g.h * g.w * g.cout * 9.0 * g.cin;
     ProfScope ps(K_TC_CONV_FWD, s, ops, 0.0);
-    cudaError_t e = fuse ? launch_gemm_pb<TC_FWD>(n, pb, ma, mb, a, s)
-                         : launch_gemm_pb<TC_FWDZ>(n, pb, ma, mb, a, s);
+    cudaError_t e = !fuse ? launch_gemm_pb<TC_FWDZ>(n, pb, ma, mb, a, s)
+                          : (a.ksplit > 1 ? launch_gemm_pb<TC_FWDK>(n, pb, ma, mb, a, s)
+                                          : launch_gemm_pb<TC_FWD>(n, pb, ma, mb, a, s));
     if (e == cudaSuccess) {
         *done = true;
         *fused = fuse;
