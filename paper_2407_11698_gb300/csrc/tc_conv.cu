@@ -26,9 +26,10 @@ namespace nitro {
 namespace {
 
 // TC_FWD: forward with the fused NITRO-Scaling / NITRO-ReLU / max-pool epilogue;
-// TC_FWDK: the same with a tile's K shared out over a cluster; TC_FWDZ: the forward
-// contraction with int64 sums as its output.
-enum TcMode : int { TC_FWD = 0, TC_WGRAD = 1, TC_DGRAD = 2, TC_GEMM = 3, TC_FWDZ = 4, TC_FWDK = 5 };
+// TC_FWDK: the same with a tile's K shared out over a cluster; TC_DGRAD: input gradient
+// with the fused routing into the lower layer's delta; TC_FWDZ, TC_DGRADZ: the same
+// contractions with int64 sums as their output.
+enum TcMode : int { TC_FWD = 0, TC_WGRAD = 1, TC_DGRAD = 2, TC_GEMM = 3, TC_FWDZ = 4, TC_FWDK = 5, TC_DGRADZ = 6 };
 
 constexpr int kBM = 128;              // rows per tile (TMEM lanes)
 constexpr int kBK = 64;               // K elements per block (one 128-byte row)
@@ -248,7 +249,6 @@ struct TcArgs {
     uint32_t* status;
     int atomic_out;
     int out_vec;           // int64 rows are 32-byte aligned: four values a store
-    int fuse;              // input gradient: fused epilogue
     int ksplit;            // fused forward: CTAs of a cluster that share a tile's K (1: none)
     // forward with fused NITRO-Scaling / NITRO-ReLU / max-pool epilogue
     FloorDiv alpha;        // divide by alpha_inv
@@ -312,13 +312,21 @@ __device__ __forceinline__ void st8(int8_t* dst, const uint32_t* w) {
 __device__ __forceinline__ void st16(int8_t* dst, const uint32_t* w) {
     *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
 }
+// eight words, one 32-byte store
+__device__ __forceinline__ void st_u32x8(void* dst, const uint32_t* w) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]),
+                 "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                 : "memory");
+}
+// all bits of the word set where byte e of a byte mask is
+__device__ __forceinline__ int32_t byte_mask(uint32_t mask, int e) {
+    return (int32_t)__byte_perm(mask, 0, 0x8888u + 0x1111u * (uint32_t)e);
+}
 // 32 int8 values (8 packed words): one 32-byte store (a whole sector) when the
 // destination is 32-byte aligned, else two of 16 bytes
 __device__ __forceinline__ void st32(int8_t* dst, const uint32_t* w, bool aligned32) {
     if (aligned32) {
-        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]),
-                     "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
-                     : "memory");
+        st_u32x8(dst, w);
     } else {
         st16(dst, w);
         st16(dst + 16, w + 4);
@@ -397,6 +405,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr int NH = N / 4;            // columns per epilogue warp
     constexpr bool kFused = MODE == TC_FWD || MODE == TC_FWDK;
     constexpr bool kFwd = kFused || MODE == TC_FWDZ;
+    constexpr bool kDgrad = MODE == TC_DGRAD || MODE == TC_DGRADZ;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -457,11 +466,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         // of 2^32.  They matter only for deciding OVERFLOW, so once that bit
         // is latched they are skipped.  Read once per CTA so that all roles
         // walk the same passes (CTAs may differ; each result is the same).
-        *hiskip_slot = (MODE == TC_DGRAD && args.fuse)
+        *hiskip_slot = MODE == TC_DGRAD
             ? ((*reinterpret_cast<volatile uint32_t*>(args.status) & ST_OVERFLOW) != 0) : 0;
     }
     // int32 x int32 contraction: flag when max|delta| max|W| 9 Cout >= 2^63
-    if (MODE == TC_DGRAD && args.fuse && blockIdx.x == 0 && threadIdx.x == 64 &&
+    if (MODE == TC_DGRAD && blockIdx.x == 0 && threadIdx.x == 64 &&
         int64_bound_exceeded(*args.bound_a, *args.bound_b, 9LL * args.Cout))
         atomicOr(args.status, ST_OVERFLOW);
     tc_fence_before();
@@ -525,7 +534,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // cb fastest, walked incrementally
                     const int knc = kFwd ? args.cin_k / kBK : (args.Cout + kBK - 1) / kBK;
                     int kt = 0, kcb = 0;
-                    if (kFwd || MODE == TC_DGRAD) {
+                    if (kFwd || kDgrad) {
                         kt = T.kb0 / knc;
                         kcb = T.kb0 - kt * knc;
                     }
@@ -551,7 +560,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                             // PB limb tiles [limb][N rows][64 k], one box
                             tma_load_3d(b_dst, &tmB, fb, t * args.cin_k + cb * kBK, n0, lb0);
                             if (++kcb == knc) { kcb = 0; ++kt; }
-                        } else if (MODE == TC_DGRAD) {
+                        } else if (kDgrad) {
                             const int t = kt, cb = kcb, ky = t / 3, kx = t - 3 * ky;
                             if (++kcb == knc) { kcb = 0; ++kt; }
                             tma_load_5d(a_dst, &tmA, fb, cb * kBK, x0 - kx + 1, y0 - ky + 1, b0, la);
@@ -596,14 +605,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             uint32_t idesc_nb[PB + 1];
 #pragma unroll
             for (int j = 1; j <= PB; ++j)
-                idesc_nb[j] = idesc_bf16(kBM, j * N, MODE == TC_WGRAD, MODE == TC_WGRAD || MODE == TC_DGRAD);
+                idesc_nb[j] = idesc_bf16(kBM, j * N, MODE == TC_WGRAD, MODE == TC_WGRAD || kDgrad);
             // K-major: a K-step of 16 is 32 bytes along each row; MN-major: 16
             // rows, two 1024-byte row groups, and 64-wide blocks along M / N 8 KB
             // apart.  Only the address field (bytes / 16, below 2^14 since shared
             // memory is below 256 KB) moves per K-step and per ring stage, so the
             // descriptors of stage 0 are built once and offset per K-block.
             constexpr bool a_mn = MODE == TC_WGRAD;
-            constexpr bool b_mn = MODE == TC_WGRAD || MODE == TC_DGRAD;
+            constexpr bool b_mn = MODE == TC_WGRAD || kDgrad;
             constexpr uint32_t kStepA = a_mn ? 2048 / 16 : 32 / 16;
             constexpr uint32_t kStepB = b_mn ? 2048 / 16 : 32 / 16;
             constexpr uint32_t kStageD = C::STAGE / 16;
@@ -675,6 +684,224 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int q = warp & 3;                     // TMEM lane quadrant this warp may read
         const int half = (warp - kEpiWarp0) >> 2;   // which quarter of the N columns
         int chunk = 0;
+        if constexpr (MODE == TC_DGRAD) {
+            // Fused input gradient: gradient at the lower layer's (pooled) output -> int32
+            // with the OVERFLOW rule -> max-pool backward (to the recorded window
+            // position) -> NITRO-ReLU backward -> lower delta.
+            //
+            // The delta is the low 32 bits of the sum, kept as they are; OVERFLOW needs the
+            // rest only as far as the sum being those 32 bits or 2^32 and more away from
+            // them, so an fp32 sum that is off by less than 2^31 decides it (form 1).  With
+            // the bit latched it is not needed (form 0); where the bound of its error is
+            // too large (six limbs and more together) the sums are 64 bits wide (form 2).
+            // The bound: every chunk of every pass rounds a pair of limb sums and the
+            // running sum, which stays below cpp csz 2^20 2^(8 (LA + LB - 2)) (1 + 2^-5).
+            // Bound by the latency of the epilogue's chains.  64-bit sums throughout, an
+            // atomic maximum a warp and tile and 16-byte stores: 128 -> 128 at 16 x 16, 256
+            // -> 256 at 8 x 8, batch 128, latched, 51.6 and 47.0 us, now 41.2 and 38.8.
+            const int ccpp = (args.kb_total + kChunkBlocks - 1) / kChunkBlocks;
+            const int ccsz = ccpp ? (args.kb_total + ccpp - 1) / ccpp : 0;
+            const float derr = exp2f((float)(8 * (LA + LB - 2))) * 1.04f / 16.0f * (float)ccsz * (float)ccpp *
+                               (float)(LA * LB) * (float)(ccpp + 1);
+            const int form = hiskip ? 0 : (derr < 2.0e9f ? 1 : 2);
+            const int npos = args.low_pool ? 4 : 1;
+            const int Cl = args.Cin;
+            bool ovf = false;
+            uint32_t mx = 0;
+            for (int tile = tile0; tile < args.total_tiles; tile += tile_step) {
+                const Tile T = decode_tile(args, tile);
+                const int r = 32 * q + lane;   // output row of this thread
+                const int col0 = T.nt * N + half * NH;
+                const int mq = udiv32(args.dv_ntx, T.mt), tb = udiv32(args.dv_nty, mq);
+                const int tx = T.mt - mq * args.ntx, ty = mq - tb * args.nty;
+                const int xx = r & ((1 << args.lg_wb) - 1);
+                const int yy = (r >> args.lg_wb) & ((1 << args.lg_hb) - 1);
+                const int bbx = r >> (args.lg_wb + args.lg_hb);
+                const int x = tx * args.wb + xx, y = ty * args.hb + yy, b = tb * args.bb + bbx;
+                const bool valid = x < args.W && y < args.H && b < args.B;
+                // element offsets (below 2^31, checked when the block is made) of this
+                // thread's channels at the gradient's position and the window's positions
+                const uint32_t opix = (uint32_t)((b * args.H + y) * args.W + x) * Cl + col0;
+                const uint32_t p0 = args.low_pool
+                    ? (uint32_t)((b * args.low_h + 2 * y) * args.low_w + 2 * x) * Cl + col0 : opix;
+                const uint32_t prow = (uint32_t)args.low_w * Cl;
+                // argmax and region codes of 16 channels; with 16 columns a thread they are
+                // loaded before the sums are waited for
+                uint4 am, rg[4];
+                const auto load_codes = [&](int k16) {
+                    const bool in = valid && col0 + 16 * k16 < Cl;
+                    am = in && npos == 4 ? *reinterpret_cast<const uint4*>(args.low_argmax + opix + 16 * k16)
+                                         : make_uint4(0, 0, 0, 0);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        rg[k] = in && k < npos
+                            ? *reinterpret_cast<const uint4*>(args.low_region + p0 + 16 * k16 + (k >> 1) * prow +
+                                                              (k & 1) * Cl)
+                            : make_uint4(0, 0, 0, 0);
+                };
+                if constexpr (NH == 16) load_codes(0);
+                uint32_t lo[NH];
+                float zf[NH];
+                // body(address of limb 0's columns, limbs, shift of the first) for every
+                // chunk of every pass
+                const auto chunks = [&](auto body) -> bool {
+                    const int cpp = (T.kb1 - T.kb0 + kChunkBlocks - 1) / kChunkBlocks;
+                    for (int la = 0; la < LA; ++la)
+                    for (int lb0 = 0; lb0 < lb_limit(la); lb0 += PB) {
+                        const int nb = min(PB, lb_limit(la) - lb0);
+                        for (int c = 0; c < cpp; ++c, ++chunk) {
+                            const int buf = chunk % NBUF;
+                            if (!mbar_wait(tfull_bar(buf), (chunk / NBUF) & 1, abort_flag, args.status))
+                                return false;
+                            tc_fence_after();
+                            // 64-column blocks ordered [channel block][limb of this pass]
+                            const int hb = (half * NH) / 64;
+                            const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) +
+                                (uint32_t)(buf * PB * N + hb * nb * 64 + half * NH - hb * 64);
+                            body(base, nb, 8 * (la + lb0));
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(tempty_bar(buf));
+                        }
+                    }
+                    return true;
+                };
+                // sums modulo 2^32, and with kFp the fp32 sums, a limb pair at a time
+                const auto narrow = [&](auto kFp) -> bool {
+                    constexpr int CW = 8;
+#pragma unroll
+                    for (int i = 0; i < NH; ++i) {
+                        lo[i] = 0;
+                        if (kFp()) zf[i] = 0.0f;
+                    }
+                    return chunks([&](uint32_t base, int nb, int shift0) {
+#pragma unroll
+                        for (int j = 0; j < NH / CW; ++j)
+                            for (int jb = 0; jb < nb; jb += 2) {
+                                const bool two = jb + 1 < nb;
+                                const uint32_t m = 1u << (shift0 + 8 * jb);
+                                const float mf = (float)m;
+                                uint32_t v[2 * CW];
+                                tmem_ld8_nowait(base + 64 * jb + CW * j, v);
+                                if (two) tmem_ld8_nowait(base + 64 * (jb + 1) + CW * j, v + CW);
+                                tmem_wait_ld<2 * CW>(v);
+                                if (two) {
+#pragma unroll
+                                    for (int i = 0; i < CW; ++i) {
+                                        const float v0 = __uint_as_float(v[i]), v1 = __uint_as_float(v[CW + i]);
+                                        const uint32_t w = ((uint32_t)__float2int_rz(v1) << 8) + (uint32_t)__float2int_rz(v0);
+                                        lo[CW * j + i] += w * m;
+                                        if (kFp()) zf[CW * j + i] = fmaf(fmaf(v1, 256.0f, v0), mf, zf[CW * j + i]);
+                                    }
+                                } else {
+#pragma unroll
+                                    for (int i = 0; i < CW; ++i) {
+                                        const float v0 = __uint_as_float(v[i]);
+                                        lo[CW * j + i] += (uint32_t)__float2int_rz(v0) * m;
+                                        if (kFp()) zf[CW * j + i] = fmaf(v0, mf, zf[CW * j + i]);
+                                    }
+                                }
+                            }
+                    });
+                };
+                bool ok;
+                if (form == 0) {
+                    ok = narrow(std::false_type());
+                } else if (form == 1) {
+                    ok = narrow(std::true_type());
+#pragma unroll
+                    for (int i = 0; i < NH; ++i)
+                        ovf |= valid && col0 + i < Cl && fabsf(zf[i] - (float)(int32_t)lo[i]) > 2147483648.0f;
+                } else {
+                    uint64_t acc[NH];
+#pragma unroll
+                    for (int i = 0; i < NH; ++i) acc[i] = 0;
+                    ok = chunks([&](uint32_t base, int nb, int shift0) {
+                        for (int jb = 0; jb < nb; ++jb)
+#pragma unroll
+                            for (int j = 0; j < NH / 8; ++j) {
+                                uint32_t v[8];
+                                tmem_ld8_nowait(base + 64 * jb + 8 * j, v);
+                                tmem_wait_ld<8>(v);
+#pragma unroll
+                                for (int i = 0; i < 8; ++i)
+                                    acc[8 * j + i] += (uint64_t)(int64_t)__float2int_rz(__uint_as_float(v[i]))
+                                                      << (shift0 + 8 * jb);
+                            }
+                    });
+#pragma unroll
+                    for (int i = 0; i < NH; ++i) {
+                        ovf |= valid && col0 + i < Cl && !fits_i32((int64_t)acc[i]);
+                        lo[i] = (uint32_t)acc[i];
+                    }
+                }
+                if (!ok) break;
+                // Eight channels at a time: NITRO-ReLU backward once, by the region code at the
+                // recorded position, then each window position gets it or zero.  Codes are
+                // 0..3: the byte masks of one code value come from its two bits.
+                const auto route = [&](auto kPool) {
+                    constexpr int NP = kPool() ? 4 : 1;
+#pragma unroll
+                    for (int k16 = 0; k16 < NH / 16; ++k16) {
+                        if (col0 + 16 * k16 >= Cl) break;   // uniform across the warp
+                        if constexpr (NH != 16) load_codes(k16);
+                        const uint32_t amw[4] = {am.x, am.y, am.z, am.w};
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            int32_t v[8];
+                            uint32_t at[2][NP];
+#pragma unroll
+                            for (int e4 = 0; e4 < 2; ++e4) {
+                                const int w = 2 * h + e4;
+                                const uint32_t r0[4] = {rg[0].x, rg[0].y, rg[0].z, rg[0].w};
+                                uint32_t code = r0[w];
+                                if constexpr (kPool()) {
+                                    const uint32_t a0 = amw[w], a1 = amw[w] >> 1;
+                                    at[e4][0] = (~a0 & ~a1 & 0x01010101u) * 255u;
+                                    at[e4][1] = (a0 & ~a1 & 0x01010101u) * 255u;
+                                    at[e4][2] = (~a0 & a1 & 0x01010101u) * 255u;
+                                    at[e4][3] = (a0 & a1 & 0x01010101u) * 255u;
+                                    code = 0;
+#pragma unroll
+                                    for (int k = 0; k < 4; ++k) {
+                                        const uint32_t rw[4] = {rg[k].x, rg[k].y, rg[k].z, rg[k].w};
+                                        code |= rw[w] & at[e4][k];
+                                    }
+                                }
+                                const uint32_t m1 = (code & ~(code >> 1) & 0x01010101u) * 255u;
+                                const uint32_t m2 = (~code & (code >> 1) & 0x01010101u) * 255u;
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    const int32_t g = (int32_t)lo[16 * k16 + 8 * h + 4 * e4 + e];
+                                    const int32_t gq = args.alpha32.floor_div(g);
+                                    v[4 * e4 + e] = (gq & byte_mask(m1, e)) | (g & byte_mask(m2, e));
+                                }
+                            }
+                            if (!valid) continue;
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) mx = max(mx, abs_u32(v[e]));
+#pragma unroll
+                            for (int k = 0; k < NP; ++k) {
+                                uint32_t o[8];
+#pragma unroll
+                                for (int e = 0; e < 8; ++e)
+                                    o[e] = kPool() ? (uint32_t)(v[e] & byte_mask(at[e >> 2][k], e & 3)) : (uint32_t)v[e];
+                                st_u32x8(reinterpret_cast<uint32_t*>(args.low_delta) + p0 + 16 * k16 + 8 * h +
+                                             (k >> 1) * prow + (k & 1) * Cl, o);
+                            }
+                        }
+                    }
+                };
+                if (args.low_pool) route(std::true_type());
+                else route(std::false_type());
+            }
+            mx = __reduce_max_sync(0xffffffffu, mx);
+            ovf = __any_sync(0xffffffffu, ovf);
+            if (lane == 0) {
+                if (mx) atomicMax(args.low_maxabs, mx);
+                if (ovf) atomicOr(args.status, ST_OVERFLOW);
+            }
+        } else {
         // Fused forward: bound of the error of its fp32 sums.  A chunk of csz K-blocks
         // has limb sums below csz 2^20 2^(8 limb).  Per chunk at most two roundings (of
         // 2^-24) hit the running sum, which stays below c csz 2^20 2^(8 (LB - 1)) (1 +
@@ -719,7 +946,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // ordered [channel block][limb of this pass]
                     auto limb_base = [&](int jb) -> uint32_t {
                         const int hb = (half * NH) / 64;
-                        const int colj = (MODE == TC_WGRAD || MODE == TC_DGRAD)
+                        const int colj = (MODE == TC_WGRAD || kDgrad)
                             ? (hb * pbw + jb) * 64 + (half * NH - hb * 64)
                             : jb * N + half * NH;
                         return tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * PB * N + colj);
@@ -1071,104 +1298,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 if (col0 + 8 * k < C) st8_bf16(args.next_nhwc + o + 8 * k, vpk + 2 * k);
                         }
                     }
-                } else if (MODE == TC_DGRAD && args.fuse) {
-                    // gradient at the lower layer's (pooled) output -> int32 with
-                    // the OVERFLOW rule -> max-pool backward (to the recorded
-                    // window position) -> NITRO-ReLU backward -> lower delta.
-                    const int mq = udiv32(args.dv_ntx, T.mt), tb = udiv32(args.dv_nty, mq);
-                    const int tx = T.mt - mq * args.ntx, ty = mq - tb * args.nty;
-                    const int xx = r & ((1 << args.lg_wb) - 1);
-                    const int yy = (r >> args.lg_wb) & ((1 << args.lg_hb) - 1);
-                    const int bbx = r >> (args.lg_wb + args.lg_hb);
-                    const int x = tx * args.wb + xx, y = ty * args.hb + yy, b = tb * args.bb + bbx;
-                    const bool valid = x < args.W && y < args.H && b < args.B;
-                    const int Cl = args.Cin;
-                    bool ovf = false;
-                    uint32_t mx = 0;
-                    if (valid) {
-                        const int64_t opix = ((int64_t)b * args.H + y) * args.W + x;
-                        const int npos = args.low_pool ? 4 : 1;
-                        int64_t ppix[4];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            ppix[k] = args.low_pool
-                                ? ((int64_t)b * args.low_h + 2 * y + (k >> 1)) * args.low_w + 2 * x + (k & 1)
-                                : opix;
-                        // the int32 values first (storage rule), then the argmax and
-                        // region words of all the thread's channels and window positions
-                        // in one batch of 16-byte loads, then per 4 channels the floor
-                        // quotient by alpha_inv, the routing and the stores
-                        constexpr int NG16 = NH / 16;
-                        int32_t gsv[NH];
-#pragma unroll
-                        for (int i = 0; i < NH; ++i) {
-                            const int64_t gv = (int64_t)acc[i];
-                            ovf |= col0 + i < Cl && !fits_i32(gv);
-                            gsv[i] = (int32_t)gv;
-                        }
-                        // two groups of 16 channels per batch of code loads
-#pragma unroll
-                        for (int kp = 0; kp < NG16; kp += 2) {
-                            if (col0 + 16 * kp >= Cl) break;   // uniform across the warp
-                            uint4 amv[2], rgv[2][4];
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                const int c16 = col0 + 16 * (kp + h);
-                                const bool in = kp + h < NG16 && c16 < Cl;
-                                amv[h] = (args.low_pool && in)
-                                    ? *reinterpret_cast<const uint4*>(args.low_argmax + opix * Cl + c16)
-                                    : make_uint4(0, 0, 0, 0);
-#pragma unroll
-                                for (int k = 0; k < 4; ++k)
-                                    rgv[h][k] = (k < npos && in)
-                                        ? *reinterpret_cast<const uint4*>(args.low_region + ppix[k] * Cl + c16)
-                                        : make_uint4(0, 0, 0, 0);
-                            }
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                const int k16 = kp + h;
-                                const int c16 = col0 + 16 * k16;
-                                if (k16 >= NG16 || c16 >= Cl) break;
-                                const uint32_t amw4[4] = {amv[h].x, amv[h].y, amv[h].z, amv[h].w};
-#pragma unroll
-                                for (int e4 = 0; e4 < 4; ++e4) {
-                                    const int c0 = c16 + 4 * e4;
-                                    int32_t gs[4], gq[4];   // gradient and floor(gradient / alpha_inv)
-#pragma unroll
-                                    for (int e = 0; e < 4; ++e) {
-                                        gs[e] = gsv[16 * k16 + 4 * e4 + e];
-                                        gq[e] = args.alpha32.floor_div(gs[e]);
-                                    }
-                                    const uint32_t amw = amw4[e4];
-#pragma unroll
-                                    for (int k = 0; k < 4; ++k) {
-                                        if (k >= npos) break;
-                                        const uint32_t rw[4] = {rgv[h][k].x, rgv[h][k].y, rgv[h][k].z,
-                                                                rgv[h][k].w};
-                                        const uint32_t rgw = rw[e4];
-                                        int32_t dv[4];
-#pragma unroll
-                                        for (int e = 0; e < 4; ++e) {
-                                            const int reg = (int)((rgw >> (8 * e)) & 255u);
-                                            const int am = (int)((amw >> (8 * e)) & 255u);
-                                            const int32_t v = am != k ? 0 : (reg == 1 ? gq[e] : (reg == 2 ? gs[e] : 0));
-                                            dv[e] = v;
-                                            mx = max(mx, abs_u32(v));
-                                        }
-                                        *reinterpret_cast<int4*>(args.low_delta + ppix[k] * Cl + c0) =
-                                            make_int4(dv[0], dv[1], dv[2], dv[3]);
-                                    }
-                                }
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int off = 16; off; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-                    ovf = __any_sync(0xffffffffu, ovf);
-                    if (lane == 0) {
-                        if (mx) atomicMax(args.low_maxabs, mx);
-                        if (ovf) atomicOr(args.status, ST_OVERFLOW);
-                    }
                 } else {
                     const int mq = udiv32(args.dv_ntx, T.mt), tb = udiv32(args.dv_nty, mq);
                     const int tx = T.mt - mq * args.ntx, ty = mq - tb * args.nty;
@@ -1190,8 +1319,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
         }
-    epi_done:
+    epi_done:;
         for (; barriers > 0; --barriers) cluster_barrier();   // a wait gave up: the peers still count on it
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -1424,6 +1554,25 @@ __global__ void k_pack_weights(const int32_t* __restrict__ W, int Cout, int Cin,
 
 }
 
+// Maximum over a launch: the CTA's into scratch[0] (one atomic a CTA), and the last
+// CTA, by the ticket in scratch[1], stores it to *out and leaves both words zero.
+__device__ __forceinline__ void publish_max(uint32_t m, uint32_t* out, uint32_t* scratch) {
+    __shared__ uint32_t cta_max;
+    if (threadIdx.x == 0) cta_max = 0;
+    __syncthreads();
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(&cta_max, m);
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    if (cta_max) atomicMax(&scratch[0], cta_max);
+    __threadfence();
+    if (atomicAdd(&scratch[1], 1u) == gridDim.x - 1) {
+        __threadfence();
+        *out = atomicExch(&scratch[0], 0u);
+        scratch[1] = 0;
+    }
+}
+
 // The same into all four planes, eight entries a thread, zeros where the rows are
 // padded, and *out = max |W| (maximum and CTA ticket in scratch[0], scratch[1],
 // zero between launches): one launch for planes whose memory holds anything.
@@ -1449,17 +1598,7 @@ __global__ void __launch_bounds__(256) k_pack_weights_pad(const int32_t* __restr
                 make_uint4(limb_bf16x2(v[0], v[1], l), limb_bf16x2(v[2], v[3], l),
                            limb_bf16x2(v[4], v[5], l), limb_bf16x2(v[6], v[7], l));
     }
-    mx = __reduce_max_sync(0xffffffffu, mx);
-    if ((threadIdx.x & 31) == 0) {
-        if (mx) atomicMax(&scratch[0], mx);
-        __threadfence();     // this warp's maximum, before the CTA's ticket
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && atomicAdd(&scratch[1], 1u) == gridDim.x - 1) {
-        __threadfence();
-        *out = atomicExch(&scratch[0], 0u);
-        scratch[1] = 0;
-    }
+    publish_max(mx, out, scratch);
 }
 
 // ------------------------------------------------------------------ host side
@@ -2032,8 +2171,8 @@ cudaError_t tc_conv_dgrad(TcLayer& t, const LayerGeom& g, int batch, int64_t* g6
     a.out_vec = ((uintptr_t)g64 & 31) == 0 && g.cin % 4 == 0;
     a.status = status;
     a.atomic_out = 0;
-    if (fo && g.cin % 16 == 0) {
-        a.fuse = 1;
+    const bool fuse = fo && g.cin % 16 == 0;
+    if (fuse) {
         a.alpha32 = FloorDiv32::make((uint32_t)fo->alpha_inv);
         a.bound_a = fo->maxabs_delta;
         a.bound_b = fo->maxabs_w;
@@ -2067,10 +2206,11 @@ cudaError_t tc_conv_dgrad(TcLayer& t, const LayerGeom& g, int batch, int64_t* g6
         return cudaErrorInvalidValue;
     const double ops = 2.0 * batch * g.h * g.w * g.cin * 9.0 * g.cout;
     ProfScope ps(K_TC_CONV_DGRAD, s, ops, 0.0);
-    cudaError_t e = launch_gemm_pb<TC_DGRAD>(n, pb, ma, mb, a, s);
+    cudaError_t e = fuse ? launch_gemm_pb<TC_DGRAD>(n, pb, ma, mb, a, s)
+                         : launch_gemm_pb<TC_DGRADZ>(n, pb, ma, mb, a, s);
     if (e == cudaSuccess) {
         *done = true;
-        *fused = a.fuse != 0;
+        *fused = fuse;
     }
     return e;
 }
@@ -2109,18 +2249,7 @@ __global__ void __launch_bounds__(256) k_maxabs(const int32_t* __restrict__ x, i
     for (; i < n4; i += stride) take(xv[i]);
     if (tid < head) m = max(m, abs_u32(x[tid]));
     if (tid < n - tail) m = max(m, abs_u32(x[tail + tid]));
-#pragma unroll
-    for (int off = 16; off; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if ((threadIdx.x & 31) == 0) {
-        if (m) atomicMax(&scratch[0], m);
-        __threadfence();     // this warp's maximum, before the CTA's ticket
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && atomicAdd(&scratch[1], 1u) == gridDim.x - 1) {
-        __threadfence();
-        *out = atomicExch(&scratch[0], 0u);
-        scratch[1] = 0;
-    }
+    publish_max(m, out, scratch);
 }
 }  // namespace
 
