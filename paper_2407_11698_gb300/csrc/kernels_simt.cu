@@ -363,23 +363,20 @@ __global__ void __launch_bounds__(256) k_learn_fwd(const LearnArgs p, FloorDiv d
                                                    int32_t* __restrict__ grad_l,
                                                    const uint32_t* maxabs_wlr, uint32_t* status,
                                                    uint32_t* zero_words, int n_zero,
-                                                   int64_t* zero_dwlr) {
+                                                   uint32_t* gl_bound) {
     namespace cg = cooperative_groups;
     const cg::cluster_group cluster = cg::this_cluster();
     const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     __shared__ __align__(16) uint32_t ws[4 * kLfG * 64];
     __shared__ long long part[kLfSamples][kMaxClasses];
     const int u = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int group = blockIdx.x / S, groups = gridDim.x / S;
+    const int group = blockIdx.x / S;
     const int b = group * kLfSamples + u;
     pdl_wait();
     const int limbs = limb_count(*maxabs_wlr);
     // nothing in this launch reads what is cleared here
     if (blockIdx.x == 0 && threadIdx.x < n_zero) zero_words[threadIdx.x] = 0;
     const int j0 = rank * p.per, j1 = min(p.d, j0 + p.per);
-    if (zero_dwlr)
-        for (int g = group; g < p.G; g += groups)
-            for (int j = j0 + threadIdx.x; j < j1; j += 256) zero_dwlr[(int64_t)g * p.d + j] = 0;
     for (int gc = 0; gc < p.G; gc += kLfG) {
         const long long z = p.G <= 10 ? learn_pass<10>(p, limbs, b, gc, j0, j1, ws)
                                       : learn_pass<kLfG>(p, limbs, b, gc, j0, j1, ws);
@@ -387,6 +384,7 @@ __global__ void __launch_bounds__(256) k_learn_fwd(const LearnArgs p, FloorDiv d
     }
     cluster.sync();
     // sample v of the group is finished by CTA v mod S
+    uint32_t mx = 0;
     for (int i = threadIdx.x; i < kLfSamples * p.G; i += 256) {
         const int v = i / p.G, g = i - v * p.G, bb = group * kLfSamples + v;
         if (v % S != rank || bb >= p.B) continue;
@@ -400,7 +398,10 @@ __global__ void __launch_bounds__(256) k_learn_fwd(const LearnArgs p, FloorDiv d
         if (bad && g == 0) atomicOr(status, ST_BAD_LABEL);
         if (!fits_i32(t)) atomicOr(status, ST_OVERFLOW);
         grad_l[(int64_t)bb * p.G + g] = (int32_t)t;
+        mx = max(mx, abs_u32((int32_t)t));
     }
+    mx = __reduce_max_sync(kFull, mx);
+    if (lane == 0 && mx) atomicMax(gl_bound, mx);
     cluster.sync();      // the partial sums stay until every CTA has read them
 }
 
@@ -502,10 +503,10 @@ __global__ void __launch_bounds__(256) k_lin_wgrad(const int8_t* __restrict__ a,
         if (i0 + 4 * q + k < in) row[i0 + 4 * q + k] = acc[k];
 }
 
-// The last CTA column of the kernel after k_learn_fwd: SSE, loss = floor(SSE / 2),
-// max |grad_L| and, with wlr_max != null, the int64 exactness bound of grad_L W_lr.
-// One CTA forms them up to kTailValues values; above, the column's CTAs add their
-// shares into *sse and *maxabs_gl (cleared by k_learn_fwd) and the last one ends.
+// The last CTAs of the kernel after k_learn_fwd: SSE, loss = floor(SSE / 2), max
+// |grad_L| and, with wlr_max != null, the int64 exactness bound of grad_L W_lr.
+// One CTA forms them up to kTailValues values; above, several add their shares
+// into *sse and *maxabs_gl (cleared by k_learn_fwd) and the last one ends.
 struct LossTail {
     const int32_t* grad_l;
     int B, G;
@@ -517,13 +518,11 @@ struct LossTail {
     uint32_t* status;
 };
 constexpr int kTailValues = 8192;
-__device__ __forceinline__ void loss_tail(const LossTail& t) {
+__device__ __forceinline__ void loss_tail(const LossTail& t, int cta, int ctas) {
     const int64_t n = (int64_t)t.B * t.G;
-    const int ctas = (int)min((int64_t)gridDim.y, (n + kTailValues - 1) / kTailValues);
-    if ((int)blockIdx.y >= ctas) return;
     unsigned long long ss = 0;
     uint32_t mx = 0;
-    for (int64_t i = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; i < n; i += (int64_t)ctas * blockDim.x) {
+    for (int64_t i = (int64_t)cta * blockDim.x + threadIdx.x; i < n; i += (int64_t)ctas * blockDim.x) {
         const int32_t v = t.grad_l[i];
         ss += (unsigned long long)((int64_t)v * v);              // modulo 2^64
         mx = max(mx, abs_u32(v));
@@ -563,23 +562,6 @@ __device__ __forceinline__ void loss_tail(const LossTail& t) {
     }
 }
 
-// dW_lr[g][j] = sum_b grad_l[b][g] * a[b][j]; the last CTA column forms the loss
-__global__ void k_learn_dw(const int8_t* __restrict__ a, const int32_t* __restrict__ grad_l,
-                           int B, int d, int G, int64_t* __restrict__ dwlr, const LossTail tail) {
-    pdl_wait();
-    if (blockIdx.x == gridDim.x - 1) {
-        loss_tail(tail);
-        return;
-    }
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int g = blockIdx.y;
-    if (j >= d) return;
-    int64_t s = 0;
-#pragma unroll 8
-    for (int b = 0; b < B; ++b) s += (int64_t)grad_l[(int64_t)b * G + g] * a[(int64_t)b * d + j];
-    dwlr[(int64_t)g * d + j] = s;
-}
-
 // ---------------------------------------------------------------------------
 // Gradient at a layer output -> delta at its pre-activation.
 // ---------------------------------------------------------------------------
@@ -598,17 +580,7 @@ __global__ void k_grad_to_delta(DeltaSrc src, LayerGeom g, int B, int alpha_inv,
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = i / out_f, q = i - b * out_f;
-        int64_t gv;
-        if (src.wlr) {
-            uint64_t acc = 0;  // modulo 2^64, exact below the bound
-#pragma unroll 16
-            for (int k = 0; k < src.G; ++k)
-                acc += (uint64_t)(int64_t)src.grad_l[b * src.G + k] *
-                       (uint64_t)(int64_t)src.wlr[(int64_t)k * out_f + q];
-            gv = (int64_t)acc;
-        } else {
-            gv = src.g64[i];
-        }
+        const int64_t gv = src.g64[i];
         ovf |= !fits_i32(gv);
         const int32_t gs = (int32_t)gv;
         if (g.pool) {
@@ -973,6 +945,7 @@ __global__ void __launch_bounds__(256) k_integersgd(const SgdBatch bt) {
         *bt.t[threadIdx.x].maxabs_w = atomicExch(&bt.scratch[threadIdx.x], 0u);
     if (threadIdx.x == 0) {
         bt.scratch[kMaxSgdTensors] = 0;
+        bt.scratch[kMaxSgdTensors + 1] = 0;    // the bound of |grad_L|, of the step that ends
         // one block step taken: advance the dropout step counter
         if (bt.step) *bt.step += 1u;
     }
@@ -982,243 +955,227 @@ __global__ void __launch_bounds__(256) k_integersgd(const SgdBatch bt) {
 }
 
 // ---------------------------------------------------------------------------
-// Learning-layer backward, fused, for G <= 16.  CTA: 64 features q of the
-// block output x 16 samples; grad_L and the 16 x 64 slice of a are staged in
-// shared memory.  dW_lr[g][q] partials over the 16 samples are dot products
-// out of shared memory, added to a zeroed dW_lr with 64-bit atomics.  With a
-// forward layer below (has_delta): thread (q, lane) forms delta_fw[b][q] =
-// sum_g grad_L[b][g] W_lr[g][q] (int32 storage rule) for samples lane,
-// lane + 4, ... and routes it through max-pool backward and NITRO-ReLU
-// backward into that layer's delta; the region bytes of its four samples are
-// loaded before any is used.
+// Learning-layer backward, one launch of three kinds of CTAs that wait on nothing
+// of one another:
+//   dW_lr[g][q] = sum_b grad_L[b][g] a[b][q] for 16 V features, all samples: sixteen
+//     sample lanes with the sums of GM classes in registers, added through shared
+//     memory, written once (no K split, no clearing, no atomics);
+//   delta_fw[b][q] = sum_g grad_L[b][g] W_lr[g][q] (int32 storage rule) for 16 V features
+//     x 16 samples, routed through max-pool backward and NITRO-ReLU backward into the
+//     last layer's delta, every position written, with the delta's bf16 limb planes
+//     (planes != null; as many as G max|grad_L| max|W_lr| can need), so that no pass
+//     reads delta again; these CTAs also clear zero[0..n_zero);
+//   the loss (loss_tail).
+// V features a thread: four channels of one output position when the channel count is
+// a multiple of 4 and the arrays are aligned for it, else one.  dW_lr sums in 32 bits
+// where gl_bound allows (ten classes a pass, four in 64 bits), which leaves room for
+// three CTAs an SM: with 64-bit sums of ten classes and one CTA an SM the first block
+// of a 64-channel 32x32 network (2 M features) took 64 us, so 33.  Bound by the
+// instructions and latency of the delta part.  One CTA doing both parts for 64
+// features x 32 samples around a barrier, dW_lr by atomics into an array cleared
+// before, and a pass that split delta: VGG-style graph 479 us a step, odd block 173,
+// small CNN 101, VGG8B 727; so 478, 164, 95, 721.
 // ---------------------------------------------------------------------------
-constexpr int kLbQ = 64;                         // features per CTA
-constexpr int kLbLanes = 4;                      // sample lanes per feature
-constexpr int kLbPer = 4;                        // samples per lane
-constexpr int kLbSamples = kLbLanes * kLbPer;    // samples per CTA
-constexpr int kLbMaxG = 16;
+struct LrBackArgs {
+    const int8_t* a;
+    const int32_t* gl;
+    const int32_t* wlr;
+    int B, G, d;
+    int64_t* dwlr;
+    // delta part (delta null: dW_lr only)
+    LayerGeom lg;
+    FloorDiv32 alpha, dv_c, dv_ow;
+    const int8_t* region;
+    const int8_t* argmax;
+    int32_t* delta;
+    uint16_t* planes;
+    int64_t plane;
+    int64_t* zero;
+    int64_t n_zero;
+    const uint32_t* gl_bound;      // >= max |grad_L|
+    const uint32_t* maxabs_wlr;
+    uint32_t* maxabs_delta;
+    uint32_t* status;
+    int dw_ctas, delta_x, delta_ctas, tail_ctas;
+};
+constexpr int kLbSlab = 256;       // samples taken at once: sixteen a thread
+union LrShared {
+    int32_t gl[kLbSlab][16];
+    long long red[8][4][64];
+};
 
-template <int GM>   // classes held in registers: G <= GM
-__global__ void __launch_bounds__(256) k_lr_backward(const int8_t* __restrict__ a,
-                                                     const int32_t* __restrict__ gl,
-                                                     const int32_t* __restrict__ wlr, int B, int G,
-                                                     int d, int has_delta, LayerGeom lg,
-                                                     FloorDiv32 alpha,
-                                                     const int8_t* __restrict__ region,
-                                                     const int8_t* __restrict__ argmax,
-                                                     int32_t* __restrict__ delta,
-                                                     unsigned long long* __restrict__ dwlr,
-                                                     uint32_t* maxabs_delta, uint32_t* status,
-                                                     const LossTail tail) {
-    pdl_wait();
-    if (blockIdx.x == gridDim.x - 1) {        // the last column of the grid: the loss
-        loss_tail(tail);
-        return;
-    }
-    __shared__ int32_t gls[kLbSamples][GM];
-    __shared__ int8_t as[kLbSamples][kLbQ];
-    const int ql = threadIdx.x % kLbQ, sl = threadIdx.x / kLbQ;
-    const int q0 = blockIdx.x * kLbQ, q = q0 + ql;
-    const int b0 = blockIdx.y * kLbSamples;
-    const int nb = min(kLbSamples, B - b0);
-    for (int i = threadIdx.x; i < kLbSamples * GM; i += blockDim.x) {
-        const int u = i / GM, g = i % GM;
-        gls[u][g] = (u < nb && g < G) ? gl[(int64_t)(b0 + u) * G + g] : 0;
-    }
+// T int32 where the sums of a thread's samples fit
+template <int V, int GM, typename T>
+__device__ __forceinline__ void lr_dw(const LrBackArgs& p, LrShared& sm) {
+    const int quad = threadIdx.x & 15, lane_s = threadIdx.x >> 4, warp = threadIdx.x >> 5;
+    const int q0 = blockIdx.x * 16 * V, q = q0 + quad * V;
+    for (int gc = 0; gc < p.G; gc += GM) {
+        T acc[GM][V];
 #pragma unroll
-    for (int i = 0; i < kLbPer; ++i) {
-        const int u = sl + kLbLanes * i;
-        as[u][ql] = (u < nb && q < d) ? a[(int64_t)(b0 + u) * d + q] : (int8_t)0;
-    }
-    // loads of the delta path (W_lr column, argmax, region bytes) go out with
-    // the staging loads, before the barrier
-    const bool act = has_delta && q < d;
-    int32_t w[GM];
-    int rgv[kLbPer], am[kLbPer];
-    int64_t img = 0, p00 = 0, dx = 0, dy = 0;
+        for (int g = 0; g < GM; ++g)
 #pragma unroll
-    for (int g = 0; g < GM; ++g) w[g] = (act && g < G) ? wlr[(int64_t)g * d + q] : 0;
-    if (act) {
-        // position of feature q in the (pooled) output grid
-        const int c = q % lg.cout;
-        const int r = q / lg.cout;
-        const int ox = r % lg.ow, oy = r / lg.ow;
-        // element offsets of the (up to) four pre-pool positions within one image
-        img = lg.pool ? (int64_t)lg.h * lg.w * lg.cout : (int64_t)d;
-        p00 = lg.pool ? ((int64_t)(2 * oy) * lg.w + 2 * ox) * lg.cout + c : q;
-        dx = lg.cout;
-        dy = (int64_t)lg.w * lg.cout;
-    }
+            for (int j = 0; j < V; ++j) acc[g][j] = 0;
+        for (int b0 = 0; b0 < p.B; b0 += kLbSlab) {
+            const int nb = min(kLbSlab, p.B - b0);
+            uint32_t aw[kLbSlab / 16];
 #pragma unroll
-    for (int i = 0; i < kLbPer; ++i) {
-        const int u = sl + kLbLanes * i;
-        rgv[i] = 0;
-        am[i] = 0;
-        if (act && u < nb) {
-            const int64_t base = (b0 + u) * img + p00;
-            if (lg.pool) {
-                // only the recorded window position receives the gradient
-                am[i] = argmax[(int64_t)(b0 + u) * d + q];
-                const int r0 = region[base], r1 = region[base + dx];
-                const int r2 = region[base + dy], r3 = region[base + dy + dx];
-                rgv[i] = am[i] == 0 ? r0 : (am[i] == 1 ? r1 : (am[i] == 2 ? r2 : r3));
-            } else {
-                rgv[i] = region[base];
+            for (int i = 0; i < kLbSlab / 16; ++i) {
+                const int b = lane_s + 16 * i;
+                aw[i] = 0;
+                if (b < nb && q < p.d) {
+                    const int8_t* src = p.a + (int64_t)(b0 + b) * p.d + q;
+                    aw[i] = V == 4 ? *reinterpret_cast<const uint32_t*>(src) : (uint32_t)(uint8_t)*src;
+                }
+            }
+            __syncthreads();
+            for (int i = threadIdx.x; i < nb * GM; i += 256) {
+                const int b = i / GM, g = i - b * GM;
+                sm.gl[b][g] = gc + g < p.G ? p.gl[(int64_t)(b0 + b) * p.G + gc + g] : 0;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < kLbSlab / 16; ++i) {
+                const int b = lane_s + 16 * i;
+                if (b >= nb) break;
+#pragma unroll
+                for (int g = 0; g < GM; ++g) {
+                    const T gv = sm.gl[b][g];
+#pragma unroll
+                    for (int j = 0; j < V; ++j) acc[g][j] += gv * (int8_t)(aw[i] >> (8 * j));
+                }
+            }
+        }
+        // two sample lanes of a warp, then the eight warps, four classes at a time
+#pragma unroll
+        for (int g0 = 0; g0 < GM; g0 += 4) {
+            __syncthreads();
+#pragma unroll
+            for (int g = g0; g < g0 + 4 && g < GM; ++g)
+#pragma unroll
+                for (int j = 0; j < V; ++j) {
+                    const long long t = (long long)acc[g][j] + __shfl_xor_sync(kFull, acc[g][j], 16);
+                    if ((threadIdx.x & 16) == 0) sm.red[warp][g - g0][quad * V + j] = t;
+                }
+            __syncthreads();
+            for (int i = threadIdx.x; i < 4 * 16 * V; i += 256) {
+                const int g = i / (16 * V), f = i - g * 16 * V;
+                if (g0 + g >= GM || gc + g0 + g >= p.G || q0 + f >= p.d) continue;
+                long long t = 0;
+#pragma unroll
+                for (int w = 0; w < 8; ++w) t += sm.red[w][g][f];
+                p.dwlr[(int64_t)(gc + g0 + g) * p.d + q0 + f] = t;
             }
         }
     }
-    __syncthreads();
-    // dW_lr partials: (g, q) pairs over the CTA's samples
-    for (int i = threadIdx.x; i < G * kLbQ; i += blockDim.x) {
-        const int g = i / kLbQ, qq = i - g * kLbQ;
-        if (q0 + qq >= d) continue;
-        long long t = 0;
-#pragma unroll
-        for (int u = 0; u < kLbSamples; ++u) t += (long long)gls[u][g] * as[u][qq];
-        if (t != 0) atomicAdd(&dwlr[(int64_t)g * d + q0 + qq], (unsigned long long)t);
-    }
-    if (!has_delta) return;
-    uint32_t mx = 0;
-    bool ovf = false;
-    if (q < d) {
-#pragma unroll
-        for (int i = 0; i < kLbPer; ++i) {
-            const int u = sl + kLbLanes * i;
-            if (u >= nb) break;
-            uint64_t acc = 0;     // modulo 2^64, exact below the bound
-#pragma unroll
-            for (int g = 0; g < GM; ++g) acc += (uint64_t)((int64_t)gls[u][g] * w[g]);
-            const int64_t gv = (int64_t)acc;
-            ovf |= !fits_i32(gv);
-            const int32_t gs = (int32_t)gv;
-            // NITRO-ReLU backward: piece 1 -> floor(g / alpha_inv), piece 2 -> g, else 0
-            const int32_t dvv = rgv[i] == 1 ? alpha.floor_div(gs) : (rgv[i] == 2 ? gs : 0);
-            mx = max(mx, abs_u32(dvv));
-            const int64_t base = (b0 + u) * img + p00;
-            if (lg.pool) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    delta[base + (k & 1) * dx + (k >> 1) * dy] = k == am[i] ? dvv : 0;
-            } else {
-                delta[base] = dvv;
-            }
-        }
-    }
-    block_maximum(mx, ovf, maxabs_delta, status);
 }
 
-// Same, four features per thread when the last layer's channel count is a
-// multiple of 4 (four consecutive features are then four channels of one
-// output position): thread (f4, u) takes features q0 + 4 f4 .. + 3 of sample
-// b0 + u.  The W_lr slice is staged in shared memory; the argmax codes and
-// the region bytes of the four channels are read as 4-byte words and the
-// delta written with 16-byte stores.  The dW_lr partials are those of
-// k_lr_backward.
-template <int GM, int NS>   // NS samples per CTA, 16 NS threads
-__global__ void __launch_bounds__(16 * NS) k_lr_backward4(const int8_t* __restrict__ a,
-                                                      const int32_t* __restrict__ gl,
-                                                      const int32_t* __restrict__ wlr, int B,
-                                                      int G, int d, LayerGeom lg, FloorDiv32 alpha,
-                                                      const int8_t* __restrict__ region,
-                                                      const int8_t* __restrict__ argmax,
-                                                      int32_t* __restrict__ delta,
-                                                      unsigned long long* __restrict__ dwlr,
-                                                      uint32_t* maxabs_delta, uint32_t* status,
-                                                      const LossTail tail) {
-    pdl_wait();
-    if (blockIdx.x == gridDim.x - 1) {        // the last column of the grid: the loss
-        loss_tail(tail);
-        return;
-    }
-    __shared__ int32_t gls[NS][GM];
-    __shared__ int8_t as[NS][kLbQ];
-    __shared__ __align__(16) int32_t wsl[GM][kLbQ];
-    const int f4 = threadIdx.x & 15, u = threadIdx.x >> 4;
-    const int q0 = blockIdx.x * kLbQ, q = q0 + 4 * f4;
-    const int b0 = blockIdx.y * NS;
-    const int nb = min(NS, B - b0);
-    for (int i = threadIdx.x; i < NS * GM; i += blockDim.x) {
-        const int uu = i / GM, g = i % GM;
-        gls[uu][g] = (uu < nb && g < G) ? gl[(int64_t)(b0 + uu) * G + g] : 0;
-    }
-    for (int i = threadIdx.x; i < NS * kLbQ; i += blockDim.x) {
-        const int uu = i / kLbQ, qq = i % kLbQ;
-        as[uu][qq] = (uu < nb && q0 + qq < d) ? a[(int64_t)(b0 + uu) * d + q0 + qq] : (int8_t)0;
-    }
-    for (int i = threadIdx.x; i < GM * kLbQ; i += blockDim.x) {
-        const int g = i / kLbQ, qq = i % kLbQ;
-        wsl[g][qq] = (g < G && q0 + qq < d) ? wlr[(int64_t)g * d + q0 + qq] : 0;
-    }
-    // loads of the delta path go out with the staging loads, before the barrier
-    const bool act = q < d && u < nb;      // d % 4 == 0: all four features valid
-    int64_t base = 0, dx = 0, dy = 0;
-    uint32_t amw = 0, r00 = 0, r01 = 0, r10 = 0, r11 = 0;
-    if (act) {
-        const int c = q % lg.cout;
-        const int r = q / lg.cout;
-        const int ox = r % lg.ow, oy = r / lg.ow;
-        const int64_t img = lg.pool ? (int64_t)lg.h * lg.w * lg.cout : (int64_t)d;
-        const int64_t p00 = lg.pool ? ((int64_t)(2 * oy) * lg.w + 2 * ox) * lg.cout + c : q;
-        dx = lg.cout;
-        dy = (int64_t)lg.w * lg.cout;
-        base = (b0 + u) * img + p00;
-        r00 = *reinterpret_cast<const uint32_t*>(region + base);
-        if (lg.pool) {
-            amw = *reinterpret_cast<const uint32_t*>(argmax + (int64_t)(b0 + u) * d + q);
-            r01 = *reinterpret_cast<const uint32_t*>(region + base + dx);
-            r10 = *reinterpret_cast<const uint32_t*>(region + base + dy);
-            r11 = *reinterpret_cast<const uint32_t*>(region + base + dy + dx);
-        }
-    }
-    __syncthreads();
-    // dW_lr partials: (g, q) pairs over the CTA's samples
-    for (int i = threadIdx.x; i < G * kLbQ; i += blockDim.x) {
-        const int g = i / kLbQ, qq = i - g * kLbQ;
-        if (q0 + qq >= d) continue;
-        long long t = 0;
-#pragma unroll
-        for (int uu = 0; uu < NS; ++uu) t += (long long)gls[uu][g] * as[uu][qq];
-        if (t != 0) atomicAdd(&dwlr[(int64_t)g * d + q0 + qq], (unsigned long long)t);
-    }
+template <int V>
+__device__ __forceinline__ void lr_delta(const LrBackArgs& p, int cta) {
+    for (int64_t k = (int64_t)cta * 256 + threadIdx.x; k < p.n_zero; k += (int64_t)p.delta_ctas * 256) p.zero[k] = 0;
+    const int by = cta / p.delta_x, bx = cta - by * p.delta_x;
+    const int q = (bx * 16 + (threadIdx.x & 15)) * V, b = by * 16 + (threadIdx.x >> 4);
     uint32_t mx = 0;
     bool ovf = false;
-    if (act) {
-        uint64_t acc[4] = {0, 0, 0, 0};    // modulo 2^64, exact below the bound
-#pragma unroll
-        for (int g = 0; g < GM; ++g) {
-            const int4 w4 = *reinterpret_cast<const int4*>(&wsl[g][4 * f4]);
-            const int64_t gv = gls[u][g];
-            acc[0] += (uint64_t)(gv * w4.x);
-            acc[1] += (uint64_t)(gv * w4.y);
-            acc[2] += (uint64_t)(gv * w4.z);
-            acc[3] += (uint64_t)(gv * w4.w);
-        }
-        int32_t dv[4];
-        int code[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int64_t g64 = (int64_t)acc[j];
-            ovf |= !fits_i32(g64);
-            const int32_t gs = (int32_t)g64;
-            // region byte at the recorded window position of channel j
-            code[j] = lg.pool ? (int)((amw >> (8 * j)) & 3u) : 0;
-            const uint32_t rsel = code[j] == 0 ? r00 : (code[j] == 1 ? r01 : (code[j] == 2 ? r10 : r11));
-            const int rg = (int8_t)(rsel >> (8 * j));
-            // NITRO-ReLU backward: piece 1 -> floor(g / alpha_inv), piece 2 -> g, else 0
-            dv[j] = rg == 1 ? alpha.floor_div(gs) : (rg == 2 ? gs : 0);
-            mx = max(mx, abs_u32(dv[j]));
-        }
+    if (q < p.d && b < p.B) {
+        const LayerGeom& lg = p.lg;
+        const int pix = (int)p.dv_c.udiv((uint32_t)q), c = q - pix * lg.cout;
+        const int oy = (int)p.dv_ow.udiv((uint32_t)pix), ox = pix - oy * lg.ow;
+        const int s2 = lg.pool ? 2 : 1;
+        // codes of the V channels first
+        const uint32_t base = (uint32_t)((b * lg.h + s2 * oy) * lg.w + s2 * ox) * lg.cout + c;
+        const uint32_t row = (uint32_t)lg.w * lg.cout;
+        const auto codes = [](const int8_t* at) {
+            return V == 4 ? *reinterpret_cast<const uint32_t*>(at) : (uint32_t)(uint8_t)*at;
+        };
+        uint32_t am = 0, r[4];
+        r[0] = codes(p.region + base);
         if (lg.pool) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                *reinterpret_cast<int4*>(delta + base + (k & 1) * dx + (k >> 1) * dy) =
-                    make_int4(code[0] == k ? dv[0] : 0, code[1] == k ? dv[1] : 0,
-                              code[2] == k ? dv[2] : 0, code[3] == k ? dv[3] : 0);
-        } else {
-            *reinterpret_cast<int4*>(delta + base) = make_int4(dv[0], dv[1], dv[2], dv[3]);
+            am = codes(p.argmax + (int64_t)b * p.d + q);
+            r[1] = codes(p.region + base + lg.cout);
+            r[2] = codes(p.region + base + row);
+            r[3] = codes(p.region + base + row + lg.cout);
         }
+        uint64_t acc[V];                  // modulo 2^64, exact below the bound
+#pragma unroll
+        for (int j = 0; j < V; ++j) acc[j] = 0;
+        const int32_t* wp = p.wlr + q;
+        const int32_t* gp = p.gl + (int64_t)b * p.G;
+#pragma unroll 5
+        for (int g = 0; g < p.G; ++g) {
+            const int64_t gv = gp[g];
+            if (V == 4) {
+                const int4 w = *reinterpret_cast<const int4*>(wp + (int64_t)g * p.d);
+                acc[0] += (uint64_t)(gv * w.x);
+                acc[1 % V] += (uint64_t)(gv * w.y);
+                acc[2 % V] += (uint64_t)(gv * w.z);
+                acc[3 % V] += (uint64_t)(gv * w.w);
+            } else {
+                acc[0] += (uint64_t)(gv * wp[(int64_t)g * p.d]);
+            }
+        }
+        int32_t v[4] = {0, 0, 0, 0};
+        int code[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+            const int64_t gv = (int64_t)acc[j];
+            ovf |= !fits_i32(gv);
+            const int32_t gs = (int32_t)gv;
+            code[j] = lg.pool ? (int)((am >> (8 * j)) & 3u) : 0;
+            // region byte at the recorded window position of channel j
+            const uint32_t rs = code[j] == 0 ? r[0] : (code[j] == 1 ? r[1] : (code[j] == 2 ? r[2] : r[3]));
+            const uint32_t rg = (rs >> (8 * j)) & 255u;
+            // NITRO-ReLU backward: piece 1 -> floor(g / alpha_inv), piece 2 -> g, else 0
+            v[j] = rg == 1 ? p.alpha.floor_div(gs) : (rg == 2 ? gs : 0);
+            mx = max(mx, abs_u32(v[j]));
+        }
+        int L = 0;
+        uint32_t h01[4], h23[4];
+        if (V == 4 && p.planes) {
+            const uint64_t gb = (uint64_t)*p.gl_bound * (uint64_t)p.G;
+            const uint64_t wb = *p.maxabs_wlr;
+            L = limb_count(wb && gb > 0xffffffffull / wb ? 0xffffffffu : (uint32_t)(gb * wb));
+#pragma unroll
+            for (int l = 0; l < 4; ++l) {
+                h01[l] = limb_bf16x2(v[0], v[1], l);
+                h23[l] = limb_bf16x2(v[2], v[3], l);
+            }
+        }
+        // the window, with what a floor-sized pool drops at the last row and column
+        const int ny = lg.pool ? (oy + 1 == lg.oh ? lg.h - 2 * oy : 2) : 1;
+        const int nx = lg.pool ? (ox + 1 == lg.ow ? lg.w - 2 * ox : 2) : 1;
+        for (int y = 0; y < ny; ++y)
+            for (int x = 0; x < nx; ++x) {
+                const int at = y < 2 && x < 2 ? 2 * y + x : 4;
+                const uint32_t o = base + y * row + x * lg.cout;
+                if (V == 4) {
+                    const bool k0 = code[0] == at, k1 = code[1] == at, k2 = code[2] == at, k3 = code[3] == at;
+                    *reinterpret_cast<int4*>(p.delta + o) =
+                        make_int4(k0 ? v[0] : 0, k1 ? v[1] : 0, k2 ? v[2] : 0, k3 ? v[3] : 0);
+                    const uint32_t m01 = (k0 ? 0xffffu : 0u) | (k1 ? 0xffff0000u : 0u);
+                    const uint32_t m23 = (k2 ? 0xffffu : 0u) | (k3 ? 0xffff0000u : 0u);
+#pragma unroll
+                    for (int l = 0; l < 4; ++l) {
+                        if (l >= L) break;
+                        *reinterpret_cast<uint2*>(p.planes + l * p.plane + o) = make_uint2(h01[l] & m01, h23[l] & m23);
+                    }
+                } else {
+                    p.delta[o] = code[0] == at ? v[0] : 0;
+                }
+            }
     }
-    block_maximum(mx, ovf, maxabs_delta, status);
+    block_maximum(mx, ovf, p.maxabs_delta, p.status);
+}
+
+template <int V>
+__global__ void __launch_bounds__(256, 3) k_lr_backward(const LrBackArgs p, const LossTail tail) {
+    __shared__ LrShared sm;
+    pdl_wait();
+    const int cta = blockIdx.x;
+    if (cta < p.dw_ctas) {
+        if ((uint64_t)*p.gl_bound * 128u * (uint64_t)((p.B + 15) / 16) <= 0x7fffffffull) lr_dw<V, 10, int32_t>(p, sm);
+        else lr_dw<V, 4, long long>(p, sm);
+    } else if (cta < p.dw_ctas + p.delta_ctas) lr_delta<V>(p, cta - p.dw_ctas);
+    else loss_tail(tail, cta - p.dw_ctas - p.delta_ctas, p.tail_ctas);
 }
 
 inline int grid_for(int64_t n, int threads, int cap = 152 * 16) {
@@ -1373,7 +1330,7 @@ int learn_cluster(int64_t ctas, int d) {
 
 cudaError_t simt_learn_fwd(const int8_t* a, const int32_t* wlr, const int32_t* labels, int B,
                            int d, int G, int32_t* grad_l, const uint32_t* maxabs_wlr,
-                           uint32_t* status, uint32_t* zero_words, int n_zero, int64_t* zero_dwlr,
+                           uint32_t* status, uint32_t* zero_words, int n_zero, uint32_t* gl_bound,
                            cudaStream_t s) {
     if (B <= 0) return cudaSuccess;
     if (n_zero > 256 || G > kMaxClasses) return cudaErrorInvalidValue;
@@ -1384,7 +1341,7 @@ cudaError_t simt_learn_fwd(const int8_t* a, const int32_t* wlr, const int32_t* l
     ProfScope ps(K_LEARN_FWD, s, 2.0 * B * d * G, 0.0);
     return launch_cluster(k_learn_fwd, dim3(S * ((B + kLfSamples - 1) / kLfSamples)), 256, S, s, 0, p,
                           FloorDiv::make((uint64_t)d), labels, grad_l, maxabs_wlr, status, zero_words,
-                          n_zero, zero_dwlr);
+                          n_zero, gl_bound);
 }
 
 bool simt_lin_fwd_ok(const LayerGeom& g, int B, bool tc) {
@@ -1416,20 +1373,6 @@ cudaError_t simt_lin_wgrad(const int8_t* a, const int32_t* delta, const LayerGeo
     ProfScope ps(K_SIMT_LIN_WGRAD, s, 2.0 * B * g.cin * (double)g.cout, 0.0);
     return launch_k(k_lin_wgrad, dim3((unsigned)((g.cin + 63) / 64) * (unsigned)((g.cout + 15) / 16)), 256, 0,
                     s, a, delta, B, g.cin, g.cout, dw);
-}
-
-namespace {
-LossTail loss_args(const int32_t* gl, int B, int G, const LossOut& o) {
-    return LossTail{gl, B, G, o.sse, o.loss, o.maxabs_gl, o.ticket, o.wlr_max, o.status};
-}
-}  // namespace
-
-cudaError_t simt_learn_dw(const int8_t* a, const int32_t* grad_l, int B, int d, int G,
-                          int64_t* dwlr, const LossOut& lo, cudaStream_t s) {
-    dim3 grid((d + 255) / 256 + 1, G);
-    ProfScope ps(K_LEARN_DW, s, 2.0 * B * d * G, 0.0);
-    launch_k(k_learn_dw, grid, 256, 0, s, a, grad_l, B, d, G, dwlr, loss_args(grad_l, B, G, lo));
-    return cudaGetLastError();
 }
 
 cudaError_t simt_grad_to_delta(const DeltaSrc& src, const LayerGeom& g, int B, int alpha_inv,
@@ -1479,51 +1422,46 @@ cudaError_t simt_integersgd(const SgdBatch& b_in, cudaStream_t s) {
 }
 
 
-bool simt_lr_backward_ok(int G) { return G <= kLbMaxG; }
-
-cudaError_t simt_lr_backward(const int8_t* a, const int32_t* gl, const int32_t* wlr, int B, int G,
-                             int d, const LayerGeom* lg, int alpha_inv, const int8_t* region,
-                             const int8_t* argmax, int32_t* delta, int64_t* dwlr,
-                             uint32_t* maxabs_delta, uint32_t* status, const LossOut& lo,
+cudaError_t simt_lr_backward(const int8_t* a, const int32_t* gl, const uint32_t* gl_bound, const int32_t* wlr,
+                             int B, int G, int d, int64_t* dwlr, const LrDelta* dl, uint32_t* status, const LossOut& lo,
                              cudaStream_t s) {
-    cudaError_t e = cudaSuccess;
-    if (B <= 0) return e;
-    if (lg && lg->pool && ((lg->h & 1) || (lg->w & 1))) {   // rows / columns the pool dropped
-        e = cudaMemsetAsync(delta, 0, sizeof(int32_t) * (size_t)B * lg->h * lg->w * lg->cout, s);
-        if (e != cudaSuccess) return e;
+    if (B <= 0) return cudaSuccess;
+    LrBackArgs p{};
+    p.a = a; p.gl = gl; p.wlr = wlr;
+    p.B = B; p.G = G; p.d = d;
+    p.dwlr = dwlr;
+    p.gl_bound = gl_bound;
+    bool quad = d % 4 == 0 && (((uintptr_t)a & 3) | ((uintptr_t)wlr & 15)) == 0;
+    if (dl) {
+        const LayerGeom& g = *dl->lg;
+        quad = quad && g.cout % 4 == 0 && (((uintptr_t)dl->region | (uintptr_t)dl->delta | (uintptr_t)dl->planes |
+                                            (uintptr_t)(g.pool ? dl->argmax : dl->region)) & 15) == 0;
+        p.lg = g;
+        p.alpha = FloorDiv32::make((uint32_t)dl->alpha_inv);
+        p.dv_c = FloorDiv32::make((uint32_t)g.cout);
+        p.dv_ow = FloorDiv32::make((uint32_t)g.ow);
+        p.region = dl->region; p.argmax = dl->argmax; p.delta = dl->delta;
+        if (quad && dl->planes) {
+            p.planes = dl->planes;
+            p.plane = (int64_t)B * g.h * g.w * g.cout;
+            p.zero = dl->zero;
+            p.n_zero = dl->zero ? dl->n_zero : 0;
+            *dl->planes_done = true;
+        }
+        p.maxabs_wlr = dl->maxabs_wlr;
+        p.maxabs_delta = dl->maxabs_delta;
     }
-    dim3 grid((d + kLbQ - 1) / kLbQ + 1, (B + kLbSamples - 1) / kLbSamples);   // + the loss column
-    // the four-feature kernel takes 32 samples per CTA (half the weight-gradient
-    // atomics of 16) when the batch fills them
-    constexpr int kLb4Samples = 32;
-    dim3 grid4((d + kLbQ - 1) / kLbQ + 1, (B + kLb4Samples - 1) / kLb4Samples);
-    const LossTail tail = loss_args(gl, B, G, lo);
-    ProfScope ps(K_LR_BACKWARD, s, (lg ? 4.0 : 2.0) * B * d * G, 0.0);
-    const FloorDiv32 al = FloorDiv32::make((uint32_t)(alpha_inv > 0 ? alpha_inv : 1));
-    auto* dw64 = reinterpret_cast<unsigned long long*>(dwlr);
-    const LayerGeom g0 = lg ? *lg : LayerGeom{};
-    // four features per thread: channel counts in multiples of 4 and
-    // 16-byte aligned code and delta buffers (this library's own)
-    const bool quad = lg && lg->cout % 4 == 0 && d % 4 == 0 &&
-                      (((uintptr_t)region | (uintptr_t)delta |
-                        (uintptr_t)(lg->pool ? argmax : region)) & 15) == 0;
-    if (quad) {
-        if (G <= 10)
-            launch_k(k_lr_backward4<10, kLb4Samples>, grid4, 16 * kLb4Samples, 0, s,
-                a, gl, wlr, B, G, d, g0, al, region, argmax, delta, dw64, maxabs_delta, status, tail);
-        else
-            launch_k(k_lr_backward4<kLbMaxG, kLb4Samples>, grid4, 16 * kLb4Samples, 0, s,
-                a, gl, wlr, B, G, d, g0, al, region, argmax, delta, dw64, maxabs_delta, status, tail);
-        return cudaGetLastError();
-    }
-    if (G <= 10)
-        launch_k(k_lr_backward<10>, grid, 256, 0, s, a, gl, wlr, B, G, d, lg != nullptr, g0, al, region,
-                                               argmax, delta, dw64, maxabs_delta, status, tail);
-    else
-        launch_k(k_lr_backward<kLbMaxG>, grid, 256, 0, s, a, gl, wlr, B, G, d, lg != nullptr, g0, al,
-                                                    region, argmax, delta, dw64, maxabs_delta, status,
-                                                    tail);
-    return cudaGetLastError();
+    p.status = status;
+    const int tile = quad ? 64 : 16;
+    p.dw_ctas = (d + tile - 1) / tile;
+    p.delta_x = p.dw_ctas;
+    p.delta_ctas = dl ? p.delta_x * ((B + 15) / 16) : 0;
+    p.tail_ctas = (int)(((int64_t)B * G + kTailValues - 1) / kTailValues);
+    const int grid = p.dw_ctas + p.delta_ctas + p.tail_ctas;
+    const LossTail tail{gl, B, G, lo.sse, lo.loss, lo.maxabs_gl, lo.ticket, lo.wlr_max, lo.status};
+    ProfScope ps(K_LR_BACKWARD, s, (dl ? 4.0 : 2.0) * B * d * G, 0.0);
+    return quad ? launch_k(k_lr_backward<4>, grid, 256, 0, s, p, tail)
+                : launch_k(k_lr_backward<1>, grid, 256, 0, s, p, tail);
 }
 
 }  // namespace nitro

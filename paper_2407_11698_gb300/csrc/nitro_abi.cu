@@ -433,51 +433,32 @@ nitro_status block_backward(nitro_block* b, const int8_t* a_in, const int32_t* l
                                    b->lp.ph, b->lp.pw, b->zmp, b->lr_am, s));
         a_last = b->zmp;
     }
-    // also resets the per-step words and dW_lr for the kernels below
+    // also resets the per-step words for the kernels below
+    uint32_t* gl_bound = w_sgd(b) + kMaxSgdTensors + 1;
     NITRO_TRY(simt_learn_fwd(a_last, b->Wlr, labels, batch, (int)d, G, b->grad_l, w_wlr(b),
-                             w_status(b), w_gl(b), n_words(n) - (3 + n),
-                             simt_lr_backward_ok(G) ? b->dWlr : nullptr, s));
-    // the kernel after it forms the loss; where that kernel also forms delta_fw, it
-    // checks the bound of grad_L W_lr as well
-    LossOut lo{b->sse, loss_dev, w_gl(b), b->words + n_words(n) - 1, n && !b->zmp && simt_lr_backward_ok(G) ? w_wlr(b) : nullptr,
-               w_status(b)};
-    if (b->zmp) {
-        // learning-weight gradient from z^mp, then delta_fw back through the
-        // learning pool into the last layer's delta (pre-update W_lr)
-        if (simt_lr_backward_ok(G))
-            NITRO_TRY(simt_lr_backward(a_last, b->grad_l, b->Wlr, batch, G, (int)d, nullptr,
-                                       b->desc.alpha_inv, nullptr, nullptr, nullptr, b->dWlr,
-                                       nullptr, w_status(b), lo, s));
-        else
-            NITRO_TRY(simt_learn_dw(a_last, b->grad_l, batch, (int)d, G, b->dWlr, lo, s));
-        // (and its limb planes; the launch also clears dW for a split weight gradient)
-        Layer& ly = b->L[n - 1];
-        NITRO_TRY(simt_lrpool_to_delta(b->grad_l, b->Wlr, G, (int)d, ly.g, b->lp, batch, b->lr_am,
-                                       ly.argmax, ly.region, b->desc.alpha_inv, ly.delta,
-                                       ly.tc.d_nhwc, tc_wgrad_adds(ly.tc, ly.g, batch, ly.dW),
-                                       ly.wcount, &planes_done, w_gl(b), w_wlr(b), w_delta(b, n - 1),
-                                       w_status(b), s));
-    } else if (simt_lr_backward_ok(G)) {
-        // learning-weight gradient and (below a forward layer) delta_fw -> that
-        // layer's delta in one pass
-        Layer* ly = n ? &b->L[n - 1] : nullptr;
-        NITRO_TRY(simt_lr_backward(a_last, b->grad_l, b->Wlr, batch, G, (int)d, ly ? &ly->g : nullptr,
-                                   b->desc.alpha_inv, ly ? ly->region : nullptr,
-                                   ly ? ly->argmax : nullptr, ly ? ly->delta : nullptr, b->dWlr,
-                                   n ? w_delta(b, n - 1) : nullptr, w_status(b), lo, s));
-    } else {
-        NITRO_TRY(simt_learn_dw(a_last, b->grad_l, batch, (int)d, G, b->dWlr, lo, s));
-    }
+                             w_status(b), w_gl(b), n_words(n) - (3 + n), gl_bound, s));
+    // The kernel after it forms the learning-weight gradient, the loss and (below a
+    // forward layer) delta_fw = grad_L W_lr (pre-update) into that layer's delta and limb
+    // planes, where it also clears dW for a split weight gradient and checks the bound of
+    // grad_L W_lr; with a learning pool, the launch behind it routes delta_fw.
+    const bool direct = n > 0 && !b->zmp;
+    LossOut lo{b->sse, loss_dev, w_gl(b), b->words + n_words(n) - 1, direct ? w_wlr(b) : nullptr, w_status(b)};
+    Layer* top = n ? &b->L[n - 1] : nullptr;
+    int64_t* split_dw = top ? tc_wgrad_adds(top->tc, top->g, batch, top->dW) : nullptr;
+    // a linear layer whose weight gradient stays on the CUDA cores needs no planes
+    uint16_t* planes = top && !simt_lin_wgrad_ok(top->g, batch, top->tc.wgrad) ? top->tc.d_nhwc : nullptr;
+    LrDelta dl{};
+    if (direct)
+        dl = LrDelta{&top->g, b->desc.alpha_inv, top->region, top->argmax, top->delta, planes, split_dw,
+                     top->wcount, &planes_done, w_wlr(b), w_delta(b, n - 1)};
+    NITRO_TRY(simt_lr_backward(a_last, b->grad_l, gl_bound, b->Wlr, batch, G, (int)d, b->dWlr, direct ? &dl : nullptr,
+                               w_status(b), lo, s));
+    if (b->zmp)
+        NITRO_TRY(simt_lrpool_to_delta(b->grad_l, b->Wlr, G, (int)d, top->g, b->lp, batch, b->lr_am,
+                                       top->argmax, top->region, b->desc.alpha_inv, top->delta, planes,
+                                       split_dw, top->wcount, &planes_done, w_gl(b), w_wlr(b),
+                                       w_delta(b, n - 1), w_status(b), s));
     if (n == 0) return NITRO_OK;
-    // delta_fw = grad_L W_lr (pre-update), into the last layer
-    if (!b->zmp && !simt_lr_backward_ok(G)) {
-        Layer& ly = b->L[n - 1];
-        DeltaSrc src{};
-        src.grad_l = b->grad_l; src.wlr = b->Wlr; src.G = G;
-        src.maxabs_a = w_gl(b); src.maxabs_b = w_wlr(b); src.bound_k = G;
-        NITRO_TRY(simt_grad_to_delta(src, ly.g, batch, b->desc.alpha_inv, ly.region, ly.argmax,
-                                     ly.delta, w_delta(b, n - 1), w_status(b), s));
-    }
     const int64_t gamma_fw = 64LL * b->G * b->desc.gamma_inv_lr;
     for (int i = n - 1; i >= 0; --i) {
         Layer& ly = b->L[i];

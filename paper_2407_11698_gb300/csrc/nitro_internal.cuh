@@ -270,15 +270,14 @@ cudaError_t simt_lrpool_to_delta(const int32_t* gl, const int32_t* wlr, int G, i
                                  uint32_t* status, cudaStream_t s);
 
 // Learning layer forward: grad_l = floor(a W^T / (256 d)) - 32 onehot (the limbs of
-// W from *maxabs_wlr) and status bits.  The launch also clears what the rest of the
-// backward accumulates into, which saves a memset each: zero_words[0..n_zero) and,
-// when zero_dwlr is not null, the G d values of dW_lr.
+// W from *maxabs_wlr) and status bits; *gl_bound is raised to max |grad_l|.  The launch
+// also clears zero_words[0..n_zero) for the rest of the backward, which saves a memset.
 cudaError_t simt_learn_fwd(const int8_t* a, const int32_t* wlr, const int32_t* labels, int B,
                            int d, int G, int32_t* grad_l, const uint32_t* maxabs_wlr,
-                           uint32_t* status, uint32_t* zero_words, int n_zero, int64_t* zero_dwlr,
+                           uint32_t* status, uint32_t* zero_words, int n_zero, uint32_t* gl_bound,
                            cudaStream_t s);
 
-// Written by the kernel that follows it (simt_lr_backward or simt_learn_dw): sse =
+// Written by the kernel that follows it (simt_lr_backward): sse =
 // sum grad_l^2 (mod 2^64), loss = floor(sse / 2) (may be null), max |grad_l|, and
 // OVERFLOW when max |grad_l| *wlr_max G reaches 2^63 (wlr_max null: not checked).
 struct LossOut {
@@ -289,10 +288,6 @@ struct LossOut {
     const uint32_t* wlr_max;
     uint32_t* status;
 };
-
-// dW_lr[g][j] = sum_b grad_l[b][g] a[b][j]
-cudaError_t simt_learn_dw(const int8_t* a, const int32_t* grad_l, int B, int d, int G,
-                          int64_t* dwlr, const LossOut& lo, cudaStream_t s);
 
 // Linear layer on the CUDA cores: the whole forward (scaling, NITRO-ReLU, dropout; the
 // limbs of w from *maxabs_w) and the weight gradient (dw overwritten), one launch
@@ -305,33 +300,39 @@ bool simt_lin_wgrad_ok(const LayerGeom& g, int B, bool tc);
 cudaError_t simt_lin_wgrad(const int8_t* a, const int32_t* delta, const LayerGeom& g, int B, int64_t* dw,
                            cudaStream_t s);
 
-// Gradient at the output of layer g (post-pool) -> delta at its
-// pre-activation: max-pool backward, NITRO-ReLU backward, STE.  The source
-// is either delta_fw = grad_l W_lr (lr_wlr != NULL) or an int64 dgrad output.
+// Gradient at the output of layer g (post-pool, an int64 dgrad output) -> delta at its
+// pre-activation: max-pool backward, NITRO-ReLU backward, STE.
 struct DeltaSrc {
-    const int32_t* grad_l;   // [B][G]   (learning-layer source)
-    const int32_t* wlr;      // [G][d]
-    int G;
     const uint32_t* maxabs_a;  // bound check operands: max|grad| and max|W|
     const uint32_t* maxabs_b;
     int64_t bound_k;           // contraction length for the bound
-    const int64_t* g64;      // [B][out features of the layer] (dgrad source)
+    const int64_t* g64;        // [B][out features of the layer]
 };
 cudaError_t simt_grad_to_delta(const DeltaSrc& src, const LayerGeom& g, int B, int alpha_inv,
                                const int8_t* region, const int8_t* argmax, int32_t* delta,
                                uint32_t* maxabs_delta, uint32_t* status, cudaStream_t s);
 
-// Learning-layer backward for G <= 16, fused: dW_lr (added to; zero on entry,
-// see simt_learn_fwd) and, when
-// lg (geometry of the block's last forward layer) is not null, that layer's
-// delta from delta_fw = grad_L W_lr (pre-update), with the int32 storage
-// rule, the int64 bound check, max-pool and NITRO-ReLU backward.  d: features
-// of the block output.
-bool simt_lr_backward_ok(int G);
-cudaError_t simt_lr_backward(const int8_t* a, const int32_t* gl, const int32_t* wlr, int B, int G,
-                             int d, const LayerGeom* lg, int alpha_inv, const int8_t* region,
-                             const int8_t* argmax, int32_t* delta, int64_t* dwlr,
-                             uint32_t* maxabs_delta, uint32_t* status, const LossOut& lo,
+// Learning-layer backward: dW_lr (overwritten), the loss (see LossOut) and, with dl !=
+// null, the delta of the block's last forward layer (geometry lg) from delta_fw =
+// grad_L W_lr (pre-update), with the int32 storage rule, max-pool and NITRO-ReLU
+// backward.  dl->planes (may be null): delta's limb planes [4][n], written too where the
+// layout allows (*planes_done), and zero[0..n_zero) is then cleared as well.  d:
+// features of the learning layer; *gl_bound >= max |grad_L|.
+struct LrDelta {
+    const LayerGeom* lg;
+    int alpha_inv;
+    const int8_t* region;
+    const int8_t* argmax;
+    int32_t* delta;
+    uint16_t* planes;
+    int64_t* zero;
+    int64_t n_zero;
+    bool* planes_done;
+    const uint32_t* maxabs_wlr;
+    uint32_t* maxabs_delta;
+};
+cudaError_t simt_lr_backward(const int8_t* a, const int32_t* gl, const uint32_t* gl_bound, const int32_t* wlr,
+                             int B, int G, int d, int64_t* dwlr, const LrDelta* dl, uint32_t* status, const LossOut& lo,
                              cudaStream_t s);
 
 // IntegerSGD (Algorithm 1) over up to kMaxSgdTensors tensors in one launch.
@@ -361,8 +362,9 @@ struct SgdBatch {
     int round_trunc;
     uint32_t* status;
     uint32_t* step;        // block step counter, incremented once per launch (or null)
-    // kMaxSgdTensors maxima and a CTA ticket, zero before the first launch and
-    // left zero by every launch: the last CTA stores the finished maxima into
+    // kMaxSgdTensors maxima, a CTA ticket and the step's bound of |grad_L| (see
+    // simt_learn_fwd), zero before the first launch and left zero by every launch: the
+    // last CTA stores the finished maxima into
     // each tensor's maxabs_w and copies words[0..n_words) to host_words (pinned
     // host memory; null: no copy)
     uint32_t* scratch;
@@ -371,7 +373,7 @@ struct SgdBatch {
     int n_words;
     int first[kMaxSgdTensors + 1];   // first CTA of each tensor (filled by simt_integersgd)
 };
-constexpr int kSgdScratchWords = kMaxSgdTensors + 1;
+constexpr int kSgdScratchWords = kMaxSgdTensors + 2;
 cudaError_t simt_integersgd(const SgdBatch& b, cudaStream_t s);
 
 
