@@ -383,25 +383,26 @@ __global__ void __launch_bounds__(256) k_learn_fwd(const LearnArgs p, FloorDiv d
         if (lane < min(kLfG, p.G - gc)) part[u][gc + lane] = z;
     }
     cluster.sync();
-    // sample v of the group is finished by CTA v mod S
-    uint32_t mx = 0;
-    for (int i = threadIdx.x; i < kLfSamples * p.G; i += 256) {
-        const int v = i / p.G, g = i - v * p.G, bb = group * kLfSamples + v;
-        if (v % S != rank || bb >= p.B) continue;
-        long long z = 0;
-        for (int r = 0; r < S; ++r) z += *cluster.map_shared_rank(&part[v][g], r);
-        const int lab = labels[bb];
+    // sample v of the group is finished by warp v of CTA v mod S
+    if (u % S == rank && b < p.B) {
+        const int lab = labels[b];
         const bool bad = lab < 0 || lab >= p.G;
-        // NITRO-Scaling, SF = 2^8 d: floor(floor(z / 256) / d)
-        const int64_t yhat = dv.floor_div((int64_t)z >> 8);
-        const int64_t t = yhat - ((!bad && g == lab) ? 32 : 0);
-        if (bad && g == 0) atomicOr(status, ST_BAD_LABEL);
-        if (!fits_i32(t)) atomicOr(status, ST_OVERFLOW);
-        grad_l[(int64_t)bb * p.G + g] = (int32_t)t;
-        mx = max(mx, abs_u32((int32_t)t));
+        uint64_t l1 = 0;
+        for (int g = lane; g < p.G; g += 32) {
+            long long z = 0;
+            for (int r = 0; r < S; ++r) z += *cluster.map_shared_rank(&part[u][g], r);
+            // NITRO-Scaling, SF = 2^8 d: floor(floor(z / 256) / d)
+            const int64_t yhat = dv.floor_div((int64_t)z >> 8);
+            const int64_t t = yhat - ((!bad && g == lab) ? 32 : 0);
+            if (bad && g == 0) atomicOr(status, ST_BAD_LABEL);
+            if (!fits_i32(t)) atomicOr(status, ST_OVERFLOW);
+            grad_l[(int64_t)b * p.G + g] = (int32_t)t;
+            l1 += abs_u32((int32_t)t);
+        }
+#pragma unroll
+        for (int o = 16; o; o >>= 1) l1 += __shfl_xor_sync(kFull, l1, o);
+        if (lane == 0 && l1) atomicMax(gl_bound, l1 > 0xffffffffull ? 0xffffffffu : (uint32_t)l1);
     }
-    mx = __reduce_max_sync(kFull, mx);
-    if (lane == 0 && mx) atomicMax(gl_bound, mx);
     cluster.sync();      // the partial sums stay until every CTA has read them
 }
 
@@ -739,7 +740,7 @@ __global__ void k_lrpool_to_delta(const int32_t* __restrict__ gl, const int32_t*
 // the delta stores: looking the codes up per pre-pool element instead cost a
 // chain of dependent loads for each of 8.4 M or 16.8 M elements.
 // With planes != null the thread also writes delta's bf16 limb planes (the weight
-// gradient's operand), as many as the bound G max|grad_L| max|W_lr| can need, so
+// gradient's operand), as many as gl_bound max|W_lr| can need, so
 // that no pass reads delta again; and the launch clears zero[0..n_zero).
 __global__ void __launch_bounds__(256) k_lrpool_to_delta4(
     const int32_t* __restrict__ gl, const int32_t* __restrict__ wlr, int G, int d, LayerGeom g,
@@ -747,8 +748,8 @@ __global__ void __launch_bounds__(256) k_lrpool_to_delta4(
     const uint8_t* __restrict__ lam, const int8_t* __restrict__ argmax,
     const int8_t* __restrict__ region, FloorDiv32 alpha, int32_t* __restrict__ delta,
     uint16_t* __restrict__ planes, int64_t plane, int64_t* zero, int64_t n_zero,
-    const uint32_t* maxabs_gl, const uint32_t* maxabs_wlr, uint32_t* maxabs_delta,
-    uint32_t* status) {
+    const uint32_t* maxabs_gl, const uint32_t* gl_bound, const uint32_t* maxabs_wlr,
+    uint32_t* maxabs_delta, uint32_t* status) {
     pdl_wait();
     const int C = g.cout, C4 = g.cout >> 2;
     const uint32_t n4 = (uint32_t)B * lp.ph * lp.pw * C4;
@@ -762,10 +763,9 @@ __global__ void __launch_bounds__(256) k_lrpool_to_delta4(
         atomicOr(status, ST_OVERFLOW);
     int L = 0;
     if (planes) {
-        const uint64_t gb = (uint64_t)*maxabs_gl * (uint64_t)G;           // < 2^38
-        const uint64_t wb = *maxabs_wlr;
-        const uint64_t bound = wb && gb > 0xffffffffull / wb ? 0xffffffffull : gb * wb;
-        L = limb_count((uint32_t)bound);
+        const uint32_t gb = *gl_bound;
+        const uint64_t bound = (uint64_t)gb * *maxabs_wlr;
+        L = limb_count(gb == 0xffffffffu || bound > 0xffffffffull ? 0xffffffffu : (uint32_t)bound);
     }
     uint32_t mx = 0;
     bool ovf = false;
@@ -963,18 +963,20 @@ __global__ void __launch_bounds__(256) k_integersgd(const SgdBatch bt) {
 //   delta_fw[b][q] = sum_g grad_L[b][g] W_lr[g][q] (int32 storage rule) for 16 V features
 //     x 16 samples, routed through max-pool backward and NITRO-ReLU backward into the
 //     last layer's delta, every position written, with the delta's bf16 limb planes
-//     (planes != null; as many as G max|grad_L| max|W_lr| can need), so that no pass
+//     (planes != null; as many as gl_bound max|W_lr| can need), so that no pass
 //     reads delta again; these CTAs also clear zero[0..n_zero);
 //   the loss (loss_tail).
 // V features a thread: four channels of one output position when the channel count is
 // a multiple of 4 and the arrays are aligned for it, else one.  dW_lr sums in 32 bits
-// where gl_bound allows (ten classes a pass, four in 64 bits), which leaves room for
-// three CTAs an SM: with 64-bit sums of ten classes and one CTA an SM the first block
-// of a 64-channel 32x32 network (2 M features) took 64 us, so 33.  Bound by the
-// instructions and latency of the delta part.  One CTA doing both parts for 64
-// features x 32 samples around a barrier, dW_lr by atomics into an array cleared
-// before, and a pass that split delta: VGG-style graph 479 us a step, odd block 173,
-// small CNN 101, VGG8B 727; so 478, 164, 95, 721.
+// where gl_bound allows (ten classes a pass, four in 64 bits) and delta_fw where
+// gl_bound max|W_lr| does, which leaves room for four CTAs an SM.  First block of a
+// 64-channel 32x32 network at batch 64 (2 M features): 27 us; 64-bit sums of ten
+// classes at one CTA an SM 64, 32-bit sums at three 31; five CTAs an SM with half the
+// classes a pass 25, but 4 us more where d is small.  Bound by the instructions and
+// latency of the delta part.  One CTA doing both parts for 64 features x 32 samples
+// around a barrier, dW_lr by atomics into an array cleared before, and a pass that
+// split delta: VGG-style graph 479 us a step, odd block 173, small CNN 101, VGG8B 727;
+// so 464 to 468, 164, 95, 715 to 724.
 // ---------------------------------------------------------------------------
 struct LrBackArgs {
     const int8_t* a;
@@ -992,13 +994,13 @@ struct LrBackArgs {
     int64_t plane;
     int64_t* zero;
     int64_t n_zero;
-    const uint32_t* gl_bound;      // >= max |grad_L|
+    const uint32_t* gl_bound;      // see simt_learn_fwd
     const uint32_t* maxabs_wlr;
     uint32_t* maxabs_delta;
     uint32_t* status;
     int dw_ctas, delta_x, delta_ctas, tail_ctas;
 };
-constexpr int kLbSlab = 256;       // samples taken at once: sixteen a thread
+constexpr int kLbSlab = 128;       // samples taken at once: eight a thread
 union LrShared {
     int32_t gl[kLbSlab][16];
     long long red[8][4][64];
@@ -1069,8 +1071,9 @@ __device__ __forceinline__ void lr_dw(const LrBackArgs& p, LrShared& sm) {
     }
 }
 
-template <int V>
-__device__ __forceinline__ void lr_delta(const LrBackArgs& p, int cta) {
+// T uint32 where |delta_fw| is known to fit int32, uint64 (modulo 2^64) elsewhere
+template <int V, typename T>
+__device__ __forceinline__ void lr_delta(const LrBackArgs& p, int cta, uint64_t bound) {
     for (int64_t k = (int64_t)cta * 256 + threadIdx.x; k < p.n_zero; k += (int64_t)p.delta_ctas * 256) p.zero[k] = 0;
     const int by = cta / p.delta_x, bx = cta - by * p.delta_x;
     const int q = (bx * 16 + (threadIdx.x & 15)) * V, b = by * 16 + (threadIdx.x >> 4);
@@ -1095,31 +1098,33 @@ __device__ __forceinline__ void lr_delta(const LrBackArgs& p, int cta) {
             r[2] = codes(p.region + base + row);
             r[3] = codes(p.region + base + row + lg.cout);
         }
-        uint64_t acc[V];                  // modulo 2^64, exact below the bound
+        T acc[V];
 #pragma unroll
         for (int j = 0; j < V; ++j) acc[j] = 0;
         const int32_t* wp = p.wlr + q;
         const int32_t* gp = p.gl + (int64_t)b * p.G;
+        const auto mul = [](int32_t x, int32_t y) {
+            return sizeof(T) == 4 ? (T)((uint32_t)x * (uint32_t)y) : (T)((int64_t)x * y);
+        };
 #pragma unroll 5
         for (int g = 0; g < p.G; ++g) {
-            const int64_t gv = gp[g];
+            const int32_t gv = gp[g];
             if (V == 4) {
                 const int4 w = *reinterpret_cast<const int4*>(wp + (int64_t)g * p.d);
-                acc[0] += (uint64_t)(gv * w.x);
-                acc[1 % V] += (uint64_t)(gv * w.y);
-                acc[2 % V] += (uint64_t)(gv * w.z);
-                acc[3 % V] += (uint64_t)(gv * w.w);
+                acc[0] += mul(gv, w.x);
+                acc[1 % V] += mul(gv, w.y);
+                acc[2 % V] += mul(gv, w.z);
+                acc[3 % V] += mul(gv, w.w);
             } else {
-                acc[0] += (uint64_t)(gv * wp[(int64_t)g * p.d]);
+                acc[0] += mul(gv, wp[(int64_t)g * p.d]);
             }
         }
         int32_t v[4] = {0, 0, 0, 0};
         int code[4] = {0, 0, 0, 0};
 #pragma unroll
         for (int j = 0; j < V; ++j) {
-            const int64_t gv = (int64_t)acc[j];
-            ovf |= !fits_i32(gv);
-            const int32_t gs = (int32_t)gv;
+            if (sizeof(T) == 8) ovf |= !fits_i32((int64_t)acc[j]);
+            const int32_t gs = (int32_t)acc[j];
             code[j] = lg.pool ? (int)((am >> (8 * j)) & 3u) : 0;
             // region byte at the recorded window position of channel j
             const uint32_t rs = code[j] == 0 ? r[0] : (code[j] == 1 ? r[1] : (code[j] == 2 ? r[2] : r[3]));
@@ -1131,9 +1136,7 @@ __device__ __forceinline__ void lr_delta(const LrBackArgs& p, int cta) {
         int L = 0;
         uint32_t h01[4], h23[4];
         if (V == 4 && p.planes) {
-            const uint64_t gb = (uint64_t)*p.gl_bound * (uint64_t)p.G;
-            const uint64_t wb = *p.maxabs_wlr;
-            L = limb_count(wb && gb > 0xffffffffull / wb ? 0xffffffffu : (uint32_t)(gb * wb));
+            L = limb_count(bound > 0xffffffffull ? 0xffffffffu : (uint32_t)bound);
 #pragma unroll
             for (int l = 0; l < 4; ++l) {
                 h01[l] = limb_bf16x2(v[0], v[1], l);
@@ -1167,15 +1170,21 @@ __device__ __forceinline__ void lr_delta(const LrBackArgs& p, int cta) {
 }
 
 template <int V>
-__global__ void __launch_bounds__(256, 3) k_lr_backward(const LrBackArgs p, const LossTail tail) {
+__global__ void __launch_bounds__(256, 4) k_lr_backward(const LrBackArgs p, const LossTail tail) {
     __shared__ LrShared sm;
     pdl_wait();
     const int cta = blockIdx.x;
     if (cta < p.dw_ctas) {
         if ((uint64_t)*p.gl_bound * 128u * (uint64_t)((p.B + 15) / 16) <= 0x7fffffffull) lr_dw<V, 10, int32_t>(p, sm);
         else lr_dw<V, 4, long long>(p, sm);
-    } else if (cta < p.dw_ctas + p.delta_ctas) lr_delta<V>(p, cta - p.dw_ctas);
-    else loss_tail(tail, cta - p.dw_ctas - p.delta_ctas, p.tail_ctas);
+    } else if (cta < p.dw_ctas + p.delta_ctas) {
+        const uint32_t gb = *p.gl_bound;
+        const uint64_t bound = (uint64_t)gb * *p.maxabs_wlr;
+        if (gb != 0xffffffffu && bound <= 0x7fffffffull) lr_delta<V, uint32_t>(p, cta - p.dw_ctas, bound);
+        else lr_delta<V, uint64_t>(p, cta - p.dw_ctas, gb == 0xffffffffu ? ~0ull : bound);
+    } else {
+        loss_tail(tail, cta - p.dw_ctas - p.delta_ctas, p.tail_ctas);
+    }
 }
 
 inline int grid_for(int64_t n, int threads, int cap = 152 * 16) {
@@ -1278,7 +1287,7 @@ cudaError_t simt_lrpool_to_delta(const int32_t* gl, const int32_t* wlr, int G, i
                                  const uint8_t* am, const int8_t* argmax, const int8_t* region,
                                  int alpha_inv, int32_t* delta, uint16_t* planes, int64_t* zero,
                                  int64_t n_zero, bool* planes_done, const uint32_t* maxabs_gl,
-                                 const uint32_t* maxabs_wlr, uint32_t* maxabs_delta,
+                                 const uint32_t* gl_bound, const uint32_t* maxabs_wlr, uint32_t* maxabs_delta,
                                  uint32_t* status, cudaStream_t s) {
     const int64_t n = (int64_t)B * g.h * g.w * g.cout;
     if (n <= 0) return cudaSuccess;
@@ -1306,7 +1315,7 @@ cudaError_t simt_lrpool_to_delta(const int32_t* gl, const int32_t* wlr, int G, i
             gl, wlr, G, d, g, lp, B, FloorDiv32::make((uint32_t)(g.cout / 4)),
             FloorDiv32::make((uint32_t)lp.pw), FloorDiv32::make((uint32_t)lp.ph), am, argmax, region,
             FloorDiv32::make((uint32_t)alpha_inv), delta, planes, n, zero, zero ? n_zero : (int64_t)0,
-            maxabs_gl, maxabs_wlr, maxabs_delta, status);
+            maxabs_gl, gl_bound, maxabs_wlr, maxabs_delta, status);
         *planes_done = planes != nullptr;
     } else {
         launch_k(k_lrpool_to_delta, grid_for(n, 256), 256, 0, s,

@@ -456,7 +456,7 @@ nitro_status block_backward(nitro_block* b, const int8_t* a_in, const int32_t* l
     if (b->zmp)
         NITRO_TRY(simt_lrpool_to_delta(b->grad_l, b->Wlr, G, (int)d, top->g, b->lp, batch, b->lr_am,
                                        top->argmax, top->region, b->desc.alpha_inv, top->delta, planes,
-                                       split_dw, top->wcount, &planes_done, w_gl(b), w_wlr(b),
+                                       split_dw, top->wcount, &planes_done, w_gl(b), gl_bound, w_wlr(b),
                                        w_delta(b, n - 1), w_status(b), s));
     if (n == 0) return NITRO_OK;
     const int64_t gamma_fw = 64LL * b->G * b->desc.gamma_inv_lr;

@@ -266,11 +266,13 @@ cudaError_t simt_lrpool_to_delta(const int32_t* gl, const int32_t* wlr, int G, i
                                  const uint8_t* am, const int8_t* argmax, const int8_t* region,
                                  int alpha_inv, int32_t* delta, uint16_t* planes, int64_t* zero,
                                  int64_t n_zero, bool* planes_done, const uint32_t* maxabs_gl,
-                                 const uint32_t* maxabs_wlr, uint32_t* maxabs_delta,
+                                 const uint32_t* gl_bound, const uint32_t* maxabs_wlr, uint32_t* maxabs_delta,
                                  uint32_t* status, cudaStream_t s);
 
 // Learning layer forward: grad_l = floor(a W^T / (256 d)) - 32 onehot (the limbs of
-// W from *maxabs_wlr) and status bits; *gl_bound is raised to max |grad_l|.  The launch
+// W from *maxabs_wlr) and status bits; *gl_bound is raised to the largest sum of |grad_l|
+// over a sample's classes (2^32 - 1: that or more), so that times max |W| it bounds
+// every sum of grad_l W, and more tightly than classes times max |grad_l|.  The launch
 // also clears zero_words[0..n_zero) for the rest of the backward, which saves a memset.
 cudaError_t simt_learn_fwd(const int8_t* a, const int32_t* wlr, const int32_t* labels, int B,
                            int d, int G, int32_t* grad_l, const uint32_t* maxabs_wlr,
@@ -317,7 +319,7 @@ cudaError_t simt_grad_to_delta(const DeltaSrc& src, const LayerGeom& g, int B, i
 // grad_L W_lr (pre-update), with the int32 storage rule, max-pool and NITRO-ReLU
 // backward.  dl->planes (may be null): delta's limb planes [4][n], written too where the
 // layout allows (*planes_done), and zero[0..n_zero) is then cleared as well.  d:
-// features of the learning layer; *gl_bound >= max |grad_L|.
+// features of the learning layer; gl_bound: see simt_learn_fwd.
 struct LrDelta {
     const LayerGeom* lg;
     int alpha_inv;
