@@ -1,0 +1,62 @@
+"""The one-pass fit of large datasets: sizes at its threshold, odd starts, the ends of
+the byte range where the guesses are clamped, and data whose sampled mean misses mu,
+so that the second pass runs, on one object in turn."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import oracle as O
+from paper_2407_11698_gb300 import binding as nb
+
+THRESHOLD = 96 << 20
+SAMPLES = 1 << 16
+
+
+def sampled(n, off):
+    """Start of every sampled 16-byte word (relative to x, which starts off bytes past a boundary)."""
+    k = np.arange(SAMPLES, dtype=np.uint64)
+    h = (k * np.uint64(2654435761)) & np.uint64(0xffffffff)
+    h ^= h >> np.uint64(15)
+    h = (h * np.uint64(0x85ebca6b)) & np.uint64(0xffffffff)
+    share = np.uint64(((n - 15) >> 4) // SAMPLES)
+    return (k * share + ((h * share) >> np.uint64(32))).astype(np.int64) * 16 + (-off) % 16
+
+
+def data(kind, n, off):
+    rng = np.random.default_rng(n + off)
+    if isinstance(kind, int):
+        return np.full(n, kind, dtype=np.uint8)
+    x = np.clip(rng.normal(120, 60, n), 0, 255).astype(np.uint8)
+    if kind == "miss":
+        x[sampled(n, off)[:, None] + np.arange(16)] = 255
+    elif kind == "low":
+        x = (x > 250).astype(np.uint8)
+    elif kind == "high":
+        x = 255 - (x > 250).astype(np.uint8)
+    return x
+
+
+@pytest.mark.parametrize("n,off,kinds", [(THRESHOLD - 1, 0, ["natural", "miss"]),
+                                         (THRESHOLD, 0, ["natural", "miss", 254, "miss", "high"]),
+                                         (THRESHOLD + 37, 3, ["miss", 0, 255, "low", "natural"])])
+def test_fit_matches_oracle(n, off, kinds):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    p = nb.IntPrep()
+    try:
+        for kind in kinds:
+            x = data(kind, n, off)
+            buf = torch.zeros(n + 64, dtype=torch.uint8, device="cuda")
+            xd = buf[off:off + n]
+            xd.copy_(torch.from_numpy(x))
+            p.fit(xd)
+            mu, om = O.prep_stats(x)
+            assert p.stats() == (mu, om), kind
+            out = torch.empty(n, dtype=torch.int8, device="cuda")
+            p.apply(xd, out)
+            lut = O.prep_apply(np.arange(256, dtype=np.uint8), mu, om)
+            assert np.array_equal(out.cpu().numpy(), lut.astype(np.int8)[x]), kind
+    finally:
+        p.close()
