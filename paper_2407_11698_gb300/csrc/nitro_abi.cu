@@ -290,8 +290,8 @@ nitro_status nitro_init_block(const nitro_block_desc* desc, uint64_t seed, void*
     b->z64_elems = z_need;
     for (int i = 0; ok && i < desc->n_layers; ++i) {
         Layer& ly = b->L[i];
-        ok = ly.lin_a ? tc_linear_init(ly.tc, ly.g, desc->max_batch, ly.lin_a, w_w(b, i), w_delta(b, i),
-                                       b->allocs, b->host_allocs)
+        ok = ly.lin_a ? tc_linear_init(ly.tc, ly.g, desc->max_batch, ly.lin_a, ly.lin_planes, w_w(b, i),
+                                       w_delta(b, i), b->allocs, b->host_allocs)
                       : tc_layer_init(ly.tc, ly.g, desc->max_batch, i > 0, w_w(b, i), w_delta(b, i),
                                       b->allocs, b->host_allocs);
         // one copy of all the block's words per step refreshes the layers' hints
@@ -367,15 +367,22 @@ nitro_status nitro_block_forward(nitro_block* b, const int8_t* a_in, int batch, 
             x = ly.act;
             continue;
         }
-        if (!ly.lin_planes) NITRO_TRY(tc_pack_input(ly.tc, g, x, batch, nhwc_done, s));
+        // fused scaling, activation and pool, but dropout has its own epilogue
+        const bool lin_fused = ly.lin_planes && !drop && tc_linear_fused(ly.tc, g, batch);
+        if (lin_fused) {
+            if (!nhwc_done) NITRO_TRY(tc_pack_int8(x, batch, g.cin, ly.lin_a, s));
+        } else if (!ly.lin_planes) {
+            NITRO_TRY(tc_pack_input(ly.tc, g, x, batch, nhwc_done, s));
+        }
         // the epilogue also writes the next layer's bf16 forward operand
         uint16_t* next_nhwc = nullptr;
         if (i + 1 < n && b->L[i + 1].tc.act_nhwc && !b->L[i + 1].tc.im2col &&
             b->L[i + 1].tc.cin8 == g.cout)
             next_nhwc = b->L[i + 1].tc.act_nhwc;
         TcFwdOut fo{b->desc.alpha_inv, b->mu, ly.act, out2, ly.region, ly.argmax, next_nhwc};
-        NITRO_TRY(tc_conv_forward(ly.tc, g, batch, b->z64, &fo, w_status(b), s, &done, &fused));
-        if (ly.lin_planes) {
+        if (!ly.lin_planes || lin_fused)
+            NITRO_TRY(tc_conv_forward(ly.tc, g, batch, b->z64, &fo, w_status(b), s, &done, &fused));
+        if (ly.lin_planes && !done) {
             // linear: z = a W^T on the tcgen05 GEMM (weight planes kept by IntegerSGD)
             const bool adds = tc_gemm_adds(batch, g.cout, g.cin);
             NITRO_TRY(tc_pack_int8(x, batch, g.cin, ly.lin_a, s, adds ? b->z64 : nullptr,

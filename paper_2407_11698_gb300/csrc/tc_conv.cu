@@ -1792,11 +1792,24 @@ void tc_layer_shape(TcLayer& t, const LayerGeom& g, bool has_dgrad) {
 // The forward's fused epilogue: rows of 8-byte multiples, and few enough K-blocks
 // for its error bound.
 bool tc_fwd_fused(const TcLayer& t, const LayerGeom& g) {
-    return t.fwd && g.cout % 8 == 0 && (t.im2col ? 1 : 9) * (t.cin_k / kBK) <= kFwdMaxBlocks;
+    const int taps = t.im2col || g.kind == NITRO_LINEAR ? 1 : 9;
+    return t.fwd && g.cout % 8 == 0 && taps * (t.cin_k / kBK) <= kFwdMaxBlocks;
 }
 
 size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
 }  // namespace
+
+// Linear layers: the kernel with the fused epilogue, its K split over a cluster, against
+// the GEMM into int64 that splits K over more CTAs by atomics, with a clear before and
+// the epilogue as a launch after.  Us a forward of batch x in x out at two limbs, fused
+// and not: 64 x 3000 x 3000 15.5 and 17.2, 256 x 2048 x 1024 12.1 and 20.7, 128 x 4096 x 4096
+// 18.1 and 29.0, 1024 x 1024 x 1024 14.6 and 29.9, 4096 x 1024 x 1024 21.4 and 57.9.  Few
+// tiles and a long K want the wider split: 64 x 8192 x 128 14.4 and 13.2, 128 x 8192 x 64
+// 14.7 and 12.3, 64 x 8192 x 256 14.8 and 14.0, but 64 x 6144 x 128 11.5 and 11.6.
+bool tc_linear_fused(const TcLayer& t, const LayerGeom& g, int batch) {
+    const int64_t tiles = (batch + kBM - 1) / kBM * (int64_t)((g.cout + 63) / 64);
+    return g.kind == NITRO_LINEAR && tc_fwd_fused(t, g) && (tiles > 4 || t.cin_k / kBK <= 96);
+}
 
 size_t tc_fwd_scratch(const LayerGeom& g, int batch) {
     TcLayer t;
@@ -1871,7 +1884,7 @@ bool tc_layer_init(TcLayer& t, const LayerGeom& g, int max_batch, bool has_dgrad
     return ok;
 }
 
-bool tc_linear_init(TcLayer& t, const LayerGeom& g, int max_batch, uint16_t* act_bf16,
+bool tc_linear_init(TcLayer& t, const LayerGeom& g, int max_batch, uint16_t* act_bf16, uint16_t* planes,
                     const uint32_t* maxabs_w, const uint32_t* maxabs_d,
                     std::vector<void*>& allocs, std::vector<void*>& host_allocs) {
     t = TcLayer();
@@ -1881,6 +1894,8 @@ bool tc_linear_init(TcLayer& t, const LayerGeom& g, int max_batch, uint16_t* act
     // TMA strides in multiples of 16 bytes; 8-wide output channel groups
     if (g.cin % 8 != 0 || g.cout % 8 != 0) return true;
     t.wgrad = true;
+    t.lin_planes = planes;
+    t.fwd = planes && round_up(g.cin, 64) / kBK <= kFwdMaxBlocks;
     t.cin8 = g.cin;
     t.cin_k = round_up(g.cin, 64);
     t.act_nhwc = act_bf16;       // the forward's bf16 copy of the layer input
@@ -1985,12 +2000,21 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
     *done = false;
     *fused = false;
     if (!t.fwd || batch <= 0) return cudaSuccess;
+    // A linear layer is 1 x 1 images with a single centred tap: rows = the samples
+    const bool lin = g.kind == NITRO_LINEAR;
+    if (lin && !fo) return cudaSuccess;
     TcArgs a{};
-    a.B = batch; a.H = g.h; a.W = g.w; a.Cin = g.cin; a.Cout = g.cout;
+    a.B = batch; a.H = lin ? 1 : g.h; a.W = lin ? 1 : g.w; a.Cin = g.cin; a.Cout = g.cout;
     a.Bp = round_up(batch, 8);
     a.cin_k = t.cin_k;
-    a.taps = t.im2col ? 1 : 9;
-    pixel_tiling(g, batch, a);
+    a.taps = t.im2col || lin ? 1 : 9;
+    if (lin) {
+        a.wb = a.hb = a.ntx = a.nty = 1;
+        a.bb = kBM;
+        a.tiles_m = (batch + kBM - 1) / kBM;
+    } else {
+        pixel_tiling(g, batch, a);
+    }
     a.kb_total = a.taps * (t.cin_k / kBK);
     const bool fuse = fo && tc_fwd_fused(t, g);
     int n = pick_n(g.cout);
@@ -2007,11 +2031,11 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
     a.status = status;
     a.atomic_out = 0;
     if (fuse) {
-        a.sf = 256 * 9 * g.cin;
+        a.sf = 256 * (lin ? 1 : 9) * g.cin;
         a.sf_inv = 1.0f / (float)a.sf;
         a.alpha = FloorDiv::make((uint64_t)fo->alpha_inv);
         a.mu = fo->mu;
-        a.pool = g.pool;
+        a.pool = !lin && g.pool;
         a.oh = g.oh;
         a.ow = g.ow;
         a.act = fo->act;
@@ -2025,18 +2049,19 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
         if (low & 7) return cudaErrorInvalidValue;
     }
     CUtensorMap ma, mb;
-    const uint64_t da[4] = {(uint64_t)t.cin8, (uint64_t)g.w, (uint64_t)g.h, (uint64_t)batch};
-    const uint64_t sa[3] = {(uint64_t)t.cin8, (uint64_t)g.w * t.cin8, (uint64_t)g.h * g.w * t.cin8};
+    const uint64_t da[4] = {(uint64_t)t.cin8, (uint64_t)a.W, (uint64_t)a.H, (uint64_t)batch};
+    const uint64_t sa[3] = {(uint64_t)t.cin8, (uint64_t)a.W * t.cin8, (uint64_t)a.H * a.W * t.cin8};
     const uint32_t ba[4] = {64, (uint32_t)a.wb, (uint32_t)a.hb, (uint32_t)a.bb};
-    const uint64_t kw = (uint64_t)a.taps * t.cin_k;   // w_planes row length
+    // weight plane row length (a linear layer's rows end inside a K-block: zeros follow)
+    const uint64_t kw = lin ? (uint64_t)g.cin : (uint64_t)a.taps * t.cin_k;
     const int pb = pick_pb(n, tc_limb_hint(t, 0));
     const uint64_t db[3] = {kw, (uint64_t)g.cout, (uint64_t)kMaxLimbs};
     const uint64_t sb[2] = {kw, kw * g.cout};
     const uint32_t bb[3] = {64, (uint32_t)n, (uint32_t)pb};
-    if (!make_map(&ma, t.act_nhwc, 4, da, sa, ba) || !make_map(&mb, t.w_planes, 3, db, sb, bb))
+    if (!make_map(&ma, t.act_nhwc, 4, da, sa, ba) || !make_map(&mb, lin ? t.lin_planes : t.w_planes, 3, db, sb, bb))
         return cudaErrorInvalidValue;
-    const double ops = 2.0 * batch * g.h * g.w * g.cout * 9.0 * g.cin;
-    ProfScope ps(K_TC_CONV_FWD, s, ops, 0.0);
+    const double ops = 2.0 * batch * a.H * a.W * g.cout * (lin ? 1.0 : 9.0) * g.cin;
+    ProfScope ps(lin ? K_TC_GEMM : K_TC_CONV_FWD, s, ops, 0.0);
     cudaError_t e = !fuse ? launch_gemm_pb<TC_FWDZ>(n, pb, ma, mb, a, s)
                           : (a.ksplit > 1 ? launch_gemm_pb<TC_FWDK>(n, pb, ma, mb, a, s)
                                           : launch_gemm_pb<TC_FWD>(n, pb, ma, mb, a, s));

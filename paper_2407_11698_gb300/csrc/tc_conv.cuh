@@ -41,6 +41,7 @@ struct TcLayer {
     uint16_t* act_nhwc = nullptr;
     uint16_t* d_nhwc = nullptr;
     uint16_t* w_planes = nullptr;
+    uint16_t* lin_planes = nullptr;   // linear layers: the caller's weight planes [4][Cout][Cin]
     // device words holding max |W| and max |delta| of the layer: the kernels
     // take their limb counts from them
     const uint32_t* maxabs_w = nullptr;
@@ -85,7 +86,7 @@ struct TcSgd {
 // the forward's bf16 copy of the layer input [max_batch][in] (kept by the
 // caller); the delta limb planes are allocated here.  t.wgrad is
 // false when the layer does not qualify.
-bool tc_linear_init(TcLayer& t, const LayerGeom& g, int max_batch, uint16_t* act_bf16,
+bool tc_linear_init(TcLayer& t, const LayerGeom& g, int max_batch, uint16_t* act_bf16, uint16_t* planes,
                     const uint32_t* maxabs_w, const uint32_t* maxabs_d,
                     std::vector<void*>& allocs, std::vector<void*>& host_allocs);
 
@@ -126,6 +127,9 @@ struct TcFwdOut {
     int8_t* argmax;       // [B][oh][ow][Cout] int8 if pooled
     uint16_t* next_nhwc;  // next layer's bf16 input copy, or null
 };
+
+// Whether a linear layer's forward runs on tcgen05 with its epilogue fused.
+bool tc_linear_fused(const TcLayer& t, const LayerGeom& g, int batch);
 
 // Forward contraction on tcgen05; *done = false if the layer does not run
 // there.  With fo != null and Cout % 8 == 0 (and at most 128 K-blocks) the epilogue applies
