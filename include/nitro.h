@@ -329,8 +329,8 @@ nitro_status nitro_conv3x3_forward_noalloc(const int8_t* a_in, const int32_t* we
  * 51 = floor(64 * 0.8), since the MAD of Gaussian data is ~0.8 sigma.  The
  * appendix leaves omega = 0 undefined: it is read as a divisor of 1.
  *
- * nitro_prep_fit computes mu and omega of one device buffer x [n] (two
- * passes over it) and keeps them in the handle with the 256-entry map they
+ * nitro_prep_fit computes mu and omega of one device buffer x [n] (in one
+ * pass or two over it, by size) and keeps them in the handle with the 256-entry map they
  * define; nitro_prep_apply maps any device buffer x [n] to out [n] (int8) with
  * the statistics of the last fit, so a test set can be mapped with the
  * training set's.  out may equal x (in place) but must not overlap it
