@@ -367,8 +367,7 @@ nitro_status nitro_block_forward(nitro_block* b, const int8_t* a_in, int batch, 
             x = ly.act;
             continue;
         }
-        // fused scaling, activation and pool, but dropout has its own epilogue
-        const bool lin_fused = ly.lin_planes && !drop && tc_linear_fused(ly.tc, g, batch);
+        const bool lin_fused = ly.lin_planes && tc_linear_fused(ly.tc, g, batch);
         if (lin_fused) {
             if (!nhwc_done) NITRO_TRY(tc_pack_int8(x, batch, g.cin, ly.lin_a, s));
         } else if (!ly.lin_planes) {
@@ -379,7 +378,7 @@ nitro_status nitro_block_forward(nitro_block* b, const int8_t* a_in, int batch, 
         if (i + 1 < n && b->L[i + 1].tc.act_nhwc && !b->L[i + 1].tc.im2col &&
             b->L[i + 1].tc.cin8 == g.cout)
             next_nhwc = b->L[i + 1].tc.act_nhwc;
-        TcFwdOut fo{b->desc.alpha_inv, b->mu, ly.act, out2, ly.region, ly.argmax, next_nhwc};
+        TcFwdOut fo{b->desc.alpha_inv, b->mu, ly.act, out2, ly.region, ly.argmax, next_nhwc, drop};
         if (!ly.lin_planes || lin_fused)
             NITRO_TRY(tc_conv_forward(ly.tc, g, batch, b->z64, &fo, w_status(b), s, &done, &fused));
         if (ly.lin_planes && !done) {

@@ -26,10 +26,11 @@ namespace nitro {
 namespace {
 
 // TC_FWD: forward with the fused NITRO-Scaling / NITRO-ReLU / max-pool epilogue;
-// TC_FWDK: the same with a tile's K shared out over a cluster; TC_DGRAD: input gradient
+// TC_FWDK: the same with a tile's K shared out over a cluster; TC_FWDD: linear layers
+// with dropout, either way; TC_DGRAD: input gradient
 // with the fused routing into the lower layer's delta; TC_FWDZ, TC_DGRADZ: the same
 // contractions with int64 sums as their output.
-enum TcMode : int { TC_FWD = 0, TC_WGRAD = 1, TC_DGRAD = 2, TC_GEMM = 3, TC_FWDZ = 4, TC_FWDK = 5, TC_DGRADZ = 6 };
+enum TcMode : int { TC_FWD = 0, TC_WGRAD = 1, TC_DGRAD = 2, TC_GEMM = 3, TC_FWDZ = 4, TC_FWDK = 5, TC_DGRADZ = 6, TC_FWDD = 7 };
 
 constexpr int kBM = 128;              // rows per tile (TMEM lanes)
 constexpr int kBK = 64;               // K elements per block (one 128-byte row)
@@ -256,6 +257,7 @@ struct TcArgs {
     float sf_inv;          // 1 / SF
     int out_align;         // outputs and their rows are aligned to 32, 16 or 8 bytes
     int mu, pool, oh, ow;
+    DropoutArgs drop;      // TC_FWDD
     int8_t* act;           // layer output (post-pool) int8 NHWC
     int8_t* out2;          // optional second copy of the output (caller's buffer)
     int8_t* region;        // NITRO-ReLU piece per pre-pool output
@@ -403,7 +405,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     using C = TcCfg<N, PB>;
     constexpr int S = C::S;
     constexpr int NH = N / 4;            // columns per epilogue warp
-    constexpr bool kFused = MODE == TC_FWD || MODE == TC_FWDK;
+    constexpr bool kSplitK = MODE == TC_FWDK || MODE == TC_FWDD;
+    constexpr bool kFused = MODE == TC_FWD || kSplitK;
     constexpr bool kFwd = kFused || MODE == TC_FWDZ;
     constexpr bool kDgrad = MODE == TC_DGRAD || MODE == TC_DGRADZ;
     extern __shared__ uint8_t smem_raw[];
@@ -483,11 +486,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int hiskip = *hiskip_slot;
     // Tiles of this CTA: every gridDim.x-th one, or, where a cluster shares a tile's K
     // (the ranks are the splits), one.
-    const int KS = MODE == TC_FWDK ? args.ksplit : 1;
-    const int rank = MODE == TC_FWDK ? (int)cluster_rank() : 0;
+    const int KS = kSplitK ? args.ksplit : 1;
+    const bool shared_k = MODE == TC_FWDK || (MODE == TC_FWDD && KS > 1);
+    const int rank = shared_k ? (int)cluster_rank() : 0;
     const int tile0 =
-        MODE == TC_FWDK ? rank * (args.tiles_m * args.tiles_n) + (int)blockIdx.x / KS : (int)blockIdx.x;
-    const int tile_step = MODE == TC_FWDK ? args.total_tiles : (int)gridDim.x;
+        shared_k ? rank * (args.tiles_m * args.tiles_n) + (int)blockIdx.x / KS : (int)blockIdx.x;
+    const int tile_step = shared_k ? args.total_tiles : (int)gridDim.x;
     // B limbs that pair with A limb la: all, or those with la + lb <= 3
     auto lb_limit = [&](int la) { return hiskip ? min(LB, 4 - la) : LB; };
 
@@ -674,7 +678,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             pdl_trigger();
         }
     }
-    if constexpr (MODE == TC_FWDK) {
+    if (shared_k) {
         cluster_barrier();      // the two of the epilogue's exchange
         cluster_barrier();
     }
@@ -916,7 +920,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                           (float)fcpp * ((float)fcpp + 4.2f);
         const bool tight = err <= 0.25f * (float)args.sf;
         const float far = err + 400.0f * (float)args.sf;
-        int barriers = MODE == TC_FWDK ? 2 : 0;     // cluster barriers this thread still owes
+        int barriers = shared_k ? 2 : 0;     // cluster barriers this thread still owes
         for (int tile = tile0; tile < args.total_tiles; tile += tile_step) {
             const Tile T = decode_tile(args, tile);
             const int cpp = (T.kb1 - T.kb0 + kChunkBlocks - 1) / kChunkBlocks;
@@ -1034,7 +1038,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (lane == 0) mbar_arrive(tempty_bar(buf));
                 }
             }
-            if constexpr (MODE == TC_FWDK) {
+            if (shared_k) {
+            if constexpr (kSplitK) {
                 // Partial sums of a cluster's K parts: each quarter of the columns is
                 // finished by one CTA, and the others write theirs into its ring
                 // memory, which is idle once every CTA has drained its last chunk.
@@ -1068,6 +1073,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         zf[i] += b.x; zf[i + 1] += b.y; zf[i + 2] += b.z; zf[i + 3] += b.w;
                     }
                 }
+            }
             }
             {
                 const int r = 32 * q + lane;   // output row of this thread
@@ -1252,6 +1258,19 @@ __global__ void __launch_bounds__(kThreads, 1)
                             }
                             lo[4 * g4] = e[0] | (e[1] << 16);
                             lo[4 * g4 + 1] = e[2] | (e[3] << 16);
+                        }
+                    }
+                    if constexpr (MODE == TC_FWDD) {
+                        // dropped outputs: value 0, region code 4 (element = sample, output)
+                        const uint32_t t = *args.drop.step;
+                        const uint64_t e0 = (uint64_t)pix * C + col0;
+#pragma unroll
+                        for (int k = 0; k < NH / 2; ++k) {
+                            uint32_t& w = lo[4 * (k >> 1) + (k & 1)];
+                            if (dropout_drop(args.drop.seed, t, args.drop.layer, e0 + 2 * k, args.drop.p16))
+                                w = (w & 0xffff0000u) | kRegionDropped;
+                            if (dropout_drop(args.drop.seed, t, args.drop.layer, e0 + 2 * k + 1, args.drop.p16))
+                                w = (w & 0xffffu) | ((uint32_t)kRegionDropped << 16);
                         }
                     }
                     uint32_t vpk[NH / 4], rpk[NH / 4];   // packed outputs, pieces or window positions
@@ -1695,7 +1714,7 @@ cudaError_t launch_gemm(const CUtensorMap& a, const CUtensorMap& b, const TcArgs
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    if constexpr (MODE == TC_FWDK)
+    if ((MODE == TC_FWDK || MODE == TC_FWDD) && args.ksplit > 1)
         return launch_cluster(k_tc_gemm<MODE, N, PB>, dim3(args.total_tiles), kThreads, args.ksplit, s, C::SMEM,
                               a, b, args);
     const int grid = args.total_tiles < sm_count() ? args.total_tiles : sm_count();
@@ -1819,6 +1838,8 @@ size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
 // 18.1 and 29.0, 1024 x 1024 x 1024 14.6 and 29.9, 4096 x 1024 x 1024 21.4 and 57.9.  Few
 // tiles and a long K want the wider split: 64 x 8192 x 128 14.4 and 13.2, 128 x 8192 x 64
 // 14.7 and 12.3, 64 x 8192 x 256 14.8 and 14.0, but 64 x 6144 x 128 11.5 and 11.6.
+// Dropout is drawn in the epilogue too (TC_FWDD): the wide MLP's step, 64 x 784 x 3000
+// and 64 x 3000 x 3000 twice with dropout, 217 us on the GEMM route, so 211.
 bool tc_linear_fused(const TcLayer& t, const LayerGeom& g, int batch) {
     const int64_t tiles = (batch + kBM - 1) / kBM * (int64_t)((g.cout + 63) / 64);
     return g.kind == NITRO_LINEAR && tc_fwd_fused(t, g) && (tiles > 4 || t.cin_k / kBK <= 96);
@@ -2069,6 +2090,10 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
         a.alpha = FloorDiv::make((uint64_t)fo->alpha_inv);
         a.mu = fo->mu;
         a.pool = !lin && g.pool;
+        if (fo->drop && fo->drop->p16) {
+            if (!lin || !fo->drop->step) return cudaErrorInvalidValue;
+            a.drop = *fo->drop;
+        }
         a.oh = g.oh;
         a.ow = g.ow;
         a.act = fo->act;
@@ -2096,6 +2121,7 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
     const double ops = 2.0 * batch * a.H * a.W * g.cout * (lin ? 1.0 : 9.0) * g.cin;
     ProfScope ps(lin ? K_TC_GEMM : K_TC_CONV_FWD, s, ops, 0.0);
     cudaError_t e = !fuse ? launch_gemm_pb<TC_FWDZ>(n, pb, ma, mb, a, s)
+                  : a.drop.p16 ? launch_gemm_pb<TC_FWDD>(n, pb, ma, mb, a, s)
                           : (a.ksplit > 1 ? launch_gemm_pb<TC_FWDK>(n, pb, ma, mb, a, s)
                                           : launch_gemm_pb<TC_FWD>(n, pb, ma, mb, a, s));
     if (e == cudaSuccess) {

@@ -126,6 +126,7 @@ struct TcFwdOut {
     int8_t* region;       // [B][h][w][Cout] int8
     int8_t* argmax;       // [B][oh][ow][Cout] int8 if pooled
     uint16_t* next_nhwc;  // next layer's bf16 input copy, or null
+    const DropoutArgs* drop;   // linear layers, or null
 };
 
 // Whether a linear layer's forward runs on tcgen05 with its epilogue fused.

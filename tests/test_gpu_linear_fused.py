@@ -1,7 +1,7 @@
 """Linear forwards large enough for the tensor cores, whose epilogue is fused: input
 widths that end inside a K-block and at the limit of the error bound (and the general
 route just above it), output widths inside a tile, batches around a tile, with and
-without a K split, one to four limbs, sums near zero, two layers in a row."""
+without a K split, one to four limbs, sums near zero, two layers in a row, dropout at a later step."""
 import numpy as np
 import pytest
 
@@ -26,14 +26,15 @@ SHAPES = [(129, [648, 640]), (64, [8192, 264]), (64, [8192, 104]), (70, [8200, 3
 
 @pytest.mark.parametrize("batch,widths", SHAPES)
 @pytest.mark.parametrize("kind", ["limb1", "limb2", "limb3", "limb4", "cancel"])
-def test_matches_oracle(batch, widths, kind):
+@pytest.mark.parametrize("p16", [0, 9830])
+def test_matches_oracle(batch, widths, kind, p16):
     import torch
     descs = [(L, a, b, 1, 1, 0) for a, b in zip(widths, widths[1:])]
     rng = np.random.default_rng(batch)
     top = {"limb1": 127, "limb2": 32639, "limb3": 8355711, "limb4": 2**31 - 1, "cancel": 2**30}[kind]
     x = synth.images(5, 0, batch, (widths[0],))
-    blk = nb.Block(descs, widths[0], max_batch=batch)
-    ob = O.OracleBlock([O.LayerDesc(*d) for d in descs])
+    blk = nb.Block(descs, widths[0], max_batch=batch, seed=21, dropout_p16=p16)
+    ob = O.OracleBlock([O.LayerDesc(*d) for d in descs], seed=21, dropout_p16=p16)
     try:
         for i, (a, b) in enumerate(zip(widths, widths[1:])):
             w = rng.integers(-top, top + 1, (b, a))
@@ -41,6 +42,9 @@ def test_matches_oracle(batch, widths, kind):
                 w[:, 1::2] = -w[:, ::2] + rng.integers(-4000, 4000, w[:, ::2].shape)
             blk.set(nb.NITRO_T_W, i, w.reshape(-1))
             ob.W[i] = w.astype(np.int64)
+        if p16:
+            blk.set(nb.NITRO_T_STEP, 0, np.array([5], dtype=np.uint32))
+            ob.t = 5
         if kind == "cancel":
             x[:, 1::2] = x[:, ::2]
         out = torch.empty((batch, widths[-1]), dtype=torch.int8, device="cuda")
