@@ -1838,7 +1838,7 @@ size_t align256(size_t n) { return (n + 255) & ~(size_t)255; }
 // 18.1 and 29.0, 1024 x 1024 x 1024 14.6 and 29.9, 4096 x 1024 x 1024 21.4 and 57.9.  Few
 // tiles and a long K want the wider split: 64 x 8192 x 128 14.4 and 13.2, 128 x 8192 x 64
 // 14.7 and 12.3, 64 x 8192 x 256 14.8 and 14.0, but 64 x 6144 x 128 11.5 and 11.6.
-// Dropout is drawn in the epilogue too (TC_FWDD): the wide MLP's step, 64 x 784 x 3000
+// Dropout is drawn in the epilogue too (TC_FWDD): the wide MLP's step, 64 x 1024 x 3000
 // and 64 x 3000 x 3000 twice with dropout, 217 us on the GEMM route, so 211.
 bool tc_linear_fused(const TcLayer& t, const LayerGeom& g, int batch) {
     const int64_t tiles = (batch + kBM - 1) / kBM * (int64_t)((g.cout + 63) / 64);
