@@ -589,14 +589,16 @@ __global__ void k_grad_to_delta(DeltaSrc src, LayerGeom g, int B, int alpha_inv,
             const int64_t r = q / g.cout;
             const int ox = (int)(r % g.ow), oy = (int)(r / g.ow);
             const int am = argmax[i];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int iy = 2 * oy + (k >> 1), ix = 2 * ox + (k & 1);
-                const int64_t pi = ((b * g.h + iy) * g.w + ix) * g.cout + c;
-                const int32_t dv = (k == am) ? relu_backward(gs, region[pi], alpha_inv) : 0;
-                delta[pi] = dv;
-                mx = max(mx, abs_u32(dv));
-            }
+            // the window, with what a floor-sized pool drops at the last row and column
+            const int ny = oy + 1 == g.oh ? g.h - 2 * oy : 2, nx = ox + 1 == g.ow ? g.w - 2 * ox : 2;
+            for (int y = 0; y < ny; ++y)
+                for (int x = 0; x < nx; ++x) {
+                    const int64_t pi = ((b * g.h + 2 * oy + y) * g.w + 2 * ox + x) * g.cout + c;
+                    const bool hit = y < 2 && x < 2 && 2 * y + x == am;
+                    const int32_t dv = hit ? relu_backward(gs, region[pi], alpha_inv) : 0;
+                    delta[pi] = dv;
+                    mx = max(mx, abs_u32(dv));
+                }
         } else {
             const int32_t dv = relu_backward(gs, region[i], alpha_inv);
             delta[i] = dv;
