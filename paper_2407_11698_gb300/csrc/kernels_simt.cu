@@ -792,7 +792,12 @@ __global__ void __launch_bounds__(256) k_lrpool_to_delta4(
             acc[2] += (uint64_t)(gv * w.z);
             acc[3] += (uint64_t)(gv * w.w);
         }
-        int pos[4], v[4];                     // row << 16 | column of the hit, and delta there
+        const int s2 = g.pool ? 2 : 1;
+        const int y0 = wy * lp.kh * s2, y1 = wy + 1 == lp.ph ? g.h : y0 + lp.kh * s2;
+        const int x0 = wx * lp.kw * s2, x1 = wx + 1 == lp.pw ? g.w : x0 + lp.kw * s2;
+        // row << 16 | column of the hit inside the window, and delta there: kh kw <= 256, so
+        // a window, with what the pools cut off behind the last one, has at most 1023 a side
+        int pos[4], v[4];
         uint32_t rg[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -804,7 +809,7 @@ __global__ void __launch_bounds__(256) k_lrpool_to_delta4(
                 x = 2 * x + (am & 1);
             }
             rg[j] = (uint8_t)region[((size_t)(b * g.h + y) * g.w + x) * C + c + j];
-            pos[j] = (y << 16) | x;
+            pos[j] = ((y - y0) << 16) | (x - x0);
         }
         uint32_t h01[4], h23[4];              // bf16 limbs of the four deltas
 #pragma unroll
@@ -821,13 +826,10 @@ __global__ void __launch_bounds__(256) k_lrpool_to_delta4(
             h01[l] = limb_bf16x2(v[0], v[1], l);
             h23[l] = limb_bf16x2(v[2], v[3], l);
         }
-        const int s2 = g.pool ? 2 : 1;
-        const int y0 = wy * lp.kh * s2, y1 = wy + 1 == lp.ph ? g.h : y0 + lp.kh * s2;
-        const int x0 = wx * lp.kw * s2, x1 = wx + 1 == lp.pw ? g.w : x0 + lp.kw * s2;
         for (int y = y0 + blockIdx.y; y < y1; y += gridDim.y) {
             size_t o = ((size_t)(b * g.h + y) * g.w + x0) * C + c;
             for (int x = x0; x < x1; ++x, o += C) {
-                const int at = (y << 16) | x;
+                const int at = ((y - y0) << 16) | (x - x0);
                 const bool k0 = pos[0] == at, k1 = pos[1] == at, k2 = pos[2] == at, k3 = pos[3] == at;
                 *reinterpret_cast<int4*>(delta + o) =
                     make_int4(k0 ? v[0] : 0, k1 ? v[1] : 0, k2 ? v[2] : 0, k3 ? v[3] : 0);

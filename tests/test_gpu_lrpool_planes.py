@@ -40,3 +40,16 @@ def test_matches_oracle(shape, wlr_max, fused):
             pair.compare("step %d" % s)
     finally:
         pair.close()
+
+
+# maps wider than 65536 columns, with several rows a window: (cin, cout, h, w, 2x2 pool, d_lr)
+@pytest.mark.parametrize("shape", [(1, 4, 2, 70000, 0, 8192), (1, 4, 4, 70001, 1, 8192)])
+def test_wide_map_matches_oracle(shape):
+    cin, cout, h, w, pool, d_lr = shape
+    pair = NetPair([{"layers": [(C, cin, cout, h, w, pool)], "in_features": h * w * cin}], 2, d_lr=d_lr)
+    try:
+        pair.step(synth.images(8, 0, 2, (h, w, cin)), synth.labels(8, 0, 2))
+        assert np.any(pair.ob[0].delta[0][:, :, 65536:])     # gradients land past the column in question
+        pair.compare("step 0")
+    finally:
+        pair.close()
