@@ -1,6 +1,7 @@
 // Internal declarations of the GB300 NITRO-D library (not part of the ABI).
 #pragma once
 
+#include <atomic>
 #include <cstdint>
 #include <utility>
 #include <cuda_runtime.h>
@@ -378,6 +379,24 @@ struct SgdBatch {
 constexpr int kSgdScratchWords = kMaxSgdTensors + 2;
 cudaError_t simt_integersgd(const SgdBatch& b, cudaStream_t s);
 
+
+// ---------------------------------------------------------------------------
+// A kernel's attributes belong to one device.  f() runs until it succeeds once for
+// each device that calls are made on (a bit of `done` each; two host threads that
+// meet may both run it).
+// ---------------------------------------------------------------------------
+constexpr int kMaxDevices = 64;
+template <typename F>
+inline cudaError_t once_per_device(std::atomic<uint64_t>& done, F&& f) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev >= 0 && dev < kMaxDevices ? (uint64_t)1 << dev : 0;
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = f();
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
+}
 
 // ---------------------------------------------------------------------------
 // Programmatic dependent launch.  A kernel queued with launch_k may start

@@ -26,7 +26,6 @@
 namespace {
 
 constexpr int64_t kNoallocScratchElems = (int64_t)1 << 21;   // int64 values
-constexpr int kMaxDevices = 64;
 
 // Products from which a layer with 9 Cin <= 64 runs on the tensor cores, as three
 // launches (12.7 us, host bound) instead of two: 1 x 28 x 28, 1 -> 32 channels (0.2 M
@@ -43,7 +42,7 @@ struct Scratch {
     uint32_t* words = nullptr;
 };
 std::mutex g_mu;
-Scratch g_scratch_addr[kMaxDevices];
+Scratch g_scratch_addr[nitro::kMaxDevices];
 
 // Device addresses of the arrays for the current device, looked up once; the first
 // look-up also loads the kernels, so that no later call takes memory for them.
@@ -51,7 +50,7 @@ cudaError_t scratch_for_current_device(Scratch* out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    if (dev < 0 || dev >= nitro::kMaxDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(g_mu);
     if (!g_scratch_addr[dev].z) {
         void *p = nullptr, *w = nullptr;

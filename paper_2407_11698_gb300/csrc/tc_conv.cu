@@ -16,6 +16,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <type_traits>
 
@@ -1668,13 +1669,15 @@ bool make_map(CUtensorMap* m, const void* base, int rank, const uint64_t* dims,
     return r == CUDA_SUCCESS;
 }
 
+// SMs of the current device
 int sm_count() {
-    static int n = 0;
+    static std::atomic<int> counts[kMaxDevices];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 148;
+    int n = dev < kMaxDevices ? counts[dev].load(std::memory_order_relaxed) : 0;
     if (n == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-            n = 148;
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) return 148;
+        if (dev < kMaxDevices) counts[dev].store(n, std::memory_order_relaxed);
     }
     return n;
 }
@@ -1699,21 +1702,20 @@ cudaError_t launch_gemm(const CUtensorMap& a, const CUtensorMap& b, const TcArgs
     if (args.tiles_n < 1 || args.tiles_m < 1 || args.ntx < 1 || args.nty < 1 || args.lg_wb < 0 ||
         args.lg_hb < 0)
         return cudaErrorInvalidValue;
-    static bool attr_set = false;
-    if (!attr_set) {
+    static std::atomic<uint64_t> ready{0};
+    const cudaError_t e = once_per_device(ready, [] {
         // the setmaxnreg split must fit the registers the CTA is launched with,
         // else setmaxnreg.inc would wait forever: never launch such a build
         cudaFuncAttributes fa{};
-        cudaError_t e = cudaFuncGetAttributes(&fa, k_tc_gemm<MODE, N, PB>);
-        if (e != cudaSuccess) return e;
+        const cudaError_t q = cudaFuncGetAttributes(&fa, k_tc_gemm<MODE, N, PB>);
+        if (q != cudaSuccess) return q;
         if (fa.maxThreadsPerBlock < kThreads ||
             128 * kRegsProducer + 32 * kEpiWarps * kRegsEpilogue > kThreads * fa.numRegs)
             return cudaErrorInvalidConfiguration;
-        e = cudaFuncSetAttribute(k_tc_gemm<MODE, N, PB>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+        return cudaFuncSetAttribute(k_tc_gemm<MODE, N, PB>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+    });
+    if (e != cudaSuccess) return e;
     if ((MODE == TC_FWDK || MODE == TC_FWDD) && args.ksplit > 1)
         return launch_cluster(k_tc_gemm<MODE, N, PB>, dim3(args.total_tiles), kThreads, args.ksplit, s, C::SMEM,
                               a, b, args);
