@@ -304,21 +304,34 @@ void nitro_gemm_destroy(nitro_gemm* g);
  * int8 [batch x h' x w' x cout] (pool2x2 only, else may be NULL), where
  * h' = pool2x2 ? floor(h / 2) : h and w' = pool2x2 ? floor(w / 2) : w (an odd
  * last row or column is dropped by the pool, as in the block path).  It calls no
- * cudaMalloc, cudaFree or allocating library routine: the int64
- * pre-activations go to a fixed 16 MiB array inside the library, so
- * batch*h*w*cout may be at most 2^21; larger sizes return NITRO_ERR_ARG and
- * queue nothing.  Every GPU that loads the library holds that array until the
- * process exits.  The first call on each device looks up the array's address
- * (cudaGetSymbolAddress, with that device current) and keeps it for the life
- * of the process; make that first call before any stream capture.  Calls
- * after a cudaDeviceReset of that device are not supported (the library image
- * may be reloaded elsewhere).  All calls share the one array: calls whose work
- * overlaps on the GPU (different streams, or different host threads) race
- * and give wrong results; serialise them, e.g. on one stream. */
+ * cudaMalloc, cudaFree or allocating library routine: what its kernels need
+ * between them (bf16 operands of the tensor-core forward, or the int64
+ * pre-activations of the CUDA-core one) goes to a fixed 16 MiB array inside
+ * the library, so batch*h*w*cout may be at most 2^21; larger sizes return
+ * NITRO_ERR_ARG and queue nothing.  Every GPU that loads the library holds
+ * that array until the process exits.  The first call on each device looks up
+ * the array's address (cudaGetSymbolAddress, with that device current), keeps
+ * it for the life of the process and loads the kernels; make that first call
+ * before any stream capture.  Calls after a cudaDeviceReset of that device are
+ * not supported (the library image may be reloaded elsewhere).  All calls
+ * share the one array: calls whose work overlaps on the GPU (different
+ * streams, or different host threads) race and give wrong results; serialise
+ * them, e.g. on one stream.
+ *
+ * The call is asynchronous and the waits inside its kernels are bounded, as in
+ * the block step: when one runs out, the outputs of that call are not valid
+ * and the TIMEOUT bit is latched in a status word of the device, which
+ * nitro_conv3x3_noalloc_status reads. */
 nitro_status nitro_conv3x3_forward_noalloc(const int8_t* a_in, const int32_t* weights, int batch,
                                            int h, int w, int cin, int cout, int pool2x2,
                                            int alpha_inv, int8_t* a_out, int8_t* region,
                                            int8_t* argmax, void* stream);
+
+/* Synchronises the current device and returns the latched status of the
+ * allocation-free calls made on it (NITRO_OK or NITRO_ERR_TIMEOUT); clears it
+ * if clear.  Errors: NITRO_ERR_CUDA if the device cannot be read (a stream
+ * capture in progress, for instance). */
+nitro_status nitro_conv3x3_noalloc_status(int clear);
 
 /* ---- Integer data pre-processing (App. A) ---------------------------------
  * Maps a dataset of n 8-bit values x (every element of every sample, e.g.

@@ -100,6 +100,8 @@ def lib():
     L.nitro_profile_record.restype = ctypes.c_int
     L.nitro_conv3x3_forward_noalloc.argtypes = [_VP, _VP] + [ctypes.c_int] * 7 + [_VP, _VP, _VP, _VP]
     L.nitro_conv3x3_forward_noalloc.restype = ctypes.c_int
+    L.nitro_conv3x3_noalloc_status.argtypes = [ctypes.c_int]
+    L.nitro_conv3x3_noalloc_status.restype = ctypes.c_int
     L.nitro_conv3x3_create.argtypes = [ctypes.c_int] * 5 + [ctypes.POINTER(_VP)]
     L.nitro_conv3x3_contract.argtypes = [_VP, ctypes.c_int, _VP, _VP, ctypes.c_int, _VP, _VP]
     L.nitro_conv3x3_status.argtypes = [_VP]
@@ -195,6 +197,10 @@ def nitro_conv3x3_forward_noalloc(a_in, weights, batch, h, w, cin, cout, pool2x2
     return lib().nitro_conv3x3_forward_noalloc(a_in, weights, int(batch), int(h), int(w), int(cin),
                                                int(cout), int(pool2x2), int(alpha_inv), a_out,
                                                region, argmax, stream)
+
+
+def nitro_conv3x3_noalloc_status(clear=False):
+    return lib().nitro_conv3x3_noalloc_status(1 if clear else 0)
 
 
 def nitro_destroy_block(blk):

@@ -36,6 +36,7 @@ constexpr int64_t kNoallocTcMacs = (int64_t)1 << 21;
 
 static __device__ __align__(256) int64_t g_noalloc_scratch[kNoallocScratchElems];
 static __device__ uint32_t g_noalloc_words[4];     // see tc_fwd_in_scratch
+constexpr int kStatusWord = 3;                     // latched TIMEOUT
 
 struct Scratch {
     int64_t* z = nullptr;
@@ -106,4 +107,17 @@ extern "C" nitro_status nitro_conv3x3_forward_noalloc(
         cudaSuccess)
         return NITRO_ERR_CUDA;
     return NITRO_OK;
+}
+
+extern "C" nitro_status nitro_conv3x3_noalloc_status(int clear) {
+    Scratch sc;
+    if (scratch_for_current_device(&sc) != cudaSuccess) return NITRO_ERR_CUDA;
+    uint32_t bits = 0;
+    uint32_t* word = sc.words + kStatusWord;
+    if (cudaDeviceSynchronize() != cudaSuccess ||
+        cudaMemcpy(&bits, word, sizeof(bits), cudaMemcpyDeviceToHost) != cudaSuccess)
+        return NITRO_ERR_CUDA;
+    if (clear && (cudaMemset(word, 0, sizeof(bits)) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess))
+        return NITRO_ERR_CUDA;
+    return bits & ST_TIMEOUT ? NITRO_ERR_TIMEOUT : NITRO_OK;
 }

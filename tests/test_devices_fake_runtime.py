@@ -1,8 +1,8 @@
 """Two devices in one process, on the CPU: the library's own objects linked against a
 stand-in for the CUDA runtime that, like the real one, keeps a kernel's shared-memory
 limit per device and refuses a launch above it.  Nothing runs; what is checked is
-which limits the host code has raised, and for how many SMs it sizes a grid, on the
-device that a call is made on."""
+which limits the host code has raised, for how many SMs it sizes a grid, and whose
+status word it reads, on the device that a call is made on."""
 import glob
 import os
 import shutil
@@ -10,6 +10,7 @@ import subprocess
 
 import pytest
 
+from paper_2407_11698_gb300 import binding as nb
 from paper_2407_11698_gb300 import build as nbuild
 
 FAKE = r'''
@@ -27,6 +28,7 @@ static int g_dev = 0, g_launches = 0, g_refused = 0, g_most_ctas = 0;
 static cudaError_t g_error = cudaSuccess;
 static const int kSms[2] = {152, 20};
 static std::map<std::pair<int, const void*>, int> g_limit;      // device, kernel
+static uint32_t* g_symbol[2];      // the library array looked up last on each device: the noalloc words
 
 static CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                        const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -53,7 +55,10 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
     if (c->dynamicSmemBytes > 48 * 1024 && (int)c->gridDim.x > g_most_ctas) g_most_ctas = (int)c->gridDim.x;
     return cudaSuccess;
 }
-cudaError_t cudaGetSymbolAddress(void** p, const void*) { *p = malloc(1 << 24); return cudaSuccess; }
+cudaError_t cudaGetSymbolAddress(void** p, const void*) {
+    *p = g_symbol[g_dev] = static_cast<uint32_t*>(calloc(1, 1 << 24));
+    return cudaSuccess;
+}
 cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** p, unsigned, unsigned long long,
                                              cudaDriverEntryPointQueryResult* q) {
     *p = reinterpret_cast<void*>(&encode);
@@ -64,9 +69,9 @@ cudaError_t cudaMalloc(void** p, size_t n) { *p = malloc(n); return cudaSuccess;
 cudaError_t cudaMallocHost(void** p, size_t n) { *p = malloc(n); return cudaSuccess; }
 cudaError_t cudaFree(void* p) { free(p); return cudaSuccess; }
 cudaError_t cudaFreeHost(void* p) { free(p); return cudaSuccess; }
-cudaError_t cudaMemset(void*, int, size_t) { return cudaSuccess; }
+cudaError_t cudaMemset(void* p, int v, size_t n) { memset(p, v, n); return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void*, int, size_t, cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaMemcpy(void*, const void*, size_t, cudaMemcpyKind) { return cudaSuccess; }
+cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { memcpy(d, s, n); return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void*, const void*, size_t, cudaMemcpyKind, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaGetLastError() {
     const cudaError_t e = g_error;
@@ -111,6 +116,11 @@ int main() {
         }
         printf("%d %d %d %d %d\n", g_dev, st, g_launches, g_refused, g_most_ctas);
     }
+    // a wait that ran out on the second device: the kernel sets the TIMEOUT bit of words[3]
+    g_symbol[1][3] = NITRO_STATUS_BIT_TIMEOUT;
+    for (g_dev = 0; g_dev < 2; ++g_dev)
+        for (int clear : {0, 1, 0}) printf("%d ", (int)nitro_conv3x3_noalloc_status(clear));
+    printf("\n");
     return 0;
 }
 '''
@@ -128,8 +138,11 @@ def test_calls_on_a_second_device(tmp_path):
                    sorted(glob.glob(os.path.join(nbuild.OUT_DIR, "*.o"))) + ["-o", str(exe), "-lpthread"],
                    check=True, capture_output=True, text=True)
     out = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.splitlines()
-    assert len(out) == 2
+    assert len(out) == 3
     for line, sms in zip(out, (152, 20)):
         dev, st, launches, refused, ctas = map(int, line.split())
         assert st == 0 and launches > 0 and refused == 0, out
         assert ctas == sms, out                # a persistent grid: one CTA an SM of this device
+    # the status of the allocation-free calls: latched, per device, cleared on request
+    timeout = nb.NITRO_ERR_TIMEOUT
+    assert list(map(int, out[2].split())) == [0, 0, 0, timeout, timeout, 0]

@@ -1,7 +1,7 @@
 """The allocation-free conv forward against the block forward and the oracle (GPU).
 
 nitro_conv3x3_forward_noalloc serves callers that cannot allocate device
-memory while running; it keeps its int64 scratch in a fixed array inside the
+memory while running; it keeps its scratch in a fixed array inside the
 library.  This file is named to be collected last, so a run that stops at
 the first failure has run every other test before it.
 """
@@ -140,3 +140,8 @@ def test_noalloc_call_captures_into_a_cuda_graph(torch):
                am.cpu().numpy().reshape(-1))
         _same(got, _oracle_forward(xh.astype(np.int64), w.astype(np.int64), B, h, wd, cin, cout,
                                    pool, alpha), "replay %d vs oracle" % k)
+
+
+def test_noalloc_status_is_readable(torch):
+    assert nb.nitro_conv3x3_noalloc_status(clear=True) == nb.NITRO_OK
+    assert nb.nitro_conv3x3_noalloc_status() == nb.NITRO_OK
