@@ -626,10 +626,9 @@ def run_sweep(args):
         gm.close()
         del a, b8, c
         torch.cuda.empty_cache()
-    # IntegerSGD alone: one linear layer of n x n weights (16 bytes per weight:
-    # W read + write, dW read; + 8 for the four bf16 limb planes the update
-    # writes for the tensor-core forward) and its learning layer, against the
-    # measured HBM copy bandwidth
+    # IntegerSGD alone: one linear layer of n x n weights and its learning layer, 12
+    # bytes a weight (W and dW read; with dW zero and no decay nothing is written)
+    # against the measured HBM copy bandwidth
     hbm = peaks["hbm_gbs"]
     for n in ((4096, 16384) if "sgd" in parts else ()):
         blk = nb.Block([(nb.NITRO_LINEAR, n, n, 1, 1, 0)], n, seed=1, max_batch=1)

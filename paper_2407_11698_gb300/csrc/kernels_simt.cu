@@ -1432,9 +1432,10 @@ cudaError_t simt_integersgd(const SgdBatch& b_in, cudaStream_t s) {
         }
     }
     const int grid = b.first[b.count];
+    // W and dW are read; what is written (up to 4 bytes and 8 of planes a weight) depends
+    // on the data and is not counted
     double bytes = 0;
-    for (int i = 0; i < b.count; ++i)
-        bytes += (b.t[i].planes ? 24.0 : 16.0) * b.t[i].n;   // W r+w, dW r (+ 4 bf16 planes)
+    for (int i = 0; i < b.count; ++i) bytes += 12.0 * b.t[i].n;
     ProfScope ps(K_INTEGERSGD, s, 0.0, bytes);
     launch_k(k_integersgd, grid, 256, 0, s, b);
     return cudaGetLastError();

@@ -1,6 +1,8 @@
 """IntegerSGD's 32-bit divide and the limb planes it keeps: gradients on both
 sides of 2^31, divisors around 2^31, weights that change limb count in both
 directions or not at all.  The forward after each update reads the planes."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -57,4 +59,23 @@ def test_updates_and_planes(layer, trunc, gamma_lr, eta):
                 ob.forward(x.astype(np.int64))
                 assert np.array_equal(out.cpu().numpy().reshape(-1), ob.act[0].reshape(-1))
     finally:
+        blk.close()
+
+
+def test_profile_counts_the_bytes_that_every_update_moves():
+    # 12 bytes a weight are read (W, dW); stores depend on what changes
+    lib = nb.lib()
+    blk = nb.Block([(L, 64, 72, 1, 1, 0)], 64, max_batch=2)
+    n, ms, ops, byts = ctypes.c_uint64(), ctypes.c_double(), ctypes.c_double(), ctypes.c_double()
+    names = [lib.nitro_profile_kernel_name(k) for k in range(lib.nitro_profile_kernel_count())]
+    try:
+        lib.nitro_profile_reset()
+        lib.nitro_profile_enable(1)
+        blk.sgd()
+        lib.nitro_profile_enable(0)
+        assert lib.nitro_profile_read(names.index(b"integersgd"), ctypes.byref(n), ctypes.byref(ms),
+                                      ctypes.byref(ops), ctypes.byref(byts)) == nb.NITRO_OK
+        assert (n.value, byts.value) == (1, 12.0 * (64 * 72 + 72 * 10))
+    finally:
+        lib.nitro_profile_reset()
         blk.close()
