@@ -80,6 +80,9 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_sample(const uint4* __res
                                                               PrepState* st) {
     pdl_wait();
     const uint32_t k = blockIdx.x * kPrepThreads + threadIdx.x;
+    // multiplicative hash by a prime near 2^32 over the golden ratio (Knuth, The Art of
+    // Computer Programming, vol. 3, 6.4), its upper bits folded in and mixed by the first
+    // multiplier of MurmurHash3's finalizer (Appleby)
     uint32_t h = k * 2654435761u;
     h ^= h >> 15;
     h *= 0x85ebca6bu;
@@ -332,7 +335,8 @@ nitro_status nitro_prep_fit(nitro_prep* p, const uint8_t* x, int64_t n, void* st
         launch_k(k_prep_reduce<0>, grid, kPrepThreads, 0, s, x, n, p->st);
     }
     {
-        ProfScope ps(K_PREP_MAD, s, 0.0, (double)n);
+        // after one pass the launch reads nothing unless mu was none of the guesses
+        ProfScope ps(K_PREP_MAD, s, 0.0, n >= kOnePassBytes ? 0.0 : (double)n);
         launch_k(k_prep_reduce<1>, grid, kPrepThreads, 0, s, x, n, p->st);
     }
     if (cudaGetLastError() != cudaSuccess) {

@@ -1,6 +1,8 @@
 """The one-pass fit of large datasets: sizes at its threshold, odd starts, the ends of
 the byte range where the guesses are clamped, and data whose sampled mean misses mu,
 so that the second pass runs, on one object in turn."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -59,4 +61,28 @@ def test_fit_matches_oracle(n, off, kinds):
             lut = O.prep_apply(np.arange(256, dtype=np.uint8), mu, om)
             assert np.array_equal(out.cpu().numpy(), lut.astype(np.int8)[x]), kind
     finally:
+        p.close()
+
+
+def test_profile_counts_the_bytes_that_a_fit_reads():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    lib, p = nb.lib(), nb.IntPrep()
+    names = [lib.nitro_profile_kernel_name(k) for k in range(lib.nitro_profile_kernel_count())]
+    try:
+        for n, want in ((THRESHOLD - 1, [THRESHOLD - 1] * 2), (THRESHOLD, [THRESHOLD + 16 * SAMPLES, 0])):
+            x = torch.from_numpy(data("natural", n, 0)).cuda()
+            lib.nitro_profile_reset()
+            lib.nitro_profile_enable(1)
+            p.fit(x)
+            lib.nitro_profile_enable(0)
+            got = []
+            for name in (b"prep_sum", b"prep_mad"):
+                c, ms, ops, by = ctypes.c_uint64(), ctypes.c_double(), ctypes.c_double(), ctypes.c_double()
+                assert lib.nitro_profile_read(names.index(name), ctypes.byref(c), ctypes.byref(ms),
+                                              ctypes.byref(ops), ctypes.byref(by)) == nb.NITRO_OK
+                got.append(by.value)
+            assert got == want
+    finally:
+        lib.nitro_profile_reset()
         p.close()
