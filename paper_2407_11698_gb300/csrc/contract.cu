@@ -76,10 +76,12 @@ nitro_status nitro_conv3x3_create(int max_batch, int h, int w, int cin, int cout
     if (!c) return NITRO_ERR_CUDA;
     c->g = LayerGeom{NITRO_CONV3X3, cin, cout, h, w, 0, h, w};
     c->max_batch = max_batch;
-    bool ok = dalloc(c->allocs, &c->words, 6) &&
-              tc_layer_init(c->t, c->g, max_batch, true, c->words, c->words + 1, c->allocs,
-                            c->host_allocs);
-    if (ok) ok = cudaMemset(c->words, 0, 24) == cudaSuccess;
+    bool ok = dalloc(c->allocs, &c->words, 6);
+    ok = ok && on_own_stream([&](cudaStream_t s) {
+        if (!tc_layer_init(c->t, c->g, max_batch, true, c->words, c->words + 1, c->allocs, c->host_allocs, s))
+            return cudaErrorMemoryAllocation;
+        return cudaMemsetAsync(c->words, 0, 24, s);
+    }) == cudaSuccess;
     if (!ok) {
         free_all(c->allocs);
         free_host(c->host_allocs);
@@ -162,7 +164,7 @@ nitro_status nitro_gemm_create(int max_m, int max_n, int max_k, nitro_gemm** out
     bool ok = dalloc(g->allocs, &g->a, (size_t)max_m * max_k) &&
               dalloc(g->allocs, &g->b, (size_t)kMaxLimbs * max_n * max_k) &&
               dalloc(g->allocs, &g->words, 4);
-    if (ok) ok = cudaMemset(g->words, 0, 16) == cudaSuccess;
+    ok = ok && on_own_stream([&](cudaStream_t s) { return cudaMemsetAsync(g->words, 0, 16, s); }) == cudaSuccess;
     if (!ok) {
         free_all(g->allocs);
         delete g;

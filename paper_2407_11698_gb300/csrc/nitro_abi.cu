@@ -293,12 +293,13 @@ nitro_status nitro_init_block(const nitro_block_desc* desc, uint64_t seed, void*
         ok = ly.lin_a ? tc_linear_init(ly.tc, ly.g, desc->max_batch, ly.lin_a, ly.lin_planes, w_w(b, i),
                                        w_delta(b, i), b->allocs, b->host_allocs)
                       : tc_layer_init(ly.tc, ly.g, desc->max_batch, i > 0, w_w(b, i), w_delta(b, i),
-                                      b->allocs, b->host_allocs);
+                                      b->allocs, b->host_allocs, s);
         // one copy of all the block's words per step refreshes the layers' hints
         if (ok) tc_use_external_hints(ly.tc, b->words_host + 3 + i,
                                       b->words_host + 4 + desc->n_layers + i);
     }
     if (!ok) {
+        cudaStreamSynchronize(s);      // layers made before the one that failed queued their clears
         free_all(b);
         delete b;
         return NITRO_ERR_CUDA;

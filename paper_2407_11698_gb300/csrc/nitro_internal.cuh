@@ -398,6 +398,20 @@ inline cudaError_t once_per_device(std::atomic<uint64_t>& done, F&& f) {
     return e;
 }
 
+// Runs f(s) on a stream of its own and waits for it: what a handle's creation clears is
+// then cleared when the call returns.  (A plain cudaMemset queues on the default stream
+// and may still be waiting there when the handle is used on another one.)
+template <typename F>
+inline cudaError_t on_own_stream(F&& f) {
+    cudaStream_t s = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    e = f(s);
+    const cudaError_t q = cudaStreamSynchronize(s);
+    cudaStreamDestroy(s);
+    return e != cudaSuccess ? e : q;
+}
+
 // ---------------------------------------------------------------------------
 // Programmatic dependent launch.  A kernel queued with launch_k may start
 // (get SMs, set up shared memory, barriers and TMEM) while the kernel before

@@ -310,7 +310,8 @@ nitro_status nitro_prep_create(nitro_prep** out) {
     bool ok = cudaGetDevice(&dev) == cudaSuccess &&
               cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
               cudaMalloc(&p->st, sizeof(PrepState) + (size_t)p->sms * kCtasPerSm * 32) == cudaSuccess &&
-              cudaMemset(p->st, 0, sizeof(PrepState)) == cudaSuccess;
+              on_own_stream([&](cudaStream_t s) { return cudaMemsetAsync(p->st, 0, sizeof(PrepState), s); }) ==
+                  cudaSuccess;
     if (!ok) {
         if (p->st) cudaFree(p->st);
         delete p;

@@ -1894,7 +1894,7 @@ cudaError_t tc_fwd_preload() {
 
 bool tc_layer_init(TcLayer& t, const LayerGeom& g, int max_batch, bool has_dgrad,
                    const uint32_t* maxabs_w, const uint32_t* maxabs_d,
-                   std::vector<void*>& allocs, std::vector<void*>& host_allocs) {
+                   std::vector<void*>& allocs, std::vector<void*>& host_allocs, cudaStream_t s) {
     t = TcLayer();
     t.maxabs_w = maxabs_w;
     t.maxabs_d = maxabs_d;
@@ -1916,7 +1916,7 @@ bool tc_layer_init(TcLayer& t, const LayerGeom& g, int max_batch, bool has_dgrad
             t.max_host[0] = t.max_host[1] = 0;
         }
     }
-    if (ok && t.w_planes) ok = cudaMemset(t.w_planes, 0, (size_t)kMaxLimbs * nwk * 2) == cudaSuccess;
+    if (ok && t.w_planes) ok = cudaMemsetAsync(t.w_planes, 0, (size_t)kMaxLimbs * nwk * 2, s) == cudaSuccess;
     return ok;
 }
 
