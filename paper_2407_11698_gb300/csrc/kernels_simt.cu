@@ -5,10 +5,11 @@
 // NITRO-ReLU backward and STE; the learning layer, its max-pool to d_lr and
 // the RSS loss; IntegerSGD).
 //
-// The GEMM serves the contractions the tensor-core path does not take (narrow
-// or small conv layers, linear input gradients, the kernel-level matrix product
-// where K is not a multiple of 8); the learning layer (G = 10 outputs) and
-// the element-wise stages always run here.
+// The GEMM serves the contractions the tensor-core path does not take (conv
+// gradients where Cout is not a multiple of 8 or the input is narrow, linear input
+// gradients, the kernel-level matrix product where K is not a multiple of 8, small
+// or misaligned allocation-free forwards); the learning layer (up to 64 outputs)
+// and the element-wise stages always run here.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 

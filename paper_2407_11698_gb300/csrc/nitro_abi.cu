@@ -51,7 +51,6 @@ struct nitro_block {
     int64_t* dWlr = nullptr;
     int32_t* grad_l = nullptr;      // [max_batch x G]
     int64_t* z64 = nullptr;         // scratch, int64 pre-activations / dgrad outputs
-    size_t z64_elems = 0;
     uint32_t* words = nullptr;      // [0] status [1] step counter (dropout masks)
                                     // [2] max|W_lr| [3 + i] max|W_i|    (reset by the update)
                                     // [3 + n] max|grad_l| [4 + n + i] max|delta_i|, then the
@@ -287,7 +286,6 @@ nitro_status nitro_init_block(const nitro_block_desc* desc, uint64_t seed, void*
             b->words_host = static_cast<uint32_t*>(h);
         }
     }
-    b->z64_elems = z_need;
     for (int i = 0; ok && i < desc->n_layers; ++i) {
         Layer& ly = b->L[i];
         ok = ly.lin_a ? tc_linear_init(ly.tc, ly.g, desc->max_batch, ly.lin_a, ly.lin_planes, w_w(b, i),

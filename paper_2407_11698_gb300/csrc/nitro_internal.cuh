@@ -21,7 +21,6 @@ __host__ __device__ __forceinline__ int32_t fdiv32(int32_t x, int32_t d) {
     int32_t q = x / d;
     return (x % d < 0) ? q - 1 : q;
 }
-__host__ __device__ __forceinline__ int64_t tdiv64(int64_t x, int64_t d) { return x / d; }
 
 // floor(z / (256 * k)) = floor(floor(z / 256) / k) for k > 0; the first step
 // is an arithmetic shift.

@@ -39,9 +39,9 @@ cudaEvent_t take_event() {
 
 const char* const kNames[K_COUNT] = {
     "simt_conv_fwd", "simt_conv_dgrad", "simt_conv_wgrad", "simt_linear_fwd",
-    "simt_linear_dgrad", "simt_linear_wgrad", "fwd_epilogue", "learn_partial",
-    "learn_dw", "grad_to_delta", "integersgd", "learn_finish_loss", "tc_conv_fwd",
-    "tc_conv_wgrad", "tc_conv_dgrad", "tc_pack_limbs", "tc_finish", "tc_gemm", "lr_backward",
+    "simt_linear_dgrad", "simt_linear_wgrad", "fwd_epilogue", "learn_fwd",
+    "grad_to_delta", "integersgd", "tc_conv_fwd",
+    "tc_conv_wgrad", "tc_conv_dgrad", "tc_pack_limbs", "tc_gemm", "lr_backward",
     "tc_pack_weights", "tc_pack_input", "tc_pack_delta", "prep_sum", "prep_mad",
     "prep_apply", "lr_pool", "lrpool_to_delta", "tc_timeout_probe", "tc_linear_wgrad"};
 

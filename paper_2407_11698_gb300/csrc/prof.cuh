@@ -20,15 +20,12 @@ enum KernelId : int {
     K_SIMT_LIN_WGRAD,
     K_FWD_EPILOGUE,
     K_LEARN_FWD,
-    K_LEARN_DW,
     K_GRAD_TO_DELTA,
     K_INTEGERSGD,
-    K_FINISH_LOSS,
     K_TC_CONV_FWD,
     K_TC_CONV_WGRAD,
     K_TC_CONV_DGRAD,
     K_TC_PACK,
-    K_TC_FINISH,
     K_TC_GEMM,
     K_LR_BACKWARD,
     K_TC_PACK_W,

@@ -5,9 +5,9 @@
 // A persistent CTA computes 128 x N output tiles, each over a range of
 // K-blocks (64 elements each).  Warp 0 issues TMA loads into an S-stage shared-memory ring,
 // warp 1 allocates TMEM and issues the MMAs, warps 4..19 drain the fp32 TMEM
-// accumulator every <= 16 K-blocks into int64 registers (the fused forward: into
-// z modulo 2^32 and an fp32 sum; four warps per TMEM
-// lane quadrant, each owning a quarter of the N columns).  Four TMEM accumulators
+// accumulator every <= 16 K-blocks into int64 registers (the fused forward and input
+// gradient: into the sum modulo 2^32 and an fp32 sum; four warps per TMEM lane
+// quadrant, each owning a quarter of the N columns).  Four TMEM accumulators
 // rotate so the MMAs run up to three chunks ahead of the drain.
 // Every wait on an mbarrier is bounded in time; on expiry the kernel raises
 // the TIMEOUT status bit, lets the other roles leave, frees TMEM and returns.
@@ -233,7 +233,7 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t* r) {
 
 // ------------------------------------------------------------------ kernel
 struct TcArgs {
-    int B, H, W, Cin, Cout, Bp;
+    int B, H, W, Cin, Cout;
     int cin_k;             // channels per tap in the K index (Cin rounded up to 64)
     int taps;              // 9, or 1 for im2col input (forward / wgrad: no tap shift)
     int ntx, nty;          // pixel tiles along x and y (forward / dgrad)
@@ -397,7 +397,7 @@ __device__ __forceinline__ Tile decode_tile(const TcArgs& a, int tile) {
 }
 
 // Persistent: CTA c handles tiles c, c + gridDim.x, ...; the TMA ring, the
-// MMA chunk sequence and the two TMEM accumulators run on across tiles, so
+// MMA chunk sequence and the TMEM accumulators (up to four) run on across tiles, so
 // one tile's epilogue overlaps the next tile's loads and MMAs.
 template <int MODE, int N, int PB>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -684,7 +684,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         cluster_barrier();
     }
     } else {
-        // ---------------- epilogue: warpgroups 1 and 2
+        // ---------------- epilogue: warpgroups 1 to 4
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpilogue));
         const int q = warp & 3;                     // TMEM lane quadrant this warp may read
         const int half = (warp - kEpiWarp0) >> 2;   // which quarter of the N columns
@@ -1956,12 +1956,6 @@ int tc_limb_hint(const TcLayer& t, int which) {
     return t.max_host ? limb_count(t.max_host[which]) : 1;
 }
 
-cudaError_t tc_weights_hint(TcLayer& t, cudaStream_t s) {
-    if (!t.w_planes || !t.maxabs_w || !t.own_hints) return cudaSuccess;
-    // host copy of max |W|, read later as a kernel-variant hint only
-    return cudaMemcpyAsync(t.max_host, t.maxabs_w, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
-}
-
 void tc_weight_planes(const TcLayer& t, const LayerGeom& g, uint16_t** planes, int64_t* plane,
                       int* row_k, int* tap_k) {
     *planes = t.w_planes;
@@ -2061,7 +2055,6 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
     if (lin && !fo) return cudaSuccess;
     TcArgs a{};
     a.B = batch; a.H = lin ? 1 : g.h; a.W = lin ? 1 : g.w; a.Cin = g.cin; a.Cout = g.cout;
-    a.Bp = round_up(batch, 8);
     a.cin_k = t.cin_k;
     a.taps = t.im2col || lin ? 1 : 9;
     if (lin) {
@@ -2165,7 +2158,6 @@ cudaError_t tc_conv_wgrad(TcLayer& t, const LayerGeom& g, const int32_t* delta,
     const int hw = gh * gw;
     TcArgs a{};
     a.B = nimg; a.H = gh; a.W = gw; a.Cin = g.cin; a.Cout = g.cout;
-    a.Bp = round_up(nimg, 8);
     a.cin_k = t.cin_k;
     a.taps = (t.im2col || lin) ? 1 : 9;
     a.rows = lin ? g.cin : 9 * g.cin;
@@ -2241,7 +2233,6 @@ cudaError_t tc_conv_dgrad(TcLayer& t, const LayerGeom& g, int batch, int64_t* g6
     if (!t.dgrad || batch <= 0) return cudaSuccess;
     TcArgs a{};
     a.B = batch; a.H = g.h; a.W = g.w; a.Cin = g.cin; a.Cout = g.cout;
-    a.Bp = round_up(batch, 8);
     a.cin_k = t.cin_k;
     a.taps = 9;
     pixel_tiling(g, batch, a);

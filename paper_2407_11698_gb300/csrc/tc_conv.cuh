@@ -105,9 +105,6 @@ bool tc_layer_init(TcLayer& t, const LayerGeom& g, int max_batch, bool has_dgrad
 void tc_weight_planes(const TcLayer& t, const LayerGeom& g, uint16_t** planes, int64_t* plane,
                       int* row_k, int* tap_k);
 
-// After such an update: refresh the host hint of max |W|.
-cudaError_t tc_weights_hint(TcLayer& t, cudaStream_t s);
-
 // Re-splits the layer's int32 weights into limb planes (after init, an update
 // or a checkpoint load); the limb count follows *maxabs_w unless all_planes.
 cudaError_t tc_refresh_weights(TcLayer& t, const LayerGeom& g, const int32_t* W,
@@ -141,16 +138,15 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
                             bool* fused);
 
 // Splits delta into NHWC limb planes for the wgrad and dgrad passes (limb
-// count from *maxabs_delta), unless planes_done (an earlier call split this
-// delta already), and clears zero[0..n_zero) (not with planes_done); then refreshes the host hint of max |delta|.  Writing the
-// planes from the kernels that produce delta instead (the dgrad epilogue,
-// the learning-layer backward) was measured slower than this pass.
+// count from *maxabs_delta) and clears zero[0..n_zero), unless planes_done; then
+// refreshes the host hint of max |delta|.  planes_done: the learning backward or the
+// routing through the learning pool wrote the planes with the delta (and cleared),
+// or an earlier call split it.  A delta that the input gradient produced is split
+// here: the same stores in its epilogue were measured slower than this pass.
 cudaError_t tc_pack_delta(TcLayer& t, const LayerGeom& g, const int32_t* delta,
                           const uint32_t* maxabs_delta, int batch, cudaStream_t s,
                           bool planes_done = false, int64_t* zero = nullptr, int64_t n_zero = 0);
 
-// tc_pack_delta, then, if wgrad runs on tcgen05, dW = sum_p delta (x)
-// im2col(a).  Must precede tc_conv_dgrad.
 // dW when tc_conv_wgrad adds K-split partial sums into it at this batch (it must
 // be zero before), else null.
 int64_t* tc_wgrad_adds(const TcLayer& t, const LayerGeom& g, int batch, int64_t* dW);
@@ -159,6 +155,8 @@ int64_t* tc_wgrad_adds(const TcLayer& t, const LayerGeom& g, int batch, int64_t*
 // this batch, i.e. when tc_conv_wgrad can fold IntegerSGD into it.
 bool tc_wgrad_fusable(const TcLayer& t, const LayerGeom& g, int batch);
 
+// tc_pack_delta, then, if wgrad runs on tcgen05, dW = sum_p delta (x)
+// im2col(a).  Must precede tc_conv_dgrad.
 // With sgd != null the kernel also applies IntegerSGD (see TcSgd) when the
 // weight gradient runs on tcgen05 without a K split; *sgd_done says whether
 // it did (the caller updates the layer otherwise).
