@@ -381,18 +381,15 @@ cudaError_t simt_integersgd(const SgdBatch& b, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // A kernel's attributes belong to one device.  f() runs until it succeeds once for
-// each device that calls are made on (a bit of `done` each; two host threads that
+// each device dev that calls are made on (a bit of `done` each; two host threads that
 // meet may both run it).
 // ---------------------------------------------------------------------------
 constexpr int kMaxDevices = 64;
 template <typename F>
-inline cudaError_t once_per_device(std::atomic<uint64_t>& done, F&& f) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
+inline cudaError_t once_per_device(std::atomic<uint64_t>& done, int dev, F&& f) {
     const uint64_t bit = dev >= 0 && dev < kMaxDevices ? (uint64_t)1 << dev : 0;
     if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
-    e = f();
+    const cudaError_t e = f();
     if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
     return e;
 }

@@ -1669,12 +1669,15 @@ bool make_map(CUtensorMap* m, const void* base, int rank, const uint64_t* dims,
     return r == CUDA_SUCCESS;
 }
 
-// SMs of the current device
-int sm_count() {
+// SMs of the current device, and which it is (-1: unknown).  The query takes 16 ns,
+// which eager steps of small layers feel, so callers ask once.
+int sm_count(int* device = nullptr) {
     static std::atomic<int> counts[kMaxDevices];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 148;
-    int n = dev < kMaxDevices ? counts[dev].load(std::memory_order_relaxed) : 0;
+    int dev = -1, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+    if (device) *device = dev;
+    if (dev < 0) return 148;
+    if (dev < kMaxDevices) n = counts[dev].load(std::memory_order_relaxed);
     if (n == 0) {
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) return 148;
         if (dev < kMaxDevices) counts[dev].store(n, std::memory_order_relaxed);
@@ -1703,7 +1706,9 @@ cudaError_t launch_gemm(const CUtensorMap& a, const CUtensorMap& b, const TcArgs
         args.lg_hb < 0)
         return cudaErrorInvalidValue;
     static std::atomic<uint64_t> ready{0};
-    const cudaError_t e = once_per_device(ready, [] {
+    int dev = 0;
+    const int sms = sm_count(&dev);
+    const cudaError_t e = once_per_device(ready, dev, [] {
         // the setmaxnreg split must fit the registers the CTA is launched with,
         // else setmaxnreg.inc would wait forever: never launch such a build
         cudaFuncAttributes fa{};
@@ -1719,7 +1724,7 @@ cudaError_t launch_gemm(const CUtensorMap& a, const CUtensorMap& b, const TcArgs
     if ((MODE == TC_FWDK || MODE == TC_FWDD) && args.ksplit > 1)
         return launch_cluster(k_tc_gemm<MODE, N, PB>, dim3(args.total_tiles), kThreads, args.ksplit, s, C::SMEM,
                               a, b, args);
-    const int grid = args.total_tiles < sm_count() ? args.total_tiles : sm_count();
+    const int grid = args.total_tiles < sms ? args.total_tiles : sms;
     launch_k(k_tc_gemm<MODE, N, PB>, grid, kThreads, C::SMEM, s, a, b, args);
     return cudaGetLastError();
 }
@@ -2033,10 +2038,12 @@ namespace {
 // 14.1; 64 images 512 -> 512 at 4 x 4 35.7 against 22.6.
 void fwd_split(TcArgs& a, int cout, int* n) {
     const auto tiles = [&](int w) { return a.tiles_m * ((cout + w - 1) / w); };
-    if (a.kb_total < 16 || tiles(*n) * 2 > sm_count()) return;
-    if (*n == 128 && tiles(128) * 8 < sm_count()) *n = 64;
+    if (a.kb_total < 16) return;
+    const int sms = sm_count();
+    if (tiles(*n) * 2 > sms) return;
+    if (*n == 128 && tiles(128) * 8 < sms) *n = 64;
     for (const int s : {8, 4, 2}) {
-        if ((s == 8 && (*n == 128 || tiles(*n) * 8 > 104)) || tiles(*n) * s > sm_count() || a.kb_total < 4 * s)
+        if ((s == 8 && (*n == 128 || tiles(*n) * 8 > 104)) || tiles(*n) * s > sms || a.kb_total < 4 * s)
             continue;
         a.ksplit = s;
         return;
