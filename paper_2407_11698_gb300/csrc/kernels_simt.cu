@@ -65,7 +65,7 @@ __device__ __forceinline__ int32_t load_a(const GemmParams& p, int m, int k) {
         if (iy < 0 || iy >= p.H || ix < 0 || ix >= p.W) return 0;
         const int64_t idx = ((int64_t)(b * p.H + iy) * p.W + ix) * C + c;
         return MODE == GM_CONV_FWD ? (int32_t)p.act[idx] : p.grad[idx];
-    } else if (MODE == GM_CONV_WGRAD) {
+    } else if (MODE == GM_CONV_WGRAD || MODE == GM_LIN_WGRAD) {
         return p.grad[(int64_t)k * p.Cout + m];
     } else if (MODE == GM_LIN_FWD) {
         return p.act[(int64_t)m * p.Cin + k];
@@ -90,8 +90,10 @@ __device__ __forceinline__ int32_t load_b(const GemmParams& p, int n, int k) {
         return p.act[((int64_t)(b * p.H + iy) * p.W + ix) * p.Cin + ci];
     } else if (MODE == GM_LIN_FWD) {
         return p.wts[(int64_t)n * p.Cin + k];
-    } else {  // GM_LIN_DGRAD
+    } else if (MODE == GM_LIN_DGRAD) {
         return p.wts[(int64_t)k * p.Cin + n];
+    } else {  // GM_LIN_WGRAD
+        return p.act[(int64_t)k * p.Cin + n];
     }
 }
 
@@ -241,6 +243,11 @@ constexpr int kLfSpan = 128;       // tiles per 32-bit sum
 // (batch 256, 512 x 512), 128 M 23.6 / 20.0; four limbs at 64 M 18.3 / 16.8.  Whole
 // backward: 16 M 18.2 / 19.5, 32 M 18.6 / 19.6, 64 M 26.1 / 19.5.
 constexpr int64_t kLinFwdMacs = (int64_t)48 << 20, kLinWgradMacs = (int64_t)32 << 20;
+// Products above which the weight gradient of a layer without a tensor-core form takes the
+// general GEMM, whose 4 x 4 sums a thread feed the multipliers better (the samples padded
+// to whole slabs): backward of a 1001 -> 999 layer at batch 192 57 us here, 60 there, at
+// 512 134 and 114, at 1024 263 and 203.
+constexpr int64_t kLinGemmMacs = (int64_t)192 << 20;
 
 struct LearnArgs {
     const int8_t* a;
@@ -460,14 +467,15 @@ __global__ void __launch_bounds__(256) k_lin_fwd(const LearnArgs p, const LinFwd
 
 // Weight gradient of a linear layer: dW[o][i] = sum_b d[b][o] a[b][i], 16 outputs x
 // 64 inputs per CTA, four inputs a thread, the samples in slabs through shared
-// memory; every sum is finished in one thread (no K split, no clearing).  Few
-// products: bound by latency.  A backward of 64 x 784 x 100 with it takes 13.7 us,
-// 19.7 us with the general CUDA-core GEMM, which decodes an index for every operand
-// it stages.
+// memory.  Few products: bound by latency, some 2.3 us a slab, so the slabs are shared
+// out over CTAs (blockIdx.y, `per` samples each) that add into a cleared dW.  A backward
+// of 64 x 784 x 100 with it takes 13.7 us, 19.7 us with the general CUDA-core GEMM, which
+// decodes an index for every operand it stages; of 4096 x 64 x 64 25 us, 366 with all
+// samples in one CTA a tile.
 constexpr int kLwB = 32;           // samples per slab
 __global__ void __launch_bounds__(256) k_lin_wgrad(const int8_t* __restrict__ a,
                                                    const int32_t* __restrict__ dl, int B, int in,
-                                                   int out, int64_t* __restrict__ dw) {
+                                                   int out, int per, int64_t* __restrict__ dw) {
     pdl_wait();
     __shared__ int32_t ds[kLwB][16];
     __shared__ __align__(4) int8_t as[kLwB][64];
@@ -475,34 +483,45 @@ __global__ void __launch_bounds__(256) k_lin_wgrad(const int8_t* __restrict__ a,
     const int i0 = (int)(blockIdx.x % ti) * 64, o0 = (int)(blockIdx.x / ti) * 16;
     const int oi = threadIdx.x >> 4, q = threadIdx.x & 15;
     int64_t acc[4] = {0, 0, 0, 0};
-    for (int b0 = 0; b0 < B; b0 += kLwB) {
+    const int b_end = min(B, ((int)blockIdx.y + 1) * per);
+    for (int b0 = (int)blockIdx.y * per; b0 < b_end; b0 += kLwB) {
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < kLwB * 16 / 256; ++k) {
             const int e = threadIdx.x + 256 * k, b = e >> 4, c = e & 15;
-            ds[b][c] = b0 + b < B && o0 + c < out ? dl[(int64_t)(b0 + b) * out + o0 + c] : 0;
+            ds[b][c] = b0 + b < b_end && o0 + c < out ? dl[(int64_t)(b0 + b) * out + o0 + c] : 0;
         }
 #pragma unroll
         for (int k = 0; k < kLwB * 64 / 256; ++k) {
             const int e = threadIdx.x + 256 * k, b = e >> 6, c = e & 63;
-            as[b][c] = b0 + b < B && i0 + c < in ? a[(int64_t)(b0 + b) * in + i0 + c] : (int8_t)0;
+            as[b][c] = b0 + b < b_end && i0 + c < in ? a[(int64_t)(b0 + b) * in + i0 + c] : (int8_t)0;
         }
         __syncthreads();
-#pragma unroll 8
-        for (int b = 0; b < kLwB; ++b) {
+        const auto add = [&](int b) {
             const int32_t d = ds[b][oi];
             const char4 v = *reinterpret_cast<const char4*>(&as[b][4 * q]);
             acc[0] += (int64_t)d * v.x;
             acc[1] += (int64_t)d * v.y;
             acc[2] += (int64_t)d * v.z;
             acc[3] += (int64_t)d * v.w;
+        };
+        if (b_end - b0 > 8) {                  // zeros past the last sample
+#pragma unroll 8
+            for (int b = 0; b < kLwB; ++b) add(b);
+        } else {
+            for (int b = 0; b < b_end - b0; ++b) add(b);
         }
     }
     if (o0 + oi >= out) return;
     int64_t* row = dw + (int64_t)(o0 + oi) * in;
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-        if (i0 + 4 * q + k < in) row[i0 + 4 * q + k] = acc[k];
+    for (int k = 0; k < 4; ++k) {
+        if (i0 + 4 * q + k >= in) break;
+        if (gridDim.y > 1)
+            atomicAdd(reinterpret_cast<unsigned long long*>(row + i0 + 4 * q + k), (unsigned long long)acc[k]);
+        else
+            row[i0 + 4 * q + k] = acc[k];
+    }
 }
 
 // The last CTAs of the kernel after k_learn_fwd: SSE, loss = floor(SSE / 2), max
@@ -1219,6 +1238,7 @@ cudaError_t simt_gemm(int mode, const int8_t* act, const int32_t* grad, const in
         case GM_CONV_WGRAD: p.M = Cout; p.N = 9 * Cin; p.K = P; break;
         case GM_LIN_FWD: p.M = B; p.N = Cout; p.K = Cin; break;
         case GM_LIN_DGRAD: p.M = B; p.N = Cin; p.K = Cout; break;
+        case GM_LIN_WGRAD: p.M = Cout; p.N = Cin; p.K = B; break;
         default: return cudaErrorInvalidValue;
     }
     if (p.M <= 0 || p.N <= 0) return cudaSuccess;
@@ -1230,7 +1250,7 @@ cudaError_t simt_gemm(int mode, const int8_t* act, const int32_t* grad, const in
     // batch of 64 against a linear layer, a 4 x 4 conv map).
     int splits = 1;
     const int64_t tiles = (int64_t)tiles_m * tiles_n;
-    if (mode == GM_CONV_WGRAD || tiles < 2 * 152) {
+    if (mode == GM_CONV_WGRAD || mode == GM_LIN_WGRAD || tiles < 2 * 152) {
         const int64_t want = (4 * 152 + tiles - 1) / tiles;
         const int64_t maxs = (p.K + 255) / 256;
         splits = (int)(want < maxs ? want : maxs);
@@ -1245,15 +1265,16 @@ cudaError_t simt_gemm(int mode, const int8_t* act, const int32_t* grad, const in
         if (p.K == 0) return cudaSuccess;
     }
     dim3 grid(tiles_n, tiles_m, splits);
-    static const int kIds[5] = {K_SIMT_CONV_FWD, K_SIMT_CONV_DGRAD, K_SIMT_CONV_WGRAD,
-                                K_SIMT_LIN_FWD, K_SIMT_LIN_DGRAD};
+    static const int kIds[6] = {K_SIMT_CONV_FWD, K_SIMT_CONV_DGRAD, K_SIMT_CONV_WGRAD,
+                                K_SIMT_LIN_FWD, K_SIMT_LIN_DGRAD, K_SIMT_LIN_WGRAD};
     ProfScope ps(kIds[mode], s, 2.0 * p.M * p.N * p.K, 0.0);
     switch (mode) {
         case GM_CONV_FWD: launch_k(k_gemm<GM_CONV_FWD>, grid, 256, 0, s, p); break;
         case GM_CONV_DGRAD: launch_k(k_gemm<GM_CONV_DGRAD>, grid, 256, 0, s, p); break;
         case GM_CONV_WGRAD: launch_k(k_gemm<GM_CONV_WGRAD>, grid, 256, 0, s, p); break;
         case GM_LIN_FWD: launch_k(k_gemm<GM_LIN_FWD>, grid, 256, 0, s, p); break;
-        default: launch_k(k_gemm<GM_LIN_DGRAD>, grid, 256, 0, s, p); break;
+        case GM_LIN_DGRAD: launch_k(k_gemm<GM_LIN_DGRAD>, grid, 256, 0, s, p); break;
+        default: launch_k(k_gemm<GM_LIN_WGRAD>, grid, 256, 0, s, p); break;
     }
     return cudaGetLastError();
 }
@@ -1394,9 +1415,22 @@ bool simt_lin_wgrad_ok(const LayerGeom& g, int B, bool tc) {
 
 cudaError_t simt_lin_wgrad(const int8_t* a, const int32_t* delta, const LayerGeom& g, int B, int64_t* dw,
                            cudaStream_t s) {
+    if ((int64_t)((B + kLwB - 1) / kLwB * kLwB) * g.cin * g.cout > kLinGemmMacs)
+        return simt_gemm(GM_LIN_WGRAD, a, delta, nullptr, dw, B, 1, 1, g.cin, g.cout, s);
+    // samples shared out until about six CTAs an SM run, from four slabs on (below, the
+    // clear costs what the split gives)
+    const int64_t tiles = (int64_t)((g.cin + 63) / 64) * ((g.cout + 15) / 16);
+    const int slabs = (B + kLwB - 1) / kLwB;
+    int64_t splits = slabs < 4 ? 1 : std::min<int64_t>((152 * 6 + tiles - 1) / tiles, slabs);
+    const int per = (int)((slabs + splits - 1) / splits) * kLwB;
+    splits = (B + per - 1) / per;
+    if (splits > 1) {
+        const cudaError_t e = cudaMemsetAsync(dw, 0, sizeof(int64_t) * (size_t)g.cin * g.cout, s);
+        if (e != cudaSuccess) return e;
+    }
     ProfScope ps(K_SIMT_LIN_WGRAD, s, 2.0 * B * g.cin * (double)g.cout, 0.0);
-    return launch_k(k_lin_wgrad, dim3((unsigned)((g.cin + 63) / 64) * (unsigned)((g.cout + 15) / 16)), 256, 0,
-                    s, a, delta, B, g.cin, g.cout, dw);
+    return launch_k(k_lin_wgrad, dim3((unsigned)tiles, (unsigned)splits), 256, 0, s, a, delta, B, g.cin, g.cout,
+                    per, dw);
 }
 
 cudaError_t simt_grad_to_delta(const DeltaSrc& src, const LayerGeom& g, int B, int alpha_inv,

@@ -227,7 +227,8 @@ enum GemmMode : int {
     GM_CONV_DGRAD = 1,  // C[p][ci]      = sum_(t,co) g[p - tap t][co] * W[co][t][ci]
     GM_CONV_WGRAD = 2,  // C[co][(t,ci)] = sum_p g[p][co] * a[p + tap t][ci]
     GM_LIN_FWD = 3,     // C[b][o] = sum_i a[b][i] * W[o][i]
-    GM_LIN_DGRAD = 4    // C[b][i] = sum_o g[b][o] * W[o][i]
+    GM_LIN_DGRAD = 4,   // C[b][i] = sum_o g[b][o] * W[o][i]
+    GM_LIN_WGRAD = 5    // C[o][i] = sum_b g[b][o] * a[b][i]
 };
 
 // Exact int64 implicit GEMM on CUDA cores.  act: int8 activations, grad:
@@ -292,8 +293,10 @@ struct LossOut {
 };
 
 // Linear layer on the CUDA cores: the whole forward (scaling, NITRO-ReLU, dropout; the
-// limbs of w from *maxabs_w) and the weight gradient (dw overwritten), one launch
-// each.  _ok: the layer has few products, or no tensor-core form (tc false).
+// limbs of w from *maxabs_w), one launch, and the weight gradient (dw overwritten; with
+// many samples or products a clear goes before).  _ok: the layer has few products, or
+// no tensor-core form (tc false; the forward of one with many samples and few inputs is
+// left to simt_gemm and simt_fwd_epilogue).
 bool simt_lin_fwd_ok(const LayerGeom& g, int B, bool tc);
 cudaError_t simt_lin_fwd(const int8_t* a, const int32_t* w, const uint32_t* maxabs_w, const LayerGeom& g,
                          int B, int alpha_inv, int mu, int8_t* act, int8_t* out2, int8_t* region,
