@@ -991,9 +991,10 @@ __global__ void __launch_bounds__(256, 5) k_integersgd(const SgdBatch bt) {
 // ---------------------------------------------------------------------------
 // Learning-layer backward, one launch of three kinds of CTAs that wait on nothing
 // of one another:
-//   dW_lr[g][q] = sum_b grad_L[b][g] a[b][q] for 16 V features, all samples: sixteen
-//     sample lanes with the sums of GM classes in registers, added through shared
-//     memory, written once (no K split, no clearing, no atomics);
+//   dW_lr[g][q] = sum_b grad_L[b][g] a[b][q] for 16 V features: sixteen sample lanes with
+//     the sums of GM classes in registers, added through shared memory, all samples and
+//     written once (no clearing, no atomics), or, at large batches (SHARED), some samples
+//     each and added into a cleared array;
 //   delta_fw[b][q] = sum_g grad_L[b][g] W_lr[g][q] (int32 storage rule) for 16 V features
 //     x 16 samples, routed through max-pool backward and NITRO-ReLU backward into the
 //     last layer's delta, every position written, with the delta's bf16 limb planes
@@ -1032,7 +1033,9 @@ struct LrBackArgs {
     const uint32_t* maxabs_wlr;
     uint32_t* maxabs_delta;
     uint32_t* status;
-    int dw_ctas, delta_x, delta_ctas, tail_ctas;
+    // dW_lr CTAs: dw_x along the features, for each dw_per samples (dw_ctas > dw_x: they add
+    // into a cleared dW_lr)
+    int dw_x, dw_per, dw_ctas, delta_x, delta_ctas, tail_ctas;
 };
 constexpr int kLbSlab = 128;       // samples taken at once: eight a thread
 union LrShared {
@@ -1041,18 +1044,20 @@ union LrShared {
 };
 
 // T int32 where the sums of a thread's samples fit
-template <int V, int GM, typename T>
+template <int V, int GM, typename T, bool SHARED>
 __device__ __forceinline__ void lr_dw(const LrBackArgs& p, LrShared& sm) {
     const int quad = threadIdx.x & 15, lane_s = threadIdx.x >> 4, warp = threadIdx.x >> 5;
-    const int q0 = blockIdx.x * 16 * V, q = q0 + quad * V;
+    const int part = SHARED ? (int)blockIdx.x / p.dw_x : 0;
+    const int b_begin = SHARED ? part * p.dw_per : 0, b_end = SHARED ? min(p.B, b_begin + p.dw_per) : p.B;
+    const int q0 = (SHARED ? blockIdx.x - part * p.dw_x : blockIdx.x) * 16 * V, q = q0 + quad * V;
     for (int gc = 0; gc < p.G; gc += GM) {
         T acc[GM][V];
 #pragma unroll
         for (int g = 0; g < GM; ++g)
 #pragma unroll
             for (int j = 0; j < V; ++j) acc[g][j] = 0;
-        for (int b0 = 0; b0 < p.B; b0 += kLbSlab) {
-            const int nb = min(kLbSlab, p.B - b0);
+        for (int b0 = SHARED ? b_begin : 0; b0 < (SHARED ? b_end : p.B); b0 += kLbSlab) {
+            const int nb = min(kLbSlab, (SHARED ? b_end : p.B) - b0);
             uint32_t aw[kLbSlab / 16];
 #pragma unroll
             for (int i = 0; i < kLbSlab / 16; ++i) {
@@ -1099,7 +1104,11 @@ __device__ __forceinline__ void lr_dw(const LrBackArgs& p, LrShared& sm) {
                 long long t = 0;
 #pragma unroll
                 for (int w = 0; w < 8; ++w) t += sm.red[w][g][f];
-                p.dwlr[(int64_t)(gc + g0 + g) * p.d + q0 + f] = t;
+                if constexpr (SHARED)
+                    atomicAdd(reinterpret_cast<unsigned long long*>(p.dwlr + (int64_t)(gc + g0 + g) * p.d + q0 + f),
+                              (unsigned long long)t);
+                else
+                    p.dwlr[(int64_t)(gc + g0 + g) * p.d + q0 + f] = t;
             }
         }
     }
@@ -1203,14 +1212,16 @@ __device__ __forceinline__ void lr_delta(const LrBackArgs& p, int cta, uint64_t 
     block_maximum(mx, ovf, p.maxabs_delta, p.status);
 }
 
-template <int V>
+template <int V, bool SHARED>
 __global__ void __launch_bounds__(256, 4) k_lr_backward(const LrBackArgs p, const LossTail tail) {
     __shared__ LrShared sm;
     pdl_wait();
     const int cta = blockIdx.x;
     if (cta < p.dw_ctas) {
-        if ((uint64_t)*p.gl_bound * 128u * (uint64_t)((p.B + 15) / 16) <= 0x7fffffffull) lr_dw<V, 10, int32_t>(p, sm);
-        else lr_dw<V, 4, long long>(p, sm);
+        if ((uint64_t)*p.gl_bound * 128u * (uint64_t)(((SHARED ? p.dw_per : p.B) + 15) / 16) <= 0x7fffffffull)
+            lr_dw<V, 10, int32_t, SHARED>(p, sm);
+        else
+            lr_dw<V, 4, long long, SHARED>(p, sm);
     } else if (cta < p.dw_ctas + p.delta_ctas) {
         const uint32_t gb = *p.gl_bound;
         const uint64_t bound = (uint64_t)gb * *p.maxabs_wlr;
@@ -1508,15 +1519,34 @@ cudaError_t simt_lr_backward(const int8_t* a, const int32_t* gl, const uint32_t*
     }
     p.status = status;
     const int tile = quad ? 64 : 16;
-    p.dw_ctas = (d + tile - 1) / tile;
-    p.delta_x = p.dw_ctas;
+    p.delta_x = p.dw_x = (d + tile - 1) / tile;
+    const int slabs = (B + kLbSlab - 1) / kLbSlab;
+    // Samples shared out until eight CTAs an SM form dW_lr, where a slab after another (1.7
+    // us each and ten classes) would outlast the rest: few CTAs along the features, none
+    // or few of the delta part beside them.  Us a backward, shared out and not: 64 features,
+    // 47 classes 33 and 318 at batch 4096; 1024 features 11.2 and 15.3 at 512, 21 and 78 at
+    // 4096; 16384 features 30 and 27 at 512, 136 and 150 at 4096; a conv of 64 x 16 x 16,
+    // pooled, under the learning layer 64.7 and 62.6 at 512.
+    const int few = dl ? 32 : 152 * ((G + 9) / 10);
+    const bool share = slabs >= (quad ? 4 : 6) && (p.dw_x < few || (!dl && slabs >= 32));
+    int splits = share ? std::min((152 * 8 + p.dw_x - 1) / p.dw_x, slabs) : 1;
+    p.dw_per = (slabs + splits - 1) / splits * kLbSlab;
+    splits = (B + p.dw_per - 1) / p.dw_per;
+    p.dw_ctas = p.dw_x * splits;
+    if (splits > 1) {
+        const cudaError_t e = cudaMemsetAsync(dwlr, 0, sizeof(int64_t) * (size_t)G * d, s);
+        if (e != cudaSuccess) return e;
+    }
     p.delta_ctas = dl ? p.delta_x * ((B + 15) / 16) : 0;
     p.tail_ctas = (int)(((int64_t)B * G + kTailValues - 1) / kTailValues);
     const int grid = p.dw_ctas + p.delta_ctas + p.tail_ctas;
     const LossTail tail{gl, B, G, lo.sse, lo.loss, lo.maxabs_gl, lo.ticket, lo.wlr_max, lo.status};
     ProfScope ps(K_LR_BACKWARD, s, (dl ? 4.0 : 2.0) * B * d * G, 0.0);
-    return quad ? launch_k(k_lr_backward<4>, grid, 256, 0, s, p, tail)
-                : launch_k(k_lr_backward<1>, grid, 256, 0, s, p, tail);
+    if (splits > 1)
+        return quad ? launch_k(k_lr_backward<4, true>, grid, 256, 0, s, p, tail)
+                    : launch_k(k_lr_backward<1, true>, grid, 256, 0, s, p, tail);
+    return quad ? launch_k(k_lr_backward<4, false>, grid, 256, 0, s, p, tail)
+                : launch_k(k_lr_backward<1, false>, grid, 256, 0, s, p, tail);
 }
 
 }  // namespace nitro
