@@ -248,6 +248,16 @@ constexpr int64_t kLinFwdMacs = (int64_t)48 << 20, kLinWgradMacs = (int64_t)32 <
 // to whole slabs): backward of a 1001 -> 999 layer at batch 192 57 us here, 60 there, at
 // 512 134 and 114, at 1024 263 and 203.
 constexpr int64_t kLinGemmMacs = (int64_t)192 << 20;
+// CTAs (16 outputs x 8 samples each) up to which the forward of a linear layer takes
+// k_lin_fwd.  Against the tensor cores, us: 128 x 128 at 512 CTAs 6.1 and 8.8, at 1024 10.6
+// and 8.7; 256 x 256 6.2 and 9.1, 10.8 and 9.4; 504 x 333 at 672 10.3 and 13.8.  Against the
+// general GEMM (no tensor-core form) the line rises with the inputs a CTA sums: 16 of
+// them at 256 CTAs 3.9 and 5.7, at 512 6.1 and 5.7; 60 at 1024 12.2 and 12.7, at 2048 21.4
+// and 14.2; 250 at 5376 57 and 64, at 10752 109 and 90; 1001 at 16128 394 and 392, at 32256
+// 761 and 658.
+// A cluster of eight shares the inputs; the tensor-core GEMM shares a long K wider: one
+// sample, 191 outputs, 50176 inputs 13 and 17 us, 111888 inputs 26 and 23.
+constexpr int64_t kLinFwdCtas = 896, kLinFwdCtasMin = 448, kLinFwdCtasPerIn = 24, kLinFwdIn = 65536;
 
 struct LearnArgs {
     const int8_t* a;
@@ -1401,7 +1411,11 @@ cudaError_t simt_learn_fwd(const int8_t* a, const int32_t* wlr, const int32_t* l
 }
 
 bool simt_lin_fwd_ok(const LayerGeom& g, int B, bool tc) {
-    return g.kind == NITRO_LINEAR && (!tc || (int64_t)B * g.cin * g.cout <= kLinFwdMacs);
+    // CTAs before the features are shared out over clusters
+    const int64_t ctas = (int64_t)((B + kLfSamples - 1) / kLfSamples) * ((g.cout + kLfG - 1) / kLfG);
+    if (g.kind != NITRO_LINEAR) return false;
+    return tc ? (int64_t)B * g.cin * g.cout <= kLinFwdMacs && ctas <= kLinFwdCtas && g.cin <= kLinFwdIn
+              : ctas <= std::max<int64_t>(kLinFwdCtasMin, kLinFwdCtasPerIn * g.cin);
 }
 
 cudaError_t simt_lin_fwd(const int8_t* a, const int32_t* w, const uint32_t* maxabs_w, const LayerGeom& g,

@@ -390,7 +390,8 @@ nitro_status nitro_block_forward(nitro_block* b, const int8_t* a_in, int batch, 
             done = true;
         }
         if (!done)
-            NITRO_TRY(simt_gemm(GM_CONV_FWD, x, nullptr, ly.W, b->z64, batch, g.h, g.w, g.cin, g.cout, s));
+            NITRO_TRY(simt_gemm(g.kind == NITRO_CONV3X3 ? GM_CONV_FWD : GM_LIN_FWD, x, nullptr, ly.W, b->z64, batch,
+                                g.h, g.w, g.cin, g.cout, s));
         if (!fused) {
             NITRO_TRY(simt_fwd_epilogue(b->z64, g, batch, b->desc.alpha_inv, b->mu, ly.act, out2,
                                         ly.region, ly.argmax, s, drop));
