@@ -250,7 +250,7 @@ struct TcArgs {
     int64_t* out;
     uint32_t* status;
     int atomic_out;
-    int out_vec;           // int64 rows are 32-byte aligned: four values a store
+    int out_vec;           // int64 values a store: 4 (rows 32-byte aligned), 2 (16) or 1
     int ksplit;            // fused forward: CTAs of a cluster that share a tile's K (1: none)
     // forward with fused NITRO-Scaling / NITRO-ReLU / max-pool epilogue
     FloorDiv alpha;        // divide by alpha_inv
@@ -1083,7 +1083,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const int m = T.mt * kBM + r;      // C[m][n], M rows in args.B
                     if (m < args.B) {
                         int64_t* o = args.out + (int64_t)m * args.ncols + col0;
-                        if (args.out_vec && !args.atomic_out && col0 + NH <= args.ncols) {
+                        if (args.out_vec == 4 && !args.atomic_out && col0 + NH <= args.ncols) {
 #pragma unroll
                             for (int i = 0; i < NH; i += 4) st_i64x4(o + i, acc + i);
                         } else {
@@ -1327,9 +1327,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const int x = tx * args.wb + xx, y = ty * args.hb + yy, b = tb * args.bb + bbx;
                     if (x < args.W && y < args.H && b < args.B) {
                         int64_t* o = args.out + (((int64_t)b * args.H + y) * args.W + x) * args.ncols + col0;
-                        if (args.out_vec && col0 + NH <= args.ncols) {
+                        if (args.out_vec == 4 && col0 + NH <= args.ncols) {
 #pragma unroll
                             for (int i = 0; i < NH; i += 4) st_i64x4(o + i, acc + i);
+                        } else if (args.out_vec == 2 && col0 + NH <= args.ncols) {
+#pragma unroll
+                            for (int i = 0; i < NH; i += 2)
+                                *reinterpret_cast<ulonglong2*>(o + i) = make_ulonglong2(acc[i], acc[i + 1]);
                         } else {
 #pragma unroll
                             for (int i = 0; i < NH; ++i)
@@ -1750,6 +1754,12 @@ cudaError_t launch_gemm_pb(int n, int pb, const CUtensorMap& a, const CUtensorMa
 
 int pick_n(int cols) { return cols % 128 == 0 ? 128 : 64; }
 
+// int64 values a store where every row of `cols` starts aligned for it
+int out_width(const void* out, int cols) {
+    const uintptr_t low = (uintptr_t)out | (uintptr_t)(8 * cols);
+    return (low & 31) == 0 ? 4 : ((low & 15) == 0 ? 2 : 1);
+}
+
 void pixel_tiling(const LayerGeom& g, int batch, TcArgs& a) {
     if (g.w > 8) { a.wb = 16; a.hb = 8; a.bb = 1; }
     else if (g.w > 4 || g.h > 4) { a.wb = 8; a.hb = 8; a.bb = 2; }
@@ -2083,7 +2093,7 @@ cudaError_t tc_conv_forward(TcLayer& t, const LayerGeom& g, int batch, int64_t* 
     a.max_a = nullptr;
     a.max_b = t.maxabs_w;
     a.out = z;
-    a.out_vec = ((uintptr_t)z & 31) == 0 && g.cout % 4 == 0;
+    a.out_vec = out_width(z, g.cout);
     a.status = status;
     a.atomic_out = 0;
     if (fuse) {
@@ -2252,7 +2262,7 @@ cudaError_t tc_conv_dgrad(TcLayer& t, const LayerGeom& g, int batch, int64_t* g6
     a.max_a = t.maxabs_d;
     a.max_b = t.maxabs_w;
     a.out = g64;
-    a.out_vec = ((uintptr_t)g64 & 31) == 0 && g.cin % 4 == 0;
+    a.out_vec = out_width(g64, g.cin);
     a.status = status;
     a.atomic_out = 0;
     const bool fuse = fo && g.cin % 16 == 0;
@@ -2404,7 +2414,7 @@ cudaError_t tc_gemm_run(const uint16_t* a_bf16, const uint16_t* b_planes, int M,
     a.max_a = nullptr;
     a.max_b = max_b;
     a.out = out;
-    a.out_vec = ((uintptr_t)out & 31) == 0 && N % 4 == 0;
+    a.out_vec = out_width(out, N);
     a.status = status;
     CUtensorMap ma, mb;
     const uint64_t da[2] = {(uint64_t)K, (uint64_t)M};
