@@ -55,6 +55,8 @@ nitro_status latched(uint32_t bits) {
     return NITRO_OK;
 }
 
+constexpr int64_t kFewMacs = (int64_t)64 << 20;   // see nitro_conv3x3_contract
+
 #define TRY(expr)                                      \
     do {                                               \
         if ((expr) != cudaSuccess) return NITRO_ERR_CUDA; \
@@ -107,26 +109,38 @@ nitro_status nitro_conv3x3_contract(nitro_conv* c, int mode, const void* x, cons
         return NITRO_OK;
     }
     bool done = false, fused = false;
+    // With eight channels to sum over on a small map the maxima, the packs and padded tiles
+    // cost more than the products: the one launch of the CUDA-core GEMM.  Us there and
+    // here: forward 8 -> 32 at 30 x 1, batch 256, 20 and 38; input gradient 8 -> 8 at 20 x 1,
+    // batch 60, 25 and 52, 72 -> 8 at 5 x 4, batch 95, 39 and 50.
+    // (225 x 7 x 29, 8 -> 24, 79 M products, forward 53 and 39.)
+    const bool few = (g.h < 8 || g.w < 8) && (int64_t)batch * g.h * g.w * g.cin * g.cout * 9 < kFewMacs;
     if (mode == NITRO_CONTRACT_FWD) {
         const int8_t* a = static_cast<const int8_t*>(x);
-        TRY(tc_maxabs(y, (int64_t)g.cout * 9 * g.cin, c->words, c->words + 4, s));
-        TRY(tc_refresh_weights(c->t, g, y, c->words, s));
-        TRY(tc_pack_input(c->t, g, a, batch, false, s));
-        TRY(tc_conv_forward(c->t, g, batch, out, nullptr, status, s, &done, &fused));
+        if (c->t.fwd && !(few && g.cin <= 8)) {
+            TRY(tc_maxabs(y, (int64_t)g.cout * 9 * g.cin, c->words, c->words + 4, s));
+            TRY(tc_refresh_weights(c->t, g, y, c->words, s));
+            TRY(tc_pack_input(c->t, g, a, batch, false, s));
+            TRY(tc_conv_forward(c->t, g, batch, out, nullptr, status, s, &done, &fused));
+        }
         if (!done) TRY(simt_gemm(GM_CONV_FWD, a, nullptr, y, out, batch, g.h, g.w, g.cin, g.cout, s));
     } else if (mode == NITRO_CONTRACT_WGRAD) {
         const int8_t* a = static_cast<const int8_t*>(x);
-        TRY(tc_pack_input(c->t, g, a, batch, false, s));
-        TRY(tc_maxabs(y, (int64_t)batch * g.h * g.w * g.cout, c->words + 1, c->words + 4, s));
-        TRY(tc_conv_wgrad(c->t, g, y, c->words + 1, batch, out, status, s, &done));
+        if (c->t.wgrad) {
+            TRY(tc_pack_input(c->t, g, a, batch, false, s));
+            TRY(tc_maxabs(y, (int64_t)batch * g.h * g.w * g.cout, c->words + 1, c->words + 4, s));
+            TRY(tc_conv_wgrad(c->t, g, y, c->words + 1, batch, out, status, s, &done));
+        }
         if (!done) TRY(simt_gemm(GM_CONV_WGRAD, a, y, nullptr, out, batch, g.h, g.w, g.cin, g.cout, s));
     } else {
         const int32_t* d = static_cast<const int32_t*>(x);
-        TRY(tc_maxabs(y, (int64_t)g.cout * 9 * g.cin, c->words, c->words + 4, s));
-        TRY(tc_refresh_weights(c->t, g, y, c->words, s));
-        TRY(tc_maxabs(d, (int64_t)batch * g.h * g.w * g.cout, c->words + 1, c->words + 4, s));
-        TRY(tc_pack_delta(c->t, g, d, c->words + 1, batch, s));
-        TRY(tc_conv_dgrad(c->t, g, batch, out, nullptr, status, s, &done, &fused));
+        if (c->t.dgrad && !(few && g.cout <= 8)) {
+            TRY(tc_maxabs(y, (int64_t)g.cout * 9 * g.cin, c->words, c->words + 4, s));
+            TRY(tc_refresh_weights(c->t, g, y, c->words, s));
+            TRY(tc_maxabs(d, (int64_t)batch * g.h * g.w * g.cout, c->words + 1, c->words + 4, s));
+            TRY(tc_pack_delta(c->t, g, d, c->words + 1, batch, s));
+            TRY(tc_conv_dgrad(c->t, g, batch, out, nullptr, status, s, &done, &fused));
+        }
         if (!done) TRY(simt_gemm(GM_CONV_DGRAD, nullptr, d, y, out, batch, g.h, g.w, g.cin, g.cout, s));
     }
     return NITRO_OK;
