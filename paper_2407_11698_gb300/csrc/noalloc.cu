@@ -29,10 +29,12 @@ constexpr int64_t kNoallocScratchElems = (int64_t)1 << 21;   // int64 values
 
 // Products from which a layer with 9 Cin <= 64 runs on the tensor cores, as three
 // launches (12.7 us, host bound) instead of two: 1 x 28 x 28, 1 -> 32 channels (0.2 M
-// products) takes 13.1 us there and 10.0 us on the CUDA cores, 16 x 28 x 28, 3 -> 64
-// (22 M) 12.9 and 21.4 us.  Layers with more channels always do: 1 x 8 x 8, 16 -> 16
-// (0.15 M) 12.7 against 26.1 us, 8 x 16 x 16, 64 -> 64 13.1 against 41.2 us.
-constexpr int64_t kNoallocTcMacs = (int64_t)1 << 21;
+// products) takes 13.1 us there and 10.0 us on the CUDA cores, 121 x 12 x 4, 2 -> 24 (2.5 M)
+// 12.5 and 10.7 us, 16 x 28 x 28, 3 -> 64 (22 M) 12.9 and 21.4 us.  Layers with more channels
+// do unless the map is a line that fills an eighth of a tile with a quarter of its channels:
+// 1 x 8 x 8, 16 -> 16 (0.15 M) 12.7 against 26.1 us, 8 x 16 x 16, 64 -> 64 13.1 against 41.2 us,
+// but 64 x 1 x 62, 12 -> 240 62 against 43 us.
+constexpr int64_t kNoallocTcMacs = (int64_t)1 << 22;
 
 static __device__ __align__(256) int64_t g_noalloc_scratch[kNoallocScratchElems];
 static __device__ uint32_t g_noalloc_words[4];     // see tc_fwd_in_scratch
@@ -94,7 +96,7 @@ extern "C" nitro_status nitro_conv3x3_forward_noalloc(
     const size_t need = tc_fwd_scratch(g, batch);
     const uintptr_t low = (uintptr_t)a_out | (uintptr_t)region | (pool2x2 ? (uintptr_t)argmax : 0);
     if (need && need <= sizeof(int64_t) * (size_t)kNoallocScratchElems && (low & 7) == 0 &&
-        (9 * cin > 64 || elems * 9 * cin >= kNoallocTcMacs)) {
+        (9 * cin > 64 ? cin >= 16 || (h > 1 && w > 1) : elems * 9 * cin >= kNoallocTcMacs)) {
         const TcFwdOut fo{alpha_inv, mu, a_out, nullptr, region, pool2x2 ? argmax : nullptr, nullptr};
         return tc_fwd_in_scratch(g, batch, a_in, weights, fo, z, sc.words, s) == cudaSuccess ? NITRO_OK
                                                                                             : NITRO_ERR_CUDA;

@@ -79,3 +79,10 @@ def test_noalloc_matches_oracle(shape):
             got = got.cpu().numpy()
             assert np.array_equal(got[off:off + k], want.reshape(-1))
             assert (got[:off] == 99).all() and (got[off + k:] == 99).all()
+
+
+# lines of pixels below and at 16 channels, few channels above the earlier line for narrow inputs
+@pytest.mark.parametrize("shape", [(3, 1, 62, 12, 40, 0, 0), (3, 1, 62, 16, 40, 0, 0), (2, 9, 1, 8, 16, 0, 0),
+                                   (121, 12, 4, 2, 24, 0, 0)])
+def test_noalloc_lines_match_oracle(shape):
+    test_noalloc_matches_oracle(shape)
