@@ -64,6 +64,29 @@ def test_fit_matches_oracle(n, off, kinds):
         p.close()
 
 
+# byte by byte where the offsets differ, and in two rounds of CTAs from 128 MB on
+@pytest.mark.parametrize("n,xoff,ooff", [(3000001, 0, 3), (3000001, 5, 0), (200000, 1, 2), ((1 << 27) + 19, 0, 0),
+                                         ((1 << 27) + 19, 7, 7)])
+def test_map_matches_table(n, xoff, ooff):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    p = nb.IntPrep()
+    try:
+        x = data("natural", n, xoff)
+        buf = torch.zeros(n + 16, dtype=torch.uint8, device="cuda")
+        xd = buf[xoff:xoff + n]
+        xd.copy_(torch.from_numpy(x))
+        out = torch.full((n + 16,), 99, dtype=torch.int8, device="cuda")
+        p.fit(xd)
+        p.apply(xd, out[ooff:ooff + n])
+        lut = O.prep_apply(np.arange(256, dtype=np.uint8), *O.prep_stats(x)).astype(np.int8)
+        got = out.cpu().numpy()
+        assert np.array_equal(got[ooff:ooff + n], lut[x])
+        assert (got[:ooff] == 99).all() and (got[ooff + n:] == 99).all()
+    finally:
+        p.close()
+
+
 def test_profile_counts_the_bytes_that_a_fit_reads():
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
