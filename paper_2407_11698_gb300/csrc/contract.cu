@@ -16,6 +16,7 @@ struct nitro_conv {
     TcLayer t;
     int max_batch = 0;
     uint32_t* words = nullptr;   // [0] max|W| [1] max|delta| [2] status [4, 5] tc_maxabs scratch
+    bool clean = false;          // see clear_once
     std::vector<void*> allocs;
     std::vector<void*> host_allocs;
 };
@@ -25,6 +26,7 @@ struct nitro_gemm {
     uint16_t* a = nullptr;       // bf16 [M][K]
     uint16_t* b = nullptr;       // bf16 limb planes [4][N][K]
     uint32_t* words = nullptr;   // [0] max|B| [1] status [2, 3] tc_maxabs scratch
+    bool clean = false;          // see clear_once
     std::vector<void*> allocs;
 };
 
@@ -78,12 +80,12 @@ nitro_status nitro_conv3x3_create(int max_batch, int h, int w, int cin, int cout
     if (!c) return NITRO_ERR_CUDA;
     c->g = LayerGeom{NITRO_CONV3X3, cin, cout, h, w, 0, h, w};
     c->max_batch = max_batch;
-    bool ok = dalloc(c->allocs, &c->words, 6);
-    ok = ok && on_own_stream([&](cudaStream_t s) {
-        if (!tc_layer_init(c->t, c->g, max_batch, true, c->words, c->words + 1, c->allocs, c->host_allocs, s))
-            return cudaErrorMemoryAllocation;
-        return cudaMemsetAsync(c->words, 0, 24, s);
-    }) == cudaSuccess;
+    // the status word is latched from here on; what the kernels sum into is cleared by the
+    // first call
+    bool ok = dalloc(c->allocs, &c->words, 6) &&
+              tc_layer_init(c->t, c->g, max_batch, true, c->words, c->words + 1, c->allocs,
+                            c->host_allocs) &&
+              cudaMemset(c->words + 2, 0, 4) == cudaSuccess;
     if (!ok) {
         free_all(c->allocs);
         free_host(c->host_allocs);
@@ -107,6 +109,10 @@ nitro_status nitro_conv3x3_contract(nitro_conv* c, int mode, const void* x, cons
         if (mode == NITRO_CONTRACT_WGRAD)
             TRY(cudaMemsetAsync(out, 0, sizeof(int64_t) * 9 * g.cin * g.cout, s));
         return NITRO_OK;
+    }
+    if (!c->clean) {
+        TRY(tc_clear_planes(c->t, g, s));
+        TRY(clear_once(c->clean, c->words + 4, 8, s));
     }
     bool done = false, fused = false;
     // With eight channels to sum over on a small map the maxima, the packs and padded tiles
@@ -177,8 +183,7 @@ nitro_status nitro_gemm_create(int max_m, int max_n, int max_k, nitro_gemm** out
     g->max_k = max_k;
     bool ok = dalloc(g->allocs, &g->a, (size_t)max_m * max_k) &&
               dalloc(g->allocs, &g->b, (size_t)kMaxLimbs * max_n * max_k) &&
-              dalloc(g->allocs, &g->words, 4);
-    ok = ok && on_own_stream([&](cudaStream_t s) { return cudaMemsetAsync(g->words, 0, 16, s); }) == cudaSuccess;
+              dalloc(g->allocs, &g->words, 4) && cudaMemset(g->words + 1, 0, 4) == cudaSuccess;
     if (!ok) {
         free_all(g->allocs);
         delete g;
@@ -204,6 +209,7 @@ nitro_status nitro_gemm_run(nitro_gemm* g, const int8_t* a, const int32_t* b, in
         TRY(simt_gemm(GM_LIN_FWD, a, nullptr, b, c, m, 1, 1, k, n, s));
         return NITRO_OK;
     }
+    TRY(clear_once(g->clean, g->words + 2, 8, s));
     TRY(tc_pack_int8(a, m, k, g->a, s, tc_gemm_adds(m, n, k) ? c : nullptr, (int64_t)m * n));
     TRY(tc_maxabs(b, (int64_t)n * k, g->words, g->words + 2, s));
     TRY(tc_pack_limbs(b, (int64_t)n * k, g->words, g->b, s));

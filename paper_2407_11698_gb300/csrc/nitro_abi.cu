@@ -291,13 +291,12 @@ nitro_status nitro_init_block(const nitro_block_desc* desc, uint64_t seed, void*
         ok = ly.lin_a ? tc_linear_init(ly.tc, ly.g, desc->max_batch, ly.lin_a, ly.lin_planes, w_w(b, i),
                                        w_delta(b, i), b->allocs, b->host_allocs)
                       : tc_layer_init(ly.tc, ly.g, desc->max_batch, i > 0, w_w(b, i), w_delta(b, i),
-                                      b->allocs, b->host_allocs, s);
+                                      b->allocs, b->host_allocs);
         // one copy of all the block's words per step refreshes the layers' hints
         if (ok) tc_use_external_hints(ly.tc, b->words_host + 3 + i,
                                       b->words_host + 4 + desc->n_layers + i);
     }
     if (!ok) {
-        cudaStreamSynchronize(s);      // layers made before the one that failed queued their clears
         free_all(b);
         delete b;
         return NITRO_ERR_CUDA;
@@ -317,7 +316,8 @@ nitro_status nitro_init_block(const nitro_block_desc* desc, uint64_t seed, void*
     if (e == cudaSuccess) e = cudaMemsetAsync(b->sse, 0, 8, s);
     for (int i = 0; e == cudaSuccess && i < desc->n_layers; ++i) {
         // all four limb planes: IntegerSGD stores only what changes in them
-        e = tc_refresh_weights(b->L[i].tc, b->L[i].g, b->L[i].W, w_w(b, i), s, true);
+        if (!b->L[i].lin_planes) e = tc_clear_planes(b->L[i].tc, b->L[i].g, s);
+        if (e == cudaSuccess) e = tc_refresh_weights(b->L[i].tc, b->L[i].g, b->L[i].W, w_w(b, i), s, true);
         if (e == cudaSuccess && b->L[i].lin_planes)
             e = tc_pack_limbs(b->L[i].W, b->L[i].wcount, nullptr, b->L[i].lin_planes, s);
     }

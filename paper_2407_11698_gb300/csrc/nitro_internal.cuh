@@ -397,18 +397,18 @@ inline cudaError_t once_per_device(std::atomic<uint64_t>& done, int dev, F&& f) 
     return e;
 }
 
-// Runs f(s) on a stream of its own and waits for it: what a handle's creation clears is
-// then cleared when the call returns.  (A plain cudaMemset queues on the default stream
-// and may still be waiting there when the handle is used on another one.)
-template <typename F>
-inline cudaError_t on_own_stream(F&& f) {
-    cudaStream_t s = nullptr;
-    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
-    if (e != cudaSuccess) return e;
-    e = f(s);
-    const cudaError_t q = cudaStreamSynchronize(s);
-    cudaStreamDestroy(s);
-    return e != cudaSuccess ? e : q;
+// Clears n bytes on s the first time that a handle runs; its kernels keep them clean from
+// then on.  (A clear at creation would queue on the default stream, and could still be
+// waiting there when the handle is used on another; a stream of its own to wait for
+// costs 50 us a handle.)  A captured call holds the clear too and does not count as the
+// first: its graph need not have run before the next call.
+inline cudaError_t clear_once(bool& clean, void* p, size_t n, cudaStream_t s) {
+    if (clean) return cudaSuccess;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s, &capture);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, n, s);
+    if (e == cudaSuccess && capture == cudaStreamCaptureStatusNone) clean = true;
+    return e;
 }
 
 // ---------------------------------------------------------------------------

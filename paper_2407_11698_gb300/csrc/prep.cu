@@ -309,7 +309,7 @@ constexpr int64_t kPrepMaxN = (int64_t)1 << 48;   // 255 n stays far inside uint
 struct nitro_prep {
     PrepState* st = nullptr;
     int sms = 0;
-    bool fitted = false;
+    bool fitted = false, clean = false;    // clean: see clear_once
 };
 
 extern "C" {
@@ -322,9 +322,7 @@ nitro_status nitro_prep_create(nitro_prep** out) {
     int dev = 0;
     bool ok = cudaGetDevice(&dev) == cudaSuccess &&
               cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-              cudaMalloc(&p->st, sizeof(PrepState) + (size_t)p->sms * kCtasPerSm * 32) == cudaSuccess &&
-              on_own_stream([&](cudaStream_t s) { return cudaMemsetAsync(p->st, 0, sizeof(PrepState), s); }) ==
-                  cudaSuccess;
+              cudaMalloc(&p->st, sizeof(PrepState) + (size_t)p->sms * kCtasPerSm * 32) == cudaSuccess;
     if (!ok) {
         if (p->st) cudaFree(p->st);
         delete p;
@@ -338,6 +336,7 @@ nitro_status nitro_prep_fit(nitro_prep* p, const uint8_t* x, int64_t n, void* st
     if (!p || !x || n < 1 || n > kPrepMaxN) return NITRO_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int grid = grid_for_bytes(n, p->sms);
+    if (clear_once(p->clean, p->st, sizeof(PrepState), s) != cudaSuccess) return NITRO_ERR_CUDA;
     if (n >= kOnePassBytes) {
         ProfScope ps(K_PREP_SUM, s, 0.0, (double)n + 16.0 * kSamples);
         const uint8_t* body = x + ((16 - ((uintptr_t)x & 15)) & 15);

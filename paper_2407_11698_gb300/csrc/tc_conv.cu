@@ -1909,7 +1909,7 @@ cudaError_t tc_fwd_preload() {
 
 bool tc_layer_init(TcLayer& t, const LayerGeom& g, int max_batch, bool has_dgrad,
                    const uint32_t* maxabs_w, const uint32_t* maxabs_d,
-                   std::vector<void*>& allocs, std::vector<void*>& host_allocs, cudaStream_t s) {
+                   std::vector<void*>& allocs, std::vector<void*>& host_allocs) {
     t = TcLayer();
     t.maxabs_w = maxabs_w;
     t.maxabs_d = maxabs_d;
@@ -1931,8 +1931,13 @@ bool tc_layer_init(TcLayer& t, const LayerGeom& g, int max_batch, bool has_dgrad
             t.max_host[0] = t.max_host[1] = 0;
         }
     }
-    if (ok && t.w_planes) ok = cudaMemsetAsync(t.w_planes, 0, (size_t)kMaxLimbs * nwk * 2, s) == cudaSuccess;
     return ok;
+}
+
+cudaError_t tc_clear_planes(const TcLayer& t, const LayerGeom& g, cudaStream_t s) {
+    if (!t.w_planes) return cudaSuccess;
+    const size_t nwk = (size_t)g.cout * (t.im2col ? kBK : 9 * t.cin_k);
+    return cudaMemsetAsync(t.w_planes, 0, (size_t)kMaxLimbs * nwk * 2, s);
 }
 
 bool tc_linear_init(TcLayer& t, const LayerGeom& g, int max_batch, uint16_t* act_bf16, uint16_t* planes,

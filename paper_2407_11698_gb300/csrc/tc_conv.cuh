@@ -94,10 +94,13 @@ bool tc_linear_init(TcLayer& t, const LayerGeom& g, int max_batch, uint16_t* act
 // buffers (device memory recorded in `allocs`, pinned host memory in
 // `host_allocs`).  `has_dgrad`: the layer is not the block's first, so its
 // input gradient is needed.  maxabs_w / maxabs_d: device words that will hold
-// max |W| and max |delta| of the layer.  The weight planes are cleared on s.
+// max |W| and max |delta| of the layer.
 bool tc_layer_init(TcLayer& t, const LayerGeom& g, int max_batch, bool has_dgrad,
                    const uint32_t* maxabs_w, const uint32_t* maxabs_d,
-                   std::vector<void*>& allocs, std::vector<void*>& host_allocs, cudaStream_t s);
+                   std::vector<void*>& allocs, std::vector<void*>& host_allocs);
+
+// Clears the weight planes (their padding stays zero): before the first tc_refresh_weights.
+cudaError_t tc_clear_planes(const TcLayer& t, const LayerGeom& g, cudaStream_t s);
 
 // Where IntegerSGD writes the layer's weight planes when it splits the updated
 // weights itself: planes [4][Cout][row_k], plane stride, entry (t, ci) of row

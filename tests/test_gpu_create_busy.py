@@ -1,6 +1,6 @@
 """Handles made while the default stream is busy, and used at once on another stream:
-what the calls that make them clear must be cleared when they return, not when the
-default stream gets to it."""
+what their kernels sum into must be clean then, not when the default stream gets to
+it; and a handle whose first call is captured."""
 import numpy as np
 import pytest
 
@@ -100,3 +100,25 @@ def test_gemm(side):
     finally:
         torch.cuda.synchronize()
         g.close()
+
+
+def test_first_call_captured(side):
+    # a graph captured before any eager call, launched after one: both start from clean sums
+    x = torch.randint(0, 256, (100003,), dtype=torch.uint8, device="cuda")
+    y = torch.randint(0, 40, (5000,), dtype=torch.uint8, device="cuda")
+    p = nb.IntPrep()
+    try:
+        side.wait_stream(torch.cuda.current_stream())
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.stream(side):
+            with torch.cuda.graph(graph, stream=side):
+                p.fit(x, stream=side)
+        p.fit(y)
+        assert p.stats() == O.prep_stats(y.cpu().numpy())
+        for _ in range(2):
+            graph.replay()
+            assert p.stats() == O.prep_stats(x.cpu().numpy())
+        p.fit(y)
+        assert p.stats() == O.prep_stats(y.cpu().numpy())
+    finally:
+        p.close()
